@@ -92,6 +92,8 @@ __global__ void __launch_bounds__(kBlock, (MODE == kBwdStore && !DC) ? GABM_BWD_
     const int32_t *sg = nullptr;   // scale exponents of the current graph
     int sig_t = 0;                 // sigma(t) of the current graph
     unsigned emax_w = 0u;          // largest exponent stored by this warp (+128)
+    bool rnz_w = false;            // this lane stored an r other than 0
+    unsigned live_k = 0u;          // bit k: day t + k carries adjoint (its gx is not all 0)
     float gtail = 0.f;             // m_{t+L} gD_{t+L} at day t's scale
     const bool has_next = (t + 1 < T);
     const int16_t *E = a.E;
@@ -128,8 +130,11 @@ __global__ void __launch_bounds__(kBlock, (MODE == kBwdStore && !DC) ? GABM_BWD_
                 const int sN = __reduce_add_sync(0xffffffffu, cN);
                 if (lane == 0 && sN) atomicAdd(a.newRM + (size_t)cur_g * a.ldP + t, sN);
                 flush_emax(a.emax + (size_t)cur_g * a.ld_sig + t, emax_w);
+                flush_rnz(a.rnz + (size_t)cur_g * a.ld_sig + t, rnz_w);
                 emax_w = 0u;
+                rnz_w = false;
             }
+            live_k = carries_adjoint(a.rnz + (size_t)g * a.ld_sig, t, T, L);
             // this day's scale for graph g (every warp computes the same value; the warp
             // holding the graph's first tile records it)
             sg = a.sig + (size_t)g * a.ld_sig;
@@ -155,7 +160,8 @@ __global__ void __launch_bounds__(kBlock, (MODE == kBwdStore && !DC) ? GABM_BWD_
         // soft relaxation: every agent carries susceptible mass and draws every day
         const bool isS = SOFT ? agent : live && (never || Ei >= t);
         // R/M split: rows exposed before day 0 keep gx while day t+1 is inside their window
-        const bool needA = has_next && (SOFT ? agent : (live && (never || Ei >= t + 2 - L)) ||
+        const bool gather = (live_k & 2u) != 0u;   // else gx(t+1) = 0 for every row
+        const bool needA = gather && (SOFT ? agent : (live && (never || Ei >= t + 2 - L)) ||
                                                        (FATE && agent && !never && Ei < 0 && t + 1 - Ei < L));
         if constexpr (DUR) {
             // exits at the row's drawn L_i (its first possible day is tau_EI + 1)
@@ -168,7 +174,7 @@ __global__ void __launch_bounds__(kBlock, (MODE == kBwdStore && !DC) ? GABM_BWD_
         // table adjoint: rows infectious on day t+1 (k = t+1-E in [1, L-1]) add gx(t+1) to
         // dc[k]; the non-seed ones are already gathered (needA), the seeds only for this
         const int kd = t + 1 - Ei;
-        const bool dc_row = DC && !SOFT && has_next && agent && !never && kd >= 1 && kd <= L - 1;
+        const bool dc_row = DC && !SOFT && gather && agent && !never && kd >= 1 && kd <= L - 1;
 
         // the epilogue's row loads that do not depend on the sums go out before them, so
         // that their latency overlaps the entry stream; A was stored on day E_i (soft:
@@ -192,14 +198,14 @@ __global__ void __launch_bounds__(kBlock, (MODE == kBwdStore && !DC) ? GABM_BWD_
                 row_sums<NARR>(a.m, cur.p0, cur.len, act, lane, contrib, want, sum);
         }
         float gx_mine = sum[0];
-        if (a.self_q) gx_mine = __fmaf_rn(-a.self_q[row], a.self_r[row], gx_mine);
+        if (a.self_q && gather) gx_mine = __fmaf_rn(-a.self_q[row], a.self_r[row], gx_mine);
 
         if (needA) a.ring[(size_t)slot_k[1] * a.ring_stride + row] = gx_mine;
         if constexpr (DC && !SOFT) dc_accumulate(a.dc_tile, tile, dc_row, kd, gx_mine, sg[t + 1], lane);
         if constexpr (DC && SOFT) {
             // soft: every agent's mass exposed k days before t+1 counts, n_j(d) = s_j(d) y_j(d)
             // for d >= 0 and the seeds' unit mass on their day E_j < 0 (lane k keeps k's sum)
-            const bool on = has_next && agent;
+            const bool on = gather && agent;
             if (__any_sync(0xffffffffu, on)) {
                 float mine = 0.f;
                 for (int k = 1; k < L; ++k) {
@@ -255,7 +261,7 @@ __global__ void __launch_bounds__(kBlock, (MODE == kBwdStore && !DC) ? GABM_BWD_
 #pragma unroll
                 for (int u = 0; u < RB; ++u) {
                     const int k = k0 + u;
-                    const bool ok = k < L && t + k < T;
+                    const bool ok = k < L && ((live_k >> k) & 1u);   // a day without adjoint has no ring slot
                     rv[u] = ld_if(a.ring + (size_t)slot_k[ok ? k : 0] * a.ring_stride + row, ok);
                 }
 #pragma unroll
@@ -291,17 +297,23 @@ __global__ void __launch_bounds__(kBlock, (MODE == kBwdStore && !DC) ? GABM_BWD_
             else dy = G - Apre;
             const float RS = a.R[pi + t] * a.S[inst * kAges + ai];
             const float lam = RS * Lam;
-            const float q = expf(-lam);
-            const float p = -expm1f(-lam);
-            const uint32_t id = caller_id(a.gr, row, g);
-            const float u = uniform_from_word(philox_word(a.seed, id, (uint32_t)t, (uint32_t)inst, 0u));
-            const float den = __fmaf_rn(p, 1.f - u, q * u);
-            const float dydl = (u * (1.f - u)) * q / (den * den);
-            const float glam = dy * dydl;
+            // dy = 0 and 0 <= lambda < inf: dy/dlambda is finite and >= 0, so the product is dy
+            // itself and the draw's uniform is not needed
+            float glam = dy;
+            if (!(dy == 0.f && lam >= 0.f && lam < __int_as_float(0x7f800000))) {
+                const float q = expf(-lam);
+                const float p = -expm1f(-lam);
+                const uint32_t id = caller_id(a.gr, row, g);
+                const float u = uniform_from_word(philox_word(a.seed, id, (uint32_t)t, (uint32_t)inst, 0u));
+                const float den = __fmaf_rn(p, 1.f - u, q * u);
+                const float dydl = (u * (1.f - u)) * q / (den * den);
+                glam = dy * dydl;
+            }
             const float rc = RS * glam * a.gr.inv_Dbar[g];
             a.r_cur[row] = rc;
             v = glam * Lam;
             stored = fmaxf(stored, fabsf(rc));
+            rnz_w |= !(rc == 0.f);
             emax_w = max(emax_w, (unsigned)(float_exponent(stored) + 128));
         }
 
@@ -343,7 +355,10 @@ __global__ void __launch_bounds__(kBlock, (MODE == kBwdStore && !DC) ? GABM_BWD_
     }
 
     const int sN = __reduce_add_sync(0xffffffffu, cN);
-    if (cur_g >= 0) flush_emax(a.emax + (size_t)cur_g * a.ld_sig + t, emax_w);
+    if (cur_g >= 0) {
+        flush_emax(a.emax + (size_t)cur_g * a.ld_sig + t, emax_w);
+        flush_rnz(a.rnz + (size_t)cur_g * a.ld_sig + t, rnz_w);
+    }
     if (lane == 0) { red_s[wib][0] = cur_g; red_s[wib][1] = sN; }
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -423,8 +438,9 @@ __global__ void __launch_bounds__(kBlock) k_dc_seeds(Sell m, const int16_t *E, c
 // H dphi/dm per day t_I < tau_EI (warp tree in FP64) to Pm[t_I][tile], zeroed beforehand.
 __global__ void __launch_bounds__(kBlock) k_fate_seeds(Sell m, const int16_t *E, const float *r0, const float *ring,
                                                        size_t ring_stride, int Lm1, GraphRef gr, FateRef f,
-                                                       const double *gD, const int32_t *sig, int ld_sig, int ntiles,
-                                                       int T, const float *c, double *Pm) {
+                                                       const double *gD, const int32_t *sig, int ld_sig,
+                                                       const int32_t *rnz, int ntiles, int T, const float *c,
+                                                       double *Pm) {
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const int nwarps = gridDim.x * (kBlock / 32);
     const int L = Lm1 + 1;
@@ -453,7 +469,7 @@ __global__ void __launch_bounds__(kBlock) k_fate_seeds(Sell m, const int16_t *E,
             double H = (Ei + f.L_M >= 0 && Ei + f.L_M < T) ? gD[pg + Ei + f.L_M] : 0.0;
             for (int k = Lmin; k < L; ++k) {
                 const int d = Ei + k;
-                if (d < 0 || d >= T) continue;
+                if (d < 0 || d >= T || rnz[(size_t)g * ld_sig + d] == 0) continue;   // no adjoint: gx(d) = 0
                 const float gxs = d == 0 ? sum[0] : ring[(size_t)(d % Lm1) * ring_stride + row];
                 H += sgn * (double)c[k] * ldexp((double)gxs, sg[d]);
             }
@@ -593,8 +609,10 @@ cudaError_t launch_dc_seeds(Sell m_out, const int16_t *E, const float *r0, Graph
 
 cudaError_t launch_fate_seeds(Sell m_out, const int16_t *E, const float *r0, const float *ring, size_t ring_stride,
                               int Lm1, GraphRef gr, FateRef f, const double *gD, const int32_t *sig, int ld_sig,
-                              int ntiles, int T, const float *c, double *Pm, int grid, cudaStream_t s) {
-    k_fate_seeds<<<grid, kBlock, 0, s>>>(m_out, E, r0, ring, ring_stride, Lm1, gr, f, gD, sig, ld_sig, ntiles, T, c, Pm);
+                              const int32_t *rnz, int ntiles, int T, const float *c, double *Pm, int grid,
+                              cudaStream_t s) {
+    k_fate_seeds<<<grid, kBlock, 0, s>>>(m_out, E, r0, ring, ring_stride, Lm1, gr, f, gD, sig, ld_sig, rnz, ntiles, T, c,
+                                         Pm);
     return cudaGetLastError();
 }
 

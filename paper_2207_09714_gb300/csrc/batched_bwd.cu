@@ -58,6 +58,8 @@ __global__ void __launch_bounds__(kBlock, GABM_BBWD_MINBLOCKS) k_bwd_day_b(const
     const int32_t *sg = nullptr;   // scale exponents of the current graph (shared by its sets)
     int sig_t = 0;
     unsigned emax_w = 0u;          // largest exponent stored by this warp (+128)
+    unsigned live_k = 0u;          // bit k: day t + k carries adjoint in some set
+    bool rnz_w = false;            // this lane stored an r other than 0
     uint32_t touched = 0u;         // DC: the k rows of dcs this lane added to in the current tile
     TileDispenser disp;
     disp.init(a.tile_ctr, ntiles, gridDim.x * NW, lane);
@@ -79,8 +81,11 @@ __global__ void __launch_bounds__(kBlock, GABM_BBWD_MINBLOCKS) k_bwd_day_b(const
         if (g != cur_g) {
             if (cur_g >= 0) {
                 flush_emax(a.emax + (size_t)cur_g * a.ld_sig + t, emax_w);
+                flush_rnz(a.rnz + (size_t)cur_g * a.ld_sig + t, rnz_w);
                 emax_w = 0u;
+                rnz_w = false;
             }
+            live_k = carries_adjoint(a.rnz + (size_t)g * a.ld_sig, t, T, L);
             cur_g = g;
             sg = a.sig + (size_t)g * a.ld_sig;
             sig_t = next_sigma(sg[t + 1], a.emax[(size_t)g * a.ld_sig + t + 1]);
@@ -117,7 +122,7 @@ __global__ void __launch_bounds__(kBlock, GABM_BBWD_MINBLOCKS) k_bwd_day_b(const
                 const bool never = Eh == kNever;
                 const bool live = (Eh != kPad) && (never || Eh >= 0);   // seeds are constants
                 isS[h] = live && (never || Eh >= t);
-                needA_any |= has_next && live && (never || Eh >= t + 2 - L);
+                needA_any |= (live_k & 2u) && live && (never || Eh >= t + 2 - L);
                 anyS |= isS[h];
             }
             // table adjoint: sets in which the row is infectious on day t+1 (k = t+1-E in
@@ -129,7 +134,7 @@ __global__ void __launch_bounds__(kBlock, GABM_BBWD_MINBLOCKS) k_bwd_day_b(const
             for (int h = 0; h < SPL; ++h) {
                 const int Eh = half_of(ew[h >> 1], h & 1);
                 kdh[h] = t + 1 - Eh;
-                dch[h] = DC && has_next && Eh != kPad && Eh != kNever && kdh[h] >= 1 && kdh[h] <= L - 1;
+                dch[h] = DC && (live_k & 2u) && Eh != kPad && Eh != kNever && kdh[h] >= 1 && kdh[h] <= L - 1;
                 dc_any |= dch[h];
             }
             const bool act = (group_bits<LPR>(__ballot_sync(kFull, needA_any || dc_any)) >> grp) & 1u;
@@ -201,7 +206,7 @@ __global__ void __launch_bounds__(kBlock, GABM_BBWD_MINBLOCKS) k_bwd_day_b(const
 #pragma unroll
                     for (int u = 0; u < 4; ++u) {
                         const int k = k0 + u;
-                        const bool ok = k < L && t + k < T;
+                        const bool ok = k < L && ((live_k >> k) & 1u);
                         ld_floats<SPL>(a.ring + (size_t)slot_k[ok ? k : 0] * stride + xo, ok, rv[u]);
                     }
 #pragma unroll
@@ -227,15 +232,19 @@ __global__ void __launch_bounds__(kBlock, GABM_BBWD_MINBLOCKS) k_bwd_day_b(const
                     const int inst = g * B + s0 + h;
                     const float RS = Rt[h] * a.S[inst * kAges + ai];
                     const float lam = RS * Lv[h];
-                    const float qv = expf(-lam);
-                    const float p = -expm1f(-lam);
-                    const float u = uniform_from_word(philox_word(a.seed, id, (uint32_t)t, (uint32_t)inst, 0u));
-                    const float den = __fmaf_rn(p, 1.f - u, qv * u);
-                    const float dydl = (u * (1.f - u)) * qv / (den * den);
-                    const float glam = dy * dydl;
+                    float glam = dy;   // dy = 0 and lambda finite: the product with dy/dlambda >= 0 is dy itself
+                    if (!(dy == 0.f && lam >= 0.f && lam < __int_as_float(0x7f800000))) {
+                        const float qv = expf(-lam);
+                        const float p = -expm1f(-lam);
+                        const float u = uniform_from_word(philox_word(a.seed, id, (uint32_t)t, (uint32_t)inst, 0u));
+                        const float den = __fmaf_rn(p, 1.f - u, qv * u);
+                        const float dydl = (u * (1.f - u)) * qv / (den * den);
+                        glam = dy * dydl;
+                    }
                     rc[h] = RS * glam * inv_D;
                     v[h] = glam * Lv[h];
                     stored = fmaxf(stored, fabsf(rc[h]));
+                    rnz_w |= !(rc[h] == 0.f);
                 }
                 emax_w = max(emax_w, (unsigned)(float_exponent(stored) + 128));
                 if (writeA) st_floats<SPL>(a.A + xo, Av);
@@ -286,7 +295,10 @@ __global__ void __launch_bounds__(kBlock, GABM_BBWD_MINBLOCKS) k_bwd_day_b(const
         rp_lo = nrp_lo;
         rp_hi = nrp_hi;
     }
-    if (cur_g >= 0) flush_emax(a.emax + (size_t)cur_g * a.ld_sig + t, emax_w);
+    if (cur_g >= 0) {
+        flush_emax(a.emax + (size_t)cur_g * a.ld_sig + t, emax_w);
+        flush_rnz(a.rnz + (size_t)cur_g * a.ld_sig + t, rnz_w);
+    }
 }
 
 template <int LPR, int SPL, bool KAHAN>

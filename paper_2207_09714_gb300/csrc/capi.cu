@@ -43,6 +43,7 @@ struct gabm_ctx {
     float *s_hist = nullptr, *y_hist = nullptr;                 // [Tcap][n_rows] soft histories
     double *P_nrm = nullptr, *newRM_real = nullptr;             // [Tcap][ntiles], [I][Tcap]
     int32_t *sig = nullptr, *emax = nullptr;   // [G][Tcap+1] reverse-sweep scale exponents per graph and day
+    int32_t *rnz = nullptr;                    // [G][Tcap+1] 1: some coefficient r of that day is not 0
     int tau_EI = 0, tau_IR = 0, L = 0;   // L: the table's length, the longest infectious window
     int tau_IM = 0, L_R = 0, L_M = 0;    // sampled R/M split (tau_IM > 0): exits at L_R and L_M
     bool fate = false;
@@ -571,7 +572,7 @@ gabm_status ensure_days(gabm_ctx *c, int T) {
     dfree(c, c->dR_s); dfree(c, c->dm_s); dfree(c, c->tile_ctr); dfree(c, c->bits); dfree(c, c->Pc);
     dfree(c, c->tile_new); dfree(c, c->newinf);
     dfree(c, c->s_hist); dfree(c, c->y_hist); dfree(c, c->P_nrm); dfree(c, c->newRM_real);
-    dfree(c, c->sig); dfree(c, c->emax); dfree(c, c->Pm);
+    dfree(c, c->sig); dfree(c, c->emax); dfree(c, c->rnz); dfree(c, c->Pm);
     c->Tcap = 0;
     const size_t IT = (size_t)c->I * cap;
     if (c->policy == GABM_STORE_LAMBDA) TRY(dalloc(c, &c->lam, (size_t)cap * c->n_rows * c->Bp));
@@ -603,6 +604,7 @@ gabm_status ensure_days(gabm_ctx *c, int T) {
     TRY(dalloc(c, &c->bits, (size_t)(cap + 1) * c->ntiles));
     TRY(dalloc(c, &c->sig, (size_t)c->G * (cap + 1)));
     TRY(dalloc(c, &c->emax, (size_t)c->G * (cap + 1)));
+    TRY(dalloc(c, &c->rnz, (size_t)c->G * (cap + 1)));
     CK(cudaMemsetAsync(c->D, 0, IT * sizeof(double), c->stream));
     c->Tcap = cap;
     c->T_last = -1;
@@ -781,6 +783,7 @@ gabm_status backward_days_batched(gabm_ctx *c, int T, cudaStream_t s) {
     for (int k = 0; k < kMaxL; ++k) a.c[k] = k < c->L ? c->c[k] : 0.f;
     a.sig = c->sig;
     a.emax = c->emax;
+    a.rnz = c->rnz;
     a.ld_sig = ld + 1;
     a.Bw = c->Bp;
     a.dc_tile = c->want_dc ? c->dc_tile : nullptr;
@@ -884,6 +887,7 @@ gabm_status backward_days_sirs(gabm_ctx *c, int T, cudaStream_t s) {
     a.newRM = c->newRM_b;
     a.sig = c->sig;
     a.emax = c->emax;
+    a.rnz = c->rnz;
     a.ld_sig = ld + 1;
     a.ntiles = c->ntiles;
     a.T = T;
@@ -1022,6 +1026,7 @@ gabm_status backward_days_plain(gabm_ctx *c, int T, cudaStream_t s) {
     a.hist_stride = (size_t)c->n_rows;
     a.sig = c->sig;
     a.emax = c->emax;
+    a.rnz = c->rnz;
     a.ld_sig = ld + 1;
     a.dc_tile = c->want_dc ? c->dc_tile : nullptr;
     a.self_r = a.self_q = nullptr;
@@ -1061,7 +1066,7 @@ gabm_status backward_days_plain(gabm_ctx *c, int T, cudaStream_t s) {
     }
     if (c->fate)   // the fate draws of agents exposed before day 0 (r of day 0 is in slot 0)
         LAUNCH(launch_fate_seeds(sell_view(c, true), c->e, c->r, c->ring, (size_t)c->n_rows, Lm1, graph_ref(c), a.fate,
-                                 c->gD, c->sig, ld + 1, c->ntiles, T, c->c_dev, c->Pm, c->grid_bwd, s));
+                                 c->gD, c->sig, ld + 1, c->rnz, c->ntiles, T, c->c_dev, c->Pm, c->grid_bwd, s));
     if (a.dc_tile) {   // the seeds' share through day 0 (r of day 0 is in slot 0)
         const float *r0 = c->r;
         if (c->two_hop) {
@@ -1212,6 +1217,7 @@ gabm_status backward_core(gabm_ctx *c, int T) {
     // sigma(T) = 0 and no stored exponent yet
     CK(cudaMemsetAsync(c->sig, 0, sizeof(int32_t) * (size_t)c->G * (ld + 1), s));
     CK(cudaMemsetAsync(c->emax, 0, sizeof(int32_t) * (size_t)c->G * (ld + 1), s));
+    CK(cudaMemsetAsync(c->rnz, 0, sizeof(int32_t) * (size_t)c->G * (ld + 1), s));
     if (c->soft) CK(cudaMemsetAsync(c->A, 0, sizeof(float) * (size_t)c->n_rows, s));   // dL/ds(T) = 0
 
     if (!c->batched && c->policy != GABM_STORE_LAMBDA && !c->symmetric && !c->lam_tmp)

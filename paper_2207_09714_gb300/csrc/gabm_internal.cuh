@@ -230,6 +230,7 @@ struct BwdDayArgs {
     float c[kMaxL];
     int ring_slot[kMaxL];      // ring slot holding day t + k, k = 1..L-1
     int32_t *sig, *emax;       // [G][ld_sig] scale exponent and largest stored exponent per day
+    int32_t *rnz;              // [G][ld_sig] 1: some r of that day is not 0 (see carries_adjoint)
     int ld_sig;
     double *dc_tile;           // [ntiles][kMaxL] per-tile sums of the table adjoint over days, or nullptr
     // agent-location graphs: r_next is the location adjoint gP; the agent's own share of its
@@ -321,6 +322,7 @@ struct BwdBatchArgs {
     float c[kMaxL];
     int ring_slot[kMaxL];
     int32_t *sig, *emax;         // [G][ld_sig] per graph (shared by its sets)
+    int32_t *rnz;                // [G][ld_sig] 1: some r of that day is not 0 in some set
     int ld_sig;
     int Bw, s0;                  // row width of the per-agent arrays; first set of this launch
     double *dc_tile;             // [ntiles][L][Bw] per-tile sums of the table adjoint over days, or nullptr
@@ -390,6 +392,20 @@ __device__ __forceinline__ void flush_emax(int32_t *emax_gt, unsigned em_lane) {
     }
 }
 
+// Days whose coefficients r are all exactly 0 carry no adjoint back: gx of such a day is 0
+// for every row, so the sweep neither gathers nor stores nor reads it.  The last L days of a
+// horizon are always so (an exposure there enters RM after it), and so is every day after
+// the last one the loss looks at, so the test is made on the stored coefficients
+// themselves: a launch that stores an r other than 0 (or a NaN) sets its day's flag.
+// Bit k of the result (1 <= k < L): day t + k of this graph has one.  Called by all 32 lanes.
+__device__ __forceinline__ unsigned carries_adjoint(const int32_t *rnz_g, int t, int T, int L) {
+    const int lane = threadIdx.x & 31;
+    return __ballot_sync(0xffffffffu, lane >= 1 && lane < L && t + lane < T && rnz_g[t + lane] != 0);
+}
+__device__ __forceinline__ void flush_rnz(int32_t *rnz_gt, bool any_lane) {
+    if (__any_sync(0xffffffffu, any_lane) && (threadIdx.x & 31) == 0 && *(volatile int32_t *)rnz_gt == 0) *rnz_gt = 1;
+}
+
 // Launchers (forward.cu / backward.cu)
 cudaError_t launch_init_state(int16_t *e, const int32_t *row0, const int32_t *rows, int G,
                               int64_t n_rows, int B, int Bp, int grid, cudaStream_t s);
@@ -409,7 +425,8 @@ cudaError_t launch_infectious_bits_dur(const int16_t *e, GraphRef gr, const DurR
                                        uint32_t *bits, cudaStream_t s);
 cudaError_t launch_fate_seeds(Sell m_out, const int16_t *E, const float *r0, const float *ring, size_t ring_stride,
                               int Lm1, GraphRef gr, FateRef f, const double *gD, const int32_t *sig, int ld_sig,
-                              int ntiles, int T, const float *c, double *Pm, int grid, cudaStream_t s);
+                              const int32_t *rnz, int ntiles, int T, const float *c, double *Pm, int grid,
+                              cudaStream_t s);
 cudaError_t launch_fate_dm(const double *Pm, int ntiles, const int32_t *graph_tile0, const int32_t *graph_ntiles,
                            int G, int T, double *dm, cudaStream_t s);
 cudaError_t launch_infectious_bits(const int16_t *e, int t0, int ndays, int L, int ntiles, uint32_t *bits,

@@ -159,7 +159,8 @@ __global__ void __launch_bounds__(kBlock, 3) k_bwd_day_sirs(const SirsBwdArgs a)
     };
     const bool want[1] = {true};
     int cur_g = -1, cN = 0;
-    unsigned emax_w = 0u;
+    unsigned emax_w = 0u, live_k = 0u;   // live_k bit k: day t + k carries adjoint
+    bool rnz_w = false;
     BlockTiles disp;
     disp.init(a.ntiles, lane);
     TileRows cur, nxt;
@@ -173,10 +174,13 @@ __global__ void __launch_bounds__(kBlock, 3) k_bwd_day_sirs(const SirsBwdArgs a)
                 const int sN = __reduce_add_sync(0xffffffffu, cN);
                 if (lane == 0 && sN) atomicAdd(a.newRM + (size_t)cur_g * a.ldP + t, sN);
                 flush_emax(a.emax + (size_t)cur_g * a.ld_sig + t, emax_w);
+                flush_rnz(a.rnz + (size_t)cur_g * a.ld_sig + t, rnz_w);
                 emax_w = 0u;
+                rnz_w = false;
             }
             cur_g = g;
             cN = 0;
+            live_k = carries_adjoint(a.rnz + (size_t)g * a.ld_sig, t, T, L);
         }
         const int32_t *sg = a.sig + (size_t)g * a.ld_sig;
         const int sig_t = next_sigma(sg[t + 1], a.emax[(size_t)g * a.ld_sig + t + 1]);
@@ -199,7 +203,7 @@ __global__ void __launch_bounds__(kBlock, 3) k_bwd_day_sirs(const SirsBwdArgs a)
         const int lo = max(0, t + 2 - L);
         bool covered = false;
         for (int j = 0; j < j_t; ++j) covered |= (hr[j] >= t - C + 1 && hr[j] <= lo - 1);
-        const bool act = has_next && agent && !covered;
+        const bool act = (live_k & 2u) && agent && !covered;
         float sum[1];
         row_sums<1>(a.m, cur.p0, cur.len, act, lane, contrib, want, sum,
                     [&](uint32_t j, float w) { return w * r_next[j]; });
@@ -221,7 +225,7 @@ __global__ void __launch_bounds__(kBlock, 3) k_bwd_day_sirs(const SirsBwdArgs a)
             float loc = (t + L < T) ? a.m_t[pg + t + L] * (float)a.gD[pg + t + L] * exp2i(-sig_t) : 0.f;
             if (has_next) loc = __fmaf_rn(c_s[1], gx1 * exp2i(sg[t + 1] - sig_t), loc);
             for (int k = 2; k < L; ++k)
-                if (t + k < T) loc = __fmaf_rn(c_s[k], a.ring[(size_t)slot_k[k] * a.ring_stride + row] * exp2i(sg[t + k] - sig_t), loc);
+                if ((live_k >> k) & 1u) loc = __fmaf_rn(c_s[k], a.ring[(size_t)slot_k[k] * a.ring_stride + row] * exp2i(sg[t + k] - sig_t), loc);
             const float G = loc + B_at(t + C);
             // dL/dy = G - B(t+1).  With t' the row's first exposure after t, B(t+1) = G(t'),
             // and B(t+C) = B(t'+C) when t' < t+C (the next exposure after t' is at least
@@ -239,16 +243,20 @@ __global__ void __launch_bounds__(kBlock, 3) k_bwd_day_sirs(const SirsBwdArgs a)
             const float Lam = a.lam_t[row];
             const float RS = a.R[pg + t] * a.S[g * kAges + ai];
             const float lam = RS * Lam;
-            const float q = expf(-lam);
-            const float p = -expm1f(-lam);
-            const uint32_t id = caller_id(a.gr, row, g);
-            const float u = uniform_from_word(philox_word(a.seed, id, (uint32_t)t, (uint32_t)g, 0u));
-            const float den = __fmaf_rn(p, 1.f - u, q * u);
-            const float dydl = (u * (1.f - u)) * q / (den * den);
-            const float glam = dy * dydl;
+            float glam = dy;   // dy = 0 and lambda finite: the product with dy/dlambda >= 0 is dy itself
+            if (!(dy == 0.f && lam >= 0.f && lam < __int_as_float(0x7f800000))) {
+                const float q = expf(-lam);
+                const float p = -expm1f(-lam);
+                const uint32_t id = caller_id(a.gr, row, g);
+                const float u = uniform_from_word(philox_word(a.seed, id, (uint32_t)t, (uint32_t)g, 0u));
+                const float den = __fmaf_rn(p, 1.f - u, q * u);
+                const float dydl = (u * (1.f - u)) * q / (den * den);
+                glam = dy * dydl;
+            }
             rc = RS * glam * a.gr.inv_Dbar[g];
             v = glam * Lam;
             stored = fmaxf(stored, fabsf(rc));
+            rnz_w |= !(rc == 0.f);
             emax_w = max(emax_w, (unsigned)(float_exponent(stored) + 128));
         }
         a.r_cur[row] = rc;   // 0 for rows not susceptible today (r of a later day may sit there)
@@ -262,6 +270,7 @@ __global__ void __launch_bounds__(kBlock, 3) k_bwd_day_sirs(const SirsBwdArgs a)
         const int sN = __reduce_add_sync(0xffffffffu, cN);
         if (lane == 0 && sN) atomicAdd(a.newRM + (size_t)cur_g * a.ldP + t, sN);
         flush_emax(a.emax + (size_t)cur_g * a.ld_sig + t, emax_w);
+        flush_rnz(a.rnz + (size_t)cur_g * a.ld_sig + t, rnz_w);
     }
 }
 

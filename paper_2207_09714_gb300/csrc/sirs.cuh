@@ -63,6 +63,7 @@ struct SirsBwdArgs {
     double *P_t;                // [ntiles][9] per-tile sums of gl * Lam by age
     int32_t *newRM;             // [I][ldP] recounted
     int32_t *sig, *emax;        // [G][ld_sig] per-day scale exponents
+    int32_t *rnz;               // [G][ld_sig] 1: some r of that day is not 0
     int ld_sig;
     int ntiles, t, T, tau_EI, L, cycle;
     uint64_t seed;
