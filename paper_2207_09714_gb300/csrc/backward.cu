@@ -51,13 +51,21 @@ __device__ __forceinline__ void dc_accumulate(double *dc_tile, int tile, bool ha
     if (touched) dc_tile[(size_t)tile * kMaxL + lane] += (double)mine * ldexp(1.0, sigma);
 }
 
+// One term of G_i(t): the ring slot of day t + k (an offset within the tile's slots) and
+// c[k] 2^(sigma(t+k) - sigma(t)).  Only days that carry adjoint have one.
+struct RingTerm {
+    int off;
+    float cf;
+};
+#ifndef GABM_RING_BATCH
+#define GABM_RING_BATCH 10
+#endif
+
 // DC: accumulate the table adjoint (a.dc_tile); a separate instance, so the plain sweep
 // carries none of its code.
-// Four resident blocks (64 registers) for the plain store sweep: the gathers of r want
-// the warps (79 vs 82 us per day on the 1M-agent graph at three).  The fused, soft and
-// table-adjoint instances, which spill at 64 registers, keep three.
+// Resident blocks: see the launch bounds' measurements below.
 #ifndef GABM_BWD_MINBLOCKS
-#define GABM_BWD_MINBLOCKS 4
+#define GABM_BWD_MINBLOCKS 3
 #endif
 // EXIT = kExitFate (sampled R/M split, store policy): G of an exposure today takes the
 // fate it would draw (window L_R or L_M; the death term gD_{t+L_M} only if M-fated), and
@@ -72,44 +80,50 @@ __global__ void __launch_bounds__(kBlock, (MODE == kBwdStore && !DC) ? GABM_BWD_
     k_bwd_day(const BwdDayArgs a) {
     constexpr bool FATE = EXIT == kExitFate;
     constexpr bool DUR = EXIT == kExitDur;
-    constexpr int NARR = (MODE == kBwdFused) ? 2 : 1;
     constexpr bool SOFT = MODE == kBwdSoft;
-    constexpr int RB = 8;   // ring slots loaded together in the epilogue (16: 4% slower)
+    constexpr int RB = GABM_RING_BATCH;   // ring slots loaded together in the epilogue
+    constexpr int NW = kBlock / 32;
     __shared__ float c_s[kMaxL];
-    __shared__ int slot_k[kMaxL];
-    __shared__ int32_t red_s[kBlock / 32][2];
-    __shared__ float fac_s[kBlock / 32][kMaxL];   // 2^(sigma(t+k) - sigma(t)) of the warp's graph
+    __shared__ int32_t red_s[NW][2];
+    __shared__ RingTerm term_s[NW][kMaxL];        // the warp's graph's ring terms, k ascending
+    __shared__ int term_k[FATE || DUR ? NW : 1][kMaxL];   // their k
+    __shared__ float rs_s[NW][kAges];             // R_t S_a of the warp's graph
+    __shared__ __align__(16) float bin_s[NW][kBinWords];
     __shared__ double F_s[kMaxL];
     if (threadIdx.x < kMaxL) {
         c_s[threadIdx.x] = a.c[threadIdx.x];
-        slot_k[threadIdx.x] = a.ring_slot[threadIdx.x];
         if (DUR) F_s[threadIdx.x] = a.dur.F[threadIdx.x];
     }
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    for (int i = lane; i < kBinWords; i += 32) bin_s[wib][i] = 0.f;
     __syncthreads();
 
-    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const int t = a.t, T = a.T, L = a.L, ntiles = a.ntiles;
     const int32_t *sg = nullptr;   // scale exponents of the current graph
     int sig_t = 0;                 // sigma(t) of the current graph
     unsigned emax_w = 0u;          // largest exponent stored by this warp (+128)
     bool rnz_w = false;            // this lane stored an r other than 0
     unsigned live_k = 0u;          // bit k: day t + k carries adjoint (its gx is not all 0)
+    int nterm = 0;                 // ring terms, k >= 2
     float gtail = 0.f;             // m_{t+L} gD_{t+L} at day t's scale
-    const bool has_next = (t + 1 < T);
+    float cf1 = 0.f, f1 = 0.f;     // the k = 1 term's factor, and its scale alone
+    float inv_D = 0.f;
     const int16_t *E = a.E;
-    const float *__restrict__ r_next = a.r_next;
-    const uint32_t *bits = a.bits_t;
-    // contribution 0: w * r_j(t+1) (transpose gather); contribution 1 (recompute):
-    // w * c[t - E_j] for neighbours marked infectious on day t
-    auto contrib = [&](uint32_t j, float w, bool valid, float (&out)[NARR], bool (&take)[NARR]) {
-        out[0] = w * ld_if(r_next + j, valid);
-        take[0] = valid;
-        if constexpr (NARR == 2) {
-            const bool mk = valid && marked(bits, j);
-            const int Ej = ld_if(E + j, mk, kNever);
-            out[1] = mk ? w * infectiousness(Ej, c_s, t, L) : 0.f;
-            take[1] = mk;
-        }
+    const int slot_floats = (L - 1) * kTile;
+
+    // Which of a tile's rows gather gx(t+1).  Table adjoint: rows infectious on day t+1 (k =
+    // t+1-E in [1, L-1]) add gx(t+1) to dc[k]; the non-seed ones gather anyway, the seeds only
+    // for this.  R/M split: rows exposed before day 0 keep gx while day t+1 is inside their
+    // window.  Soft relaxation: every agent carries susceptible mass and draws every day.
+    auto needs = [&](int Ei) {
+        const bool agent = Ei != kPad, never = Ei == kNever, gather = (live_k & 2u) != 0u;
+        if (SOFT) return gather && agent;
+        return gather && ((agent && (never || (Ei >= 0 && Ei >= t + 2 - L))) ||
+                          (FATE && agent && !never && Ei < 0 && t + 1 - Ei < L));
+    };
+    auto dc_row_of = [&](int Ei) {
+        const int kd = t + 1 - Ei;
+        return DC && !SOFT && (live_k & 2u) && Ei != kPad && Ei != kNever && kd >= 1 && kd <= L - 1;
     };
 
     int cur_g = -1, cN = 0;
@@ -117,12 +131,12 @@ __global__ void __launch_bounds__(kBlock, (MODE == kBwdStore && !DC) ? GABM_BWD_
     disp.init(ntiles, lane);
     TileRows cur, nxt;
     load_tile_rows(a.m, E, a.gr.tile_graph, ntiles, disp.get(), lane, cur);
-    load_tile_rows(a.m, E, a.gr.tile_graph, ntiles, disp.get(), lane, nxt);
-    prefetch_slice(a.m, cur.p0, cur.p1, lane);
+    bool have = false;   // ea holds the current tile's first pairs
+    uint4 ea[kGP];
+#pragma unroll
+    for (int u = 0; u < kGP; ++u) ea[u] = make_uint4(0u, 0u, 0u, 0u);
     while (cur.tile < ntiles) {
-        prefetch_slice(a.m, nxt.p0, nxt.p1, lane);
-        TileRows nn;
-        load_tile_rows(a.m, E, a.gr.tile_graph, ntiles, disp.get(), lane, nn);
+        load_tile_rows(a.m, E, a.gr.tile_graph, ntiles, disp.get(), lane, nxt);   // a tile ahead of use
 
         const int g = cur.g, tile = cur.tile, Ei = cur.e;
         if (g != cur_g) {
@@ -140,29 +154,37 @@ __global__ void __launch_bounds__(kBlock, (MODE == kBwdStore && !DC) ? GABM_BWD_
             sg = a.sig + (size_t)g * a.ld_sig;
             sig_t = next_sigma(sg[t + 1], a.emax[(size_t)g * a.ld_sig + t + 1]);
             if (lane == 0 && tile * kTile == a.gr.row0[g]) a.sig[(size_t)g * a.ld_sig + t] = sig_t;
-            if (lane < kMaxL)
-                fac_s[wib][lane] = (lane >= 1 && lane < L && t + lane <= T) ? exp2i(sg[t + lane] - sig_t) : 0.f;
-            {
-                const size_t pg = (size_t)g * a.ldP;
-                if constexpr (FATE)   // deaths are counted: dL/d(one M entry on day t + L_M)
-                    gtail = (t + a.fate.L_M < T) ? (float)a.gD[pg + t + a.fate.L_M] * exp2i(-sig_t) : 0.f;
-                else
-                    gtail = (t + L < T) ? a.m_t[pg + t + L] * (float)a.gD[pg + t + L] * exp2i(-sig_t) : 0.f;
+            // c[k] 2^(sigma(t+k) - sigma(t)): the power of two moves no bit of the product
+            const float fac = (lane >= 1 && lane < L && t + lane <= T) ? exp2i(sg[t + lane] - sig_t) : 0.f;
+            f1 = __shfl_sync(0xffffffffu, fac, 1);
+            cf1 = (live_k & 2u) ? c_s[1] * f1 : 0.f;
+            const unsigned tm = live_k & ~3u;
+            nterm = __popc(tm);
+            if ((tm >> lane) & 1u) {
+                const int i = __popc(tm & ((1u << lane) - 1u));
+                term_s[wib][i].off = a.ring_slot[lane] * kTile;
+                term_s[wib][i].cf = c_s[lane] * fac;
+                if (FATE || DUR) term_k[wib][i] = lane;
             }
+            const size_t pg = (size_t)g * a.ldP;
+            if (lane < kAges) rs_s[wib][lane] = a.R[pg + t] * a.S[g * kAges + lane];
+            inv_D = a.gr.inv_Dbar[g];
+            if constexpr (FATE)   // deaths are counted: dL/d(one M entry on day t + L_M)
+                gtail = (t + a.fate.L_M < T) ? (float)a.gD[pg + t + a.fate.L_M] * exp2i(-sig_t) : 0.f;
+            else
+                gtail = (t + L < T) ? a.m_t[pg + t + L] * (float)a.gD[pg + t + L] * exp2i(-sig_t) : 0.f;
             __syncwarp();
             cur_g = g;
             cN = 0;
+            have = false;
         }
         const int row = tile * kTile + lane;
         const bool agent = (Ei != kPad);
         const bool never = (Ei == kNever);
         const bool live = agent && (never || Ei >= 0);           // seeds are constants
-        // soft relaxation: every agent carries susceptible mass and draws every day
         const bool isS = SOFT ? agent : live && (never || Ei >= t);
-        // R/M split: rows exposed before day 0 keep gx while day t+1 is inside their window
         const bool gather = (live_k & 2u) != 0u;   // else gx(t+1) = 0 for every row
-        const bool needA = gather && (SOFT ? agent : (live && (never || Ei >= t + 2 - L)) ||
-                                                       (FATE && agent && !never && Ei < 0 && t + 1 - Ei < L));
+        const bool needA = needs(Ei), dc_row = dc_row_of(Ei);
         if constexpr (DUR) {
             // exits at the row's drawn L_i (its first possible day is tau_EI + 1)
             const int k = t - Ei;
@@ -171,37 +193,37 @@ __global__ void __launch_bounds__(kBlock, (MODE == kBwdStore && !DC) ? GABM_BWD_
         } else if (!SOFT) {
             cN += (agent && !never && t - Ei == L);
         }
-        // table adjoint: rows infectious on day t+1 (k = t+1-E in [1, L-1]) add gx(t+1) to
-        // dc[k]; the non-seed ones are already gathered (needA), the seeds only for this
-        const int kd = t + 1 - Ei;
-        const bool dc_row = DC && !SOFT && gather && agent && !never && kd >= 1 && kd <= L - 1;
 
-        // the epilogue's row loads that do not depend on the sums go out before them, so
-        // that their latency overlaps the entry stream; A was stored on day E_i (soft:
-        // dL/ds on day t+1) at that day's scale
-        const bool readA = SOFT || (!never && Ei != t);
-        const float A_ld = ld_if(a.A + row, isS && readA);
-        float lam_ld = 0.f;
-        if constexpr (MODE != kBwdFused) lam_ld = ld_if(a.lam_t + row, isS);
-        const int age_ld = isS ? (int)a.age[row] : 0;
+        // the row loads that do not depend on the sums go out before them, so that their
+        // latency overlaps the entry stream; A was stored on day E_i (soft: dL/ds on day
+        // t+1) at that day's scale
+        const bool readA = isS && (SOFT || (!never && Ei != t));
+        const float A_ld = readA ? a.A[row] : 0.f;
+        float Lam = 0.f;
+        if constexpr (MODE != kBwdFused) Lam = isS ? a.lam_t[row] : 0.f;
+        const int ai = isS ? (int)a.age[row] : 0;
+        const bool draws = live_k != 0u || gtail != 0.f || FATE || DUR || SOFT;   // some dy is not 0
+        uint32_t id = (isS && draws) ? caller_id(a.gr, row, g) : 0u;
 
-        float sum[NARR];
+        float gx_mine;
         {
-            const bool act = (MODE == kBwdFused) ? (needA || isS || dc_row) : (needA || dc_row);
-            bool want[NARR];
-            want[0] = needA || dc_row;
-            if constexpr (NARR == 2) want[1] = isS;
-            if constexpr (NARR == 1)   // every valid entry's w r_j(t+1) is taken
-                row_sums<1>(a.m, cur.p0, cur.len, act, lane, contrib, want, sum,
-                            [&](uint32_t j, float w) { return w * r_next[j]; });
-            else
-                row_sums<NARR>(a.m, cur.p0, cur.len, act, lane, contrib, want, sum);
+            const TileSpan sp = tile_span(a.m, cur.p0, cur.len, needA || dc_row, lane);
+            if (!have) load_pairs(sp.row, 0u, sp.lim, ea);
+            gx_mine = gather_sum(sp, a.r_next, ea);
         }
-        float gx_mine = sum[0];
         if (a.self_q && gather) gx_mine = __fmaf_rn(-a.self_q[row], a.self_r[row], gx_mine);
+        if constexpr (MODE == kBwdFused)   // lambda from the final exposure days, the forward's sum
+            Lam = marked_sum<false, 2>(a.m, cur.p0, cur.len, isS, lane, a.bits_t, E, c_s, t, L) * inv_D;
+        // the next tile's first pairs are in flight during this tile's epilogue
+        have = nxt.tile < ntiles && nxt.g == cur_g;
+        if (have) {
+            const TileSpan sp = tile_span(a.m, nxt.p0, nxt.len, needs(nxt.e) || dc_row_of(nxt.e), lane);
+            load_pairs(sp.row, 0u, sp.lim, ea);
+        }
 
-        if (needA) a.ring[(size_t)slot_k[1] * a.ring_stride + row] = gx_mine;
-        if constexpr (DC && !SOFT) dc_accumulate(a.dc_tile, tile, dc_row, kd, gx_mine, sg[t + 1], lane);
+        float *ring = a.ring + (size_t)tile * slot_floats + lane;
+        if (needA) ring[a.ring_slot[1] * kTile] = gx_mine;
+        if constexpr (DC && !SOFT) dc_accumulate(a.dc_tile, tile, dc_row, t + 1 - Ei, gx_mine, sg[t + 1], lane);
         if constexpr (DC && SOFT) {
             // soft: every agent's mass exposed k days before t+1 counts, n_j(d) = s_j(d) y_j(d)
             // for d >= 0 and the seeds' unit mass on their day E_j < 0 (lane k keeps k's sum)
@@ -225,22 +247,16 @@ __global__ void __launch_bounds__(kBlock, (MODE == kBwdStore && !DC) ? GABM_BWD_
         }
 
         float v = 0.f, pm = 0.f;
-        int ai = 0;
         if (isS) {
-            ai = age_ld;
-            const int inst = g;
-            const size_t pi = (size_t)inst * a.ldP;
-            const float Apre = readA ? A_ld * (SOFT ? fac_s[wib][1] : exp2i(sg[Ei] - sig_t)) : 0.f;
-            float Lam;
-            if constexpr (MODE == kBwdFused) Lam = sum[NARR - 1] * a.gr.inv_Dbar[g];
-            else Lam = lam_ld;
+            float Apre = 0.f;
+            if (readA) Apre = A_ld * (SOFT ? f1 : exp2i(sg[Ei] - sig_t));
             // R/M split: the fate an exposure today would draw on day t + tau_EI
             bool phi = false;
             float vf = 0.5f;
             int Lx = L;
             if constexpr (FATE) {
                 if (t + a.tau_EI < T) {
-                    vf = fate_uniform(a.fate, caller_id(a.gr, row, g), t + a.tau_EI, g);
+                    vf = fate_uniform(a.fate, id, t + a.tau_EI, g);
                     phi = vf < a.m_t[(size_t)g * a.ldP + t + a.tau_EI];
                 }
                 Lx = phi ? a.fate.L_M : a.fate.L_R;
@@ -249,28 +265,29 @@ __global__ void __launch_bounds__(kBlock, (MODE == kBwdStore && !DC) ? GABM_BWD_
             const float sgn = (FATE && a.fate.L_M > a.fate.L_R) ? 1.f : -1.f;
             if constexpr (DUR) {
                 // the window an exposure today would draw, and the death term of its exit day
-                Lx = dur_exit(a.dur, F_s, caller_id(a.gr, row, g), t, g);
+                Lx = dur_exit(a.dur, F_s, id, t, g);
                 const size_t pg = (size_t)g * a.ldP;
                 gtail = (t + Lx < T) ? a.m_t[pg + t + Lx] * (float)a.gD[pg + t + Lx] * exp2i(-sig_t) : 0.f;
             }
             float G = (FATE && !phi) ? 0.f : gtail;
             float H = gtail;
-            if (has_next) G = __fmaf_rn(c_s[1], gx_mine * fac_s[wib][1], G);
-            for (int k0 = 2; k0 < L; k0 += RB) {
+            G = __fmaf_rn(cf1, gx_mine, G);
+            for (int j0 = 0; j0 < nterm; j0 += RB) {
                 float rv[RB];
 #pragma unroll
-                for (int u = 0; u < RB; ++u) {
-                    const int k = k0 + u;
-                    const bool ok = k < L && ((live_k >> k) & 1u);   // a day without adjoint has no ring slot
-                    rv[u] = ld_if(a.ring + (size_t)slot_k[ok ? k : 0] * a.ring_stride + row, ok);
-                }
+                for (int u = 0; u < RB; ++u)
+                    if (j0 + u < nterm) rv[u] = ring[term_s[wib][j0 + u].off];
 #pragma unroll
                 for (int u = 0; u < RB; ++u) {
-                    const int k = k0 + u;
-                    if (k < L && t + k < T) {
-                        const float gk = rv[u] * fac_s[wib][k];
-                        if (!(FATE || DUR) || k < Lx) G = __fmaf_rn(c_s[k], gk, G);
-                        if (FATE && k >= Lmin) H = __fmaf_rn(sgn * c_s[k], gk, H);
+                    if (j0 + u < nterm) {
+                        const float cf = term_s[wib][j0 + u].cf;
+                        if constexpr (FATE || DUR) {
+                            const int k = term_k[wib][j0 + u];
+                            if (k < Lx) G = __fmaf_rn(cf, rv[u], G);
+                            if (FATE && k >= Lmin) H = __fmaf_rn(sgn * cf, rv[u], H);
+                        } else {
+                            G = __fmaf_rn(cf, rv[u], G);
+                        }
                     }
                 }
             }
@@ -295,7 +312,7 @@ __global__ void __launch_bounds__(kBlock, (MODE == kBwdStore && !DC) ? GABM_BWD_
             } else if (Ei == t) { a.A[row] = G; dy = G; }
             else if (never) dy = G;
             else dy = G - Apre;
-            const float RS = a.R[pi + t] * a.S[inst * kAges + ai];
+            const float RS = rs_s[wib][ai];
             const float lam = RS * Lam;
             // dy = 0 and 0 <= lambda < inf: dy/dlambda is finite and >= 0, so the product is dy
             // itself and the draw's uniform is not needed
@@ -303,13 +320,13 @@ __global__ void __launch_bounds__(kBlock, (MODE == kBwdStore && !DC) ? GABM_BWD_
             if (!(dy == 0.f && lam >= 0.f && lam < __int_as_float(0x7f800000))) {
                 const float q = expf(-lam);
                 const float p = -expm1f(-lam);
-                const uint32_t id = caller_id(a.gr, row, g);
-                const float u = uniform_from_word(philox_word(a.seed, id, (uint32_t)t, (uint32_t)inst, 0u));
+                if (!draws) id = caller_id(a.gr, row, g);
+                const float u = uniform_from_word(philox_word(a.seed, id, (uint32_t)t, (uint32_t)g, 0u));
                 const float den = __fmaf_rn(p, 1.f - u, q * u);
                 const float dydl = (u * (1.f - u)) * q / (den * den);
                 glam = dy * dydl;
             }
-            const float rc = RS * glam * a.gr.inv_Dbar[g];
+            const float rc = RS * glam * inv_D;
             a.r_cur[row] = rc;
             v = glam * Lam;
             stored = fmaxf(stored, fabsf(rc));
@@ -318,31 +335,9 @@ __global__ void __launch_bounds__(kBlock, (MODE == kBwdStore && !DC) ? GABM_BWD_
         }
 
         // per-tile sums of gl * Lam by age bin (fp32 over 32 rows, FP64 from here on)
-        // (the recomputing instance keeps a butterfly per bin: with the reduce-scatter its
-        // day took 1.37 ms against 0.92 on the 8M power-law workload)
-        static_assert(kAges <= 16, "age bins fit the warp's bin sums");
-        const unsigned smask = __ballot_sync(0xffffffffu, isS);
-        if constexpr (NARR == 1) {
-            float mine = 0.f;   // lanes 2b, 2b + 1: bin b
-            if (smask) mine = warp_bin_sums16(isS ? v : 0.f, ai, lane);
-            if (!(lane & 1) && (lane >> 1) < kAges) a.P_t[(size_t)tile * kAges + (lane >> 1)] = (double)mine;
-        } else {
-            double outv = 0.0;
-            if (smask) {
-                float vb[kAges];
-#pragma unroll
-                for (int b = 0; b < kAges; ++b) vb[b] = (isS && ai == b) ? v : 0.f;
-#pragma unroll
-                for (int b = 0; b < kAges; ++b)
-#pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) vb[b] += __shfl_xor_sync(0xffffffffu, vb[b], o);
-                float mine = 0.f;
-#pragma unroll
-                for (int b = 0; b < kAges; ++b) if (lane == b) mine = vb[b];
-                outv = (double)mine;
-            }
-            if (lane < kAges) a.P_t[(size_t)tile * kAges + lane] = outv;
-        }
+        float mine = 0.f;   // lanes 2b, 2b + 1: bin b
+        if (__any_sync(0xffffffffu, !(v == 0.f))) mine = warp_bin_sums(v, ai, lane, bin_s[wib]);
+        if (!(lane & 1) && (lane >> 1) < kAges) a.P_t[(size_t)tile * kAges + (lane >> 1)] = (double)mine;
         if constexpr (FATE) {
             // dL/dm of day t + tau_EI from this tile's exposures today (fixed tree, FP64 out)
 #pragma unroll
@@ -351,7 +346,6 @@ __global__ void __launch_bounds__(kBlock, (MODE == kBwdStore && !DC) ? GABM_BWD_
         }
 
         cur = nxt;
-        nxt = nn;
     }
 
     const int sN = __reduce_add_sync(0xffffffffu, cN);
@@ -386,22 +380,14 @@ __global__ void __launch_bounds__(kBlock) k_lam_day(Sell m, const int16_t *E, co
     __syncthreads();
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const int nwarps = gridDim.x * (kBlock / 32);
-    auto contrib = [&](uint32_t j, float w, bool valid, float (&out)[1], bool (&take)[1]) {
-        const bool mk = valid && marked(bits, j);
-        const int Ej = ld_if(E + j, mk, kNever);
-        out[0] = mk ? w * infectiousness(Ej, c_s, t, L) : 0.f;
-        take[0] = mk;
-    };
-    const bool want[1] = {true};
     for (int tile = blockIdx.x * (kBlock / 32) + wib; tile < ntiles; tile += nwarps) {
         const int row = tile * kTile + lane;
         const int Ei = E[row];
         const bool act = (Ei != kPad) && (Ei == kNever || Ei >= t);
-        float sum[1];
-        row_sums<1>(m, m.slice_ptr[tile], m.row_len[row], act, lane, contrib, want, sum);
+        const float sum = marked_sum(m, m.slice_ptr[tile], m.row_len[row], act, lane, bits, E, c_s, t, L);
         if (act) {
             const int g = gr.tile_graph ? (int)gr.tile_graph[tile] : 0;
-            lam_out[row] = sum[0] * gr.inv_Dbar[g];
+            lam_out[row] = sum * gr.inv_Dbar[g];
         }
     }
 }
@@ -414,20 +400,14 @@ __global__ void __launch_bounds__(kBlock) k_dc_seeds(Sell m, const int16_t *E, c
                                                      double *dc_tile) {
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const int nwarps = gridDim.x * (kBlock / 32);
-    auto contrib = [&](uint32_t j, float w, bool valid, float (&out)[1], bool (&take)[1]) {
-        out[0] = w * ld_if(r0 + j, valid);
-        take[0] = valid;
-    };
-    const bool want[1] = {true};
     for (int tile = blockIdx.x * (kBlock / 32) + wib; tile < ntiles; tile += nwarps) {
         const int row = tile * kTile + lane;
         const int Ei = E[row];
         const bool seed = Ei != kPad && Ei < 0 && -Ei <= L - 1;
         if (!__any_sync(0xffffffffu, seed)) continue;
-        float sum[1];
-        row_sums<1>(m, m.slice_ptr[tile], m.row_len[row], seed, lane, contrib, want, sum);
+        const float sum = gather_sum(m, m.slice_ptr[tile], m.row_len[row], seed, lane, r0);
         const int g = gr.tile_graph ? (int)gr.tile_graph[tile] : 0;
-        dc_accumulate(dc_tile, tile, seed, -Ei, sum[0], sig[(size_t)g * ld_sig], lane);
+        dc_accumulate(dc_tile, tile, seed, -Ei, sum, sig[(size_t)g * ld_sig], lane);
     }
 }
 
@@ -437,7 +417,7 @@ __global__ void __launch_bounds__(kBlock) k_dc_seeds(Sell m, const int16_t *E, c
 // (day d in slot d mod (L-1), written while the sweep ran).  Each tile adds its seeds'
 // H dphi/dm per day t_I < tau_EI (warp tree in FP64) to Pm[t_I][tile], zeroed beforehand.
 __global__ void __launch_bounds__(kBlock) k_fate_seeds(Sell m, const int16_t *E, const float *r0, const float *ring,
-                                                       size_t ring_stride, int Lm1, GraphRef gr, FateRef f,
+                                                       int Lm1, GraphRef gr, FateRef f,
                                                        const double *gD, const int32_t *sig, int ld_sig,
                                                        const int32_t *rnz, int ntiles, int T, const float *c,
                                                        double *Pm) {
@@ -446,11 +426,6 @@ __global__ void __launch_bounds__(kBlock) k_fate_seeds(Sell m, const int16_t *E,
     const int L = Lm1 + 1;
     const int Lmin = min(f.L_R, f.L_M);
     const double sgn = f.L_M > f.L_R ? 1.0 : -1.0;
-    auto contrib = [&](uint32_t j, float w, bool valid, float (&out)[1], bool (&take)[1]) {
-        out[0] = w * ld_if(r0 + j, valid);
-        take[0] = valid;
-    };
-    const bool want[1] = {true};
     for (int tile = blockIdx.x * (kBlock / 32) + wib; tile < ntiles; tile += nwarps) {
         const int row = tile * kTile + lane;
         const int Ei = E[row];
@@ -461,8 +436,7 @@ __global__ void __launch_bounds__(kBlock) k_fate_seeds(Sell m, const int16_t *E,
         const int32_t *sg = sig + (size_t)g * ld_sig;
         // gx(0), needed when day 0 lies between the two exits
         const bool at0 = seed && -Ei >= Lmin && -Ei < L;
-        float sum[1];
-        row_sums<1>(m, m.slice_ptr[tile], m.row_len[row], at0, lane, contrib, want, sum);
+        const float gx0 = gather_sum(m, m.slice_ptr[tile], m.row_len[row], at0, lane, r0);
         double pm = 0.0;
         if (seed) {
             const size_t pg = (size_t)g * f.ldP;
@@ -470,7 +444,7 @@ __global__ void __launch_bounds__(kBlock) k_fate_seeds(Sell m, const int16_t *E,
             for (int k = Lmin; k < L; ++k) {
                 const int d = Ei + k;
                 if (d < 0 || d >= T || rnz[(size_t)g * ld_sig + d] == 0) continue;   // no adjoint: gx(d) = 0
-                const float gxs = d == 0 ? sum[0] : ring[(size_t)(d % Lm1) * ring_stride + row];
+                const float gxs = d == 0 ? gx0 : ring[((size_t)tile * Lm1 + d % Lm1) * kTile + lane];
                 H += sgn * (double)c[k] * ldexp((double)gxs, sg[d]);
             }
             const float vf = fate_uniform(f, caller_id(gr, row, g), tI, g);
@@ -607,11 +581,10 @@ cudaError_t launch_dc_seeds(Sell m_out, const int16_t *E, const float *r0, Graph
     return cudaGetLastError();
 }
 
-cudaError_t launch_fate_seeds(Sell m_out, const int16_t *E, const float *r0, const float *ring, size_t ring_stride,
-                              int Lm1, GraphRef gr, FateRef f, const double *gD, const int32_t *sig, int ld_sig,
+cudaError_t launch_fate_seeds(Sell m_out, const int16_t *E, const float *r0, const float *ring, int Lm1, GraphRef gr, FateRef f, const double *gD, const int32_t *sig, int ld_sig,
                               const int32_t *rnz, int ntiles, int T, const float *c, double *Pm, int grid,
                               cudaStream_t s) {
-    k_fate_seeds<<<grid, kBlock, 0, s>>>(m_out, E, r0, ring, ring_stride, Lm1, gr, f, gD, sig, ld_sig, rnz, ntiles, T, c,
+    k_fate_seeds<<<grid, kBlock, 0, s>>>(m_out, E, r0, ring, Lm1, gr, f, gD, sig, ld_sig, rnz, ntiles, T, c,
                                          Pm);
     return cudaGetLastError();
 }

@@ -69,11 +69,10 @@ struct gabm_ctx {
     bool symmetric = false;
 
     // SELL-32 edges: in-edges, and out-edges when the weights are not symmetric
-    uint32_t *slice_ptr = nullptr, *row_len = nullptr, *scol = nullptr;
-    float *sw = nullptr;
-    uint32_t *t_slice_ptr = nullptr, *t_row_len = nullptr, *t_scol = nullptr;
-    float *t_sw = nullptr;
-    int64_t sell_entries = 0;
+    uint32_t *slice_ptr = nullptr, *row_len = nullptr;
+    uint4 *scw = nullptr;
+    uint32_t *t_slice_ptr = nullptr, *t_row_len = nullptr;
+    uint4 *t_scw = nullptr;
     // row-compressed edges (batched kernels): in-edges, and out-edges when not symmetric
     uint32_t *csr_rowptr = nullptr, *csr_col = nullptr, *t_csr_rowptr = nullptr, *t_csr_col = nullptr;
     float *csr_w = nullptr, *t_csr_w = nullptr;
@@ -127,8 +126,8 @@ struct gabm_ctx {
     bool two_hop = false;
     int64_t n_loc = 0;
     int loc_ntiles = 0, grid_loc = 0;
-    uint32_t *loc_slice_ptr = nullptr, *loc_row_len = nullptr, *loc_col = nullptr;
-    float *loc_w = nullptr;
+    uint32_t *loc_slice_ptr = nullptr, *loc_row_len = nullptr;
+    uint4 *loc_cw = nullptr;
     float *locv = nullptr;          // [loc_ntiles * 32] location pressures (forward) or adjoints (backward)
     float *self_q = nullptr;        // [n_rows] sum over the agent's locations of w_il^2
     uint32_t *big_rowptr = nullptr, *big_col = nullptr;   // locations of more than 32 members (CSR)
@@ -460,12 +459,11 @@ void group_long_rows(const HostGraph &h, std::vector<uint32_t> &order, int sigma
     }
 }
 
-// SELL-32 of a device-order CSR: slice s = rows [32 s, 32 s + 32), max_len(s) x 32
-// entries, entry k of the row in lane l at slice_ptr[s] + 32 k + l; padding has
-// column 0 and weight 0 and is never read.
+// SELL-32 of a device-order CSR in pairs of entries: slice s = rows [32 s, 32 s + 32), pair q
+// of the row in lane l at cw[slice_ptr[s] + 32 q + l]; padding has column 0 and weight 0.
 struct HostSell {
-    std::vector<uint32_t> slice_ptr, row_len, col;
-    std::vector<float> w;
+    std::vector<uint32_t> slice_ptr, row_len;
+    std::vector<uint4> cw;
 };
 
 bool build_sell(const std::vector<uint32_t> &rowptr, const std::vector<uint32_t> &col, const std::vector<float> &w,
@@ -483,17 +481,17 @@ bool build_sell(const std::vector<uint32_t> &rowptr, const std::vector<uint32_t>
             mx = std::max(mx, len);
         }
         hs.slice_ptr[sl] = (uint32_t)total;
-        total += (uint64_t)mx * kTile;
-        if (total >= ((uint64_t)1 << 32) - 64) return false;
+        total += (uint64_t)((mx + 1) / 2) * kTile;
+        if (total >= ((uint64_t)1 << 31) - 64) return false;   // 2^32 entries
     }
     hs.slice_ptr[ns] = (uint32_t)total;
-    hs.col.assign((size_t)std::max<uint64_t>(total, 32), 0u);
-    hs.w.assign((size_t)std::max<uint64_t>(total, 32), 0.f);
+    hs.cw.assign((size_t)std::max<uint64_t>(total, 32), make_uint4(0u, 0u, 0u, 0u));
     for (int64_t r = 0; r < n_rows; ++r) {
         const uint32_t base = hs.slice_ptr[r / kTile] + (uint32_t)(r % kTile);
         for (uint32_t k = 0; k < hs.row_len[r]; ++k) {
-            hs.col[base + (size_t)k * kTile] = col[rowptr[r] + k];
-            hs.w[base + (size_t)k * kTile] = w[rowptr[r] + k];
+            uint4 &p = hs.cw[base + (size_t)(k / 2) * kTile];
+            (k % 2 ? p.z : p.x) = col[rowptr[r] + k];
+            memcpy(k % 2 ? &p.w : &p.y, &w[rowptr[r] + k], sizeof(float));
         }
     }
     return true;
@@ -650,8 +648,7 @@ Sell sell_view(const gabm_ctx *c, bool out_edges) {
     Sell m;
     m.slice_ptr = out_edges ? c->t_slice_ptr : c->slice_ptr;
     m.row_len = out_edges ? c->t_row_len : c->row_len;
-    m.col = out_edges ? c->t_scol : c->scol;
-    m.w = out_edges ? c->t_sw : c->sw;
+    m.cw = out_edges ? c->t_scw : c->scw;
     return m;
 }
 
@@ -659,8 +656,7 @@ Sell loc_sell_view(const gabm_ctx *c) {
     Sell m;
     m.slice_ptr = c->loc_slice_ptr;
     m.row_len = c->loc_row_len;
-    m.col = c->loc_col;
-    m.w = c->loc_w;
+    m.cw = c->loc_cw;
     return m;
 }
 
@@ -878,7 +874,6 @@ gabm_status backward_days_sirs(gabm_ctx *c, int T, cudaStream_t s) {
     a.Gh = c->sirs_Gh;
     a.Lh = c->sirs_Lh;
     a.ring = c->ring;
-    a.ring_stride = (size_t)c->n_rows;
     a.R = c->R;
     a.m_t = c->m;
     a.S = c->S;
@@ -1003,7 +998,6 @@ gabm_status backward_days_plain(gabm_ctx *c, int T, cudaStream_t s) {
     a.gr = graph_ref(c);
     a.E = c->e;
     a.ring = c->ring;
-    a.ring_stride = (size_t)c->n_rows;
     a.A = c->A;
     a.R = c->R;
     a.m_t = c->m;
@@ -1065,7 +1059,7 @@ gabm_status backward_days_plain(gabm_ctx *c, int T, cudaStream_t s) {
         prof_end(c, 1);
     }
     if (c->fate)   // the fate draws of agents exposed before day 0 (r of day 0 is in slot 0)
-        LAUNCH(launch_fate_seeds(sell_view(c, true), c->e, c->r, c->ring, (size_t)c->n_rows, Lm1, graph_ref(c), a.fate,
+        LAUNCH(launch_fate_seeds(sell_view(c, true), c->e, c->r, c->ring, Lm1, graph_ref(c), a.fate,
                                  c->gD, c->sig, ld + 1, c->rnz, c->ntiles, T, c->c_dev, c->Pm, c->grid_bwd, s));
     if (a.dc_tile) {   // the seeds' share through day 0 (r of day 0 is in slot 0)
         const float *r0 = c->r;
@@ -1417,16 +1411,13 @@ static gabm_status create_on_device(const HostLayout &H, const gabm_model_desc *
     CCK(cudaDeviceGetAttribute(&c->num_sms, cudaDevAttrMultiProcessorCount, c->device));
 
     c->sigma = sigma;
-    c->sell_entries = batched ? 0 : (int64_t)sell_in.slice_ptr.back();
-    auto upload_sell = [&](const HostSell &hs, uint32_t *&sp, uint32_t *&rl, uint32_t *&cl, float *&ww) -> gabm_status {
+    auto upload_sell = [&](const HostSell &hs, uint32_t *&sp, uint32_t *&rl, uint4 *&cw) -> gabm_status {
         TRY(dalloc(c, &sp, hs.slice_ptr.size()));
         TRY(dalloc(c, &rl, hs.row_len.size()));
-        TRY(dalloc(c, &cl, hs.col.size()));
-        TRY(dalloc(c, &ww, hs.w.size()));
+        TRY(dalloc(c, &cw, hs.cw.size()));
         CK(cudaMemcpyAsync(sp, hs.slice_ptr.data(), sizeof(uint32_t) * hs.slice_ptr.size(), cudaMemcpyHostToDevice, c->stream));
         CK(cudaMemcpyAsync(rl, hs.row_len.data(), sizeof(uint32_t) * hs.row_len.size(), cudaMemcpyHostToDevice, c->stream));
-        CK(cudaMemcpyAsync(cl, hs.col.data(), sizeof(uint32_t) * hs.col.size(), cudaMemcpyHostToDevice, c->stream));
-        CK(cudaMemcpyAsync(ww, hs.w.data(), sizeof(float) * hs.w.size(), cudaMemcpyHostToDevice, c->stream));
+        CK(cudaMemcpyAsync(cw, hs.cw.data(), sizeof(uint4) * hs.cw.size(), cudaMemcpyHostToDevice, c->stream));
         return GABM_OK;
     };
     auto upload_csr = [&](const std::vector<uint32_t> &rp, const std::vector<uint32_t> &cl, const std::vector<float> &ww,
@@ -1449,14 +1440,13 @@ static gabm_status create_on_device(const HostLayout &H, const gabm_model_desc *
             CTRY(upload_csr(t_rowptr, t_col, t_w, c->t_csr_rowptr, c->t_csr_col, c->t_csr_w));
         }
     } else {
-        CTRY(upload_sell(sell_in, c->slice_ptr, c->row_len, c->scol, c->sw));
+        CTRY(upload_sell(sell_in, c->slice_ptr, c->row_len, c->scw));
         if (symmetric) {
             c->t_slice_ptr = c->slice_ptr;
             c->t_row_len = c->row_len;
-            c->t_scol = c->scol;
-            c->t_sw = c->sw;
+            c->t_scw = c->scw;
         } else {
-            CTRY(upload_sell(sell_out, c->t_slice_ptr, c->t_row_len, c->t_scol, c->t_sw));
+            CTRY(upload_sell(sell_out, c->t_slice_ptr, c->t_row_len, c->t_scw));
         }
     }
     CTRY(dalloc(c, &c->age, (size_t)n_rows));
@@ -1885,8 +1875,7 @@ gabm_status gabm_create_bipartite(const gabm_bipartite_desc *graphs, int num_gra
     };
     if (st == GABM_OK) st = up(c->loc_slice_ptr, loc_sell.slice_ptr);
     if (st == GABM_OK) st = up(c->loc_row_len, loc_sell.row_len);
-    if (st == GABM_OK) st = up(c->loc_col, loc_sell.col);
-    if (st == GABM_OK) st = up(c->loc_w, loc_sell.w);
+    if (st == GABM_OK) st = up(c->loc_cw, loc_sell.cw);
     if (st == GABM_OK) st = up(c->big_rowptr, brow);
     if (st == GABM_OK) st = up(c->big_col, bcol);
     if (st == GABM_OK) st = up(c->big_w, bw);

@@ -75,41 +75,30 @@ __global__ void __launch_bounds__(NT, MINB) k_fwd_day(const FwdDayArgs a) {
     const int t = a.t, L = a.L, tau_EI = a.tau_EI, ntiles = a.ntiles;
     const int16_t *e = a.e;
     const uint32_t *bits = a.bits_cur;
-    // Only neighbours infectious today contribute; their exposure day is gathered.  While
-    // few rows are infectious the day's bitmap spares the gathers of the others; once many
-    // are (use_bits false, base model only), every entry's exposure day is gathered and
-    // tested directly, which selects the same entries (an exposure during the day gives
-    // c[0] = 0) at one scattered load per entry instead of two.
+    // Only neighbours infectious today contribute.  While few rows are infectious the day's
+    // bitmap spares the gathers of the others' exposure days; once many are (use_bits
+    // false, base model only), every entry's exposure day is gathered and tested directly.
     bool use_bits = true;
-    auto contrib = [&](uint32_t j, float w, bool valid, float (&out)[1], bool (&take)[1]) {
-        if constexpr (PULL) {
-            out[0] = w * ld_if(a.pull + j, valid);
-            take[0] = valid;
-        } else {
-            const bool pre = valid && (!use_bits || (SMEM_BITS ? ((bits_s[j >> 5] >> (j & 31u)) & 1u) : marked(bits, j)));
-            const int ej = ld_if(e + j, pre, kNever);
-            const int k = t - ej;
-            const bool mk = pre && (unsigned)(k - 1) < (unsigned)(L - 1);
-            out[0] = mk ? w * c_s[k] : 0.f;
-            take[0] = mk;
-        }
+    auto contrib = [&](uint32_t j, float w, bool valid, float &out, bool &take) {
+        const bool pre = valid && (!use_bits || (SMEM_BITS ? ((bits_s[j >> 5] >> (j & 31u)) & 1u) : marked(bits, j)));
+        const int ej = ld_if(e + j, pre, kNever);
+        const int k = t - ej;
+        take = pre && (unsigned)(k - 1) < (unsigned)(L - 1);
+        out = take ? w * c_s[k] : 0.f;
     };
-    const bool want[1] = {true};
 
     int cur_g = -1;
     int cS = 0, cE = 0, cI = 0, cR = 0, cN = 0;
 
-    // Tiles come from the block's contiguous range; each tile's row data is loaded one
-    // tile ahead of use (and, when enabled, its slice prefetched into L2).
+    // Tiles come from the block's contiguous range; each tile's row data is loaded two
+    // tiles ahead of use.
     BlockTiles disp;
     disp.init(ntiles, lane);
     const uint8_t *flags = PULL ? nullptr : a.flag_cur;
     TileRows cur, nxt;
     load_tile_rows(a.m, e, a.gr.tile_graph, ntiles, disp.get(), lane, cur, flags);
     load_tile_rows(a.m, e, a.gr.tile_graph, ntiles, disp.get(), lane, nxt, flags);
-    prefetch_slice(a.m, cur.p0, cur.p1, lane);
     while (cur.tile < ntiles) {
-        prefetch_slice(a.m, nxt.p0, nxt.p1, lane);
         TileRows nn;
         load_tile_rows(a.m, e, a.gr.tile_graph, ntiles, disp.get(), lane, nn, flags);
 
@@ -152,19 +141,21 @@ __global__ void __launch_bounds__(NT, MINB) k_fwd_day(const FwdDayArgs a) {
         // the draw's row loads go out before the sums, so that their latency overlaps them
         const int age_ld = act ? (int)a.age[row] : 0;
         const uint32_t id_ld = act ? caller_id(a.gr, row, g) : 0u;
-        float sum[1];
+        float sum = 0.f;
         const unsigned amask = __ballot_sync(0xffffffffu, act);
-        if (flags && __popc(amask) <= GABM_COOP_ROWS) {   // few summing rows: warp-wide, together
-            float cs = 0.f;
-            sum[0] = 0.f;
-            if (amask) few_row_sums(a.m, cur.p0, cur.len, amask, lane, contrib, sum[0], cs);
+        if constexpr (PULL) {
+            sum = gather_sum(a.m, cur.p0, cur.len, act, lane, a.pull);
+        } else if (flags && __popc(amask) <= GABM_COOP_ROWS) {   // few summing rows: warp-wide, together
+            if (amask) sum = few_row_sums(a.m, cur.p0, cur.len, amask, lane, contrib);
+        } else if (use_bits) {
+            sum = marked_sum<SMEM_BITS>(a.m, cur.p0, cur.len, act, lane, SMEM_BITS ? bits_s : bits, e, c_s, t, L);
         } else {
-            row_sums<1>(a.m, cur.p0, cur.len, act, lane, contrib, want, sum);
+            sum = exposed_sum(a.m, cur.p0, cur.len, act, lane, e, c_s, t, L);
         }
 
         int e_next = ei;
         if (act) {
-            const float Lam = sum[0] * a.gr.inv_Dbar[g];
+            const float Lam = sum * a.gr.inv_Dbar[g];
             const int inst = g;
             const float lam = (a.R[(size_t)inst * a.ldP + t] * a.S[inst * kAges + age_ld]) * Lam;
             const float p = -expm1f(-lam);
@@ -257,11 +248,6 @@ __global__ void __launch_bounds__(kBlock, GABM_MINBLOCKS) k_fwd_day_soft(const S
     const int lane = threadIdx.x & 31;
     const int t = a.t, L = a.L, ntiles = a.ntiles;
     const float *__restrict__ x_cur = a.x_cur;
-    auto contrib = [&](uint32_t j, float w, bool valid, float (&out)[1], bool (&take)[1]) {
-        out[0] = w * ld_if(x_cur + j, valid);
-        take[0] = valid;
-    };
-    const bool want[1] = {true};
     const size_t n_rows = (size_t)ntiles * kTile;
     const int slot_t = t % L;   // holds n(t - L) before this launch overwrites it with n(t)
     BlockTiles disp;
@@ -271,11 +257,10 @@ __global__ void __launch_bounds__(kBlock, GABM_MINBLOCKS) k_fwd_day_soft(const S
         const int ei = a.e[row];
         const bool agent = ei != kPad;
         const int g = a.gr.tile_graph ? (int)a.gr.tile_graph[tile] : 0;
-        float sum[1];
-        row_sums<1>(a.m, a.m.slice_ptr[tile], a.m.row_len[row], agent, lane, contrib, want, sum);
+        const float sum = gather_sum(a.m, a.m.slice_ptr[tile], a.m.row_len[row], agent, lane, x_cur);
         float n_old = 0.f;
         if (agent) {
-            const float Lam = sum[0] * a.gr.inv_Dbar[g];
+            const float Lam = sum * a.gr.inv_Dbar[g];
             const float lam = (a.R[(size_t)g * a.ldP + t] * a.S[g * kAges + a.age[row]]) * Lam;
             const float q = expf(-lam);
             const float p = -expm1f(-lam);

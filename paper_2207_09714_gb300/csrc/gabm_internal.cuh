@@ -4,14 +4,14 @@
 //   graphs are concatenated block-diagonally, each padded to a multiple of 32
 //   rows so that a 32-row tile never straddles two graphs; padding rows have
 //   no edges and exposure day kPad.
-//   SELL-32 in-edges (row i lists its in-neighbours j with w_ji), one slice of
-//   max_len x 32 entries per 32-row tile, column-major:
-//   slice_ptr u32 [ntiles+1], row_len u32 [n_rows], col u32 / w f32 [entries]
+//   SELL-32 in-edges (row i lists its in-neighbours j with w_ji), one slice per 32-row
+//   tile, its rows padded to the longest, rounded up to pairs of entries:
+//   slice_ptr u32 [ntiles+1], row_len u32 [n_rows], cw {col, w, col, w} [pairs x 32]
 //   (the out-edges in the same layout when the weights are not symmetric)
 //   age     u8  [n_rows]
 //   e       i16 [n_rows]          exposure day (kNever = susceptible)
 //   lam     f32 [Tcap][n_rows]    normalised neighbour sums (store policy)
-//   ring    f32 [L-1][n_rows]     adjoint of infectiousness, last L-1 days
+//   ring    f32 [ntiles][L-1][32] adjoint of infectiousness, last L-1 days
 //   r       f32 [2][n_rows]       per-day transpose-gather coefficients
 //   P       f64 [Tcap][ntiles][9] per-tile, per-age partial gradient sums
 #pragma once
@@ -147,10 +147,10 @@ enum { kExitBase = 0, kExitFate = 1, kExitDur = 2 };
 
 // Edges of one orientation in SELL-32 layout (one slice per 32-row tile).
 struct Sell {
-    const uint32_t *slice_ptr;  // [ntiles+1] first entry of each slice
+    const uint32_t *slice_ptr;  // [ntiles+1] first element of each slice in cw
     const uint32_t *row_len;    // [n_rows] entries of each row
-    const uint32_t *col;        // [entries] column (neighbour row) of each entry
-    const float *w;             // [entries] weight of each entry (0 in padding)
+    const uint4 *cw;            // entries 2q, 2q+1 of the row in lane l at slice_ptr + 32 q + l: column
+                                // (neighbour row) and weight bits of each (0 in padding)
 };
 
 struct FwdDayArgs {
@@ -213,8 +213,7 @@ struct BwdDayArgs {
     const float *lam_t;        // stored normalised sums for day t (store policy) or nullptr
     const float *r_next;       // coefficients of day t+1 [n_rows]
     float *r_cur;              // coefficients of day t   [n_rows]
-    float *ring;               // [L-1][n_rows]
-    size_t ring_stride;
+    float *ring;               // [ntiles][L-1][32]: a tile's slots lie together
     float *A;                  // [n_rows] adjoint of s carried back from the infection day (soft: dL/ds(t+1))
     const float *s_hist_t, *y_hist_t;   // soft mode: s_i(t), y_i(t)
     const float *s_hist, *y_hist;       // soft mode, table adjoint: all days [T][hist_stride]
@@ -423,8 +422,7 @@ cudaError_t launch_infectious_bits_fate(const int16_t *e, GraphRef gr, FateRef f
                                         cudaStream_t s);
 cudaError_t launch_infectious_bits_dur(const int16_t *e, GraphRef gr, const DurRef &d, int t, int ntiles,
                                        uint32_t *bits, cudaStream_t s);
-cudaError_t launch_fate_seeds(Sell m_out, const int16_t *E, const float *r0, const float *ring, size_t ring_stride,
-                              int Lm1, GraphRef gr, FateRef f, const double *gD, const int32_t *sig, int ld_sig,
+cudaError_t launch_fate_seeds(Sell m_out, const int16_t *E, const float *r0, const float *ring, int Lm1, GraphRef gr, FateRef f, const double *gD, const int32_t *sig, int ld_sig,
                               const int32_t *rnz, int ntiles, int T, const float *c, double *Pm, int grid,
                               cudaStream_t s);
 cudaError_t launch_fate_dm(const double *Pm, int ntiles, const int32_t *graph_tile0, const int32_t *graph_ntiles,

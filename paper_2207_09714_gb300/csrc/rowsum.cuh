@@ -1,34 +1,31 @@
 // rowsum.cuh -- device helpers shared by the forward and backward day kernels.
 //
-// Edge storage is SELL-32 (sliced ELLPACK, one slice per 32-row warp tile):
-// slice s holds max_len(s) x 32 entries, column-major, so entry k of the row in
-// lane l of the slice sits at slice_ptr[s] + 32 k + l.  A warp reads entry k of
-// its 32 rows with one coalesced 128-byte load per array, and every lane sums
-// its own row in entry order.  The sum of a row therefore depends only on the
-// row (the same operation sequence wherever and whenever it is computed), so a
-// sum recomputed in the backward is bitwise the forward's.  Rows are laid out
-// so that a slice holds rows of similar length (little padding).
+// Edge storage is SELL-32 (sliced ELLPACK, one slice per 32-row warp tile) in pairs of
+// entries: pair q of the row in lane l of a slice sits at cw[slice_ptr[s] + 32 q + l] and
+// holds {column, weight, column, weight} of entries 2q and 2q + 1.  A warp reads two
+// entries of its 32 rows with one 16-byte load per lane (512 consecutive bytes), where
+// separate column and weight arrays took four loads and their addresses; the day kernels
+// issue about as many instructions as they wait for memory, so the count matters.  Every
+// lane sums its own row in entry order.  The sum of a row therefore depends only on the
+// row (the same operation sequence wherever and whenever it is computed), so a sum
+// recomputed in the backward is bitwise the forward's.  Rows are laid out so that a slice
+// holds rows of similar length (little padding).
 #pragma once
-
-#include <type_traits>
 
 #include "gabm_internal.cuh"
 
 namespace gabm {
 
-#ifndef GABM_UNROLL
-#define GABM_UNROLL 8
-#endif
-#ifndef GABM_PIPE
-#define GABM_PIPE 1
-#endif
-#ifndef GABM_PREFETCH
-#define GABM_PREFETCH 0
+#ifndef GABM_GATHER_PAIRS
+#define GABM_GATHER_PAIRS 2
 #endif
 #ifndef GABM_MINBLOCKS
 #define GABM_MINBLOCKS 3
 #endif
-constexpr int kUnroll = GABM_UNROLL;   // entries per lane loaded ahead of use
+// Pairs of entries per lane loaded ahead of use: by the gathers (whose kernels have little
+// register room left) and by the marked sums.
+constexpr int kGP = GABM_GATHER_PAIRS;
+constexpr int kMP = 4;
 
 __device__ __forceinline__ void kahan_add(float &s, float &c, float x) {
     const float y = __fsub_rn(x, c);
@@ -52,6 +49,12 @@ __device__ __forceinline__ float infectiousness(int e_j, const float *c_s, int t
     const int k = t - e_j;
     return ((unsigned)(k - 1) < (unsigned)(L - 1)) ? c_s[k] : 0.f;
 }
+
+// A compile-time width.
+template <int N>
+struct Width {
+    static constexpr int value = N;
+};
 
 // Whether row j is marked in a per-day bitmap of infectious rows (read-only during the launch).
 __device__ __forceinline__ bool marked(const uint32_t *__restrict__ bits, uint32_t j) {
@@ -97,9 +100,9 @@ struct TileDispenser {
     }
 };
 
-// Hands each block one contiguous range of tiles, claimed tile by tile by its
-// warps through a shared-memory counter.  Rows are laid out breadth-first, so
-// the neighbours of a range's rows mostly lie in and around the same range:
+// Hands each block one contiguous range of tiles; its warps take the first two rounds in
+// order and the rest one at a time through a shared-memory counter.  Rows are laid out in
+// groups, so the neighbours of a range's rows mostly lie in and around the same range:
 // the warps of a block gather from lines their own SM has just cached, where a
 // launch-wide counter would spread consecutive tiles over all SMs.  (Measured
 // on the 1M-agent typed graph: 10% shorter day kernels than the launch-wide
@@ -109,57 +112,65 @@ struct TileDispenser {
 // imbalance cost 7%.)  Called by every thread of the block (init holds a barrier).
 struct BlockTiles {
     int *ctr;          // the block's counter (shared memory)
-    int end, ntiles, lane, pend;
+    int end, ntiles, lane, pend, given, first, nw;
     __device__ __forceinline__ void init(int nt, int ln) {
         __shared__ int s_ctr;
         ntiles = nt;
         lane = ln;
+        nw = (int)(blockDim.x >> 5);
         const int b0 = (int)(((long long)blockIdx.x * nt) / gridDim.x);
         end = (int)(((long long)(blockIdx.x + 1) * nt) / gridDim.x);
-        if (threadIdx.x == 0) s_ctr = b0;
+        first = b0 + (int)(threadIdx.x >> 5);
+        given = 0;
+        pend = 0;
+        if (threadIdx.x == 0) s_ctr = b0 + 2 * nw;
         __syncthreads();
         ctr = &s_ctr;
-        pend = (lane == 0) ? atomicAdd(ctr, 1) : 0;
     }
     // the next tile of this warp, or ntiles when the block's range is done
     __device__ __forceinline__ int get() {
-        const int tile = __shfl_sync(0xffffffffu, pend, 0);
-        if (tile >= end) return ntiles;
-        if (lane == 0) pend = atomicAdd(ctr, 1);
-        return tile;
+        int tile;
+        if (given < 2) {
+            tile = first + given * nw;
+            if (++given == 2 && lane == 0) pend = atomicAdd(ctr, 1);
+        } else {
+            tile = __shfl_sync(0xffffffffu, pend, 0);
+            if (tile < end && lane == 0) pend = atomicAdd(ctr, 1);
+        }
+        return tile < end ? tile : ntiles;
     }
 };
 
-// Ask L2 to fetch one slice (entries [p0, p1) of both arrays) ahead of use.
-// Slices start on 128-byte boundaries and hold multiples of 32 entries.
-__device__ __forceinline__ void prefetch_slice(const Sell &m, uint32_t p0, uint32_t p1, int lane) {
-    if (GABM_PREFETCH == 0) return;
-    if (lane == 0 && p1 > p0) {
-        const uint32_t bytes = (p1 - p0) * 4u;
-        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;\n" ::"l"(m.col + p0), "r"(bytes) : "memory");
-        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;\n" ::"l"(m.w + p0), "r"(bytes) : "memory");
-    }
-}
-
-// Warp sums of v by bin (bins 0..15; lanes with nothing to add pass v = 0): a
-// reduce-scatter over the lanes, each step keeping half of a lane's bins and receiving
-// the same half from the partner lane, 16 shuffles for all 16 bins (a butterfly per bin
-// would take 80).  On return lanes 2b and 2b + 1 hold bin b's sum.  The addition tree is
-// fixed, so the sums do not depend on anything but the inputs.  Called by all 32 lanes.
-__device__ __forceinline__ float warp_bin_sums16(float v, int bin, int lane) {
+// Warp sums of v by age bin.  Bin b's 32 values lie in shared memory (the warp's `cells`,
+// zero outside this call), even lanes' in its row 2b, odd lanes' in row 2b + 1; lane r < 2
+// kAges sums row r with four 16-byte loads and the two rows' sums meet in one shuffle: lanes
+// 2b and 2b + 1 return bin b's sum.  About 30 instructions for all bins, where a
+// reduce-scatter over the lanes took 100 and a butterfly per bin 200.  The addition tree is
+// the butterfly's (lanes 16 apart first, neighbours last), so the sums do not depend on
+// anything but the inputs.  Rows are 20 words apart: eight lanes' 16-byte loads then cover
+// all banks once.  Called by all 32 lanes; lanes with nothing to add pass v = 0.
+constexpr int kBinStride = 20;
+constexpr int kBinWords = 2 * kAges * kBinStride;   // shared-memory words per warp
+__device__ __forceinline__ float warp_bin_sums(float v, int bin, int lane, float *cells) {
+    float *cell = cells + (2 * bin + (lane & 1)) * kBinStride + (lane >> 1);
+    *cell = v;
+    __syncwarp();
     float x[16];
+    if (lane < 2 * kAges) {
 #pragma unroll
-    for (int b = 0; b < 16; ++b) x[b] = (bin == b) ? v : 0.f;
-#pragma unroll
-    for (int h = 8, o = 16; h >= 1; h >>= 1, o >>= 1) {
-        const bool hi = (lane & o) != 0;
-#pragma unroll
-        for (int i = 0; i < h; ++i) {
-            const float send = hi ? x[i] : x[i + h];
-            const float keep = hi ? x[i + h] : x[i];
-            x[i] = __fadd_rn(keep, __shfl_xor_sync(0xffffffffu, send, o));
+        for (int i = 0; i < 4; ++i) {
+            const float4 q = *reinterpret_cast<const float4 *>(cells + lane * kBinStride + 4 * i);
+            x[4 * i] = q.x; x[4 * i + 1] = q.y; x[4 * i + 2] = q.z; x[4 * i + 3] = q.w;
         }
+#pragma unroll
+        for (int h = 8; h >= 1; h >>= 1)
+#pragma unroll
+            for (int i = 0; i < h; ++i) x[i] = __fadd_rn(x[i], x[i + h]);
+    } else {
+        x[0] = 0.f;
     }
+    __syncwarp();
+    *cell = 0.f;
     return __fadd_rn(x[0], __shfl_xor_sync(0xffffffffu, x[0], 1));
 }
 
@@ -168,7 +179,7 @@ struct TileRows {
     int tile;
     int e;            // exposure day of this lane's row
     uint32_t len;     // entries of this lane's row
-    uint32_t p0, p1;  // the tile's slice bounds
+    uint32_t p0;      // the tile's slice
     int g;            // graph of the tile
     bool flag;        // the row has an infectious in-neighbour today (true without flags)
 };
@@ -179,7 +190,7 @@ __device__ __forceinline__ void load_tile_rows(const Sell &m, const int16_t *e, 
     tr.tile = tile;
     tr.e = kPad;
     tr.len = 0;
-    tr.p0 = tr.p1 = 0;
+    tr.p0 = 0;
     tr.g = 0;
     tr.flag = true;
     if (tile < ntiles) {
@@ -187,27 +198,47 @@ __device__ __forceinline__ void load_tile_rows(const Sell &m, const int16_t *e, 
         tr.e = e[row];
         tr.len = m.row_len[row];
         tr.p0 = m.slice_ptr[tile];
-        tr.p1 = m.slice_ptr[tile + 1];
         tr.g = tile_graph ? (int)tile_graph[tile] : 0;
         if (flags) tr.flag = flags[row] != 0;
     }
 }
 
+// The column and weight of entry k of the row in lane r of a slice.
+__device__ __forceinline__ const uint2 *entry_ptr(const Sell &m, uint32_t p0, uint32_t k, int r) {
+    return reinterpret_cast<const uint2 *>(m.cw + p0 + 32u * (k >> 1) + (uint32_t)r) + (k & 1u);
+}
+
 // Sets flags[j] = 1 for every out-neighbour j of the tile rows whose lane has `push`
-// (one byte store each: every writer stores the same value, so the result does not
-// depend on their order).  The warp takes those rows one at a time, its lanes splitting
-// the row's entries (entry k of tile row r sits at slice_ptr[tile] + 32 k + r), so a
-// row costs a load round trip per 32 entries.  Called by all 32 lanes.
+// (byte stores: every writer stores the same value, so the result does not depend on
+// their order).  Up to two rows: one at a time, the lanes splitting the row's entries.
+// More: every lane walks its own row, kMP pairs in flight; taken one at a time, the rows
+// of a tile with a dozen infectious agents would cost a dozen load round trips in a row.
+// Called by all 32 lanes.
 __device__ __forceinline__ void push_flags(const Sell &m_out, int tile, int lane, bool push, uint8_t *flags) {
     unsigned rows = __ballot_sync(0xffffffffu, push);
     if (!rows) return;
     const uint32_t base = m_out.slice_ptr[tile];
     const uint32_t my_len = push ? m_out.row_len[tile * kTile + lane] : 0u;
-    while (rows) {
-        const int r = __ffs(rows) - 1;
-        rows &= rows - 1u;
-        const uint32_t len = __shfl_sync(0xffffffffu, my_len, r);
-        for (uint32_t k = (uint32_t)lane; k < len; k += 32u) flags[__ldg(m_out.col + base + 32u * k + (uint32_t)r)] = 1;
+    if (__popc(rows) <= 2) {
+        while (rows) {
+            const int r = __ffs(rows) - 1;
+            rows &= rows - 1u;
+            const uint32_t len = __shfl_sync(0xffffffffu, my_len, r);
+            for (uint32_t k = (uint32_t)lane; k < len; k += 32u) flags[__ldg(&entry_ptr(m_out, base, k, r)->x)] = 1;
+        }
+        return;
+    }
+    const uint32_t np = (my_len + 1u) >> 1;
+    const uint4 *row = m_out.cw + base + (uint32_t)lane;
+    for (uint32_t q0 = 0; q0 < np; q0 += kMP) {
+        uint4 v[kMP];
+#pragma unroll
+        for (int u = 0; u < kMP; ++u) v[u] = __ldg(row + 32u * min(q0 + (uint32_t)u, np - 1u));
+#pragma unroll
+        for (int u = 0; u < kMP; ++u) {
+            if (q0 + (uint32_t)u < np) flags[v[u].x] = 1;
+            if (2u * (q0 + (uint32_t)u) + 1u < my_len) flags[v[u].z] = 1;
+        }
     }
 }
 
@@ -245,105 +276,209 @@ __device__ __forceinline__ int ld_if(const int16_t *p, bool pred, int dflt) {
     return v;
 }
 
-// For this lane's row (when act), sum[a] = the sum of contribution a over the
-// row's entries in entry order, with compensated summation; f(j, w, valid, out, take)
-// writes the NARR contributions of the entry with column j and weight w and whether
-// each is added (it is also called for invalid entries -- padding, other rows'
-// tails -- and must then touch no memory beyond the slice and take nothing), and
-// want[a] says whether sum a is taken for this row.  A sum of marked neighbours'
-// infectiousness takes the marked entries only: the compensated sum of a row is then
-// a function of its marked entries in entry order, however they are visited
-// (row_sums here, or a warp walking one row).  Called by all 32 lanes; the batch runs
-// without branches.
-// No all-taken contribution: every batch goes through f.
-struct NoFull {};
+// ---- sums over a tile's rows ------------------------------------------------
+// What a tile's 32 lanes sum, worked out once per tile by all of them.
+struct TileSpan {
+    const uint4 *row;   // pair q of this lane's row at row[32 q]
+    uint32_t len;       // entries this lane sums (0: nothing)
+    uint32_t lim;       // pairs this lane loads: mostly-active slices are read whole, sparse ones row by row
+    uint32_t np;        // pairs of the longest summing row (warp-uniform)
+    uint32_t kfull;     // entries below this are valid in every lane (warp-uniform)
+};
 
-template <int NARR, class F, class FF = NoFull>
-__device__ __forceinline__ void row_sums(const Sell &m, uint32_t p0, uint32_t len, bool act, int lane, F f,
-                                         const bool (&want)[NARR], float (&sum)[NARR], FF ff = NoFull{}) {
-    constexpr bool HAS_FULL = !std::is_same<FF, NoFull>::value;
-    static_assert(!HAS_FULL || NARR == 1, "the all-taken path sums one contribution");
-    float comp[NARR];
+__device__ __forceinline__ TileSpan tile_span(const Sell &m, uint32_t p0, uint32_t len, bool act, int lane) {
+    TileSpan s;
+    s.row = m.cw + p0 + (uint32_t)lane;
+    s.len = act ? len : 0u;
+    s.np = (__reduce_max_sync(0xffffffffu, s.len) + 1u) >> 1;
+    s.kfull = __reduce_min_sync(0xffffffffu, s.len);
+    s.lim = __popc(__ballot_sync(0xffffffffu, act)) >= 24 ? s.np : (s.len + 1u) >> 1;
+    return s;
+}
+
+// Pairs [q0, q0 + UP) of the lane's row below its limit; the others keep what they held
+// (columns of some row, or 0: nothing is added for them).
+template <int UP>
+__device__ __forceinline__ void load_pairs(const uint4 *row, uint32_t q0, uint32_t lim, uint4 (&v)[UP]) {
 #pragma unroll
-    for (int a = 0; a < NARR; ++a) { sum[a] = 0.f; comp[a] = 0.f; }
-    const unsigned amask = __ballot_sync(0xffffffffu, act);
-    const uint32_t kmax = __reduce_max_sync(0xffffffffu, act ? len : 0u);
-    // Mostly-active slices are read whole (padding and inactive rows included: every
-    // entry below kmax lies inside the slice); sparse ones with predicated loads.
-    const bool dense = __popc(amask) >= 24;
-    // Batches wholly below every lane's row length (all lanes summing) have every entry
-    // valid: with ff (the contribution of a valid entry when every valid entry is taken,
-    // ff(j, w) = what f gives) they run without predicates or selects; the operations
-    // and their order are those of the predicated path, so the sums are bitwise equal.
-    uint32_t kfull = 0u;
-    if constexpr (HAS_FULL) {
-        const unsigned fmask = __ballot_sync(0xffffffffu, act && want[0]);
-        kfull = __reduce_min_sync(0xffffffffu, (fmask == 0xffffffffu) ? len : 0u);
-    }
-    auto load_batch = [&](uint32_t k0, uint32_t (&jv)[kUnroll], float (&wv)[kUnroll]) {
-        if (HAS_FULL && dense && k0 + (uint32_t)kUnroll <= kmax) {   // inside the slice: no predicates
+    for (int u = 0; u < UP; ++u)
+        if (q0 + (uint32_t)u < lim) v[u] = __ldcs(row + 32u * (q0 + (uint32_t)u));
+}
+
+// sum of w x[j] over the lane's entries, in entry order with compensated summation.  `ea`
+// holds the first kGP pairs (load_pairs(row, 0, lim, ea), issued by the caller well ahead:
+// before the previous tile's epilogue).  The next batch of pairs is in flight while one is
+// used.  Batches in which every lane's entries are valid run without predicates; in the
+// others an invalid entry adds y = 0, which leaves the sum as it is (entries are invalid
+// from some k on, so the compensation it spoils is not used again).
+__device__ __forceinline__ float gather_sum(const TileSpan &s, const float *__restrict__ x, uint4 (&ea)[kGP]) {
+    float sum = 0.f, comp = 0.f;
+    auto use = [&](uint32_t q0, const uint4 (&v)[kGP]) {
+        float g[2 * kGP];
+        if (2u * q0 + 2u * kGP <= s.kfull) {
 #pragma unroll
-            for (int u = 0; u < kUnroll; ++u) {
-                const uint32_t idx = p0 + (k0 + (uint32_t)u) * 32u + (uint32_t)lane;
-                jv[u] = __ldcs(m.col + idx);
-                wv[u] = __ldcs(m.w + idx);
+            for (int u = 0; u < kGP; ++u) {
+                g[2 * u] = x[v[u].x];
+                g[2 * u + 1] = x[v[u].z];
+            }
+#pragma unroll
+            for (int u = 0; u < kGP; ++u) {
+                kahan_add(sum, comp, __uint_as_float(v[u].y) * g[2 * u]);
+                kahan_add(sum, comp, __uint_as_float(v[u].w) * g[2 * u + 1]);
             }
             return;
         }
 #pragma unroll
-        for (int u = 0; u < kUnroll; ++u) {
-            const uint32_t k = k0 + (uint32_t)u;
-            const uint32_t idx = p0 + k * 32u + (uint32_t)lane;
-            if (dense) {
-                const bool in = k < kmax;
-                jv[u] = ld_cs_if(m.col + idx, in);
-                wv[u] = ld_cs_if(m.w + idx, in);
-            } else {
-                const bool v = act && k < len;
-                jv[u] = ld_cs_if(m.col + idx, v);
-                wv[u] = ld_cs_if(m.w + idx, v);
-            }
+        for (int u = 0; u < kGP; ++u) {
+            const uint32_t k = 2u * (q0 + (uint32_t)u);
+            g[2 * u] = k < s.len ? x[v[u].x] : 0.f;
+            g[2 * u + 1] = k + 1u < s.len ? x[v[u].z] : 0.f;
+        }
+#pragma unroll
+        for (int i = 0; i < 2 * kGP; ++i) {
+            const float w = __uint_as_float((i & 1) ? v[i >> 1].w : v[i >> 1].y);
+            const float y = (2u * q0 + (uint32_t)i < s.len) ? __fsub_rn(w * g[i], comp) : 0.f;
+            const float t = __fadd_rn(sum, y);
+            comp = __fsub_rn(__fsub_rn(t, sum), y);
+            sum = t;
         }
     };
-    auto use_batch = [&](uint32_t k0, const uint32_t (&jv)[kUnroll], const float (&wv)[kUnroll]) {
-        if constexpr (HAS_FULL) {
-            if (k0 + (uint32_t)kUnroll <= kfull) {
+    uint4 eb[kGP];
 #pragma unroll
-                for (int u = 0; u < kUnroll; ++u) kahan_add(sum[0], comp[0], ff(jv[u], wv[u]));
-                return;
-            }
+    for (int u = 0; u < kGP; ++u) eb[u] = make_uint4(0u, 0u, 0u, 0u);
+    for (uint32_t q = 0; q < s.np; q += 2 * kGP) {
+        if (q + kGP < s.np) load_pairs(s.row, q + kGP, s.lim, eb);
+        use(q, ea);
+        if (q + kGP >= s.np) break;
+        if (q + 2 * kGP < s.np) load_pairs(s.row, q + 2 * kGP, s.lim, ea);
+        use(q + kGP, eb);
+    }
+    return sum;
+}
+
+// gather_sum that loads its own first pairs.
+__device__ __forceinline__ float gather_sum(const Sell &m, uint32_t p0, uint32_t len, bool act, int lane,
+                                            const float *__restrict__ x) {
+    const TileSpan s = tile_span(m, p0, len, act, lane);
+    uint4 ea[kGP];
+#pragma unroll
+    for (int u = 0; u < kGP; ++u) ea[u] = make_uint4(0u, 0u, 0u, 0u);
+    load_pairs(s.row, 0u, s.lim, ea);
+    return gather_sum(s, x, ea);
+}
+
+// sum of w c[t - e_j] over the lane's entries whose neighbour j is infectious on day t: marked
+// in `bits` and 1 <= t - e_j < L.  Only those entries are added, in entry order with
+// compensated summation, so a row's value is a function of its marked entries however
+// they are visited.  Entries go 32 at a time: first every entry's bit is tested (the
+// bitmap is small enough for L1) and the marks collected in one word per lane; then the
+// lanes walk their marks, two or four at a time, reading the entry again and the
+// neighbour's exposure day.  On a typical day one entry in twenty is marked, and the
+// longest lane has three or four marks, so this runs about a third of the instructions of
+// a pass that carries every entry through the lookup and the compensated addition.
+template <bool SHARED_BITS = false, int UP = kMP>
+__device__ __forceinline__ float marked_sum(const Sell &m, uint32_t p0, uint32_t len, bool act, int lane,
+                                            const uint32_t *bits, const int16_t *e, const float *c_s, int t, int L) {
+    const TileSpan s = tile_span(m, p0, len, act, lane);
+    float sum = 0.f, comp = 0.f;
+    uint4 ea[UP], eb[UP];
+#pragma unroll
+    for (int u = 0; u < UP; ++u) ea[u] = eb[u] = make_uint4(0u, 0u, 0u, 0u);
+    load_pairs(s.row, 0u, s.lim, ea);
+    uint32_t mask = 0u;
+    auto word = [&](uint32_t j) { return (SHARED_BITS ? bits[j >> 5] : __ldg(bits + (j >> 5))) >> (j & 31u); };
+    auto test = [&](uint32_t q0, const uint4 (&v)[UP]) {
+        uint32_t w[2 * UP];
+#pragma unroll
+        for (int u = 0; u < UP; ++u) {
+            const uint32_t k = 2u * (q0 + (uint32_t)u);
+            w[2 * u] = k < s.len ? word(v[u].x) : 0u;
+            w[2 * u + 1] = k + 1u < s.len ? word(v[u].z) : 0u;
+        }
+        const uint32_t sh = (2u * q0) & 31u;
+        uint32_t mk = 0u;
+#pragma unroll
+        for (int i = 0; i < 2 * UP; ++i) mk |= (w[i] & 1u) << i;
+        mask |= mk << sh;
+    };
+    auto take = [&](uint32_t k0, auto width) {
+        constexpr int W = decltype(width)::value;
+        uint2 v[W];
+        int ej[W];
+        bool ok[W];
+#pragma unroll
+        for (int i = 0; i < W; ++i) {
+            ok[i] = mask != 0u;
+            const uint32_t k = k0 + (uint32_t)(ok[i] ? __ffs(mask) - 1 : 0);
+            mask &= mask - 1u;
+            v[i] = make_uint2(0u, 0u);
+            if (ok[i]) v[i] = __ldg(reinterpret_cast<const uint2 *>(s.row + 32u * (k >> 1)) + (k & 1u));
         }
 #pragma unroll
-        for (int u = 0; u < kUnroll; ++u) {
-            const uint32_t k = k0 + (uint32_t)u;
-            const bool valid = act && k < len;
-            float out[NARR];
-            bool take[NARR];
-            f(jv[u], wv[u], valid, out, take);
+        for (int i = 0; i < W; ++i) ej[i] = ok[i] ? (int)e[v[i].x] : kNever;
 #pragma unroll
-            for (int a = 0; a < NARR; ++a) kahan_add_if(sum[a], comp[a], out[a], take[a] && want[a]);
+        for (int i = 0; i < W; ++i) {
+            const int k = t - ej[i];
+            const bool tk = (unsigned)(k - 1) < (unsigned)(L - 1);
+            kahan_add_if(sum, comp, tk ? __uint_as_float(v[i].y) * c_s[k] : 0.f, tk);
         }
     };
-    if (GABM_PIPE) {
-        // the next batch is in flight while the current one is used
-        uint32_t ja[kUnroll], jb[kUnroll];
-        float wa[kUnroll], wb[kUnroll];
-        if (kmax > 0) load_batch(0, ja, wa);
-        for (uint32_t k0 = 0; k0 < kmax; k0 += 2 * kUnroll) {
-            if (k0 + kUnroll < kmax) load_batch(k0 + kUnroll, jb, wb);
-            use_batch(k0, ja, wa);
-            if (k0 + kUnroll >= kmax) break;
-            if (k0 + 2 * kUnroll < kmax) load_batch(k0 + 2 * kUnroll, ja, wa);
-            use_batch(k0 + kUnroll, jb, wb);
-        }
-    } else {
-        for (uint32_t k0 = 0; k0 < kmax; k0 += kUnroll) {
-            uint32_t jv[kUnroll];
-            float wv[kUnroll];
-            load_batch(k0, jv, wv);
-            use_batch(k0, jv, wv);
+    for (uint32_t q = 0; q < s.np; q += 2 * UP) {
+        if (q + UP < s.np) load_pairs(s.row, q + UP, s.lim, eb);
+        test(q, ea);
+        if (q + 2 * UP < s.np) load_pairs(s.row, q + 2 * UP, s.lim, ea);
+        if (q + UP < s.np) test(q + UP, eb);
+        if (((q + 2 * UP) & 15u) == 0u || q + 2 * UP >= s.np) {   // 32 entries tested, or the last
+            const uint32_t k0 = (2u * q) & ~31u;
+            for (unsigned n = __reduce_max_sync(0xffffffffu, (unsigned)__popc(mask)); n > 0u;) {
+                if (n > 2u) {
+                    take(k0, Width<4>{});
+                    n = n > 4u ? n - 4u : 0u;
+                } else {
+                    take(k0, Width<2>{});
+                    n = 0u;
+                }
+            }
         }
     }
+    return sum;
+}
+
+// marked_sum without the bitmap: every entry's exposure day is gathered and tested, which
+// takes the same entries (an exposure during day t itself gives t - e_j = 0).  One
+// scattered load per entry: the cheaper way once a good share of the rows is infectious.
+__device__ __forceinline__ float exposed_sum(const Sell &m, uint32_t p0, uint32_t len, bool act, int lane,
+                                             const int16_t *e, const float *c_s, int t, int L) {
+    const TileSpan s = tile_span(m, p0, len, act, lane);
+    float sum = 0.f, comp = 0.f;
+    uint4 ea[kMP], eb[kMP];
+#pragma unroll
+    for (int u = 0; u < kMP; ++u) ea[u] = eb[u] = make_uint4(0u, 0u, 0u, 0u);
+    load_pairs(s.row, 0u, s.lim, ea);
+    auto use = [&](uint32_t q0, const uint4 (&v)[kMP]) {
+        int ej[2 * kMP];
+#pragma unroll
+        for (int u = 0; u < kMP; ++u) {
+            const uint32_t k = 2u * (q0 + (uint32_t)u);
+            ej[2 * u] = k < s.len ? (int)e[v[u].x] : kNever;
+            ej[2 * u + 1] = k + 1u < s.len ? (int)e[v[u].z] : kNever;
+        }
+#pragma unroll
+        for (int i = 0; i < 2 * kMP; ++i) {
+            const float w = __uint_as_float((i & 1) ? v[i >> 1].w : v[i >> 1].y);
+            const int k = t - ej[i];
+            const bool tk = (unsigned)(k - 1) < (unsigned)(L - 1);
+            kahan_add_if(sum, comp, tk ? w * c_s[k] : 0.f, tk);
+        }
+    };
+    for (uint32_t q = 0; q < s.np; q += 2 * kMP) {
+        if (q + kMP < s.np) load_pairs(s.row, q + kMP, s.lim, eb);
+        use(q, ea);
+        if (q + kMP >= s.np) break;
+        if (q + 2 * kMP < s.np) load_pairs(s.row, q + 2 * kMP, s.lim, ea);
+        use(q + kMP, eb);
+    }
+    return sum;
 }
 
 // Tiles with at most this many summing rows have them summed one row at a time by the
@@ -353,50 +488,44 @@ __device__ __forceinline__ void row_sums(const Sell &m, uint32_t p0, uint32_t le
 #endif
 
 // The sum of one row's taken contributions by the whole warp: the row of tile lane r
-// (entries [0, len) at p0 + 32 k + r), the result in lane r's sum / comp.  The lanes
-// load 32 entries at a time and evaluate f as row_sums does; lane r then adds the taken
-// ones in entry order with the same compensated addition, so the value is row_sums'.
-// Called by all 32 lanes.
+// (entries [k_first, len)), the result in lane r's sum / comp.  The lanes load 32 entries at
+// a time and f(j, w, valid, out, take) gives an entry's contribution and whether it is
+// added; lane r then adds the taken ones in entry order with the same compensated
+// addition, so the value is marked_sum's.  Called by all 32 lanes.
 template <class F>
 __device__ __forceinline__ void warp_row_sum_from(const Sell &m, uint32_t p0, uint32_t len, uint32_t k_first, int r,
                                                   int lane, F f, float &sum, float &comp) {
     for (uint32_t k0 = k_first; k0 < len; k0 += 32u) {
         const uint32_t k = k0 + (uint32_t)lane;
         const bool valid = k < len;
-        const uint32_t idx = p0 + k * 32u + (uint32_t)r;
-        const uint32_t j = ld_cs_if(m.col + idx, valid);
-        const float w = ld_cs_if(m.w + idx, valid);
-        float out[1];
-        bool take[1];
-        f(j, w, valid, out, take);
-        unsigned mm = __ballot_sync(0xffffffffu, take[0]);
+        uint2 v = make_uint2(0u, 0u);
+        if (valid) v = __ldg(entry_ptr(m, p0, k, r));
+        float out;
+        bool take;
+        f(v.x, __uint_as_float(v.y), valid, out, take);
+        unsigned mm = __ballot_sync(0xffffffffu, take);
         while (mm) {
             const int src = __ffs(mm) - 1;
             mm &= mm - 1u;
-            const float v = __shfl_sync(0xffffffffu, out[0], src);
-            if (lane == r) kahan_add(sum, comp, v);
+            const float x = __shfl_sync(0xffffffffu, out, src);
+            if (lane == r) kahan_add(sum, comp, x);
         }
     }
 }
 
-template <class F>
-__device__ __forceinline__ void warp_row_sum(const Sell &m, uint32_t p0, uint32_t len, int r, int lane, F f,
-                                             float &sum, float &comp) {
-    warp_row_sum_from(m, p0, len, 0u, r, lane, f, sum, comp);
-}
-
-// warp_row_sum for up to GABM_COOP_ROWS rows of a tile at once (the rows of `amask`), so
+// warp_row_sum_from for up to GABM_COOP_ROWS rows of a tile at once (the rows of `amask`), so
 // that their loads overlap: the first 32 entries of every row are loaded, tested and
-// gathered together, then each row's lane adds its taken contributions in entry order;
-// entries past the first 32 go through warp_row_sum.  Each row's value is row_sums'.
-// sum / comp: this lane's row (lanes without a row keep 0).  Called by all 32 lanes.
+// gathered together, then each row's lane adds its taken contributions in entry order.
+// Each row's value is marked_sum's.  Lanes without a row return 0.  Called by all 32 lanes.
 template <class F>
-__device__ __forceinline__ void few_row_sums(const Sell &m, uint32_t p0, uint32_t my_len, unsigned amask, int lane,
-                                             F f, float &sum, float &comp) {
+__device__ __forceinline__ float few_row_sums(const Sell &m, uint32_t p0, uint32_t my_len, unsigned amask, int lane,
+                                              F f) {
     constexpr int K = GABM_COOP_ROWS;
+    float sum = 0.f, comp = 0.f;
     int r[K];
-    uint32_t len[K], j[K];
-    float w[K], out[K];
+    uint32_t len[K];
+    uint2 v[K];
+    float out[K];
     bool take[K];
     unsigned mm = amask;
 #pragma unroll
@@ -405,33 +534,25 @@ __device__ __forceinline__ void few_row_sums(const Sell &m, uint32_t p0, uint32_
         mm &= mm - 1u;
         len[i] = __shfl_sync(0xffffffffu, my_len, r[i] < 0 ? 0 : r[i]);
         if (r[i] < 0) len[i] = 0u;
-        const bool valid = (uint32_t)lane < len[i];
-        const uint32_t idx = p0 + (uint32_t)lane * 32u + (uint32_t)(r[i] < 0 ? 0 : r[i]);
-        j[i] = ld_cs_if(m.col + idx, valid);
-        w[i] = ld_cs_if(m.w + idx, valid);
+        v[i] = make_uint2(0u, 0u);
+        if ((uint32_t)lane < len[i]) v[i] = __ldg(entry_ptr(m, p0, (uint32_t)lane, r[i]));
     }
 #pragma unroll
-    for (int i = 0; i < K; ++i) {
-        float o[1];
-        bool tk[1];
-        f(j[i], w[i], (uint32_t)lane < len[i], o, tk);
-        out[i] = o[0];
-        take[i] = tk[0];
-    }
+    for (int i = 0; i < K; ++i) f(v[i].x, __uint_as_float(v[i].y), (uint32_t)lane < len[i], out[i], take[i]);
 #pragma unroll
     for (int i = 0; i < K; ++i) {
         unsigned tm = __ballot_sync(0xffffffffu, take[i]);
         while (tm) {
             const int src = __ffs(tm) - 1;
             tm &= tm - 1u;
-            const float v = __shfl_sync(0xffffffffu, out[i], src);
-            if (lane == r[i]) kahan_add(sum, comp, v);
+            const float x = __shfl_sync(0xffffffffu, out[i], src);
+            if (lane == r[i]) kahan_add(sum, comp, x);
         }
     }
 #pragma unroll
     for (int i = 0; i < K; ++i)
-        if (__shfl_sync(0xffffffffu, len[i], 0) > 32u)   // len[i] is warp-uniform
-            warp_row_sum_from(m, p0, len[i], 32u, r[i], lane, f, sum, comp);
+        if (len[i] > 32u) warp_row_sum_from(m, p0, len[i], 32u, r[i], lane, f, sum, comp);   // len[i]: warp-uniform
+    return sum;
 }
 
 }  // namespace gabm

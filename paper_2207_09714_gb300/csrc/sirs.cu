@@ -1,7 +1,7 @@
 // sirs.cu -- forward and reverse day kernels of SIRS reinfection (see sirs.cuh).
 //
 // Each warp holds one 32-row tile at a time.  The sums
-// are those of the base model's kernels -- the same row_sums over the same SELL entries,
+// are those of the base model's kernels -- the same row sums over the same SELL entries,
 // the same fused multiply-adds in the same order for G -- so with nobody returning
 // within the horizon the results are bitwise the base model's.
 #include "sirs.cuh"
@@ -53,13 +53,11 @@ __global__ void __launch_bounds__(kBlock, 3) k_fwd_day_sirs(const SirsFwdArgs a)
     const uint32_t *bits = a.bits_cur;
     const int16_t *e = a.e;
     // neighbours marked infectious today (never written by this launch) contribute
-    auto contrib = [&](uint32_t j, float w, bool valid, float (&out)[1], bool (&take)[1]) {
-        const bool mk = valid && marked(bits, j);
-        const int ej = ld_if(e + j, mk, kNever);
-        out[0] = mk ? w * infectiousness(ej, c_s, t, L) : 0.f;
-        take[0] = mk;
+    auto contrib = [&](uint32_t j, float w, bool valid, float &out, bool &take) {
+        take = valid && marked(bits, j);
+        const int ej = ld_if(e + j, take, kNever);
+        out = take ? w * infectiousness(ej, c_s, t, L) : 0.f;
     };
-    const bool want[1] = {true};
     int cur_g = -1, cS = 0, cE = 0, cI = 0, cR = 0, cN = 0;
     BlockTiles disp;
     disp.init(ntiles, lane);
@@ -86,18 +84,16 @@ __global__ void __launch_bounds__(kBlock, 3) k_fwd_day_sirs(const SirsFwdArgs a)
         }
         cS += isS;
         const bool act = isS && cur.flag;
-        float sum[1];
+        float sum = 0.f;
         const unsigned amask = __ballot_sync(0xffffffffu, act);
         if (a.flag_cur && __popc(amask) <= GABM_COOP_ROWS) {   // few summing rows: warp-wide, together
-            float cs = 0.f;
-            sum[0] = 0.f;
-            if (amask) few_row_sums(a.m, cur.p0, cur.len, amask, lane, contrib, sum[0], cs);
+            if (amask) sum = few_row_sums(a.m, cur.p0, cur.len, amask, lane, contrib);
         } else {
-            row_sums<1>(a.m, cur.p0, cur.len, act, lane, contrib, want, sum);
+            sum = marked_sum(a.m, cur.p0, cur.len, act, lane, bits, e, c_s, t, L);
         }
         int e_next = ei;
         if (act) {
-            const float Lam = sum[0] * a.gr.inv_Dbar[g];
+            const float Lam = sum * a.gr.inv_Dbar[g];
             const float lam = (a.R[(size_t)g * a.ldP + t] * a.S[g * kAges + a.age[row]]) * Lam;
             const float p = -expm1f(-lam);
             const uint32_t id = caller_id(a.gr, row, g);
@@ -142,22 +138,20 @@ __device__ __forceinline__ TileRows nn_next(const SirsBwdArgs &a, BlockTiles &di
 // day t the adjoint of the draw, with the return terms B(t+1) and B(t+cycle) read from
 // the G stored at the row's later exposures.
 __global__ void __launch_bounds__(kBlock, 3) k_bwd_day_sirs(const SirsBwdArgs a) {
-    __shared__ float c_s[kMaxL];
-    __shared__ int slot_k[kMaxL];
-    if (threadIdx.x < kMaxL) {
-        c_s[threadIdx.x] = a.c[threadIdx.x];
-        slot_k[threadIdx.x] = a.ring_slot[threadIdx.x];
-    }
-    __syncthreads();
-    const int lane = threadIdx.x & 31;
+    constexpr int NW = kBlock / 32;
+    constexpr int RB = 8;   // ring slots loaded together
+    __shared__ float cf_s[NW][kMaxL];    // c[k] 2^(sigma(t+k) - sigma(t)) of the days that carry adjoint,
+    __shared__ int off_s[NW][kMaxL];     // and their slots' offsets, k ascending from 2
+    __shared__ float rs_s[NW][kAges];    // R_t S_a of the warp's graph
+    __shared__ __align__(16) float bin_s[NW][kBinWords];
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    for (int i = lane; i < kBinWords; i += 32) bin_s[wib][i] = 0.f;
+    __syncwarp();
     const int t = a.t, T = a.T, L = a.L, C = a.cycle, H = a.H;
-    const bool has_next = t + 1 < T;
-    const float *__restrict__ r_next = a.r_next;
-    auto contrib = [&](uint32_t j, float w, bool valid, float (&out)[1], bool (&take)[1]) {
-        out[0] = w * ld_if(r_next + j, valid);
-        take[0] = valid;
-    };
-    const bool want[1] = {true};
+    const int slot_floats = (L - 1) * kTile;
+    float cf1 = 0.f, gtail = 0.f, inv_D = 0.f;
+    int nterm = 0, sig_t = 0;
+    const int32_t *sg = nullptr;
     int cur_g = -1, cN = 0;
     unsigned emax_w = 0u, live_k = 0u;   // live_k bit k: day t + k carries adjoint
     bool rnz_w = false;
@@ -181,10 +175,25 @@ __global__ void __launch_bounds__(kBlock, 3) k_bwd_day_sirs(const SirsBwdArgs a)
             cur_g = g;
             cN = 0;
             live_k = carries_adjoint(a.rnz + (size_t)g * a.ld_sig, t, T, L);
+            sg = a.sig + (size_t)g * a.ld_sig;
+            sig_t = next_sigma(sg[t + 1], a.emax[(size_t)g * a.ld_sig + t + 1]);
+            if (lane == 0 && tile * kTile == a.gr.row0[g]) a.sig[(size_t)g * a.ld_sig + t] = sig_t;
+            const float cf = ((live_k >> lane) & 1u) ? a.c[lane] * exp2i(sg[t + lane] - sig_t) : 0.f;
+            cf1 = __shfl_sync(0xffffffffu, cf, 1);
+            const unsigned tm = live_k & ~3u;
+            nterm = __popc(tm);
+            __syncwarp();
+            if ((tm >> lane) & 1u) {
+                const int i = __popc(tm & ((1u << lane) - 1u));
+                off_s[wib][i] = a.ring_slot[lane] * kTile;
+                cf_s[wib][i] = cf;
+            }
+            const size_t pg = (size_t)g * a.ldP;
+            if (lane < kAges) rs_s[wib][lane] = a.R[pg + t] * a.S[g * kAges + lane];
+            inv_D = a.gr.inv_Dbar[g];
+            gtail = (t + L < T) ? a.m_t[pg + t + L] * (float)a.gD[pg + t + L] * exp2i(-sig_t) : 0.f;
+            __syncwarp();
         }
-        const int32_t *sg = a.sig + (size_t)g * a.ld_sig;
-        const int sig_t = next_sigma(sg[t + 1], a.emax[(size_t)g * a.ld_sig + t + 1]);
-        if (lane == 0 && tile * kTile == a.gr.row0[g]) a.sig[(size_t)g * a.ld_sig + t] = sig_t;
 
         const int row = tile * kTile + lane;
         const bool agent = cur.e != kPad;
@@ -204,28 +213,32 @@ __global__ void __launch_bounds__(kBlock, 3) k_bwd_day_sirs(const SirsBwdArgs a)
         bool covered = false;
         for (int j = 0; j < j_t; ++j) covered |= (hr[j] >= t - C + 1 && hr[j] <= lo - 1);
         const bool act = (live_k & 2u) && agent && !covered;
-        float sum[1];
-        row_sums<1>(a.m, cur.p0, cur.len, act, lane, contrib, want, sum,
-                    [&](uint32_t j, float w) { return w * r_next[j]; });
-        const float gx1 = sum[0];
-        if (act) a.ring[(size_t)slot_k[1] * a.ring_stride + row] = gx1;
+        // the row loads that do not depend on the sum go out before it
+        const float Lam = isS ? a.lam_t[row] : 0.f;
+        const int ai = isS ? (int)a.age[row] : 0;
+        const float gx1 = gather_sum(a.m, cur.p0, cur.len, act, lane, a.r_next);
+        float *ring = a.ring + (size_t)tile * slot_floats + lane;
+        if (act) ring[a.ring_slot[1] * kTile] = gx1;
 
         float v = 0.f, rc = 0.f;
-        int ai = 0;
         if (isS) {
-            ai = a.age[row];
             // B(t'): G at the row's first exposure on or after day t' (0 if none), at day t's scale
             auto B_at = [&](int tp) -> float {
                 int j = j_t;
                 while (j < n_e && hr[j] < tp) ++j;
                 return j < n_e ? a.Gh[(size_t)row * H + j] * exp2i(sg[hr[j]] - sig_t) : 0.f;
             };
-            const size_t pg = (size_t)g * a.ldP;
             // the day's own terms: the death term and the infectiousness it would cause
-            float loc = (t + L < T) ? a.m_t[pg + t + L] * (float)a.gD[pg + t + L] * exp2i(-sig_t) : 0.f;
-            if (has_next) loc = __fmaf_rn(c_s[1], gx1 * exp2i(sg[t + 1] - sig_t), loc);
-            for (int k = 2; k < L; ++k)
-                if ((live_k >> k) & 1u) loc = __fmaf_rn(c_s[k], a.ring[(size_t)slot_k[k] * a.ring_stride + row] * exp2i(sg[t + k] - sig_t), loc);
+            float loc = __fmaf_rn(cf1, gx1, gtail);
+            for (int j0 = 0; j0 < nterm; j0 += RB) {
+                float rv[RB];
+#pragma unroll
+                for (int u = 0; u < RB; ++u)
+                    if (j0 + u < nterm) rv[u] = ring[off_s[wib][j0 + u]];
+#pragma unroll
+                for (int u = 0; u < RB; ++u)
+                    if (j0 + u < nterm) loc = __fmaf_rn(cf_s[wib][j0 + u], rv[u], loc);
+            }
             const float G = loc + B_at(t + C);
             // dL/dy = G - B(t+1).  With t' the row's first exposure after t, B(t+1) = G(t'),
             // and B(t+C) = B(t'+C) when t' < t+C (the next exposure after t' is at least
@@ -240,8 +253,7 @@ __global__ void __launch_bounds__(kBlock, 3) k_bwd_day_sirs(const SirsBwdArgs a)
                 a.Lh[(size_t)row * H + j_t] = loc;
             }
             float stored = fmaxf(fabsf(G), fabsf(loc));
-            const float Lam = a.lam_t[row];
-            const float RS = a.R[pg + t] * a.S[g * kAges + ai];
+            const float RS = rs_s[wib][ai];
             const float lam = RS * Lam;
             float glam = dy;   // dy = 0 and lambda finite: the product with dy/dlambda >= 0 is dy itself
             if (!(dy == 0.f && lam >= 0.f && lam < __int_as_float(0x7f800000))) {
@@ -253,7 +265,7 @@ __global__ void __launch_bounds__(kBlock, 3) k_bwd_day_sirs(const SirsBwdArgs a)
                 const float dydl = (u * (1.f - u)) * q / (den * den);
                 glam = dy * dydl;
             }
-            rc = RS * glam * a.gr.inv_Dbar[g];
+            rc = RS * glam * inv_D;
             v = glam * Lam;
             stored = fmaxf(stored, fabsf(rc));
             rnz_w |= !(rc == 0.f);
@@ -261,9 +273,8 @@ __global__ void __launch_bounds__(kBlock, 3) k_bwd_day_sirs(const SirsBwdArgs a)
         }
         a.r_cur[row] = rc;   // 0 for rows not susceptible today (r of a later day may sit there)
 
-        const unsigned smask = __ballot_sync(0xffffffffu, isS);
         float mine = 0.f;   // lanes 2b, 2b + 1: bin b (the base kernel's tree)
-        if (smask) mine = warp_bin_sums16(isS ? v : 0.f, ai, lane);
+        if (__any_sync(0xffffffffu, !(v == 0.f))) mine = warp_bin_sums(v, ai, lane, bin_s[wib]);
         if (!(lane & 1) && (lane >> 1) < kAges) a.P_t[(size_t)tile * kAges + (lane >> 1)] = (double)mine;
     }
     if (cur_g >= 0) {

@@ -54,8 +54,7 @@ struct SirsBwdArgs {
     const float *lam_t;         // stored normalised sums of day t
     const float *r_next;        // r of day t + 1
     float *r_cur;               // r of day t (0 for rows not susceptible on day t)
-    float *ring;                // [L-1][n_rows] gx of the next L-1 days
-    size_t ring_stride;
+    float *ring;                // [ntiles][L-1][32] gx of the next L-1 days
     int ring_slot[kMaxL];       // slot of day t + k
     const float *R, *m_t, *S;
     const double *gD;

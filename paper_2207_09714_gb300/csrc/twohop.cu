@@ -28,26 +28,13 @@ __global__ void __launch_bounds__(kBlock) k_loc_sum(Sell ml, int nloc_tiles, con
     if (threadIdx.x < kMaxL) c_s[threadIdx.x] = c[threadIdx.x];
     __syncthreads();
     const int lane = threadIdx.x & 31;
-    auto contrib = [&](uint32_t j, float w, bool valid, float (&o)[1], bool (&take)[1]) {
-        if constexpr (FWD) {
-            const bool mk = valid && marked(bits, j);
-            const int ej = ld_if(e + j, mk, kNever);
-            o[0] = mk ? w * infectiousness(ej, c_s, t, L) : 0.f;
-            take[0] = mk;
-        } else {
-            o[0] = w * ld_if(r + j, valid);
-            take[0] = valid;
-        }
-    };
-    const bool want[1] = {true};
     BlockTiles disp;
     disp.init(nloc_tiles, lane);
     for (int tile = disp.get(); tile < nloc_tiles; tile = disp.get()) {
         const int row = tile * kTile + lane;
         const uint32_t len = ml.row_len[row];
-        float sum[1];
-        row_sums<1>(ml, ml.slice_ptr[tile], len, len > 0, lane, contrib, want, sum);
-        out[row] = sum[0];
+        out[row] = FWD ? marked_sum(ml, ml.slice_ptr[tile], len, len > 0, lane, bits, e, c_s, t, L)
+                       : gather_sum(ml, ml.slice_ptr[tile], len, len > 0, lane, r);
     }
 }
 
