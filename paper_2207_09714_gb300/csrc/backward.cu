@@ -77,19 +77,20 @@ struct RingTerm {
 // day; the exits recounted for dm are at each row's drawn L_i.
 template <int MODE, bool DC, int EXIT = kExitBase>
 __global__ void __launch_bounds__(kBlock, (MODE == kBwdStore && !DC) ? GABM_BWD_MINBLOCKS : GABM_MINBLOCKS)
-    k_bwd_day(const BwdDayArgs a) {
+    k_bwd_day(BwdDayArgs a) {
     constexpr bool FATE = EXIT == kExitFate;
     constexpr bool DUR = EXIT == kExitDur;
     constexpr bool SOFT = MODE == kBwdSoft;
     constexpr int RB = GABM_RING_BATCH;   // ring slots loaded together in the epilogue
     constexpr int NW = kBlock / 32;
     __shared__ float c_s[kMaxL];
-    __shared__ int32_t red_s[NW][2];
+    __shared__ int32_t red_s[NW][4];
     __shared__ RingTerm term_s[NW][kMaxL];        // the warp's graph's ring terms, k ascending
     __shared__ int term_k[FATE || DUR ? NW : 1][kMaxL];   // their k
     __shared__ float rs_s[NW][kAges];             // R_t S_a of the warp's graph
     __shared__ __align__(16) float bin_s[NW][kBinWords];
     __shared__ double F_s[kMaxL];
+    pdl_trigger();
     if (threadIdx.x < kMaxL) {
         c_s[threadIdx.x] = a.c[threadIdx.x];
         if (DUR) F_s[threadIdx.x] = a.dur.F[threadIdx.x];
@@ -131,10 +132,18 @@ __global__ void __launch_bounds__(kBlock, (MODE == kBwdStore && !DC) ? GABM_BWD_
     disp.init(ntiles, lane);
     TileRows cur, nxt;
     load_tile_rows(a.m, E, a.gr.tile_graph, ntiles, disp.get(), lane, cur);
-    bool have = false;   // ea holds the current tile's first pairs
     uint4 ea[kGP];
 #pragma unroll
     for (int u = 0; u < kGP; ++u) ea[u] = make_uint4(0u, 0u, 0u, 0u);
+    // the first tile's first pairs before the wait, as if its rows gather (they do, but for
+    // the last days of a horizon); the final exposure days are not written by the sweep
+    live_k = 2u;
+    {
+        const TileSpan sp = tile_span(a.m, cur.p0, cur.len, needs(cur.e) || dc_row_of(cur.e), lane);
+        load_pairs(sp.row, 0u, sp.lim, ea);
+    }
+    bool have = true;   // ea holds the current tile's first pairs
+    pdl_wait();
     while (cur.tile < ntiles) {
         load_tile_rows(a.m, E, a.gr.tile_graph, ntiles, disp.get(), lane, nxt);   // a tile ahead of use
 
@@ -148,14 +157,26 @@ __global__ void __launch_bounds__(kBlock, (MODE == kBwdStore && !DC) ? GABM_BWD_
                 emax_w = 0u;
                 rnz_w = false;
             }
-            live_k = carries_adjoint(a.rnz + (size_t)g * a.ld_sig, t, T, L);
+            const bool first = cur_g < 0;
+            // every load of this block goes out before any is used
+            const size_t pg = (size_t)g * a.ldP, ps = (size_t)g * a.ld_sig;
+            sg = a.sig + ps;
+            const bool in = lane >= 1 && lane < L && t + lane < T;
+            const int32_t nz_ld = in ? a.rnz[ps + t + lane] : 0;
+            const int32_t sg_ld = (lane >= 1 && lane < L && t + lane <= T) ? sg[t + lane] : 0;
+            const int32_t em_ld = a.emax[ps + t + 1];
+            const float RS_ld = lane < kAges ? a.R[pg + t] * a.S[g * kAges + lane] : 0.f;
+            const int td = t + (FATE ? a.fate.L_M : L);   // the day today's exposures die on
+            const float gt_ld = td < T ? (FATE ? 1.f : a.m_t[pg + td]) * (float)a.gD[pg + td] : 0.f;
+            inv_D = a.gr.inv_Dbar[g];
+            const int row0_ld = a.gr.row0[g];
+            live_k = __ballot_sync(0xffffffffu, nz_ld != 0);   // days that carry adjoint (flush_rnz)
             // this day's scale for graph g (every warp computes the same value; the warp
             // holding the graph's first tile records it)
-            sg = a.sig + (size_t)g * a.ld_sig;
-            sig_t = next_sigma(sg[t + 1], a.emax[(size_t)g * a.ld_sig + t + 1]);
-            if (lane == 0 && tile * kTile == a.gr.row0[g]) a.sig[(size_t)g * a.ld_sig + t] = sig_t;
+            sig_t = next_sigma(__shfl_sync(0xffffffffu, sg_ld, 1), em_ld);
+            if (lane == 0 && tile * kTile == row0_ld) a.sig[ps + t] = sig_t;
             // c[k] 2^(sigma(t+k) - sigma(t)): the power of two moves no bit of the product
-            const float fac = (lane >= 1 && lane < L && t + lane <= T) ? exp2i(sg[t + lane] - sig_t) : 0.f;
+            const float fac = (lane >= 1 && lane < L && t + lane <= T) ? exp2i(sg_ld - sig_t) : 0.f;
             f1 = __shfl_sync(0xffffffffu, fac, 1);
             cf1 = (live_k & 2u) ? c_s[1] * f1 : 0.f;
             const unsigned tm = live_k & ~3u;
@@ -166,17 +187,12 @@ __global__ void __launch_bounds__(kBlock, (MODE == kBwdStore && !DC) ? GABM_BWD_
                 term_s[wib][i].cf = c_s[lane] * fac;
                 if (FATE || DUR) term_k[wib][i] = lane;
             }
-            const size_t pg = (size_t)g * a.ldP;
-            if (lane < kAges) rs_s[wib][lane] = a.R[pg + t] * a.S[g * kAges + lane];
-            inv_D = a.gr.inv_Dbar[g];
-            if constexpr (FATE)   // deaths are counted: dL/d(one M entry on day t + L_M)
-                gtail = (t + a.fate.L_M < T) ? (float)a.gD[pg + t + a.fate.L_M] * exp2i(-sig_t) : 0.f;
-            else
-                gtail = (t + L < T) ? a.m_t[pg + t + L] * (float)a.gD[pg + t + L] * exp2i(-sig_t) : 0.f;
+            if (lane < kAges) rs_s[wib][lane] = RS_ld;
+            gtail = gt_ld * exp2i(-sig_t);   // R/M split: deaths are counted, dL/d(one M entry on day t + L_M)
             __syncwarp();
             cur_g = g;
             cN = 0;
-            have = false;
+            if (!first) have = false;
         }
         const int row = tile * kTile + lane;
         const bool agent = (Ei != kPad);
@@ -199,6 +215,7 @@ __global__ void __launch_bounds__(kBlock, (MODE == kBwdStore && !DC) ? GABM_BWD_
         // t+1) at that day's scale
         const bool readA = isS && (SOFT || (!never && Ei != t));
         const float A_ld = readA ? a.A[row] : 0.f;
+        const int sgE_ld = (readA && !SOFT) ? sg[Ei] : 0;
         float Lam = 0.f;
         if constexpr (MODE != kBwdFused) Lam = isS ? a.lam_t[row] : 0.f;
         const int ai = isS ? (int)a.age[row] : 0;
@@ -213,7 +230,7 @@ __global__ void __launch_bounds__(kBlock, (MODE == kBwdStore && !DC) ? GABM_BWD_
         }
         if (a.self_q && gather) gx_mine = __fmaf_rn(-a.self_q[row], a.self_r[row], gx_mine);
         if constexpr (MODE == kBwdFused)   // lambda from the final exposure days, the forward's sum
-            Lam = marked_sum<false, 2>(a.m, cur.p0, cur.len, isS, lane, a.bits_t, E, c_s, t, L) * inv_D;
+            Lam = marked_sum<2>(a.m, cur.p0, cur.len, isS, lane, a.bits_t, E, c_s, t, L) * inv_D;
         // the next tile's first pairs are in flight during this tile's epilogue
         have = nxt.tile < ntiles && nxt.g == cur_g;
         if (have) {
@@ -249,7 +266,7 @@ __global__ void __launch_bounds__(kBlock, (MODE == kBwdStore && !DC) ? GABM_BWD_
         float v = 0.f, pm = 0.f;
         if (isS) {
             float Apre = 0.f;
-            if (readA) Apre = A_ld * (SOFT ? f1 : exp2i(sg[Ei] - sig_t));
+            if (readA) Apre = A_ld * (SOFT ? f1 : exp2i(sgE_ld - sig_t));
             // R/M split: the fate an exposure today would draw on day t + tau_EI
             bool phi = false;
             float vf = 0.5f;
@@ -348,24 +365,37 @@ __global__ void __launch_bounds__(kBlock, (MODE == kBwdStore && !DC) ? GABM_BWD_
         cur = nxt;
     }
 
+    // the block's counts and flags of its warps' last graphs: one thread, without reading
+    // what is there first (each warp reading, then writing, held the block's end for two
+    // round trips)
     const int sN = __reduce_add_sync(0xffffffffu, cN);
-    if (cur_g >= 0) {
-        flush_emax(a.emax + (size_t)cur_g * a.ld_sig + t, emax_w);
-        flush_rnz(a.rnz + (size_t)cur_g * a.ld_sig + t, rnz_w);
+    const unsigned em = __reduce_max_sync(0xffffffffu, emax_w);
+    const bool nz = __any_sync(0xffffffffu, rnz_w);
+    if (lane == 0) {
+        red_s[wib][0] = cur_g;
+        red_s[wib][1] = sN;
+        red_s[wib][2] = (int)em - 128;
+        red_s[wib][3] = nz;
     }
-    if (lane == 0) { red_s[wib][0] = cur_g; red_s[wib][1] = sN; }
     __syncthreads();
     if (threadIdx.x == 0) {
-        int g = -1;
-        int32_t acc = 0;
-        for (int w = 0; w <= kBlock / 32; ++w) {
-            const int gw = (w < kBlock / 32) ? red_s[w][0] : -2;
+        int g = -1, acc = 0, top = 0, any = 0;
+        for (int w = 0; w <= NW; ++w) {
+            const int gw = (w < NW) ? red_s[w][0] : -2;
             if (gw != g) {
-                if (g >= 0 && acc) atomicAdd(a.newRM + (size_t)g * a.ldP + t, acc);
+                if (g >= 0) {
+                    if (acc) atomicAdd(a.newRM + (size_t)g * a.ldP + t, acc);
+                    if (top > 0) atomicMax(a.emax + (size_t)g * a.ld_sig + t, top);   // stored maxima start at 0
+                    if (any) a.rnz[(size_t)g * a.ld_sig + t] = 1;
+                }
                 g = gw;
-                acc = 0;
+                acc = top = any = 0;
             }
-            if (w < kBlock / 32 && gw >= 0) acc += red_s[w][1];
+            if (w < NW && gw >= 0) {
+                acc += red_s[w][1];
+                top = max(top, red_s[w][2]);
+                any |= red_s[w][3];
+            }
         }
     }
 }
@@ -549,30 +579,19 @@ __global__ void __launch_bounds__(256) k_bwd_finalize(const double *Q, const flo
 
 }  // namespace
 
-cudaError_t launch_bwd_day(const BwdDayArgs &a, int grid, cudaStream_t s) {
+cudaError_t launch_bwd_day(const BwdDayArgs &a, int grid, bool overlap, cudaStream_t s) {
     const bool dc = a.dc_tile != nullptr;
+    auto go = [&](void (*k)(BwdDayArgs)) { return launch_day(k, grid, kBlock, 0, s, overlap, a); };
     if (a.fate.L_M > 0 || a.dur.n > 0) {   // store policy, plain instance only (checked at creation)
         if (a.mode != kBwdStore || dc) return cudaErrorInvalidValue;
-        if (a.fate.L_M > 0) k_bwd_day<kBwdStore, false, kExitFate><<<grid, kBlock, 0, s>>>(a);
-        else k_bwd_day<kBwdStore, false, kExitDur><<<grid, kBlock, 0, s>>>(a);
-        return cudaGetLastError();
+        return a.fate.L_M > 0 ? go(k_bwd_day<kBwdStore, false, kExitFate>) : go(k_bwd_day<kBwdStore, false, kExitDur>);
     }
     switch (a.mode) {
-        case kBwdStore:
-            if (dc) k_bwd_day<kBwdStore, true><<<grid, kBlock, 0, s>>>(a);
-            else k_bwd_day<kBwdStore, false><<<grid, kBlock, 0, s>>>(a);
-            break;
-        case kBwdFused:
-            if (dc) k_bwd_day<kBwdFused, true><<<grid, kBlock, 0, s>>>(a);
-            else k_bwd_day<kBwdFused, false><<<grid, kBlock, 0, s>>>(a);
-            break;
-        case kBwdSoft:
-            if (dc) k_bwd_day<kBwdSoft, true><<<grid, kBlock, 0, s>>>(a);
-            else k_bwd_day<kBwdSoft, false><<<grid, kBlock, 0, s>>>(a);
-            break;
+        case kBwdStore: return dc ? go(k_bwd_day<kBwdStore, true>) : go(k_bwd_day<kBwdStore, false>);
+        case kBwdFused: return dc ? go(k_bwd_day<kBwdFused, true>) : go(k_bwd_day<kBwdFused, false>);
+        case kBwdSoft: return dc ? go(k_bwd_day<kBwdSoft, true>) : go(k_bwd_day<kBwdSoft, false>);
         default: return cudaErrorInvalidValue;
     }
-    return cudaGetLastError();
 }
 
 cudaError_t launch_dc_seeds(Sell m_out, const int16_t *E, const float *r0, GraphRef gr, const int32_t *sig,

@@ -17,6 +17,9 @@
 
 using namespace gabm;
 
+// Warps of a day kernel an SM holds (three blocks).
+#define GABM_RESIDENT_WARPS (3 * kBlock / 32)
+
 #ifndef GABM_DAY_WAVES
 #define GABM_DAY_WAVES 1
 #endif
@@ -119,6 +122,7 @@ struct gabm_ctx {
     int lam_from = -1;
     int bits_from = -1;             // first day whose infectious bitmap the last forward wrote
 
+    bool overlap = false;           // day launches overlap at their edges (see pdl_wait)
     int grid_fwd = 0, grid_bwd = 0, grid_bwd_dc = 0;   // grid_bwd_dc: the table-adjoint instance
     int grid_bwd_fate = 0;                              // the sampled R/M split's instance
     bool smem_bits = false;         // forward keeps the infectious bitmap in shared memory
@@ -854,7 +858,7 @@ gabm_status forward_days_sirs(gabm_ctx *c, int t0, int T, cudaStream_t s) {
         a.flag_next = c->flags ? fbuf(t + 1) : nullptr;
         a.flag_clear = c->flags ? fbuf(t + 2) : nullptr;
         prof_begin(c, 0);
-        LAUNCH(launch_fwd_day_sirs(a, c->grid_sirs_f, s));
+        LAUNCH(launch_fwd_day_sirs(a, c->grid_sirs_f, c->overlap && t > 0, s));
         prof_end(c, 0);
     }
     return GABM_OK;
@@ -900,7 +904,7 @@ gabm_status backward_days_sirs(gabm_ctx *c, int T, cudaStream_t s) {
         a.P_t = c->P + (size_t)t * c->ntiles * kAges;
         for (int k = 0; k < kMaxL; ++k) a.ring_slot[k] = (k >= 1 && k < c->L) ? (t + k) % Lm1 : 0;
         prof_begin(c, 1);
-        LAUNCH(launch_bwd_day_sirs(a, c->grid_sirs_b, s));
+        LAUNCH(launch_bwd_day_sirs(a, c->grid_sirs_b, c->overlap && t < T - 1, s));
         prof_end(c, 1);
     }
     LAUNCH(launch_bwd_reduce(c->P, c->ntiles, ld, c->d_tile0, c->d_ntiles, T, c->I, c->sig, ld + 1, c->Q, s));
@@ -979,7 +983,7 @@ gabm_status forward_days_plain(gabm_ctx *c, int t0, int T, cudaStream_t s) {
                                        c->grid_loc, s));
             a.pull = c->locv;
         }
-        LAUNCH(launch_fwd_day(a, c->grid_fwd, c->smem_bits, s));
+        LAUNCH(launch_fwd_day(a, c->grid_fwd, c->smem_bits, c->overlap && t > t0, s));
         prof_end(c, 0);
     }
     return GABM_OK;
@@ -1055,7 +1059,7 @@ gabm_status backward_days_plain(gabm_ctx *c, int T, cudaStream_t s) {
         if (c->fate) a.Pm_t = (t + c->tau_EI < T) ? c->Pm + (size_t)(t + c->tau_EI) * c->ntiles : nullptr;
         for (int k = 0; k < kMaxL; ++k) a.ring_slot[k] = (k >= 1 && k < c->L) ? (t + k) % Lm1 : 0;
         prof_begin(c, 1);
-        LAUNCH(launch_bwd_day(a, grid, s));
+        LAUNCH(launch_bwd_day(a, grid, c->overlap && t < T - 1 && mode != kBwdSplit, s));
         prof_end(c, 1);
     }
     if (c->fate)   // the fate draws of agents exposed before day 0 (r of day 0 is in slot 0)
@@ -1255,6 +1259,8 @@ void apply_schedule(gabm_ctx *c) {
     if (c->grid_bwd_fate > max_grid) c->grid_bwd_fate = max_grid;
     c->grid_sirs_f = std::min(max_grid, c->num_sms * occupancy_sirs(false));
     c->grid_sirs_b = std::min(max_grid, c->num_sms * occupancy_sirs(true));
+    c->overlap = !c->batched && !c->soft && !c->two_hop &&
+                 c->ntiles <= kOverlapRounds * c->num_sms * GABM_RESIDENT_WARPS;
     for (auto &g : c->loop_graph) drop_graph(g);   // captured launches carry the old schedule
 }
 

@@ -58,17 +58,20 @@ __device__ __forceinline__ void flush_counts_warp(int32_t *counts, int32_t *newR
 // durations): the exit is the row's drawn L_i (drawn again from its first possible day
 // on); deaths stay m_t newRM(t).
 template <bool SMEM_BITS, int NT, int MINB, bool PULL = false, int EXIT = kExitBase>
-__global__ void __launch_bounds__(NT, MINB) k_fwd_day(const FwdDayArgs a) {
+__global__ void __launch_bounds__(NT, MINB) k_fwd_day(FwdDayArgs a) {
     constexpr int NW = NT / 32;
     extern __shared__ uint32_t bits_s[];
     constexpr bool FATE = EXIT == kExitFate;
+    pdl_trigger();
     __shared__ float c_s[kMaxL];
     __shared__ double F_s[kMaxL];
     __shared__ int32_t red_s[NW][6];
     if (threadIdx.x < kMaxL) c_s[threadIdx.x] = a.c[threadIdx.x];
     if (EXIT == kExitDur && threadIdx.x < kMaxL) F_s[threadIdx.x] = a.dur.F[threadIdx.x];
-    if (SMEM_BITS)
+    if (SMEM_BITS) {
+        pdl_wait();
         for (int i = threadIdx.x; i < a.ntiles; i += NT) bits_s[i] = __ldcg(a.bits_cur + i);
+    }
     __syncthreads();
 
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
@@ -96,8 +99,11 @@ __global__ void __launch_bounds__(NT, MINB) k_fwd_day(const FwdDayArgs a) {
     disp.init(ntiles, lane);
     const uint8_t *flags = PULL ? nullptr : a.flag_cur;
     TileRows cur, nxt;
-    load_tile_rows(a.m, e, a.gr.tile_graph, ntiles, disp.get(), lane, cur, flags);
-    load_tile_rows(a.m, e, a.gr.tile_graph, ntiles, disp.get(), lane, nxt, flags);
+    load_tile_layout(a.m, a.gr.tile_graph, ntiles, disp.get(), lane, cur);
+    load_tile_layout(a.m, a.gr.tile_graph, ntiles, disp.get(), lane, nxt);
+    if (!SMEM_BITS) pdl_wait();
+    load_tile_state(e, ntiles, lane, cur, flags);
+    load_tile_state(e, ntiles, lane, nxt, flags);
     while (cur.tile < ntiles) {
         TileRows nn;
         load_tile_rows(a.m, e, a.gr.tile_graph, ntiles, disp.get(), lane, nn, flags);
@@ -148,7 +154,7 @@ __global__ void __launch_bounds__(NT, MINB) k_fwd_day(const FwdDayArgs a) {
         } else if (flags && __popc(amask) <= GABM_COOP_ROWS) {   // few summing rows: warp-wide, together
             if (amask) sum = few_row_sums(a.m, cur.p0, cur.len, amask, lane, contrib);
         } else if (use_bits) {
-            sum = marked_sum<SMEM_BITS>(a.m, cur.p0, cur.len, act, lane, SMEM_BITS ? bits_s : bits, e, c_s, t, L);
+            sum = marked_sum(a.m, cur.p0, cur.len, act, lane, SMEM_BITS ? bits_s : bits, e, c_s, t, L);
         } else {
             sum = exposed_sum(a.m, cur.p0, cur.len, act, lane, e, c_s, t, L);
         }
@@ -698,20 +704,18 @@ cudaError_t launch_flags_from_bits(const uint32_t *bits_t, Sell m_out, int ntile
     return cudaGetLastError();
 }
 
-cudaError_t launch_fwd_day(const FwdDayArgs &a, int grid, bool smem_bits, cudaStream_t s) {
+cudaError_t launch_fwd_day(const FwdDayArgs &a, int grid, bool smem_bits, bool overlap, cudaStream_t s) {
     if (a.fate.L_M > 0) {
-        k_fwd_day<false, kBlock, GABM_MINBLOCKS, false, kExitFate><<<grid, kBlock, 0, s>>>(a);
+        return launch_day(k_fwd_day<false, kBlock, GABM_MINBLOCKS, false, kExitFate>, grid, kBlock, 0, s, overlap, a);
     } else if (a.dur.n > 0) {
-        k_fwd_day<false, kBlock, GABM_MINBLOCKS, false, kExitDur><<<grid, kBlock, 0, s>>>(a);
+        return launch_day(k_fwd_day<false, kBlock, GABM_MINBLOCKS, false, kExitDur>, grid, kBlock, 0, s, overlap, a);
     } else if (smem_bits && !a.pull) {
         const size_t bytes = (size_t)a.ntiles * sizeof(uint32_t);
-        k_fwd_day<true, kBitsBlock, 1><<<grid, kBitsBlock, bytes, s>>>(a);
+        return launch_day(k_fwd_day<true, kBitsBlock, 1>, grid, kBitsBlock, bytes, s, overlap, a);
     } else if (a.pull) {
-        k_fwd_day<false, kBlock, GABM_MINBLOCKS, true><<<grid, kBlock, 0, s>>>(a);
-    } else {
-        k_fwd_day<false, kBlock, GABM_MINBLOCKS><<<grid, kBlock, 0, s>>>(a);
+        return launch_day(k_fwd_day<false, kBlock, GABM_MINBLOCKS, true>, grid, kBlock, 0, s, overlap, a);
     }
-    return cudaGetLastError();
+    return launch_day(k_fwd_day<false, kBlock, GABM_MINBLOCKS>, grid, kBlock, 0, s, overlap, a);
 }
 
 // Blocks per SM of the forward day kernel (global bitmap), or, for the

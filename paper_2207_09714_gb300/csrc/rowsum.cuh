@@ -57,8 +57,8 @@ struct Width {
 };
 
 // Whether row j is marked in a per-day bitmap of infectious rows (read-only during the launch).
-__device__ __forceinline__ bool marked(const uint32_t *__restrict__ bits, uint32_t j) {
-    return (__ldg(bits + (j >> 5)) >> (j & 31u)) & 1u;
+__device__ __forceinline__ bool marked(const uint32_t *bits, uint32_t j) {
+    return (bits[j >> 5] >> (j & 31u)) & 1u;
 }
 
 // Hands tiles to a warp in runs claimed with one atomic each from the launch's
@@ -184,23 +184,36 @@ struct TileRows {
     bool flag;        // the row has an infectious in-neighbour today (true without flags)
 };
 
-__device__ __forceinline__ void load_tile_rows(const Sell &m, const int16_t *e, const uint16_t *tile_graph,
-                                               int ntiles, int tile, int lane, TileRows &tr,
-                                               const uint8_t *flags = nullptr) {
+// What no launch of a day loop writes (row layout), and the rest.
+__device__ __forceinline__ void load_tile_layout(const Sell &m, const uint16_t *tile_graph, int ntiles, int tile,
+                                                 int lane, TileRows &tr) {
     tr.tile = tile;
-    tr.e = kPad;
     tr.len = 0;
     tr.p0 = 0;
     tr.g = 0;
-    tr.flag = true;
     if (tile < ntiles) {
-        const int row = tile * kTile + lane;
-        tr.e = e[row];
-        tr.len = m.row_len[row];
+        tr.len = m.row_len[tile * kTile + lane];
         tr.p0 = m.slice_ptr[tile];
         tr.g = tile_graph ? (int)tile_graph[tile] : 0;
+    }
+}
+
+__device__ __forceinline__ void load_tile_state(const int16_t *e, int ntiles, int lane, TileRows &tr,
+                                                const uint8_t *flags = nullptr) {
+    tr.e = kPad;
+    tr.flag = true;
+    if (tr.tile < ntiles) {
+        const int row = tr.tile * kTile + lane;
+        tr.e = e[row];
         if (flags) tr.flag = flags[row] != 0;
     }
+}
+
+__device__ __forceinline__ void load_tile_rows(const Sell &m, const int16_t *e, const uint16_t *tile_graph,
+                                               int ntiles, int tile, int lane, TileRows &tr,
+                                               const uint8_t *flags = nullptr) {
+    load_tile_layout(m, tile_graph, ntiles, tile, lane, tr);
+    load_tile_state(e, ntiles, lane, tr, flags);
 }
 
 // The column and weight of entry k of the row in lane r of a slice.
@@ -311,7 +324,7 @@ __device__ __forceinline__ void load_pairs(const uint4 *row, uint32_t q0, uint32
 // used.  Batches in which every lane's entries are valid run without predicates; in the
 // others an invalid entry adds y = 0, which leaves the sum as it is (entries are invalid
 // from some k on, so the compensation it spoils is not used again).
-__device__ __forceinline__ float gather_sum(const TileSpan &s, const float *__restrict__ x, uint4 (&ea)[kGP]) {
+__device__ __forceinline__ float gather_sum(const TileSpan &s, const float *x, uint4 (&ea)[kGP]) {
     float sum = 0.f, comp = 0.f;
     auto use = [&](uint32_t q0, const uint4 (&v)[kGP]) {
         float g[2 * kGP];
@@ -358,7 +371,7 @@ __device__ __forceinline__ float gather_sum(const TileSpan &s, const float *__re
 
 // gather_sum that loads its own first pairs.
 __device__ __forceinline__ float gather_sum(const Sell &m, uint32_t p0, uint32_t len, bool act, int lane,
-                                            const float *__restrict__ x) {
+                                            const float *x) {
     const TileSpan s = tile_span(m, p0, len, act, lane);
     uint4 ea[kGP];
 #pragma unroll
@@ -376,7 +389,7 @@ __device__ __forceinline__ float gather_sum(const Sell &m, uint32_t p0, uint32_t
 // neighbour's exposure day.  On a typical day one entry in twenty is marked, and the
 // longest lane has three or four marks, so this runs about a third of the instructions of
 // a pass that carries every entry through the lookup and the compensated addition.
-template <bool SHARED_BITS = false, int UP = kMP>
+template <int UP = kMP>
 __device__ __forceinline__ float marked_sum(const Sell &m, uint32_t p0, uint32_t len, bool act, int lane,
                                             const uint32_t *bits, const int16_t *e, const float *c_s, int t, int L) {
     const TileSpan s = tile_span(m, p0, len, act, lane);
@@ -386,7 +399,7 @@ __device__ __forceinline__ float marked_sum(const Sell &m, uint32_t p0, uint32_t
     for (int u = 0; u < UP; ++u) ea[u] = eb[u] = make_uint4(0u, 0u, 0u, 0u);
     load_pairs(s.row, 0u, s.lim, ea);
     uint32_t mask = 0u;
-    auto word = [&](uint32_t j) { return (SHARED_BITS ? bits[j >> 5] : __ldg(bits + (j >> 5))) >> (j & 31u); };
+    auto word = [&](uint32_t j) { return bits[j >> 5] >> (j & 31u); };
     auto test = [&](uint32_t q0, const uint4 (&v)[UP]) {
         uint32_t w[2 * UP];
 #pragma unroll

@@ -44,8 +44,9 @@ __global__ void k_sirs_hist_init(const int16_t *e, int64_t n_rows, int H, int16_
 // contiguous range of tiles (neighbours stay in its SM's L1), each warp's next tile is
 // read one tile ahead, and a susceptible row with no infectious in-neighbour (flag_cur)
 // reads no entries: its lambda is 0 exactly.
-__global__ void __launch_bounds__(kBlock, 3) k_fwd_day_sirs(const SirsFwdArgs a) {
+__global__ void __launch_bounds__(kBlock, 3) k_fwd_day_sirs(SirsFwdArgs a) {
     __shared__ float c_s[kMaxL];
+    pdl_trigger();
     if (threadIdx.x < kMaxL) c_s[threadIdx.x] = a.c[threadIdx.x];
     __syncthreads();
     const int lane = threadIdx.x & 31;
@@ -62,8 +63,11 @@ __global__ void __launch_bounds__(kBlock, 3) k_fwd_day_sirs(const SirsFwdArgs a)
     BlockTiles disp;
     disp.init(ntiles, lane);
     TileRows cur, nxt;
-    load_tile_rows(a.m, e, a.gr.tile_graph, ntiles, disp.get(), lane, cur, a.flag_cur);
-    load_tile_rows(a.m, e, a.gr.tile_graph, ntiles, disp.get(), lane, nxt, a.flag_cur);
+    load_tile_layout(a.m, a.gr.tile_graph, ntiles, disp.get(), lane, cur);
+    load_tile_layout(a.m, a.gr.tile_graph, ntiles, disp.get(), lane, nxt);
+    pdl_wait();
+    load_tile_state(e, ntiles, lane, cur, a.flag_cur);
+    load_tile_state(e, ntiles, lane, nxt, a.flag_cur);
     while (cur.tile < ntiles) {
         TileRows nn;
         load_tile_rows(a.m, e, a.gr.tile_graph, ntiles, disp.get(), lane, nn, a.flag_cur);
@@ -137,7 +141,8 @@ __device__ __forceinline__ TileRows nn_next(const SirsBwdArgs &a, BlockTiles &di
 // Reverse day t: gx(t+1) of every agent into the ring, then for rows susceptible on
 // day t the adjoint of the draw, with the return terms B(t+1) and B(t+cycle) read from
 // the G stored at the row's later exposures.
-__global__ void __launch_bounds__(kBlock, 3) k_bwd_day_sirs(const SirsBwdArgs a) {
+__global__ void __launch_bounds__(kBlock, 3) k_bwd_day_sirs(SirsBwdArgs a) {
+    pdl_trigger();
     constexpr int NW = kBlock / 32;
     constexpr int RB = 8;   // ring slots loaded together
     __shared__ float cf_s[NW][kMaxL];    // c[k] 2^(sigma(t+k) - sigma(t)) of the days that carry adjoint,
@@ -160,6 +165,7 @@ __global__ void __launch_bounds__(kBlock, 3) k_bwd_day_sirs(const SirsBwdArgs a)
     TileRows cur, nxt;
     load_tile_rows(a.m, a.E, a.gr.tile_graph, a.ntiles, disp.get(), lane, cur);
     load_tile_rows(a.m, a.E, a.gr.tile_graph, a.ntiles, disp.get(), lane, nxt);
+    pdl_wait();   // the layout, the final state and the histories are not written by the sweep
     for (; cur.tile < a.ntiles; cur = nxt, nxt = nn_next(a, disp, lane)) {
         const int tile = cur.tile;
         const int g = cur.g;
@@ -294,14 +300,12 @@ cudaError_t launch_sirs_hist_init(const int16_t *e, int64_t n_rows, int H, int16
     return cudaGetLastError();
 }
 
-cudaError_t launch_fwd_day_sirs(const SirsFwdArgs &a, int grid, cudaStream_t s) {
-    k_fwd_day_sirs<<<grid, kBlock, 0, s>>>(a);
-    return cudaGetLastError();
+cudaError_t launch_fwd_day_sirs(const SirsFwdArgs &a, int grid, bool overlap, cudaStream_t s) {
+    return launch_day(k_fwd_day_sirs, grid, kBlock, 0, s, overlap, a);
 }
 
-cudaError_t launch_bwd_day_sirs(const SirsBwdArgs &a, int grid, cudaStream_t s) {
-    k_bwd_day_sirs<<<grid, kBlock, 0, s>>>(a);
-    return cudaGetLastError();
+cudaError_t launch_bwd_day_sirs(const SirsBwdArgs &a, int grid, bool overlap, cudaStream_t s) {
+    return launch_day(k_bwd_day_sirs, grid, kBlock, 0, s, overlap, a);
 }
 
 int occupancy_sirs(bool backward) {

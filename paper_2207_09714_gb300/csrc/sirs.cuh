@@ -71,8 +71,8 @@ struct SirsBwdArgs {
 
 cudaError_t launch_sirs_hist_init(const int16_t *e, int64_t n_rows, int H, int16_t *hist, uint16_t *cnt,
                                   cudaStream_t s);
-cudaError_t launch_fwd_day_sirs(const SirsFwdArgs &a, int grid, cudaStream_t s);
-cudaError_t launch_bwd_day_sirs(const SirsBwdArgs &a, int grid, cudaStream_t s);
+cudaError_t launch_fwd_day_sirs(const SirsFwdArgs &a, int grid, bool overlap, cudaStream_t s);
+cudaError_t launch_bwd_day_sirs(const SirsBwdArgs &a, int grid, bool overlap, cudaStream_t s);
 int occupancy_sirs(bool backward);
 
 }  // namespace gabm
