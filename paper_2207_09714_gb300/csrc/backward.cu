@@ -228,9 +228,13 @@ __global__ void __launch_bounds__(kBlock, (MODE == kBwdStore && !DC) ? GABM_BWD_
             if (!have) load_pairs(sp.row, 0u, sp.lim, ea);
             gx_mine = gather_sum(sp, a.r_next, ea);
         }
+        if ((cur.len & kLongBit) && gather) gx_mine = a.long_gx[cur.len & ~kLongBit];
         if (a.self_q && gather) gx_mine = __fmaf_rn(-a.self_q[row], a.self_r[row], gx_mine);
-        if constexpr (MODE == kBwdFused)   // lambda from the final exposure days, the forward's sum
-            Lam = marked_sum<2>(a.m, cur.p0, cur.len, isS, lane, a.bits_t, E, c_s, t, L) * inv_D;
+        if constexpr (MODE == kBwdFused) {   // lambda from the final exposure days, the forward's sum
+            Lam = marked_sum<2>(a.m, cur.p0, cur.len, isS, lane, a.bits_t, E, c_s, t, L);
+            if (cur.len & kLongBit) Lam = a.long_lam[cur.len & ~kLongBit];
+            Lam *= inv_D;
+        }
         // the next tile's first pairs are in flight during this tile's epilogue
         have = nxt.tile < ntiles && nxt.g == cur_g;
         if (have) {
@@ -404,7 +408,8 @@ __global__ void __launch_bounds__(kBlock, (MODE == kBwdStore && !DC) ? GABM_BWD_
 // exposure days (used when the in- and out-edges differ, ahead of the backward day
 // kernel of day t); the same per-row summation as the forward.
 __global__ void __launch_bounds__(kBlock) k_lam_day(Sell m, const int16_t *E, const uint32_t *bits, GraphRef gr,
-                                                    int t, int L, int ntiles, const float *c, float *lam_out) {
+                                                    int t, int L, int ntiles, const float *c, const float *long_lam,
+                                                    float *lam_out) {
     __shared__ float c_s[kMaxL];
     if (threadIdx.x < kMaxL) c_s[threadIdx.x] = c[threadIdx.x];
     __syncthreads();
@@ -414,7 +419,11 @@ __global__ void __launch_bounds__(kBlock) k_lam_day(Sell m, const int16_t *E, co
         const int row = tile * kTile + lane;
         const int Ei = E[row];
         const bool act = (Ei != kPad) && (Ei == kNever || Ei >= t);
-        const float sum = marked_sum(m, m.slice_ptr[tile], m.row_len[row], act, lane, bits, E, c_s, t, L);
+        uint32_t len;
+        int lrow;
+        split_len(m.row_len[row], len, lrow);
+        float sum = marked_sum(m, m.slice_ptr[tile], len, act, lane, bits, E, c_s, t, L);
+        if (lrow >= 0) sum = long_lam[lrow];
         if (act) {
             const int g = gr.tile_graph ? (int)gr.tile_graph[tile] : 0;
             lam_out[row] = sum * gr.inv_Dbar[g];
@@ -427,7 +436,7 @@ __global__ void __launch_bounds__(kBlock) k_lam_day(Sell m, const int16_t *E, co
 // scale 2^sigma(0)).  Only tiles holding a seed do any work.
 __global__ void __launch_bounds__(kBlock) k_dc_seeds(Sell m, const int16_t *E, const float *r0, GraphRef gr,
                                                      const int32_t *sig, int ld_sig, int ntiles, int L,
-                                                     double *dc_tile) {
+                                                     const float *long_gx, double *dc_tile) {
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const int nwarps = gridDim.x * (kBlock / 32);
     for (int tile = blockIdx.x * (kBlock / 32) + wib; tile < ntiles; tile += nwarps) {
@@ -435,7 +444,11 @@ __global__ void __launch_bounds__(kBlock) k_dc_seeds(Sell m, const int16_t *E, c
         const int Ei = E[row];
         const bool seed = Ei != kPad && Ei < 0 && -Ei <= L - 1;
         if (!__any_sync(0xffffffffu, seed)) continue;
-        const float sum = gather_sum(m, m.slice_ptr[tile], m.row_len[row], seed, lane, r0);
+        uint32_t len;
+        int lrow;
+        split_len(m.row_len[row], len, lrow);
+        float sum = gather_sum(m, m.slice_ptr[tile], len, seed, lane, r0);
+        if (lrow >= 0) sum = long_gx[lrow];
         const int g = gr.tile_graph ? (int)gr.tile_graph[tile] : 0;
         dc_accumulate(dc_tile, tile, seed, -Ei, sum, sig[(size_t)g * ld_sig], lane);
     }
@@ -450,7 +463,7 @@ __global__ void __launch_bounds__(kBlock) k_fate_seeds(Sell m, const int16_t *E,
                                                        int Lm1, GraphRef gr, FateRef f,
                                                        const double *gD, const int32_t *sig, int ld_sig,
                                                        const int32_t *rnz, int ntiles, int T, const float *c,
-                                                       double *Pm) {
+                                                       const float *long_gx, double *Pm) {
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const int nwarps = gridDim.x * (kBlock / 32);
     const int L = Lm1 + 1;
@@ -466,7 +479,11 @@ __global__ void __launch_bounds__(kBlock) k_fate_seeds(Sell m, const int16_t *E,
         const int32_t *sg = sig + (size_t)g * ld_sig;
         // gx(0), needed when day 0 lies between the two exits
         const bool at0 = seed && -Ei >= Lmin && -Ei < L;
-        const float gx0 = gather_sum(m, m.slice_ptr[tile], m.row_len[row], at0, lane, r0);
+        uint32_t len;
+        int lrow;
+        split_len(m.row_len[row], len, lrow);
+        float gx0 = gather_sum(m, m.slice_ptr[tile], len, at0, lane, r0);
+        if (lrow >= 0) gx0 = long_gx[lrow];
         double pm = 0.0;
         if (seed) {
             const size_t pg = (size_t)g * f.ldP;
@@ -595,15 +612,16 @@ cudaError_t launch_bwd_day(const BwdDayArgs &a, int grid, bool overlap, cudaStre
 }
 
 cudaError_t launch_dc_seeds(Sell m_out, const int16_t *E, const float *r0, GraphRef gr, const int32_t *sig,
-                            int ld_sig, int ntiles, int L, double *dc_tile, int grid, cudaStream_t s) {
-    k_dc_seeds<<<grid, kBlock, 0, s>>>(m_out, E, r0, gr, sig, ld_sig, ntiles, L, dc_tile);
+                            int ld_sig, int ntiles, int L, const float *long_gx, double *dc_tile, int grid,
+                            cudaStream_t s) {
+    k_dc_seeds<<<grid, kBlock, 0, s>>>(m_out, E, r0, gr, sig, ld_sig, ntiles, L, long_gx, dc_tile);
     return cudaGetLastError();
 }
 
 cudaError_t launch_fate_seeds(Sell m_out, const int16_t *E, const float *r0, const float *ring, int Lm1, GraphRef gr, FateRef f, const double *gD, const int32_t *sig, int ld_sig,
-                              const int32_t *rnz, int ntiles, int T, const float *c, double *Pm, int grid,
-                              cudaStream_t s) {
-    k_fate_seeds<<<grid, kBlock, 0, s>>>(m_out, E, r0, ring, Lm1, gr, f, gD, sig, ld_sig, rnz, ntiles, T, c,
+                              const int32_t *rnz, int ntiles, int T, const float *c, const float *long_gx, double *Pm,
+                              int grid, cudaStream_t s) {
+    k_fate_seeds<<<grid, kBlock, 0, s>>>(m_out, E, r0, ring, Lm1, gr, f, gD, sig, ld_sig, rnz, ntiles, T, c, long_gx,
                                          Pm);
     return cudaGetLastError();
 }
@@ -621,8 +639,8 @@ cudaError_t launch_dc_reduce(const double *dc_tile, const int32_t *graph_tile0, 
 }
 
 cudaError_t launch_lam_day(Sell m, const int16_t *E, const uint32_t *bits, GraphRef gr, int t, int L, int ntiles,
-                           const float *c, float *lam_out, int grid, cudaStream_t s) {
-    k_lam_day<<<grid, kBlock, 0, s>>>(m, E, bits, gr, t, L, ntiles, c, lam_out);
+                           const float *c, const float *long_lam, float *lam_out, int grid, cudaStream_t s) {
+    k_lam_day<<<grid, kBlock, 0, s>>>(m, E, bits, gr, t, L, ntiles, c, long_lam, lam_out);
     return cudaGetLastError();
 }
 

@@ -76,6 +76,10 @@ struct gabm_ctx {
     uint4 *scw = nullptr;
     uint32_t *t_slice_ptr = nullptr, *t_row_len = nullptr;
     uint4 *t_scw = nullptr;
+    // long rows of both orientations, and their sums of the running day [2][max(n_in, n_out)]
+    LongRows long_in{}, long_out{};
+    float *long_sums = nullptr;
+    int long_cap = 0;
     // row-compressed edges (batched kernels): in-edges, and out-edges when not symmetric
     uint32_t *csr_rowptr = nullptr, *csr_col = nullptr, *t_csr_rowptr = nullptr, *t_csr_col = nullptr;
     float *csr_w = nullptr, *t_csr_w = nullptr;
@@ -468,10 +472,12 @@ void group_long_rows(const HostGraph &h, std::vector<uint32_t> &order, int sigma
 struct HostSell {
     std::vector<uint32_t> slice_ptr, row_len;
     std::vector<uint4> cw;
+    std::vector<uint32_t> lrow, lptr;   // long rows (LongRows), kept out of the slices
+    std::vector<uint2> lcw;
 };
 
 bool build_sell(const std::vector<uint32_t> &rowptr, const std::vector<uint32_t> &col, const std::vector<float> &w,
-                int64_t n_rows, HostSell &hs) {
+                int64_t n_rows, HostSell &hs, bool long_rows) {
     const int64_t ns = n_rows / kTile;
     hs.slice_ptr.assign((size_t)ns + 1, 0u);
     hs.row_len.assign((size_t)n_rows, 0u);
@@ -482,6 +488,11 @@ bool build_sell(const std::vector<uint32_t> &rowptr, const std::vector<uint32_t>
             const int64_t r = sl * kTile + l;
             const uint32_t len = rowptr[r + 1] - rowptr[r];
             hs.row_len[r] = len;
+            if (long_rows && len > kLongEntries) {
+                hs.row_len[r] = kLongBit | (uint32_t)hs.lrow.size();
+                hs.lrow.push_back((uint32_t)r);
+                continue;
+            }
             mx = std::max(mx, len);
         }
         hs.slice_ptr[sl] = (uint32_t)total;
@@ -490,7 +501,17 @@ bool build_sell(const std::vector<uint32_t> &rowptr, const std::vector<uint32_t>
     }
     hs.slice_ptr[ns] = (uint32_t)total;
     hs.cw.assign((size_t)std::max<uint64_t>(total, 32), make_uint4(0u, 0u, 0u, 0u));
+    hs.lptr.assign(1, 0u);
+    for (uint32_t r : hs.lrow) {
+        for (uint32_t p = rowptr[r]; p < rowptr[r + 1]; ++p) {
+            uint2 v = make_uint2(col[p], 0u);
+            memcpy(&v.y, &w[p], sizeof(float));
+            hs.lcw.push_back(v);
+        }
+        hs.lptr.push_back((uint32_t)hs.lcw.size());
+    }
     for (int64_t r = 0; r < n_rows; ++r) {
+        if (hs.row_len[r] & kLongBit) continue;
         const uint32_t base = hs.slice_ptr[r / kTile] + (uint32_t)(r % kTile);
         for (uint32_t k = 0; k < hs.row_len[r]; ++k) {
             uint4 &p = hs.cw[base + (size_t)(k / 2) * kTile];
@@ -716,6 +737,46 @@ Csr csr_view(const gabm_ctx *c, bool out_edges) {
     return m;
 }
 
+// The long rows' launch of one day (nothing to do without any): out = what it computes.
+LongArgs long_args(const gabm_ctx *c, int t) {
+    LongArgs a{};
+    a.in = c->long_in;
+    a.out = c->long_out;
+    a.e = c->e;
+    a.tile_graph = c->G > 1 ? c->d_tile_graph : nullptr;
+    a.ld_sig = c->Tcap + 1;
+    a.t = t;
+    a.L = c->L;
+    a.c = c->c_dev;
+    return a;
+}
+float *long_lam_buf(const gabm_ctx *c) { return c->long_sums; }
+float *long_gx_buf(const gabm_ctx *c) { return c->long_sums + c->long_cap; }
+
+// Sums of w x[j] over the long out-rows, into long_gx_buf.
+gabm_status long_gather(gabm_ctx *c, const float *x, const int32_t *rnz, int t, bool overlap, cudaStream_t s) {
+    if (!c->long_cap) return GABM_OK;
+    LongArgs a = long_args(c, t);
+    a.in.n = 0;
+    a.x = x;
+    a.gx = long_gx_buf(c);
+    a.rnz = rnz;
+    LAUNCH(launch_long(a, overlap, s));
+    return GABM_OK;
+}
+
+// Sums over the long in-rows' marked neighbours, into long_lam_buf.
+gabm_status long_lambda(gabm_ctx *c, const uint32_t *bits, uint8_t *flags, int t, bool overlap, cudaStream_t s) {
+    if (!c->long_cap) return GABM_OK;
+    LongArgs a = long_args(c, t);
+    if (!flags) a.out.n = 0;
+    a.bits = bits;
+    a.lam = long_lam_buf(c);
+    a.flags = flags;
+    LAUNCH(launch_long(a, overlap, s));
+    return GABM_OK;
+}
+
 // Day loop of the forward for B > 1 sets per graph (parameters already staged).
 gabm_status forward_days_batched(gabm_ctx *c, int t0, int T, cudaStream_t s) {
     const size_t nb = (size_t)c->n_rows * c->Bp;
@@ -857,7 +918,9 @@ gabm_status forward_days_sirs(gabm_ctx *c, int t0, int T, cudaStream_t s) {
         a.flag_cur = c->flags ? fbuf(t) : nullptr;
         a.flag_next = c->flags ? fbuf(t + 1) : nullptr;
         a.flag_clear = c->flags ? fbuf(t + 2) : nullptr;
+        a.long_sum = long_lam_buf(c);
         prof_begin(c, 0);
+        TRY(long_lambda(c, a.bits_cur, c->flags ? fbuf(t) : nullptr, t, c->overlap && t > 0, s));
         LAUNCH(launch_fwd_day_sirs(a, c->grid_sirs_f, c->overlap && t > 0, s));
         prof_end(c, 0);
     }
@@ -903,7 +966,9 @@ gabm_status backward_days_sirs(gabm_ctx *c, int T, cudaStream_t s) {
         a.r_cur = c->r + (size_t)(t & 1) * c->n_rows;
         a.P_t = c->P + (size_t)t * c->ntiles * kAges;
         for (int k = 0; k < kMaxL; ++k) a.ring_slot[k] = (k >= 1 && k < c->L) ? (t + k) % Lm1 : 0;
+        a.long_gx = long_gx_buf(c);
         prof_begin(c, 1);
+        if (t < T - 1) TRY(long_gather(c, a.r_next, c->rnz, t, c->overlap, s));
         LAUNCH(launch_bwd_day_sirs(a, c->grid_sirs_b, c->overlap && t < T - 1, s));
         prof_end(c, 1);
     }
@@ -983,6 +1048,8 @@ gabm_status forward_days_plain(gabm_ctx *c, int t0, int T, cudaStream_t s) {
                                        c->grid_loc, s));
             a.pull = c->locv;
         }
+        a.long_sum = long_lam_buf(c);
+        TRY(long_lambda(c, a.bits_cur, a.flag_cur ? fbuf(t) : nullptr, t, c->overlap && t > t0, s));
         LAUNCH(launch_fwd_day(a, c->grid_fwd, c->smem_bits, c->overlap && t > t0, s));
         prof_end(c, 0);
     }
@@ -1043,9 +1110,12 @@ gabm_status backward_days_plain(gabm_ctx *c, int T, cudaStream_t s) {
             a.s_hist_t = c->s_hist + (size_t)t * c->n_rows;
             a.y_hist_t = c->y_hist + (size_t)t * c->n_rows;
         }
-        if (mode == kBwdSplit)
+        const bool overlap = c->overlap && t < T - 1 && mode != kBwdSplit;
+        if (mode == kBwdSplit) {
+            TRY(long_lambda(c, c->bits + (size_t)t * c->ntiles, nullptr, t, false, s));
             LAUNCH(launch_lam_day(sell_view(c, false), c->e, c->bits + (size_t)t * c->ntiles, graph_ref(c), t, c->L,
-                                  c->ntiles, c->c_dev, c->lam_tmp, c->grid_bwd, s));
+                                  c->ntiles, c->c_dev, long_lam_buf(c), c->lam_tmp, c->grid_bwd, s));
+        }
         a.r_next = c->r + (size_t)((t + 1) & 1) * c->n_rows;
         a.r_cur = c->r + (size_t)(t & 1) * c->n_rows;
         if (c->two_hop) {   // the location hop of the transpose gather: gP = sum over members of w r(t+1)
@@ -1059,12 +1129,32 @@ gabm_status backward_days_plain(gabm_ctx *c, int T, cudaStream_t s) {
         if (c->fate) a.Pm_t = (t + c->tau_EI < T) ? c->Pm + (size_t)(t + c->tau_EI) * c->ntiles : nullptr;
         for (int k = 0; k < kMaxL; ++k) a.ring_slot[k] = (k >= 1 && k < c->L) ? (t + k) % Lm1 : 0;
         prof_begin(c, 1);
-        LAUNCH(launch_bwd_day(a, grid, c->overlap && t < T - 1 && mode != kBwdSplit, s));
+        a.long_gx = long_gx_buf(c);
+        a.long_lam = long_lam_buf(c);
+        if (c->long_cap) {   // the long rows' gx(t+1), and their lambda sums when not stored
+            LongArgs la = long_args(c, t);
+            la.rnz = c->rnz;
+            if (t < T - 1) {
+                la.x = a.r_next;
+                la.gx = long_gx_buf(c);
+            } else {
+                la.out.n = 0;
+            }
+            if (mode == kBwdFused) {
+                la.bits = a.bits_t;
+                la.lam = long_lam_buf(c);
+            } else {
+                la.in.n = 0;
+            }
+            if (la.in.n + la.out.n > 0) LAUNCH(launch_long(la, overlap, s));
+        }
+        LAUNCH(launch_bwd_day(a, grid, overlap, s));
         prof_end(c, 1);
     }
+    if (c->fate || a.dc_tile) TRY(long_gather(c, c->r, nullptr, 0, false, s));   // the long rows' gx(0)
     if (c->fate)   // the fate draws of agents exposed before day 0 (r of day 0 is in slot 0)
         LAUNCH(launch_fate_seeds(sell_view(c, true), c->e, c->r, c->ring, Lm1, graph_ref(c), a.fate,
-                                 c->gD, c->sig, ld + 1, c->rnz, c->ntiles, T, c->c_dev, c->Pm, c->grid_bwd, s));
+                                 c->gD, c->sig, ld + 1, c->rnz, c->ntiles, T, c->c_dev, long_gx_buf(c), c->Pm, c->grid_bwd, s));
     if (a.dc_tile) {   // the seeds' share through day 0 (r of day 0 is in slot 0)
         const float *r0 = c->r;
         if (c->two_hop) {
@@ -1073,7 +1163,7 @@ gabm_status backward_days_plain(gabm_ctx *c, int T, cudaStream_t s) {
             r0 = c->locv;
         }
         LAUNCH(launch_dc_seeds(sell_view(c, true), c->e, r0, graph_ref(c), c->sig, ld + 1, c->ntiles, c->L,
-                               c->dc_tile, c->grid_bwd, s));
+                               long_gx_buf(c), c->dc_tile, c->grid_bwd, s));
     }
     LAUNCH(launch_bwd_reduce(c->P, c->ntiles, ld, c->d_tile0, c->d_ntiles, T, c->I, c->sig, ld + 1, c->Q, s));
     return GABM_OK;
@@ -1105,7 +1195,16 @@ gabm_status forward_days_soft(gabm_ctx *c, int T, cudaStream_t s) {
         a.y_hist_t = c->y_hist + (size_t)t * n;
         a.lam_t = c->lam + (size_t)t * n;
         a.P_nrm_t = c->P_nrm + (size_t)t * c->ntiles;
+        a.long_sum = long_lam_buf(c);
         prof_begin(c, 0);
+        if (c->long_cap) {   // the long in-rows' sums of x(t)
+            LongArgs la = long_args(c, t);
+            la.out = c->long_in;
+            la.in.n = 0;
+            la.x = a.x_cur;
+            la.gx = long_lam_buf(c);
+            LAUNCH(launch_long(la, false, s));
+        }
         LAUNCH(launch_fwd_day_soft(a, c->grid_fwd, s));
         prof_end(c, 0);
     }
@@ -1447,6 +1546,27 @@ static gabm_status create_on_device(const HostLayout &H, const gabm_model_desc *
         }
     } else {
         CTRY(upload_sell(sell_in, c->slice_ptr, c->row_len, c->scw));
+        auto upload_long = [&](const HostSell &hs, LongRows &lr) -> gabm_status {
+            uint32_t *row = nullptr, *ptr = nullptr;
+            uint2 *cw = nullptr;
+            lr.n = (int)hs.lrow.size();
+            if (lr.n == 0) return GABM_OK;
+            TRY(dalloc(c, &row, hs.lrow.size()));
+            TRY(dalloc(c, &ptr, hs.lptr.size()));
+            TRY(dalloc(c, &cw, hs.lcw.size()));
+            CK(cudaMemcpyAsync(row, hs.lrow.data(), sizeof(uint32_t) * hs.lrow.size(), cudaMemcpyHostToDevice, c->stream));
+            CK(cudaMemcpyAsync(ptr, hs.lptr.data(), sizeof(uint32_t) * hs.lptr.size(), cudaMemcpyHostToDevice, c->stream));
+            CK(cudaMemcpyAsync(cw, hs.lcw.data(), sizeof(uint2) * hs.lcw.size(), cudaMemcpyHostToDevice, c->stream));
+            lr.row = row;
+            lr.ptr = ptr;
+            lr.cw = cw;
+            return GABM_OK;
+        };
+        CTRY(upload_long(sell_in, c->long_in));
+        if (symmetric) c->long_out = c->long_in;
+        else CTRY(upload_long(sell_out, c->long_out));
+        c->long_cap = std::max(c->long_in.n, c->long_out.n);
+        if (c->long_cap) CTRY(dalloc(c, &c->long_sums, (size_t)2 * c->long_cap));
         if (symmetric) {
             c->t_slice_ptr = c->slice_ptr;
             c->t_row_len = c->row_len;
@@ -1632,8 +1752,8 @@ gabm_status gabm_create(const gabm_graph_desc *graphs, int num_graphs, int sets_
     const bool batched = sets_per_graph > 1;
     if (batched && model->lambda_policy != GABM_STORE_LAMBDA && !symmetric)
         return fail(nullptr, GABM_EUNSUPPORTED, "sets_per_graph > 1 with GABM_RECOMPUTE needs symmetric weights in this build");
-    if (!batched && (!build_sell(h_rowptr, h_col, h_w, n_rows, sell_in) ||
-                     (!symmetric && !build_sell(t_rowptr, t_col, t_w, n_rows, sell_out))))
+    if (!batched && (!build_sell(h_rowptr, h_col, h_w, n_rows, sell_in, true) ||
+                     (!symmetric && !build_sell(t_rowptr, t_col, t_w, n_rows, sell_out, true))))
         return fail(nullptr, GABM_EUNSUPPORTED, "SELL-32 layout needs >= 2^32 entries");
     uint32_t max_degree = 0;
     for (int64_t r = 0; r < n_rows; ++r) {
@@ -1839,7 +1959,8 @@ gabm_status gabm_create_bipartite(const gabm_bipartite_desc *graphs, int num_gra
             }
     }
     HostSell loc_sell;
-    if (!build_sell(H.h_rowptr, H.h_col, H.h_w, n_rows, H.sell_in) || !build_sell(lrow, lcol, lw, ns_rows, loc_sell))
+    if (!build_sell(H.h_rowptr, H.h_col, H.h_w, n_rows, H.sell_in, false) ||
+        !build_sell(lrow, lcol, lw, ns_rows, loc_sell, false))
         return fail(nullptr, GABM_EUNSUPPORTED, "SELL-32 layout needs >= 2^32 entries");
     H.t_rowptr = H.h_rowptr;
     H.t_col = H.h_col;
@@ -2118,8 +2239,9 @@ gabm_status gabm_get_lambda(gabm_ctx *ctx, int t, float *lam_out, int mem_space)
         if (!c->lam_tmp) TRY(dalloc(c, &c->lam_tmp, (size_t)c->n_rows));
         uint32_t *bits_t = c->bits + (size_t)c->Tcap * c->ntiles;   // the last day slot, free after a forward
         LAUNCH(launch_infectious_bits(c->e, t, 1, c->L, c->ntiles, bits_t, (size_t)c->ntiles, c->stream));
+        TRY(long_lambda(c, bits_t, nullptr, t, false, c->stream));
         LAUNCH(launch_lam_day(sell_view(c, false), c->e, bits_t, graph_ref(c), t, c->L, c->ntiles, c->c_dev,
-                              c->lam_tmp, c->grid_bwd, c->stream));
+                              long_lam_buf(c), c->lam_tmp, c->grid_bwd, c->stream));
         lam_t = c->lam_tmp;
     }
     LAUNCH(launch_get_lambda(lam_t, c->e, c->age, graph_ref(c), c->R, c->S, c->Tcap, t,

@@ -159,6 +159,7 @@ __global__ void __launch_bounds__(NT, MINB) k_fwd_day(FwdDayArgs a) {
             sum = exposed_sum(a.m, cur.p0, cur.len, act, lane, e, c_s, t, L);
         }
 
+        if (cur.len & kLongBit) sum = a.long_sum[cur.len & ~kLongBit];
         int e_next = ei;
         if (act) {
             const float Lam = sum * a.gr.inv_Dbar[g];
@@ -263,7 +264,11 @@ __global__ void __launch_bounds__(kBlock, GABM_MINBLOCKS) k_fwd_day_soft(const S
         const int ei = a.e[row];
         const bool agent = ei != kPad;
         const int g = a.gr.tile_graph ? (int)a.gr.tile_graph[tile] : 0;
-        const float sum = gather_sum(a.m, a.m.slice_ptr[tile], a.m.row_len[row], agent, lane, x_cur);
+        uint32_t len;
+        int lrow;
+        split_len(a.m.row_len[row], len, lrow);
+        float sum = gather_sum(a.m, a.m.slice_ptr[tile], len, agent, lane, x_cur);
+        if (lrow >= 0) sum = a.long_sum[lrow];
         float n_old = 0.f;
         if (agent) {
             const float Lam = sum * a.gr.inv_Dbar[g];

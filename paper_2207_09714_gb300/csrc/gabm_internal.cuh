@@ -148,10 +148,43 @@ enum { kExitBase = 0, kExitFate = 1, kExitDur = 2 };
 // Edges of one orientation in SELL-32 layout (one slice per 32-row tile).
 struct Sell {
     const uint32_t *slice_ptr;  // [ntiles+1] first element of each slice in cw
-    const uint32_t *row_len;    // [n_rows] entries of each row
+    const uint32_t *row_len;    // [n_rows] entries of each row; a long row's (LongRows) is kLongBit | its index
     const uint4 *cw;            // entries 2q, 2q+1 of the row in lane l at slice_ptr + 32 q + l: column
                                 // (neighbour row) and weight bits of each (0 in padding)
 };
+
+// Rows of more than kLongEntries entries (the hubs of a power-law contact graph) are kept out
+// of the SELL slices and summed by a block each, in a launch before the day kernel
+// (longrows.cu): in a slice, one lane walks its row and the whole tile waits for it -- on
+// the 300k-agent power-law graph (90 days, recompute policy) a step took 30.7 ms that way
+// and takes 8.0 (with rows of more than 32, 48 and 96 entries taken out: 13.1, 7.7 and 8.8; at
+// 48 the 1M-agent typed graph, whose longest rows hold about 50, loses 4%).  The sum of a long row is compensated per thread and over a fixed tree.
+constexpr uint32_t kLongEntries = 64;
+constexpr uint32_t kLongBit = 0x80000000u;
+struct LongRows {
+    const uint32_t *row;      // [n] device row of each
+    const uint32_t *ptr;      // [n + 1]
+    const uint2 *cw;          // column and weight bits of each entry
+    int n;
+};
+
+// One launch over a ctx's long rows.  Each part runs when its output is given:
+// lam[i] = sum over in-row i of w c[t - e_j] over the neighbours marked in bits (marked_sum);
+// gx[i] = sum over out-row i of w x[j], 0 when rnz says that day t + 1 carries no adjoint;
+// flags: out-neighbours of the out-rows marked in bits get flag 1.
+struct LongArgs {
+    LongRows in, out;
+    const uint32_t *bits;
+    const int16_t *e;
+    const float *x;
+    float *lam, *gx;
+    uint8_t *flags;
+    const int32_t *rnz;       // [G][ld_sig] or nullptr: gather always
+    const uint16_t *tile_graph;
+    int ld_sig, t, L;
+    const float *c;           // device table [kMaxL]
+};
+cudaError_t launch_long(const LongArgs &a, bool overlap, cudaStream_t s);
 
 struct FwdDayArgs {
     Sell m;               // in-edges: row i lists j with w_ji
@@ -175,6 +208,7 @@ struct FwdDayArgs {
     const uint8_t *flag_cur;
     uint8_t *flag_next, *flag_clear;
     Sell m_out;                 // out-edges (the in-edges when the weights are symmetric)
+    const float *long_sum;      // the long in-rows' sums of today (or nullptr: there are none)
     int t_first;                // first day of this forward (counts of earlier days are not its own)
     int ntiles, t, tau_EI, L;   // L: the longest infectious window (the table's length)
     uint64_t seed;
@@ -193,6 +227,7 @@ struct SoftDayArgs {
     const int16_t *e;        // exposure days after seeding (padding rows: kPad)
     const float *x_cur;      // [n_rows] x_i(t)
     float *x_next;           // [n_rows] x_i(t+1)
+    const float *long_sum;   // the long rows' sums
     float *s;                // [n_rows] susceptible mass
     float *nh;               // [L][n_rows] n_i(d) in slot d mod L
     float *s_hist_t, *y_hist_t, *lam_t;   // day-t histories [n_rows]: s_i(t), y_i(t), Lam_i(t)
@@ -212,6 +247,7 @@ struct BwdDayArgs {
     const uint32_t *bits_t;    // [ntiles] rows infectious on day t (recompute policy) or nullptr
     const float *lam_t;        // stored normalised sums for day t (store policy) or nullptr
     const float *r_next;       // coefficients of day t+1 [n_rows]
+    const float *long_gx, *long_lam;   // the long rows' gx(t+1), and (recompute policy) lambda sums of day t
     float *r_cur;              // coefficients of day t   [n_rows]
     float *ring;               // [ntiles][L-1][32]: a tile's slots lie together
     float *A;                  // [n_rows] adjoint of s carried back from the infection day (soft: dL/ds(t+1))
@@ -459,8 +495,8 @@ cudaError_t launch_infectious_bits_fate(const int16_t *e, GraphRef gr, FateRef f
 cudaError_t launch_infectious_bits_dur(const int16_t *e, GraphRef gr, const DurRef &d, int t, int ntiles,
                                        uint32_t *bits, cudaStream_t s);
 cudaError_t launch_fate_seeds(Sell m_out, const int16_t *E, const float *r0, const float *ring, int Lm1, GraphRef gr, FateRef f, const double *gD, const int32_t *sig, int ld_sig,
-                              const int32_t *rnz, int ntiles, int T, const float *c, double *Pm, int grid,
-                              cudaStream_t s);
+                              const int32_t *rnz, int ntiles, int T, const float *c, const float *long_gx, double *Pm,
+                              int grid, cudaStream_t s);
 cudaError_t launch_fate_dm(const double *Pm, int ntiles, const int32_t *graph_tile0, const int32_t *graph_ntiles,
                            int G, int T, double *dm, cudaStream_t s);
 cudaError_t launch_infectious_bits(const int16_t *e, int t0, int ndays, int L, int ntiles, uint32_t *bits,
@@ -474,7 +510,8 @@ cudaError_t launch_bwd_day(const BwdDayArgs &a, int grid, bool overlap, cudaStre
 // Adjoint of the infectiousness table (hard mode, one set per graph): the seeds'
 // share through their day-0 infectiousness, then the per-graph sums of dc_tile.
 cudaError_t launch_dc_seeds(Sell m_out, const int16_t *E, const float *r0, GraphRef gr, const int32_t *sig,
-                            int ld_sig, int ntiles, int L, double *dc_tile, int grid, cudaStream_t s);
+                            int ld_sig, int ntiles, int L, const float *long_gx, double *dc_tile, int grid,
+                            cudaStream_t s);
 cudaError_t launch_dc_reduce(const double *dc_tile, const int32_t *graph_tile0, const int32_t *graph_ntiles, int G,
                              int L, double *dc, cudaStream_t s);
 cudaError_t launch_dc_seeds_b(Csr m_out, const int16_t *E, const float *r0, GraphRef gr, const int32_t *sig,
@@ -496,7 +533,7 @@ cudaError_t launch_loc_adjoint(Sell ml, int nloc_tiles, LocCsr big, const float 
                                int grid, cudaStream_t s);
 int occupancy_loc();
 cudaError_t launch_lam_day(Sell m, const int16_t *E, const uint32_t *bits, GraphRef gr, int t, int L, int ntiles,
-                           const float *c, float *lam_out, int grid, cudaStream_t s);
+                           const float *c, const float *long_lam, float *lam_out, int grid, cudaStream_t s);
 // Q[g][t][a] = 2^sigma_g(t) x (sum over graph g's tiles of P[t][tile][a]), FP64.
 cudaError_t launch_bwd_reduce(const double *P, int ntiles, int ldP, const int32_t *graph_tile0,
                               const int32_t *graph_ntiles, int T, int I, const int32_t *sig, int ld_sig,

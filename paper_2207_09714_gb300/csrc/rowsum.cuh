@@ -178,11 +178,18 @@ __device__ __forceinline__ float warp_bin_sums(float v, int bin, int lane, float
 struct TileRows {
     int tile;
     int e;            // exposure day of this lane's row
-    uint32_t len;     // entries of this lane's row
+    uint32_t len;     // this lane's row_len word: entries in the slice, or a long row's index (see split_len)
     uint32_t p0;      // the tile's slice
     int g;            // graph of the tile
     bool flag;        // the row has an infectious in-neighbour today (true without flags)
 };
+
+// A row_len word: entries in the slice, and the index of a long row or -1.
+__device__ __forceinline__ void split_len(uint32_t v, uint32_t &len, int &lrow) {
+    const bool lng = (v & kLongBit) != 0u;
+    len = lng ? 0u : v;
+    lrow = lng ? (int)(v & ~kLongBit) : -1;
+}
 
 // What no launch of a day loop writes (row layout), and the rest.
 __device__ __forceinline__ void load_tile_layout(const Sell &m, const uint16_t *tile_graph, int ntiles, int tile,
@@ -231,7 +238,8 @@ __device__ __forceinline__ void push_flags(const Sell &m_out, int tile, int lane
     unsigned rows = __ballot_sync(0xffffffffu, push);
     if (!rows) return;
     const uint32_t base = m_out.slice_ptr[tile];
-    const uint32_t my_len = push ? m_out.row_len[tile * kTile + lane] : 0u;
+    uint32_t my_len = push ? m_out.row_len[tile * kTile + lane] : 0u;
+    if (my_len & kLongBit) my_len = 0u;   // the next day's long-row launch pushes these
     if (__popc(rows) <= 2) {
         while (rows) {
             const int r = __ffs(rows) - 1;
@@ -302,7 +310,7 @@ struct TileSpan {
 __device__ __forceinline__ TileSpan tile_span(const Sell &m, uint32_t p0, uint32_t len, bool act, int lane) {
     TileSpan s;
     s.row = m.cw + p0 + (uint32_t)lane;
-    s.len = act ? len : 0u;
+    s.len = act && !(len & kLongBit) ? len : 0u;   // a long row is summed elsewhere
     s.np = (__reduce_max_sync(0xffffffffu, s.len) + 1u) >> 1;
     s.kfull = __reduce_min_sync(0xffffffffu, s.len);
     s.lim = __popc(__ballot_sync(0xffffffffu, act)) >= 24 ? s.np : (s.len + 1u) >> 1;
@@ -535,6 +543,7 @@ __device__ __forceinline__ float few_row_sums(const Sell &m, uint32_t p0, uint32
                                               F f) {
     constexpr int K = GABM_COOP_ROWS;
     float sum = 0.f, comp = 0.f;
+    if (my_len & kLongBit) my_len = 0u;
     int r[K];
     uint32_t len[K];
     uint2 v[K];

@@ -95,6 +95,7 @@ __global__ void __launch_bounds__(kBlock, 3) k_fwd_day_sirs(SirsFwdArgs a) {
         } else {
             sum = marked_sum(a.m, cur.p0, cur.len, act, lane, bits, e, c_s, t, L);
         }
+        if (cur.len & kLongBit) sum = a.long_sum[cur.len & ~kLongBit];
         int e_next = ei;
         if (act) {
             const float Lam = sum * a.gr.inv_Dbar[g];
@@ -222,7 +223,8 @@ __global__ void __launch_bounds__(kBlock, 3) k_bwd_day_sirs(SirsBwdArgs a) {
         // the row loads that do not depend on the sum go out before it
         const float Lam = isS ? a.lam_t[row] : 0.f;
         const int ai = isS ? (int)a.age[row] : 0;
-        const float gx1 = gather_sum(a.m, cur.p0, cur.len, act, lane, a.r_next);
+        float gx1 = gather_sum(a.m, cur.p0, cur.len, act, lane, a.r_next);
+        if ((cur.len & kLongBit) && act) gx1 = a.long_gx[cur.len & ~kLongBit];
         float *ring = a.ring + (size_t)tile * slot_floats + lane;
         if (act) ring[a.ring_slot[1] * kTile] = gx1;
 

@@ -37,6 +37,7 @@ struct SirsFwdArgs {
     const uint8_t *flag_cur;    // rows with an infectious in-neighbour on day t (or nullptr: all)
     uint8_t *flag_next, *flag_clear;   // day t + 1's flags (set here), day t + 2's (cleared here)
     Sell m_out;                 // out-edges
+    const float *long_sum;      // the long in-rows' sums of today
     int ntiles, t, tau_EI, L, cycle;
     uint64_t seed;
     float c[kMaxL];
@@ -53,6 +54,7 @@ struct SirsBwdArgs {
     float *Gh, *Lh;
     const float *lam_t;         // stored normalised sums of day t
     const float *r_next;        // r of day t + 1
+    const float *long_gx;       // the long rows' gx(t+1)
     float *r_cur;               // r of day t (0 for rows not susceptible on day t)
     float *ring;                // [ntiles][L-1][32] gx of the next L-1 days
     int ring_slot[kMaxL];       // slot of day t + k
