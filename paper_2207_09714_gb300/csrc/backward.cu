@@ -215,7 +215,8 @@ __global__ void __launch_bounds__(kBlock, (MODE == kBwdStore && !DC) ? GABM_BWD_
         // t+1) at that day's scale
         const bool readA = isS && (SOFT || (!never && Ei != t));
         const float A_ld = readA ? a.A[row] : 0.f;
-        const int sgE_ld = (readA && !SOFT) ? sg[Ei] : 0;
+        // (sigma grows towards day 0, so sigma(t) = 0 means that it is 0 on every later day)
+        const int sgE_ld = (readA && !SOFT && sig_t != 0) ? sg[Ei] : 0;
         float Lam = 0.f;
         if constexpr (MODE != kBwdFused) Lam = isS ? a.lam_t[row] : 0.f;
         const int ai = isS ? (int)a.age[row] : 0;
@@ -358,7 +359,7 @@ __global__ void __launch_bounds__(kBlock, (MODE == kBwdStore && !DC) ? GABM_BWD_
         // per-tile sums of gl * Lam by age bin (fp32 over 32 rows, FP64 from here on)
         float mine = 0.f;   // lanes 2b, 2b + 1: bin b
         if (__any_sync(0xffffffffu, !(v == 0.f))) mine = warp_bin_sums(v, ai, lane, bin_s[wib]);
-        if (!(lane & 1) && (lane >> 1) < kAges) a.P_t[(size_t)tile * kAges + (lane >> 1)] = (double)mine;
+        if (!(lane & 1) && (lane >> 1) < kAges) a.P_t[(size_t)tile * kAges + (lane >> 1)] = mine;
         if constexpr (FATE) {
             // dL/dm of day t + tau_EI from this tile's exposures today (fixed tree, FP64 out)
 #pragma unroll
@@ -542,33 +543,46 @@ __global__ void __launch_bounds__(256) k_dc_reduce(const double *dc_tile, const 
     if (threadIdx.x == 0) dc[(size_t)g * L + k] = s[0];
 }
 
-// Q[inst][t][a] = sum over the graph's tiles of P[t][tile][a], fixed order, FP64.
-__global__ void __launch_bounds__(256) k_bwd_reduce(const double *P, int ntiles, const int32_t *graph_tile0,
-                                                    const int32_t *graph_ntiles, int T, const int32_t *sig,
-                                                    int ld_sig, double *Q) {
-    __shared__ double s[256][kAges];
-    const int t = blockIdx.x, inst = blockIdx.y;
-    const int g = inst;
-    const int tile0 = graph_tile0[g], nt = graph_ntiles[g];
-    double acc[kAges];
+// parts[t][inst][c][a] = sum over the c-th of kReduceParts shares of the graph's tiles of
+// P[t][tile][a], fixed order, FP64.  The shares' elements are taken in a row by kReduceBlock
+// threads, a multiple of nine, so a thread keeps one age bin and the loads are coalesced; one
+// block of 256 threads a day with nine accumulators each took 130 us on the 1M-agent graph.
+constexpr int kReduceBlock = 9 * 56;
+__global__ void __launch_bounds__(kReduceBlock) k_bwd_reduce(const float *P, int ntiles, const int32_t *graph_tile0,
+                                                             const int32_t *graph_ntiles, double *parts) {
+    __shared__ double s[kReduceBlock];
+    const int t = blockIdx.x, inst = blockIdx.y, c = blockIdx.z, tid = threadIdx.x;
+    const int tile0 = graph_tile0[inst], nt = graph_ntiles[inst];
+    const int i0 = (int)((long long)nt * c / kReduceParts), i1 = (int)((long long)nt * (c + 1) / kReduceParts);
+    const float *p = P + ((size_t)t * ntiles + tile0 + i0) * kAges;
+    const int n = (i1 - i0) * kAges;
+    double acc = 0.0;
+    int i = tid;
+    for (; i + 3 * kReduceBlock < n; i += 4 * kReduceBlock) {
+        float v[4];
 #pragma unroll
-    for (int b = 0; b < kAges; ++b) acc[b] = 0.0;
-    const double *Pt = P + (size_t)t * ntiles * kAges;
-    for (int i = threadIdx.x; i < nt; i += blockDim.x) {
-        const double *p = Pt + (size_t)(tile0 + i) * kAges;
+        for (int u = 0; u < 4; ++u) v[u] = p[i + u * kReduceBlock];
 #pragma unroll
-        for (int b = 0; b < kAges; ++b) acc[b] += p[b];
+        for (int u = 0; u < 4; ++u) acc += (double)v[u];
     }
-#pragma unroll
-    for (int b = 0; b < kAges; ++b) s[threadIdx.x][b] = acc[b];
+    for (; i < n; i += kReduceBlock) acc += (double)p[i];
+    s[tid] = acc;
     __syncthreads();
-    for (int h = 128; h > 0; h >>= 1) {
-        if ((int)threadIdx.x < h)
-            for (int b = 0; b < kAges; ++b) s[threadIdx.x][b] += s[threadIdx.x + h][b];
-        __syncthreads();
+    if (tid < kAges) {   // 56 values of bin tid, in order
+        double v = 0.0;
+        for (int k = 0; k < kReduceBlock / kAges; ++k) v += s[k * kAges + tid];
+        parts[(((size_t)t * gridDim.y + inst) * kReduceParts + c) * kAges + tid] = v;
     }
-    if (threadIdx.x < kAges)
-        Q[((size_t)inst * T + t) * kAges + threadIdx.x] = ldexp(s[0][threadIdx.x], sig[(size_t)g * ld_sig + t]);
+}
+
+// Q[inst][t][a] = 2^sigma(t) x the sum of the shares, in order.
+__global__ void k_bwd_reduce_parts(const double *parts, int T, int I, const int32_t *sig, int ld_sig, double *Q) {
+    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
+    if (idx >= T * I * kAges) return;
+    const int a = idx % kAges, ti = idx / kAges, inst = ti % I, t = ti / I;
+    double v = 0.0;
+    for (int c = 0; c < kReduceParts; ++c) v += parts[((size_t)ti * kReduceParts + c) * kAges + a];
+    Q[((size_t)inst * T + t) * kAges + a] = ldexp(v, sig[(size_t)inst * ld_sig + t]);
 }
 
 // dR_t = sum_a S_a Q[t][a];  dS_a = sum_t R_t Q[t][a];  dm_t = gD_t newRM(t) (not written
@@ -670,11 +684,10 @@ int occupancy_bwd(int mode, bool dc, int exit_mode) {
     return blocks > 0 ? blocks : 1;
 }
 
-cudaError_t launch_bwd_reduce(const double *P, int ntiles, int ldP, const int32_t *graph_tile0,
-                              const int32_t *graph_ntiles, int T, int I, const int32_t *sig, int ld_sig,
-                              double *Q, cudaStream_t s) {
-    (void)ldP;
-    k_bwd_reduce<<<dim3(T, I), 256, 0, s>>>(P, ntiles, graph_tile0, graph_ntiles, T, sig, ld_sig, Q);
+cudaError_t launch_bwd_reduce(const float *P, int ntiles, const int32_t *graph_tile0, const int32_t *graph_ntiles,
+                              int T, int I, const int32_t *sig, int ld_sig, double *parts, double *Q, cudaStream_t s) {
+    k_bwd_reduce<<<dim3(T, I, kReduceParts), kReduceBlock, 0, s>>>(P, ntiles, graph_tile0, graph_ntiles, parts);
+    k_bwd_reduce_parts<<<(T * I * kAges + 255) / 256, 256, 0, s>>>(parts, T, I, sig, ld_sig, Q);
     return cudaGetLastError();
 }
 

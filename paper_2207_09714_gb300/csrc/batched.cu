@@ -7,9 +7,11 @@
 // agent-major, [n_rows][Bp], so a neighbour's values for every set are one
 // contiguous gather (Bp * 2 bytes of e, Bp * 4 bytes of r).
 //
-// A warp works on a 32-row tile.  A "group" of LPR = Bp/SPL lanes shares one
+// A warp works on a unit of 32, 16 or 8 rows: whole tiles while there are enough of them
+// for the chip, parts of tiles on small graphs, where a tile a warp left most warps without
+// one and the others with a long chain of passes.  A "group" of LPR = Bp/SPL lanes shares one
 // row, lane q of the group owning the SPL sets [q SPL, (q+1) SPL); 32/LPR rows
-// are in flight per warp and the tile takes LPR passes.  For each chunk of LPR
+// are in flight per warp and the unit takes as many passes as that needs.  For each chunk of LPR
 // entries of the row, the group loads the columns and weights coalesced, tests
 // each neighbour against the day's bitmap (rows infectious in some set, or
 // susceptible in some set in the backward), compacts the marked entries with a
@@ -53,7 +55,8 @@ __global__ void __launch_bounds__(kBlock, GABM_BFWD_MINBLOCKS) k_fwd_day_b(const
     __syncthreads();
 
     const int grp = lane / LPR, q = lane % LPR;
-    const int t = a.t, L = a.L, B = a.B, ntiles = a.ntiles;
+    const int t = a.t, L = a.L, B = a.B, nunits = a.nunits, ru = a.ru;
+    const bool in_unit = grp < ru;       // a pass of more rows than the unit leaves groups idle
     uint32_t *e32 = reinterpret_cast<uint32_t *>(a.e);
     const uint32_t *e32r = e32;
     constexpr int WPR = Bp / 2;   // 32-bit words per row of e
@@ -62,35 +65,36 @@ __global__ void __launch_bounds__(kBlock, GABM_BFWD_MINBLOCKS) k_fwd_day_b(const
     auto val = [&](const EWords<SPL> &r, int h) { return infect_lut(half_of(r.w[h >> 1], h & 1), c_s, t, (unsigned)L); };
 
     TileDispenser disp;
-    disp.init(a.tile_ctr, ntiles, gridDim.x * NW, lane);
-    // row bounds of the tile's 32 rows (lane r: rows r and r + 1), one tile ahead
-    int tile = disp.get();
+    disp.init(a.tile_ctr, nunits, gridDim.x * NW, lane);
+    // row bounds of the unit's rows (lane r: rows r and r + 1), one unit ahead
+    int unit = disp.get();
     uint32_t rp_lo = 0u, rp_hi = 0u;
-    if (tile < ntiles) {
-        rp_lo = a.m.rowptr[tile * kTile + lane];
-        rp_hi = a.m.rowptr[tile * kTile + lane + 1];
+    if (unit < nunits && lane < ru) {
+        rp_lo = a.m.rowptr[unit * ru + lane];
+        rp_hi = a.m.rowptr[unit * ru + lane + 1];
     }
-    while (tile < ntiles) {
-        const int ntile = disp.get();
+    while (unit < nunits) {
+        const int next_unit = disp.get();
         uint32_t nrp_lo = 0u, nrp_hi = 0u;
-        if (ntile < ntiles) {
-            nrp_lo = a.m.rowptr[ntile * kTile + lane];
-            nrp_hi = a.m.rowptr[ntile * kTile + lane + 1];
+        if (next_unit < nunits && lane < ru) {
+            nrp_lo = a.m.rowptr[next_unit * ru + lane];
+            nrp_hi = a.m.rowptr[next_unit * ru + lane + 1];
         }
-        const int g = a.gr.tile_graph ? (int)a.gr.tile_graph[tile] : 0;
+        const int row0 = unit * ru;
+        const int g = a.gr.tile_graph ? (int)a.gr.tile_graph[row0 / kTile] : 0;
         const float inv_D = a.gr.inv_Dbar[g];
         uint32_t word = 0u;
         int nnew[SPL];
 #pragma unroll
         for (int h = 0; h < SPL; ++h) nnew[h] = 0;
-        PassRow<SPL> nx;
-        load_pass_row<SPL>(a.m, e32 + (size_t)(tile * kTile + grp) * WPR + q * (SPL / 2), rp_lo, rp_hi, grp, q, nx);
-        for (int pass = 0; pass < LPR; ++pass) {
-            const int row = tile * kTile + pass * RPW + grp;
+        PassRow<LPR, SPL, 1> nx;
+        load_pass_row<LPR, SPL, 1>(a.m, e32 + (size_t)(row0 + grp) * WPR + q * (SPL / 2), in_unit, rp_lo, rp_hi, grp, q, nx);
+        for (int pass = 0; pass * RPW < ru; ++pass) {
+            const int row = row0 + pass * RPW + grp;
             uint32_t *mine_p = e32 + (size_t)row * WPR + q * (SPL / 2);
-            const PassRow<SPL> cu = nx;
-            if (pass + 1 < LPR)   // the next pass's row in flight while this one is summed
-                load_pass_row<SPL>(a.m, mine_p + (size_t)RPW * WPR, rp_lo, rp_hi, (pass + 1) * RPW + grp, q, nx);
+            const PassRow<LPR, SPL, 1> cu = nx;
+            if ((pass + 1) * RPW < ru)   // the next pass's row in flight while this one is summed
+                load_pass_row<LPR, SPL, 1>(a.m, mine_p + (size_t)RPW * WPR, true, rp_lo, rp_hi, (pass + 1) * RPW + grp, q, nx);
             uint32_t ew[SPL / 2];
 #pragma unroll
             for (int k = 0; k < SPL / 2; ++k) ew[k] = cu.ew[k];
@@ -103,7 +107,7 @@ __global__ void __launch_bounds__(kBlock, GABM_BFWD_MINBLOCKS) k_fwd_day_b(const
             }
             const bool act = (group_bits<LPR>(__ballot_sync(kFull, mine)) >> grp) & 1u;
             float sum[SPL];
-            group_row_sums<LPR, SPL, KAHAN, EWords<SPL>>(a.m, cu.p0, act ? cu.len : 0u, cu.j0, cu.w0, a.bits_cur, lane,
+            group_row_sums<LPR, SPL, 1, KAHAN, EWords<SPL>>(a.m, cu.p0, act ? cu.len : 0u, cu.j0, cu.w0, a.bits_cur, lane,
                                                          ld, val, sum);
 
             // lambda of each susceptible set with an infectious neighbour; only those draw
@@ -142,7 +146,7 @@ __global__ void __launch_bounds__(kBlock, GABM_BFWD_MINBLOCKS) k_fwd_day_b(const
                     }
                     if (pi < ndraw) {
                         const int src = nth_set_bit(msel, pi - before);
-                        const int srow = tile * kTile + pass * RPW + src / LPR;
+                        const int srow = row0 + pass * RPW + src / LPR;
                         const int inst = g * B + (src % LPR) * SPL + hs;
                         const float lam = (a.R[(size_t)inst * a.ldP + t] * a.S[inst * kAges + a.age[srow]]) *
                                           lam_w[hs * 32 + src];
@@ -190,16 +194,20 @@ __global__ void __launch_bounds__(kBlock, GABM_BFWD_MINBLOCKS) k_fwd_day_b(const
             }
             word |= group_bits<LPR>(__ballot_sync(kFull, inf)) << (pass * RPW);
         }
-        if (lane == 0) a.bits_next[tile] = word;
-        // exposures of this tile by set (at most 32 each)
+        if (lane == 0) {
+            if (ru == 32) a.bits_next[unit] = word;
+            else if (ru == 16) reinterpret_cast<uint16_t *>(a.bits_next)[unit] = (uint16_t)word;
+            else reinterpret_cast<uint8_t *>(a.bits_next)[unit] = (uint8_t)word;
+        }
+        // exposures of this unit by set (at most 32 each)
 #pragma unroll
         for (int h = 0; h < SPL; ++h) nnew[h] = group_reduce<LPR>(nnew[h]);
         if (grp == 0) {
-            uint8_t *dst = a.tile_new + (size_t)tile * Bp + q * SPL;
+            uint8_t *dst = a.unit_new + (size_t)unit * Bp + q * SPL;
 #pragma unroll
             for (int h = 0; h < SPL; ++h) dst[h] = (uint8_t)nnew[h];
         }
-        tile = ntile;
+        unit = next_unit;
         rp_lo = nrp_lo;
         rp_hi = nrp_hi;
     }
@@ -242,14 +250,14 @@ __global__ void k_exposure_hist_b(const int16_t *e, GraphRef gr, int64_t n_rows,
 
 // New exposures per instance and day: sum of the per-tile bytes over the tiles of
 // a chunk, added to newinf[inst][t] (integer sums: the order does not matter).
-__global__ void k_newinf_b(const uint8_t *tile_new, int ntiles, const int32_t *tile0, const int32_t *ntl, int B,
+__global__ void k_newinf_b(const uint8_t *unit_new, int nunits, const int32_t *unit0, const int32_t *nu, int B,
                            int Bp, int t0, int ldP, int32_t *newinf) {
     const int c = blockIdx.x, d = blockIdx.y, g = blockIdx.z;
     const int t = t0 + d;
-    const int nt = ntl[g];
+    const int nt = nu[g];
     const int i0 = c * kReduceChunkTiles * 4, i1 = min(nt, i0 + kReduceChunkTiles * 4);
     if (i0 >= nt) return;
-    const uint8_t *base = tile_new + ((size_t)t * ntiles + tile0[g]) * Bp;
+    const uint8_t *base = unit_new + ((size_t)t * nunits + unit0[g]) * Bp;
     for (int s = threadIdx.x; s < B; s += blockDim.x) {
         int acc = 0;
         for (int i = i0; i < i1; ++i) acc += base[(size_t)i * Bp + s];
@@ -287,16 +295,24 @@ __global__ void k_counts_b(const int32_t *H, const int32_t *newinf, const int32_
 
 // Level 1 of the parameter-gradient reduction: Pc[t][g][c][a][s] = sum over the
 // tiles [c K, min((c+1) K, ntiles_g)) of graph g of P[t][tile][a][s], K = kReduceChunkTiles.
-__global__ void k_reduce_b1(const double *P, int ntiles, const int32_t *tile0, const int32_t *ntl, int G, int Bp,
+__global__ void k_reduce_b1(const float *P, int nunits, const int32_t *unit0, const int32_t *nu, int G, int Bp,
                             int max_chunks, double *Pc) {
     const int c = blockIdx.x, t = blockIdx.y, g = blockIdx.z;
     const int wdt = kAges * Bp;
-    const int nt = ntl[g];
+    const int nt = nu[g];
     const int i0 = c * kReduceChunkTiles, i1 = min(nt, i0 + kReduceChunkTiles);
-    const double *base = P + ((size_t)t * ntiles + tile0[g]) * wdt;
+    const float *base = P + ((size_t)t * nunits + unit0[g]) * wdt;
     for (int k = threadIdx.x; k < wdt; k += blockDim.x) {
         double acc = 0.0;
-        for (int i = i0; i < i1; ++i) acc += base[(size_t)i * wdt + k];
+        int i = i0;
+        for (; i + 4 <= i1; i += 4) {
+            float v[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) v[u] = base[(size_t)(i + u) * wdt + k];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) acc += (double)v[u];
+        }
+        for (; i < i1; ++i) acc += (double)base[(size_t)i * wdt + k];
         Pc[(((size_t)t * G + g) * max_chunks + c) * wdt + k] = acc;
     }
 }
@@ -320,21 +336,21 @@ __global__ void k_reduce_b2(const double *Pc, int G, int B, int Bp, int T, int m
 // out-edges of w r(0) (r(0) at scale 2^sigma(0) of its graph).  The thread adds its
 // tile's seeds in row order, so the sums do not depend on scheduling.
 __global__ void k_dc_seeds_b(Csr m, const int16_t *E, const float *r0, GraphRef gr, const int32_t *sig,
-                             int ld_sig, int ntiles, int L, int B, int Bp, double *dc_tile) {
-    const int64_t total = (int64_t)ntiles * B;
+                             int ld_sig, int nunits, int ru, int L, int B, int Bp, double *dc_tile) {
+    const int64_t total = (int64_t)nunits * B;
     for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < total;
          idx += (int64_t)gridDim.x * blockDim.x) {
-        const int tile = (int)(idx / B), s = (int)(idx - (int64_t)tile * B);
-        const int g = gr.tile_graph ? (int)gr.tile_graph[tile] : 0;
+        const int unit = (int)(idx / B), s = (int)(idx - (int64_t)unit * B);
+        const int g = gr.tile_graph ? (int)gr.tile_graph[unit * ru / kTile] : 0;
         const double scale = ldexp(1.0, sig[(size_t)g * ld_sig]);
-        for (int r = 0; r < kTile; ++r) {
-            const int row = tile * kTile + r;
+        for (int r = 0; r < ru; ++r) {
+            const int row = unit * ru + r;
             const int Eh = E[(size_t)row * Bp + s];
             if (Eh == kPad || Eh >= 0 || -Eh > L - 1) continue;
             float gx = 0.f;
             for (uint32_t p = m.rowptr[row]; p < m.rowptr[row + 1]; ++p)
                 gx = __fmaf_rn(m.w[p], r0[(size_t)m.col[p] * Bp + s], gx);
-            dc_tile[((size_t)tile * L - Eh) * Bp + s] += (double)gx * scale;
+            dc_tile[((size_t)unit * L - Eh) * Bp + s] += (double)gx * scale;
         }
     }
 }
@@ -408,13 +424,13 @@ cudaError_t launch_exposure_hist_b(const int16_t *e, GraphRef gr, int64_t n_rows
     return cudaGetLastError();
 }
 
-cudaError_t launch_counts_b(const uint8_t *tile_new, int ntiles, const int32_t *d_tile0, const int32_t *d_ntiles,
-                            const int32_t *d_rows, int G, int B, int Bp, int max_tiles, int t0, int T, int ldP,
+cudaError_t launch_counts_b(const uint8_t *unit_new, int nunits, const int32_t *d_unit0, const int32_t *d_nunits,
+                            const int32_t *d_rows, int G, int B, int Bp, int max_units, int t0, int T, int ldP,
                             int tau_EI, int L, const int32_t *H, int32_t *newinf, int32_t *counts, int32_t *newRM,
                             cudaStream_t s) {
     if (T > t0) {
-        const int chunks = (max_tiles + kReduceChunkTiles * 4 - 1) / (kReduceChunkTiles * 4);
-        k_newinf_b<<<dim3(std::max(chunks, 1), T - t0, G), 64, 0, s>>>(tile_new, ntiles, d_tile0, d_ntiles, B, Bp, t0,
+        const int chunks = (max_units + kReduceChunkTiles * 4 - 1) / (kReduceChunkTiles * 4);
+        k_newinf_b<<<dim3(std::max(chunks, 1), T - t0, G), 64, 0, s>>>(unit_new, nunits, d_unit0, d_nunits, B, Bp, t0,
                                                                         ldP, newinf);
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
@@ -424,12 +440,12 @@ cudaError_t launch_counts_b(const uint8_t *tile_new, int ntiles, const int32_t *
     return cudaGetLastError();
 }
 
-cudaError_t launch_bwd_reduce_b(const double *P, int ntiles, const int32_t *d_tile0, const int32_t *d_ntiles, int G,
+cudaError_t launch_bwd_reduce_b(const float *P, int nunits, const int32_t *d_tile0, const int32_t *d_ntiles, int G,
                                 int B, int Bp, int T, double *scratch, int max_chunks, const int32_t *sig,
                                 int ld_sig, double *Q, cudaStream_t s) {
     const int wdt = kAges * Bp;
     const int threads = std::min(1024, (wdt + 31) / 32 * 32);
-    k_reduce_b1<<<dim3(max_chunks, T, G), threads, 0, s>>>(P, ntiles, d_tile0, d_ntiles, G, Bp, max_chunks, scratch);
+    k_reduce_b1<<<dim3(max_chunks, T, G), threads, 0, s>>>(P, nunits, d_tile0, d_ntiles, G, Bp, max_chunks, scratch);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     k_reduce_b2<<<dim3(T, G), threads, 0, s>>>(scratch, G, B, Bp, T, max_chunks, sig, ld_sig, Q);
@@ -437,10 +453,10 @@ cudaError_t launch_bwd_reduce_b(const double *P, int ntiles, const int32_t *d_ti
 }
 
 cudaError_t launch_dc_seeds_b(Csr m_out, const int16_t *E, const float *r0, GraphRef gr, const int32_t *sig,
-                              int ld_sig, int ntiles, int L, int B, int Bp, double *dc_tile, cudaStream_t s) {
-    const int64_t total = (int64_t)ntiles * B;
+                              int ld_sig, int nunits, int ru, int L, int B, int Bp, double *dc_tile, cudaStream_t s) {
+    const int64_t total = (int64_t)nunits * B;
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((total + 255) / 256, 65535));
-    k_dc_seeds_b<<<grid, 256, 0, s>>>(m_out, E, r0, gr, sig, ld_sig, ntiles, L, B, Bp, dc_tile);
+    k_dc_seeds_b<<<grid, 256, 0, s>>>(m_out, E, r0, gr, sig, ld_sig, nunits, ru, L, B, Bp, dc_tile);
     return cudaGetLastError();
 }
 

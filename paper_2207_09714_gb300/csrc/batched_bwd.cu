@@ -17,10 +17,13 @@ namespace {
 // symmetric weights): lambda is not stored but summed again from the final exposure
 // days over the same entries, with the forward's marking (a.bits_t) and order, so it
 // is bitwise the forward's.
+// Eight sets a lane need 125 registers (two blocks an SM; at three they spill), four or two
+// fit three blocks.
 template <int LPR, int SPL, bool KAHAN, bool DC, bool REC = false>
-__global__ void __launch_bounds__(kBlock, GABM_BBWD_MINBLOCKS) k_bwd_day_b(const BwdBatchArgs a) {
+__global__ void __launch_bounds__(kBlock, SPL <= 4 ? 3 : 2) k_bwd_day_b(const BwdBatchArgs a) {
     constexpr int RPW = 32 / LPR;
     constexpr int Bc = LPR * SPL;        // sets of this launch (a chunk of the row's Bw)
+    constexpr int CPL = chunk_per_lane<LPR>();
     constexpr int NW = kBlock / 32;
     // DC: per-warp tile sums [L][Bc] of gx at the rows' infectious days, by k = t + 1 - E
     extern __shared__ float dcs_all[];
@@ -28,6 +31,7 @@ __global__ void __launch_bounds__(kBlock, GABM_BBWD_MINBLOCKS) k_bwd_day_b(const
     __shared__ int slot_k[kMaxL];
     __shared__ float pacc[NW][kAges][Bc];   // per-warp tile sums of gl * Lam by age and set
     __shared__ float fac_s[NW][kMaxL];       // 2^(sigma(t+k) - sigma(t)) of the warp's graph
+    __shared__ int kl_s[NW][kMaxL];          // the k >= 2 whose days carry adjoint, ascending
     if (threadIdx.x < kMaxL) {
         c_s[threadIdx.x] = a.c[threadIdx.x];
         slot_k[threadIdx.x] = a.ring_slot[threadIdx.x];
@@ -41,15 +45,13 @@ __global__ void __launch_bounds__(kBlock, GABM_BBWD_MINBLOCKS) k_bwd_day_b(const
     __syncthreads();
 
     const int grp = lane / LPR, q = lane % LPR;
-    const int t = a.t, T = a.T, L = a.L, B = a.B, ntiles = a.ntiles;
+    const int t = a.t, T = a.T, L = a.L, B = a.B, nunits = a.nunits, ru = a.ru;
+    const bool in_unit = grp < ru;       // a pass of more rows than the unit leaves groups idle
     const bool has_next = t + 1 < T;
     const uint32_t *E32 = reinterpret_cast<const uint32_t *>(a.E);
     const int Bw = a.Bw;                 // row width of the per-agent arrays
     const int s0 = a.s0 + q * SPL;       // this lane's first set
     const size_t stride = a.ring_stride;
-
-    auto ld = [&](uint32_t j, bool ok, FVec<SPL> &r) { ld_floats<SPL>(a.r_next + (size_t)j * Bw + s0, ok, r.v); };
-    auto val = [](const FVec<SPL> &r, int h) { return r.v[h]; };
 
     int cur_g = -1;
     float Rt[SPL], Gtail[SPL];
@@ -62,22 +64,23 @@ __global__ void __launch_bounds__(kBlock, GABM_BBWD_MINBLOCKS) k_bwd_day_b(const
     bool rnz_w = false;            // this lane stored an r other than 0
     uint32_t touched = 0u;         // DC: the k rows of dcs this lane added to in the current tile
     TileDispenser disp;
-    disp.init(a.tile_ctr, ntiles, gridDim.x * NW, lane);
-    // row bounds of the tile's 32 rows (lane r: rows r and r + 1), one tile ahead
-    int tile = disp.get();
+    disp.init(a.tile_ctr, nunits, gridDim.x * NW, lane);
+    // row bounds of the unit's rows (lane r: rows r and r + 1), one unit ahead
+    int unit = disp.get();
     uint32_t rp_lo = 0u, rp_hi = 0u;
-    if (tile < ntiles) {
-        rp_lo = a.m.rowptr[tile * kTile + lane];
-        rp_hi = a.m.rowptr[tile * kTile + lane + 1];
+    if (unit < nunits && lane < ru) {
+        rp_lo = a.m.rowptr[unit * ru + lane];
+        rp_hi = a.m.rowptr[unit * ru + lane + 1];
     }
-    while (tile < ntiles) {
-        const int ntile = disp.get();
+    while (unit < nunits) {
+        const int next_unit = disp.get();
         uint32_t nrp_lo = 0u, nrp_hi = 0u;
-        if (ntile < ntiles) {
-            nrp_lo = a.m.rowptr[ntile * kTile + lane];
-            nrp_hi = a.m.rowptr[ntile * kTile + lane + 1];
+        if (next_unit < nunits && lane < ru) {
+            nrp_lo = a.m.rowptr[next_unit * ru + lane];
+            nrp_hi = a.m.rowptr[next_unit * ru + lane + 1];
         }
-        const int g = a.gr.tile_graph ? (int)a.gr.tile_graph[tile] : 0;
+        const int row0 = unit * ru;
+        const int g = a.gr.tile_graph ? (int)a.gr.tile_graph[row0 / kTile] : 0;
         if (g != cur_g) {
             if (cur_g >= 0) {
                 flush_emax(a.emax + (size_t)cur_g * a.ld_sig + t, emax_w);
@@ -86,10 +89,11 @@ __global__ void __launch_bounds__(kBlock, GABM_BBWD_MINBLOCKS) k_bwd_day_b(const
                 rnz_w = false;
             }
             live_k = carries_adjoint(a.rnz + (size_t)g * a.ld_sig, t, T, L);
+            if (((live_k & ~3u) >> lane) & 1u) kl_s[wib][__popc(live_k & ~3u & ((1u << lane) - 1u))] = lane;
             cur_g = g;
             sg = a.sig + (size_t)g * a.ld_sig;
             sig_t = next_sigma(sg[t + 1], a.emax[(size_t)g * a.ld_sig + t + 1]);
-            if (lane == 0 && tile * kTile == a.gr.row0[g]) a.sig[(size_t)g * a.ld_sig + t] = sig_t;  // one writer
+            if (lane == 0 && row0 == a.gr.row0[g]) a.sig[(size_t)g * a.ld_sig + t] = sig_t;  // one writer
             if (lane < kMaxL)
                 fac_s[wib][lane] = (lane >= 1 && lane < L && t + lane <= T) ? exp2i(sg[t + lane] - sig_t) : 0.f;
             __syncwarp();
@@ -102,15 +106,14 @@ __global__ void __launch_bounds__(kBlock, GABM_BBWD_MINBLOCKS) k_bwd_day_b(const
             }
         }
         const float inv_D = a.gr.inv_Dbar[g];
-        uint32_t word = 0u;
-        PassRow<SPL> nx;
-        load_pass_row<SPL>(a.m, E32 + ((size_t)(tile * kTile + grp) * Bw + s0) / 2, rp_lo, rp_hi, grp, q, nx);
-        for (int pass = 0; pass < LPR; ++pass) {
-            const int row = tile * kTile + pass * RPW + grp;
+        PassRow<LPR, SPL, CPL> nx;
+        load_pass_row<LPR, SPL, CPL>(a.m, E32 + ((size_t)(row0 + grp) * Bw + s0) / 2, in_unit, rp_lo, rp_hi, grp, q, nx);
+        for (int pass = 0; pass * RPW < ru; ++pass) {
+            const int row = row0 + pass * RPW + grp;
             const size_t xo = (size_t)row * Bw + s0;   // this lane's first slot
-            const PassRow<SPL> cu = nx;
-            if (pass + 1 < LPR)   // the next pass's row in flight while this one is summed
-                load_pass_row<SPL>(a.m, E32 + (xo + (size_t)RPW * Bw) / 2, rp_lo, rp_hi, (pass + 1) * RPW + grp, q, nx);
+            const PassRow<LPR, SPL, CPL> cu = nx;
+            if ((pass + 1) * RPW < ru)   // the next pass's row in flight while this one is summed
+                load_pass_row<LPR, SPL, CPL>(a.m, E32 + (xo + (size_t)RPW * Bw) / 2, true, rp_lo, rp_hi, (pass + 1) * RPW + grp, q, nx);
             uint32_t ew[SPL / 2];
 #pragma unroll
             for (int k = 0; k < SPL / 2; ++k) ew[k] = cu.ew[k];
@@ -138,9 +141,21 @@ __global__ void __launch_bounds__(kBlock, GABM_BBWD_MINBLOCKS) k_bwd_day_b(const
                 dc_any |= dch[h];
             }
             const bool act = (group_bits<LPR>(__ballot_sync(kFull, needA_any || dc_any)) >> grp) & 1u;
+            // the pass's lines of the ring, A and lambda into L2 while its rows are gathered: they
+            // come from DRAM (the ring alone is many times L2), and the rows of a pass are
+            // consecutive, SPL 128-byte lines of each array
+            if (Bw == Bc && RPW <= ru && (live_k != 0u || __any_sync(kFull, anyS))) {
+                const size_t base = (size_t)(row0 + pass * RPW) * Bw;
+                const int nk = __popc(live_k & ~3u);
+                for (int i = lane; i < (nk + 2) * SPL; i += 32) {
+                    const int k = i / SPL;
+                    const float *p = k < nk ? a.ring + (size_t)slot_k[kl_s[wib][k]] * stride
+                                            : (k == nk ? a.A : (REC ? a.A : a.lam_t));
+                    asm volatile("prefetch.global.L2 [%0];" ::"l"(p + base + (size_t)(i % SPL) * 32));
+                }
+            }
             float gx[SPL];
-            group_row_sums<LPR, SPL, KAHAN, FVec<SPL>>(a.m, cu.p0, act ? cu.len : 0u, cu.j0, cu.w0, a.rbits_next, lane,
-                                                       ld, val, gx);
+            group_gather_sums<LPR, SPL, CPL, KAHAN>(a.m, cu.p0, act ? cu.len : 0u, cu.j0, cu.w0, a.r_next + s0, Bw, lane, gx);
             if (needA_any) st_floats<SPL>(a.ring + (size_t)slot_k[1] * stride + xo, gx);
             if constexpr (DC) {
                 // the groups add their rows in a fixed order
@@ -167,7 +182,7 @@ __global__ void __launch_bounds__(kBlock, GABM_BBWD_MINBLOCKS) k_bwd_day_b(const
                 auto vale = [&](const EWords<SPL> &rw, int h) {
                     return infect_lut(half_of(rw.w[h >> 1], h & 1), c_s, t, (unsigned)L);
                 };
-                group_row_sums<LPR, SPL, KAHAN, EWords<SPL>>(a.m, cu.p0, actl ? cu.len : 0u, cu.j0, cu.w0, a.bits_t,
+                group_row_sums<LPR, SPL, CPL, KAHAN, EWords<SPL>>(a.m, cu.p0, actl ? cu.len : 0u, cu.j0, cu.w0, a.bits_t,
                                                              lane, lde, vale, Lrec);
 #pragma unroll
                 for (int h = 0; h < SPL; ++h) Lrec[h] = Lrec[h] * inv_D;
@@ -217,33 +232,37 @@ __global__ void __launch_bounds__(kBlock, GABM_BBWD_MINBLOCKS) k_bwd_day_b(const
                             for (int h = 0; h < SPL; ++h) G[h] = __fmaf_rn(c_s[k], rv[u][h] * fac_s[wib][k], G[h]);
                     }
                 }
-                float rc[SPL];
+                // Every set's own chain (the window of A, then exp, Philox and the division) without
+                // a branch between the sets, so that the eight chains overlap.
+                float rc[SPL], dy[SPL], RS[SPL];
                 float stored = 0.f;
+                bool draw = false;   // some set's dL/dy is not 0 (or its lambda not finite)
 #pragma unroll
                 for (int h = 0; h < SPL; ++h) {
-                    rc[h] = 0.f;
-                    if (!isS[h]) continue;
                     const int Eh = half_of(ew[h >> 1], h & 1);
-                    float dy;
-                    if (Eh == t) { Av[h] = G[h]; dy = G[h]; }
-                    else if (Eh == kNever) dy = G[h];
-                    else dy = G[h] - Av[h] * exp2i(sg[Eh] - sig_t);   // A was stored on day Eh
-                    stored = fmaxf(stored, fabsf(G[h]));
-                    const int inst = g * B + s0 + h;
-                    const float RS = Rt[h] * a.S[inst * kAges + ai];
-                    const float lam = RS * Lv[h];
-                    float glam = dy;   // dy = 0 and lambda finite: the product with dy/dlambda >= 0 is dy itself
-                    if (!(dy == 0.f && lam >= 0.f && lam < __int_as_float(0x7f800000))) {
+                    float As = Av[h];   // stored on day Eh; sigma(t) = 0 means 0 on every later day too
+                    if (sig_t != 0 && isS[h] && Eh != kNever && Eh != t) As *= exp2i(sg[Eh] - sig_t);
+                    dy[h] = (Eh == t || Eh == kNever) ? G[h] : G[h] - As;
+                    if (isS[h] && Eh == t) Av[h] = G[h];
+                    RS[h] = Rt[h] * (isS[h] ? a.S[(g * B + s0 + h) * kAges + ai] : 0.f);
+                    const float lam = RS[h] * Lv[h];
+                    draw |= isS[h] && !(dy[h] == 0.f && lam >= 0.f && lam < __int_as_float(0x7f800000));
+                }
+#pragma unroll
+                for (int h = 0; h < SPL; ++h) {
+                    float glam = dy[h];   // dy = 0 and lambda finite: the product with dy/dlambda >= 0 is dy itself
+                    if (draw) {
+                        const float lam = RS[h] * Lv[h];
                         const float qv = expf(-lam);
                         const float p = -expm1f(-lam);
-                        const float u = uniform_from_word(philox_word(a.seed, id, (uint32_t)t, (uint32_t)inst, 0u));
+                        const float u = uniform_from_word(philox_word(a.seed, id, (uint32_t)t, (uint32_t)(g * B + s0 + h), 0u));
                         const float den = __fmaf_rn(p, 1.f - u, qv * u);
                         const float dydl = (u * (1.f - u)) * qv / (den * den);
-                        glam = dy * dydl;
+                        glam = dy[h] * dydl;
                     }
-                    rc[h] = RS * glam * inv_D;
-                    v[h] = glam * Lv[h];
-                    stored = fmaxf(stored, fabsf(rc[h]));
+                    rc[h] = isS[h] ? RS[h] * glam * inv_D : 0.f;
+                    v[h] = isS[h] ? glam * Lv[h] : 0.f;
+                    stored = fmaxf(stored, isS[h] ? fmaxf(fabsf(G[h]), fabsf(rc[h])) : 0.f);
                     rnz_w |= !(rc[h] == 0.f);
                 }
                 emax_w = max(emax_w, (unsigned)(float_exponent(stored) + 128));
@@ -258,17 +277,15 @@ __global__ void __launch_bounds__(kBlock, GABM_BBWD_MINBLOCKS) k_bwd_day_b(const
                     for (int h = 0; h < SPL; ++h) pacc[wib][ai][q * SPL + h] += v[h];
                 __syncwarp();
             }
-            word |= group_bits<LPR>(__ballot_sync(kFull, anyS)) << (pass * RPW);
         }
-        // per-tile sums by age and set: fp32 over the tile's 32 rows, FP64 from here on
-        double *Pt = a.P_t + (size_t)tile * kAges * Bw + a.s0;
+        // per-unit sums by age and set: fp32 over the unit's rows, FP64 from the reduction on
+        float *Pt = a.P_t + (size_t)unit * kAges * Bw + a.s0;
         for (int i = lane; i < kAges * Bc; i += 32) {
             float *cell = &pacc[wib][0][0] + i;
-            Pt[(i / Bc) * Bw + (i % Bc)] = (double)*cell;
+            Pt[(i / Bc) * Bw + (i % Bc)] = *cell;
             *cell = 0.f;
         }
         __syncwarp();
-        if (lane == 0) a.rbits_cur[tile] = word;
         if constexpr (DC) {
             // the tile's sums of the table adjoint, at the scale of day t+1, into FP64 (the
             // warp holding the tile is the only writer of its accumulators on this day)
@@ -276,7 +293,7 @@ __global__ void __launch_bounds__(kBlock, GABM_BBWD_MINBLOCKS) k_bwd_day_b(const
             touched = 0u;
             if (tm) {
                 const double scale = ldexp(1.0, sg[t + 1]);
-                double *dt = a.dc_tile + (size_t)tile * L * Bw + a.s0;
+                double *dt = a.dc_tile + (size_t)unit * L * Bw + a.s0;
                 while (tm) {
                     const int k = __ffs(tm) - 1;
                     tm &= tm - 1u;
@@ -291,7 +308,7 @@ __global__ void __launch_bounds__(kBlock, GABM_BBWD_MINBLOCKS) k_bwd_day_b(const
                 __syncwarp();
             }
         }
-        tile = ntile;
+        unit = next_unit;
         rp_lo = nrp_lo;
         rp_hi = nrp_hi;
     }

@@ -13,9 +13,6 @@
 #ifndef GABM_BFWD_MINBLOCKS
 #define GABM_BFWD_MINBLOCKS 3
 #endif
-#ifndef GABM_BBWD_MINBLOCKS
-#define GABM_BBWD_MINBLOCKS 2
-#endif
 
 namespace gabm {
 
@@ -102,37 +99,60 @@ __device__ __forceinline__ float infect_lut(int e, const float *c_s, int t, unsi
     return c_s[min((unsigned)(t - e), L)];
 }
 
+// A group of LPR lanes holds CPL entries of its row a lane at a time (a chunk: entry i LPR + q
+// is lane q's i-th).  The reverse sweep, which gathers for nearly every entry, holds at
+// least eight: with one a lane and two lanes a row, a row of 22 entries was eleven rounds
+// of dependent loads.  The forward keeps one: it gathers few of its entries, and the
+// selection among several cost it more (53 to 65 us a day on 50k agents x 12 sets).
+template <int LPR>
+constexpr int chunk_per_lane() { return LPR >= 8 ? 1 : 8 / LPR; }
+
 // Row data of one pass (one row per group), loaded a pass ahead of use: the
 // lane's exposure words of its row, the row's entry range and the first chunk
-// of its entries (entry q for lane q of the group).
-template <int SPL>
+// of its entries.
+template <int LPR, int SPL, int CPL>
 struct PassRow {
     uint32_t ew[SPL / 2];
     uint32_t p0, len;      // entries [p0, p0 + len)
-    uint32_t j0;           // column and weight of entry q, when q < len
-    float w0;
+    uint32_t j0[CPL];
+    float w0[CPL];
 };
 
-// Loads the pass row of tile row r (0..31) into pr; lane r holds the row bounds
-// (rowptr of tile row r and r + 1) in rp_lo / rp_hi.  Called by all 32 lanes.
-template <int SPL>
-__device__ __forceinline__ void load_pass_row(const Csr &m, const uint32_t *ew_ptr, uint32_t rp_lo, uint32_t rp_hi,
-                                              int r, int q, PassRow<SPL> &pr) {
+// This lane's entries of the chunk at k0 of a row of len entries at p0 (0 past its end).
+template <int LPR, int CPL>
+__device__ __forceinline__ void load_chunk(const Csr &m, uint32_t p0, uint32_t len, uint32_t k0, int q,
+                                           uint32_t (&j)[CPL], float (&w)[CPL]) {
+#pragma unroll
+    for (int i = 0; i < CPL; ++i) {
+        const uint32_t k = k0 + (uint32_t)(i * LPR + q);
+        j[i] = ld_cs_if(m.col + p0 + k, k < len);
+        w[i] = ld_cs_if(m.w + p0 + k, k < len);
+    }
+}
+
+// Loads the pass row of unit row r into pr, or an empty padding row when !ok; lane r holds the
+// row bounds (rowptr of unit row r and r + 1; 0 past the unit) in rp_lo / rp_hi.  Called by all 32 lanes.
+template <int LPR, int SPL, int CPL>
+__device__ __forceinline__ void load_pass_row(const Csr &m, const uint32_t *ew_ptr, bool ok, uint32_t rp_lo, uint32_t rp_hi,
+                                              int r, int q, PassRow<LPR, SPL, CPL> &pr) {
     pr.p0 = __shfl_sync(kFull, rp_lo, r);
     pr.len = __shfl_sync(kFull, rp_hi, r) - pr.p0;
-    ld_words<SPL>(ew_ptr, true, pr.ew);
-    const bool v = (uint32_t)q < pr.len;
-    pr.j0 = ld_cs_if(m.col + pr.p0 + q, v);
-    pr.w0 = ld_cs_if(m.w + pr.p0 + q, v);
+    ld_words<SPL>(ew_ptr, ok, pr.ew);
+    if (!ok) {   // no row: every set a padding one
+#pragma unroll
+        for (int k = 0; k < SPL / 2; ++k) pr.ew[k] = 0x80008000u;
+    }
+    load_chunk<LPR, CPL>(m, pr.p0, pr.len, 0u, q, pr.j0, pr.w0);
 }
 
 // V marked entries of the current chunk, taken from mm in entry order (lowest lane
 // of the group first): their columns and weights broadcast from the lanes holding
 // them, every lane's gathers issued before any of their values is used, then the
 // sums.  Slots past the group's last marked entry carry weight 0 and load nothing.
-template <int V, int LPR, int SPL, bool KAHAN, class Raw, class Ld, class Val>
-__device__ __forceinline__ void gather_batch(unsigned &mm, uint32_t j, float w, Ld &ld, Val &val, float (&sum)[SPL],
-                                             float (&comp)[SPL]) {
+template <int V, int LPR, int SPL, int CPL, bool KAHAN, class Raw, class Ld, class Val>
+__device__ __forceinline__ void gather_batch(unsigned &mm, const uint32_t (&j)[CPL],
+                                             const float (&w)[CPL], Ld &ld, Val &val,
+                                             float (&sum)[SPL], float (&comp)[SPL]) {
     uint32_t jv[V];
     float wv[V];
     bool ok[V];
@@ -141,8 +161,16 @@ __device__ __forceinline__ void gather_batch(unsigned &mm, uint32_t j, float w, 
         ok[u] = mm != 0u;
         const int src = ok[u] ? __ffs(mm) - 1 : 0;
         mm &= mm - 1u;
-        jv[u] = __shfl_sync(kFull, j, src, LPR);
-        const float ws = __shfl_sync(kFull, w, src, LPR);
+        uint32_t js = j[0];   // the group's lanes agree on src, so each offers its entry of that round
+        float wsl = w[0];
+#pragma unroll
+        for (int i = 1; i < CPL; ++i)
+            if (src / LPR == i) {
+                js = j[i];
+                wsl = w[i];
+            }
+        jv[u] = __shfl_sync(kFull, js, src % LPR, LPR);
+        const float ws = __shfl_sync(kFull, wsl, src % LPR, LPR);
         wv[u] = ok[u] ? ws : 0.f;   // a zero weight leaves a plain sum unchanged
     }
     Raw rv[V];
@@ -157,15 +185,17 @@ __device__ __forceinline__ void gather_batch(unsigned &mm, uint32_t j, float w, 
 // For this lane's group row (entries [p0, p0 + len)), sum[h] = sum over the
 // entries whose column is marked in `bits` of w * x_h(j), in entry order, where
 // ld(j, ok, raw) gathers column j's values for this lane's sets (predicated by
-// ok) and val(raw, h) is set h's value.  (j0, w0) is the row's entry q, loaded
-// by the caller; each later chunk of LPR entries is in flight while the one
-// before it is used.  A chunk's marked entries go in batches of U gathers in
+// ok) and val(raw, h) is set h's value.  (j0, w0) are this lane's
+// entries of the first chunk, loaded by the caller; each later chunk is in flight while
+// the one before it is used.  A chunk's marked entries go in batches of U gathers in
 // flight, and the rest (fewer than U, counted by the group with the most) in
 // batches of U/2, U/4, ..., 1: where few neighbours are marked, as early in an
 // epidemic, a batch no larger than needed is most of the saving.  Called by all
 // 32 lanes.
-template <int LPR, int SPL, bool KAHAN, class Raw, class Ld, class Val>
-__device__ __forceinline__ void group_row_sums(const Csr &m, uint32_t p0, uint32_t len, uint32_t j0, float w0,
+template <int LPR, int SPL, int CPL, bool KAHAN, class Raw, class Ld, class Val>
+__device__ __forceinline__ void group_row_sums(const Csr &m, uint32_t p0, uint32_t len,
+                                               const uint32_t (&j0)[CPL],
+                                               const float (&w0)[CPL],
                                                const uint32_t *__restrict__ bits, int lane, Ld ld, Val val,
                                                float (&sum)[SPL]) {
     constexpr int U = (SPL == 8) ? 4 : 8;
@@ -175,26 +205,92 @@ __device__ __forceinline__ void group_row_sums(const Csr &m, uint32_t p0, uint32
 #pragma unroll
     for (int h = 0; h < SPL; ++h) sum[h] = comp[h] = 0.f;
     const uint32_t kmax = __reduce_max_sync(kFull, len);
-    uint32_t jn = j0;
-    float wn = w0;
-    for (uint32_t k0 = 0; k0 < kmax; k0 += LPR) {
-        const uint32_t kk = k0 + (uint32_t)q;
-        const bool valid = kk < len;
-        const uint32_t j = jn;
-        const float w = wn;
-        const bool vn = kk + LPR < len;
-        jn = ld_cs_if(m.col + p0 + kk + LPR, vn);
-        wn = ld_cs_if(m.w + p0 + kk + LPR, vn);
-        const bool mk = valid && marked(bits, j);
-        unsigned mm = (__ballot_sync(kFull, mk) >> (grp * LPR)) & gmask;
+    constexpr int CH = CPL * LPR;
+    uint32_t jn[CPL];
+    float wn[CPL];
+#pragma unroll
+    for (int i = 0; i < CPL; ++i) {
+        jn[i] = j0[i];
+        wn[i] = w0[i];
+    }
+    for (uint32_t k0 = 0; k0 < kmax; k0 += CH) {
+        uint32_t j[CPL];
+        float w[CPL];
+#pragma unroll
+        for (int i = 0; i < CPL; ++i) {
+            j[i] = jn[i];
+            w[i] = wn[i];
+        }
+        load_chunk<LPR, CPL>(m, p0, len, k0 + CH, q, jn, wn);
+        bool mk[CPL];
+#pragma unroll
+        for (int i = 0; i < CPL; ++i) mk[i] = k0 + (uint32_t)(i * LPR + q) < len && marked(bits, j[i]);
+        unsigned mm = 0u;   // the group's marked entries of the chunk, in entry order
+#pragma unroll
+        for (int i = 0; i < CPL; ++i) mm |= ((__ballot_sync(kFull, mk[i]) >> (grp * LPR)) & gmask) << (i * LPR);
         const int nmax = (int)__reduce_max_sync(kFull, (unsigned)__popc(mm));
         int i0 = 0;
-        for (; i0 + U <= nmax; i0 += U) gather_batch<U, LPR, SPL, KAHAN, Raw>(mm, j, w, ld, val, sum, comp);
+        for (; i0 + U <= nmax; i0 += U) gather_batch<U, LPR, SPL, CPL, KAHAN, Raw>(mm, j, w, ld, val, sum, comp);
         const int rest = nmax - i0;   // < U, warp-uniform
         if constexpr (U >= 8)
-            if (rest & 4) gather_batch<4, LPR, SPL, KAHAN, Raw>(mm, j, w, ld, val, sum, comp);
-        if (rest & 2) gather_batch<2, LPR, SPL, KAHAN, Raw>(mm, j, w, ld, val, sum, comp);
-        if (rest & 1) gather_batch<1, LPR, SPL, KAHAN, Raw>(mm, j, w, ld, val, sum, comp);
+            if (rest & 4) gather_batch<4, LPR, SPL, CPL, KAHAN, Raw>(mm, j, w, ld, val, sum, comp);
+        if (rest & 2) gather_batch<2, LPR, SPL, CPL, KAHAN, Raw>(mm, j, w, ld, val, sum, comp);
+        if (rest & 1) gather_batch<1, LPR, SPL, CPL, KAHAN, Raw>(mm, j, w, ld, val, sum, comp);
+    }
+}
+
+// sum[h] = sum over the row's entries of w x_h(j), in entry order, with no bitmap: for
+// values that are 0 where a bitmap would leave a neighbour out (the reverse sweep's
+// coefficients, which are 0 from the start for rows not yet reached).  Nearly every
+// neighbour counts there, so a test of each, its compaction and its round trip cost more than
+// the few gathers of zeros.  U gathers a lane are in flight.  Called by all 32 lanes.
+template <int LPR, int SPL, int CPL, bool KAHAN>
+__device__ __forceinline__ void group_gather_sums(const Csr &m, uint32_t p0, uint32_t len,
+                                                  const uint32_t (&j0)[CPL],
+                                                  const float (&w0)[CPL], const float *x, int Bw,
+                                                  int lane, float (&sum)[SPL]) {
+    constexpr int U = (SPL == 8) ? 4 : 8;
+    constexpr int CH = CPL * LPR;
+    const int q = lane % LPR;
+    float comp[SPL];
+#pragma unroll
+    for (int h = 0; h < SPL; ++h) sum[h] = comp[h] = 0.f;
+    const uint32_t kmax = __reduce_max_sync(kFull, len);
+    uint32_t jn[CPL];
+    float wn[CPL];
+#pragma unroll
+    for (int i = 0; i < CPL; ++i) {
+        jn[i] = j0[i];
+        wn[i] = w0[i];
+    }
+    for (uint32_t k0 = 0; k0 < kmax; k0 += CH) {
+        uint32_t j[CPL];
+        float w[CPL];
+#pragma unroll
+        for (int i = 0; i < CPL; ++i) {
+            j[i] = jn[i];
+            w[i] = wn[i];
+        }
+        load_chunk<LPR, CPL>(m, p0, len, k0 + CH, q, jn, wn);
+#pragma unroll
+        for (int u0 = 0; u0 < CH; u0 += U) {
+            if (k0 + (uint32_t)u0 >= kmax) break;
+            float rv[U][SPL];
+            float wv[U];
+            bool ok[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int c = u0 + u;   // entry c of the chunk: lane c % LPR's (c / LPR)-th
+                ok[u] = k0 + (uint32_t)c < len;
+                const uint32_t jv = __shfl_sync(kFull, j[c / LPR], c % LPR, LPR);
+                wv[u] = __shfl_sync(kFull, w[c / LPR], c % LPR, LPR);
+                ld_floats<SPL>(x + (size_t)jv * Bw, ok[u], rv[u]);
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+#pragma unroll
+                for (int h = 0; h < SPL; ++h) acc_add<KAHAN>(sum[h], comp[h], wv[u], rv[u][h], ok[u]);
+        }
     }
 }
 

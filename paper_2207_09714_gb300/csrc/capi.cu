@@ -83,10 +83,11 @@ struct gabm_ctx {
     // row-compressed edges (batched kernels): in-edges, and out-edges when not symmetric
     uint32_t *csr_rowptr = nullptr, *csr_col = nullptr, *t_csr_rowptr = nullptr, *t_csr_col = nullptr;
     float *csr_w = nullptr, *t_csr_w = nullptr;
-    uint32_t *rbits = nullptr;      // [Bp/2][2][ntiles] rows susceptible in some set of a chunk (batched backward)
     double *Pc = nullptr;           // [Tcap][G][max_chunks][9][Bp] first-level gradient sums (batched)
-    int max_chunks = 0, max_graph_tiles = 0;
-    uint8_t *tile_new = nullptr;    // [Tcap][ntiles][Bp] exposures per tile, set and day (batched)
+    int max_chunks = 0, max_graph_units = 0;
+    int ru = kTile, nunits = 0;     // batched: rows of a warp's unit of work, and the units (see unit_rows)
+    int32_t *d_unit0 = nullptr, *d_nunits = nullptr;   // [G] first unit of each graph and its units
+    uint8_t *unit_new = nullptr;    // [Tcap][nunits][Bp] exposures per unit, set and day (batched)
     int32_t *hist0 = nullptr;       // [I][L+2] exposure-day histogram of the forward's starting state
     int32_t *newinf = nullptr;      // [I][Tcap] exposures per instance and day
     int sigma = 1024;
@@ -101,7 +102,8 @@ struct gabm_ctx {
     int Tcap = 0;
     float *lam = nullptr;
     int32_t *counts = nullptr, *newRM = nullptr, *newRM_b = nullptr;
-    double *D = nullptr, *gD = nullptr, *y = nullptr, *P = nullptr, *Q = nullptr;
+    double *D = nullptr, *gD = nullptr, *y = nullptr, *Q = nullptr, *Qp = nullptr;   // Qp [Tcap][I][kReduceParts][9] (one set per graph)
+    float *P = nullptr;
     float *R = nullptr, *m = nullptr, *S = nullptr;
     double *dR_s = nullptr, *dm_s = nullptr, *dS_s = nullptr, *loss_s = nullptr;
     double *dc_tile = nullptr;      // [ntiles][kMaxL] table-adjoint accumulators (on request)
@@ -580,6 +582,19 @@ HostGraph permute_graph(const HostGraph &h, const std::vector<uint32_t> &order) 
     return o;
 }
 
+// Rows of a warp's unit of work in the batched kernels: 8, as long as a pass of at least two
+// sets a lane fills the unit, and 16 or 32 on graphs with so many tiles that each resident
+// warp of the backward (16 an SM) has eight units of those.  A whole tile a warp left a third
+// of the warps of a 50k-agent graph x 12 sets without one and gave the others a chain of
+// passes (day 56 + 53 us; now 34 + 39), and on 200k agents x 64 sets the last of two and a
+// half rounds ran nearly empty (forward 190 us a day, 129 with 16 rows, 116 with 8; backward
+// 306, 254, 238).  Smaller units cost memory and reduction time of the per-unit gradient sums.
+int unit_rows(int ntiles, int Bp, int num_sms) {
+    int ru = kTile;
+    while (ru > 8 && (int64_t)ntiles * (kTile / ru) < 8 * 16 * (int64_t)num_sms && Bp * (ru / 2) / 32 >= 2) ru /= 2;
+    return ru;
+}
+
 // Launches per backward day at most (the batched backward may split a row's sets).
 int max_bwd_chunks(const gabm_ctx *c) { return c->batched ? std::max(1, c->Bp / 2) : 1; }
 
@@ -590,10 +605,10 @@ gabm_status ensure_days(gabm_ctx *c, int T) {
     if (cap > GABM_MAX_DAYS) cap = GABM_MAX_DAYS;
     CK(cudaStreamSynchronize(c->stream));
     dfree(c, c->lam); dfree(c, c->counts); dfree(c, c->newRM); dfree(c, c->newRM_b);
-    dfree(c, c->D); dfree(c, c->gD); dfree(c, c->y); dfree(c, c->P); dfree(c, c->Q);
+    dfree(c, c->D); dfree(c, c->gD); dfree(c, c->y); dfree(c, c->P); dfree(c, c->Q); dfree(c, c->Qp);
     dfree(c, c->R); dfree(c, c->m);
     dfree(c, c->dR_s); dfree(c, c->dm_s); dfree(c, c->tile_ctr); dfree(c, c->bits); dfree(c, c->Pc);
-    dfree(c, c->tile_new); dfree(c, c->newinf);
+    dfree(c, c->unit_new); dfree(c, c->newinf);
     dfree(c, c->s_hist); dfree(c, c->y_hist); dfree(c, c->P_nrm); dfree(c, c->newRM_real);
     dfree(c, c->sig); dfree(c, c->emax); dfree(c, c->rnz); dfree(c, c->Pm);
     c->Tcap = 0;
@@ -605,7 +620,8 @@ gabm_status ensure_days(gabm_ctx *c, int T) {
     TRY(dalloc(c, &c->D, IT));
     TRY(dalloc(c, &c->gD, IT));
     TRY(dalloc(c, &c->y, IT));
-    TRY(dalloc(c, &c->P, (size_t)cap * c->ntiles * kAges * c->Bp));
+    TRY(dalloc(c, &c->P, (size_t)cap * (c->batched ? c->nunits : c->ntiles) * kAges * c->Bp));
+    if (!c->batched) TRY(dalloc(c, &c->Qp, IT * kAges * kReduceParts));
     if (c->fate) TRY(dalloc(c, &c->Pm, (size_t)cap * c->ntiles));
     if (c->soft) {
         TRY(dalloc(c, &c->s_hist, (size_t)cap * c->n_rows));
@@ -615,7 +631,7 @@ gabm_status ensure_days(gabm_ctx *c, int T) {
     }
     if (c->batched) {
         TRY(dalloc(c, &c->Pc, (size_t)cap * c->G * c->max_chunks * kAges * c->Bp));
-        TRY(dalloc(c, &c->tile_new, (size_t)cap * c->ntiles * c->Bp));
+        TRY(dalloc(c, &c->unit_new, (size_t)cap * c->nunits * c->Bp));
         TRY(dalloc(c, &c->newinf, IT));
     }
     TRY(dalloc(c, &c->Q, IT * kAges));
@@ -788,7 +804,8 @@ gabm_status forward_days_batched(gabm_ctx *c, int t0, int T, cudaStream_t s) {
     a.R = c->R;
     a.S = c->S;
     a.ldP = c->Tcap;
-    a.ntiles = c->ntiles;
+    a.nunits = c->nunits;
+    a.ru = c->ru;
     a.tau_EI = c->tau_EI;
     a.L = c->L;
     a.B = c->B;
@@ -805,13 +822,13 @@ gabm_status forward_days_batched(gabm_ctx *c, int t0, int T, cudaStream_t s) {
         a.tile_ctr = c->tile_ctr + t;
         a.bits_cur = c->bits + (size_t)t * c->ntiles;
         a.bits_next = c->bits + (size_t)(t + 1) * c->ntiles;
-        a.tile_new = c->tile_new + (size_t)t * c->ntiles * c->Bp;
+        a.unit_new = c->unit_new + (size_t)t * c->nunits * c->Bp;
         prof_begin(c, 0);
         LAUNCH(launch_fwd_day_b(a, c->Bp, c->spl_fwd, c->kahan_b, c->grid_fwd, s));
         prof_end(c, 0);
     }
-    LAUNCH(launch_counts_b(c->tile_new, c->ntiles, c->d_tile0, c->d_ntiles, c->d_rows, c->G, c->B, c->Bp,
-                           c->max_graph_tiles, t0, T, c->Tcap, c->tau_EI, c->L, c->hist0, c->newinf, c->counts,
+    LAUNCH(launch_counts_b(c->unit_new, c->nunits, c->d_unit0, c->d_nunits, c->d_rows, c->G, c->B, c->Bp,
+                           c->max_graph_units, t0, T, c->Tcap, c->tau_EI, c->L, c->hist0, c->newinf, c->counts,
                            c->newRM, s));
     return GABM_OK;
 }
@@ -821,7 +838,6 @@ gabm_status backward_days_batched(gabm_ctx *c, int T, cudaStream_t s) {
     const int ld = c->Tcap;
     const size_t nb = (size_t)c->n_rows * c->Bp;
     const int nch = c->Bp / c->bwd_chunk;
-    CK(cudaMemsetAsync(c->rbits, 0, sizeof(uint32_t) * 2 * (size_t)c->ntiles * nch, s));
     BwdBatchArgs a;
     a.m = csr_view(c, true);
     a.age = c->age;
@@ -835,7 +851,8 @@ gabm_status backward_days_batched(gabm_ctx *c, int T, cudaStream_t s) {
     a.S = c->S;
     a.gD = c->gD;
     a.ldP = ld;
-    a.ntiles = c->ntiles;
+    a.nunits = c->nunits;
+    a.ru = c->ru;
     a.T = T;
     a.tau_EI = c->tau_EI;
     a.L = c->L;
@@ -857,23 +874,20 @@ gabm_status backward_days_batched(gabm_ctx *c, int T, cudaStream_t s) {
         a.r_next = c->r + (size_t)((t + 1) & 1) * nb;
         a.r_cur = c->r + (size_t)(t & 1) * nb;
 
-        a.P_t = c->P + (size_t)t * c->ntiles * kAges * c->Bp;
+        a.P_t = c->P + (size_t)t * c->nunits * kAges * c->Bp;
         for (int k = 0; k < kMaxL; ++k) a.ring_slot[k] = (k >= 1 && k < c->L) ? (t + k) % Lm1 : 0;
         prof_begin(c, 1);
         for (int ch = 0; ch < nch; ++ch) {   // the row's sets in launches of bwd_chunk sets
             a.s0 = ch * c->bwd_chunk;
-            uint32_t *rb = c->rbits + (size_t)ch * 2 * c->ntiles;
-            a.rbits_next = rb + (size_t)((t + 1) & 1) * c->ntiles;
-            a.rbits_cur = rb + (size_t)(t & 1) * c->ntiles;
             a.tile_ctr = c->tile_ctr + (size_t)(1 + ch) * ld + t;
             LAUNCH(launch_bwd_day_b(a, c->bwd_chunk, c->spl_bwd, c->kahan_b, c->grid_bwd, s));
         }
         prof_end(c, 1);
     }
     if (a.dc_tile)   // the seeds' share through day 0 (r of day 0 is in slot 0)
-        LAUNCH(launch_dc_seeds_b(csr_view(c, true), c->e, c->r, graph_ref(c), c->sig, ld + 1, c->ntiles, c->L, c->B,
-                                 c->Bp, c->dc_tile, s));
-    LAUNCH(launch_bwd_reduce_b(c->P, c->ntiles, c->d_tile0, c->d_ntiles, c->G, c->B, c->Bp, T, c->Pc, c->max_chunks,
+        LAUNCH(launch_dc_seeds_b(csr_view(c, true), c->e, c->r, graph_ref(c), c->sig, ld + 1, c->nunits,
+                                 c->ru, c->L, c->B, c->Bp, c->dc_tile, s));
+    LAUNCH(launch_bwd_reduce_b(c->P, c->nunits, c->d_unit0, c->d_nunits, c->G, c->B, c->Bp, T, c->Pc, c->max_chunks,
                                c->sig, ld + 1, c->Q, s));
     return GABM_OK;
 }
@@ -972,7 +986,7 @@ gabm_status backward_days_sirs(gabm_ctx *c, int T, cudaStream_t s) {
         LAUNCH(launch_bwd_day_sirs(a, c->grid_sirs_b, c->overlap && t < T - 1, s));
         prof_end(c, 1);
     }
-    LAUNCH(launch_bwd_reduce(c->P, c->ntiles, ld, c->d_tile0, c->d_ntiles, T, c->I, c->sig, ld + 1, c->Q, s));
+    LAUNCH(launch_bwd_reduce(c->P, c->ntiles, c->d_tile0, c->d_ntiles, T, c->I, c->sig, ld + 1, c->Qp, c->Q, s));
     return GABM_OK;
 }
 
@@ -1165,7 +1179,7 @@ gabm_status backward_days_plain(gabm_ctx *c, int T, cudaStream_t s) {
         LAUNCH(launch_dc_seeds(sell_view(c, true), c->e, r0, graph_ref(c), c->sig, ld + 1, c->ntiles, c->L,
                                long_gx_buf(c), c->dc_tile, c->grid_bwd, s));
     }
-    LAUNCH(launch_bwd_reduce(c->P, c->ntiles, ld, c->d_tile0, c->d_ntiles, T, c->I, c->sig, ld + 1, c->Q, s));
+    LAUNCH(launch_bwd_reduce(c->P, c->ntiles, c->d_tile0, c->d_ntiles, T, c->I, c->sig, ld + 1, c->Qp, c->Q, s));
     return GABM_OK;
 }
 
@@ -1351,7 +1365,7 @@ void apply_schedule(gabm_ctx *c) {
         const int units = std::max(c->loc_ntiles, c->n_big);   // warp work units of the larger launch
         c->grid_loc = std::min(c->num_sms * occupancy_loc(), std::max(1, (units + kBlock / 32 - 1) / (kBlock / 32)));
     }
-    const int max_grid = (c->ntiles + kBlock / 32 - 1) / (kBlock / 32);
+    const int max_grid = ((c->batched ? c->nunits : c->ntiles) + kBlock / 32 - 1) / (kBlock / 32);
     if (!c->smem_bits && c->grid_fwd > max_grid) c->grid_fwd = max_grid;
     if (c->grid_bwd > max_grid) c->grid_bwd = max_grid;
     if (c->grid_bwd_dc > max_grid) c->grid_bwd_dc = max_grid;
@@ -1445,17 +1459,7 @@ static gabm_status create_on_device(const HostLayout &H, const gabm_model_desc *
     {
         int mx = 1;
         for (int g = 0; g < num_graphs; ++g) mx = std::max(mx, ntl[g]);
-        c->max_chunks = (mx + kReduceChunkTiles - 1) / kReduceChunkTiles;
-        c->max_graph_tiles = mx;
-    }
-    if (batched) {
-        // widest vectors first: eight sets per lane keeps 32 / (Bp / 8) rows in flight per warp
-        c->spl_fwd = c->spl_bwd = std::min(c->Bp, 8);
-        c->bwd_chunk = c->Bp;
-        if (const char *f = getenv("GABM_BATCH_SPL")) {
-            const int v = atoi(f);
-            if (batch_config_ok(c->Bp, v)) c->spl_fwd = c->spl_bwd = v;
-        }
+        c->max_graph_units = mx;
     }
     c->tau_EI = model->tau_EI;
     c->tau_IR = model->tau_IR;
@@ -1514,6 +1518,25 @@ static gabm_status create_on_device(const HostLayout &H, const gabm_model_desc *
 
     CCK(cudaGetDevice(&c->device));
     CCK(cudaDeviceGetAttribute(&c->num_sms, cudaDevAttrMultiProcessorCount, c->device));
+    if (batched) {
+        c->ru = unit_rows(ntiles, c->Bp, c->num_sms);
+        c->nunits = ntiles * (kTile / c->ru);
+        c->max_graph_units *= kTile / c->ru;
+        c->max_chunks = (c->max_graph_units + kReduceChunkTiles - 1) / kReduceChunkTiles;
+        // widest vectors first: eight sets per lane keeps 32 / (Bp / 8) rows in flight per warp,
+        // as far as the unit has that many
+        c->spl_fwd = c->spl_bwd = std::max(2, std::min(std::min(c->Bp, 8), c->Bp * c->ru / 32));
+        // the backward: four, whose kernel fits three blocks an SM instead of two, once there are
+        // two units for each of those warps (200k agents x 64 sets: 238 us a day against 267,
+        // 100k x 32: 79 against 85); with fewer units the longer rows of lanes only lengthen
+        // each warp's chain (20k x 64: 80 against 71)
+        if (c->Bp >= 8 && c->nunits >= 2 * 24 * c->num_sms) c->spl_bwd = std::min(c->spl_bwd, 4);
+        c->bwd_chunk = c->Bp;
+        if (const char *f = getenv("GABM_BATCH_SPL")) {
+            const int v = atoi(f);
+            if (batch_config_ok(c->Bp, v)) c->spl_fwd = c->spl_bwd = v;
+        }
+    }
 
     c->sigma = sigma;
     auto upload_sell = [&](const HostSell &hs, uint32_t *&sp, uint32_t *&rl, uint4 *&cw) -> gabm_status {
@@ -1588,6 +1611,15 @@ static gabm_status create_on_device(const HostLayout &H, const gabm_model_desc *
     CTRY(dalloc(c, &c->d_inv_Dbar, (size_t)num_graphs));
     CTRY(dalloc(c, &c->d_tile_graph, (size_t)ntiles));
     CTRY(dalloc(c, &c->d_goff, (size_t)num_graphs));
+    std::vector<int32_t> unit0(tile0), nun(ntl);
+    if (batched) {
+        for (auto &u : unit0) u *= kTile / c->ru;
+        for (auto &u : nun) u *= kTile / c->ru;
+        CTRY(dalloc(c, &c->d_unit0, (size_t)num_graphs));
+        CTRY(dalloc(c, &c->d_nunits, (size_t)num_graphs));
+        CCK(cudaMemcpyAsync(c->d_unit0, unit0.data(), sizeof(int32_t) * num_graphs, cudaMemcpyHostToDevice, c->stream));
+        CCK(cudaMemcpyAsync(c->d_nunits, nun.data(), sizeof(int32_t) * num_graphs, cudaMemcpyHostToDevice, c->stream));
+    }
     CCK(cudaMemcpyAsync(c->d_goff, goff.data(), sizeof(int64_t) * num_graphs, cudaMemcpyHostToDevice, c->stream));
     if (reorder) {
         CTRY(dalloc(c, &c->d_orig_id, (size_t)n_rows));
@@ -1609,7 +1641,6 @@ static gabm_status create_on_device(const HostLayout &H, const gabm_model_desc *
     CTRY(dalloc(c, &c->rows_e, nb));
     CTRY(dalloc(c, &c->stage_f, nb));
     if (batched) {
-        CTRY(dalloc(c, &c->rbits, (size_t)2 * ntiles * std::max(1, c->Bp / 2)));
         CTRY(dalloc(c, &c->hist0, (size_t)c->I * (c->L + 2)));
     } else if (!c->soft) {
         CTRY(dalloc(c, &c->flags, (size_t)3 * n_rows));
@@ -2134,8 +2165,8 @@ static gabm_status backward_impl(gabm_ctx *c, const double *gD, double *dR, doub
     cudaStream_t s = c->stream;
     CK(cudaMemcpy2DAsync(c->gD, ld * sizeof(double), gD, T * sizeof(double), T * sizeof(double), c->I, h2d_kind(mem_space), s));
     c->gD_staged = true;
-    // table-adjoint accumulators: [ntiles][kMaxL] (one set per graph) or [ntiles][L][Bp]
-    const size_t dc_len = c->batched ? (size_t)c->ntiles * c->L * c->Bp : (size_t)c->ntiles * kMaxL;
+    // table-adjoint accumulators: [ntiles][kMaxL] (one set per graph) or [nunits][L][Bp]
+    const size_t dc_len = c->batched ? (size_t)c->nunits * c->L * c->Bp : (size_t)c->ntiles * kMaxL;
     if (dc) {
         if (!c->dc_tile) TRY(dalloc(c, &c->dc_tile, dc_len));
         if (!c->dc_s) TRY(dalloc(c, &c->dc_s, (size_t)c->I * c->L));
@@ -2148,7 +2179,7 @@ static gabm_status backward_impl(gabm_ctx *c, const double *gD, double *dR, doub
     const bool dev = mem_space == GABM_DEVICE;
     if (dc) {
         double *out = dev ? dc : c->dc_s;
-        if (c->batched) LAUNCH(launch_dc_reduce_b(c->dc_tile, c->d_tile0, c->d_ntiles, c->G, c->B, c->Bp, c->L, out, s));
+        if (c->batched) LAUNCH(launch_dc_reduce_b(c->dc_tile, c->d_unit0, c->d_nunits, c->G, c->B, c->Bp, c->L, out, s));
         else LAUNCH(launch_dc_reduce(c->dc_tile, c->d_tile0, c->d_ntiles, c->G, c->L, out, s));
     }
     LAUNCH(launch_bwd_finalize(c->Q, c->R, c->S, c->gD,

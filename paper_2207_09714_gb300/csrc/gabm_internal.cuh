@@ -13,7 +13,7 @@
 //   lam     f32 [Tcap][n_rows]    normalised neighbour sums (store policy)
 //   ring    f32 [ntiles][L-1][32] adjoint of infectiousness, last L-1 days
 //   r       f32 [2][n_rows]       per-day transpose-gather coefficients
-//   P       f64 [Tcap][ntiles][9] per-tile, per-age partial gradient sums
+//   P       f32 [Tcap][ntiles][9] per-tile, per-age partial gradient sums (fp32 sums, FP64 from there on)
 #pragma once
 
 #include <cuda_runtime.h>
@@ -257,7 +257,7 @@ struct BwdDayArgs {
     const float *R, *m_t, *S;  // R and mortality [I][ldP], susceptibility [I][9]
     const double *gD;          // [I][ldP]
     int ldP;
-    double *P_t;               // [ntiles][9] partial sums of gl * Lam for day t
+    float *P_t;                // [ntiles][9] partial sums of gl * Lam for day t
     int32_t *newRM;            // [I][ldP]
     int ntiles, t, T, tau_EI, L;
     int mode;                  // kBwdStore, kBwdFused or kBwdSplit
@@ -325,11 +325,11 @@ struct FwdBatchArgs {
     float *lam_out;              // day-t slice [n_rows][Bp] of the lambda store, or nullptr
     const float *R, *S;          // [I][ldP], [I][9]
     int ldP;
-    uint8_t *tile_new;           // [ntiles][Bp] agents exposed on day t, by tile and set
+    uint8_t *unit_new;           // [nunits][Bp] agents exposed on day t, by unit and set
     int *tile_ctr;
     const uint32_t *bits_cur;    // [ntiles] rows infectious on day t in any set
     uint32_t *bits_next;         // the same for day t + 1
-    int ntiles, t, tau_EI, L, B;
+    int nunits, ru, t, tau_EI, L, B;   // units of ru rows (see unit_rows)
     uint64_t seed;
     float c[kMaxL];
 };
@@ -340,19 +340,17 @@ struct BwdBatchArgs {
     GraphRef gr;
     const int16_t *E;            // [n_rows][Bp] final exposure days
     const float *lam_t;          // [n_rows][Bp] stored normalised sums of day t
-    const float *r_next;         // [n_rows][Bp] coefficients of day t+1
+    const float *r_next;         // [n_rows][Bp] coefficients of day t+1 (0 for rows not susceptible then)
     float *r_cur;                // [n_rows][Bp] coefficients of day t
-    const uint32_t *rbits_next;  // [ntiles] rows susceptible on day t+1 in some set
-    uint32_t *rbits_cur;         // the same for day t
     float *ring;                 // [L-1][n_rows][Bp]
     size_t ring_stride;
     float *A;                    // [n_rows][Bp]
     const float *R, *m_t, *S;
     const double *gD;
     int ldP;
-    double *P_t;                 // [ntiles][9][Bp] per-tile partial sums of gl * Lam
+    float *P_t;                  // [nunits][9][Bp] per-unit partial sums of gl * Lam
     int *tile_ctr;
-    int ntiles, t, T, tau_EI, L, B;
+    int nunits, ru, t, T, tau_EI, L, B;
     uint64_t seed;
     float c[kMaxL];
     int ring_slot[kMaxL];
@@ -360,7 +358,7 @@ struct BwdBatchArgs {
     int32_t *rnz;                // [G][ld_sig] 1: some r of that day is not 0 in some set
     int ld_sig;
     int Bw, s0;                  // row width of the per-agent arrays; first set of this launch
-    double *dc_tile;             // [ntiles][L][Bw] per-tile sums of the table adjoint over days, or nullptr
+    double *dc_tile;             // [nunits][L][Bw] per-unit sums of the table adjoint over days, or nullptr
     const uint32_t *bits_t;      // recompute policy (lam_t == nullptr): [ntiles] rows infectious on day t in any set
 };
 
@@ -378,14 +376,14 @@ cudaError_t launch_infectious_bits_b(const int16_t *e, int Bp, int t0, int L, in
 cudaError_t launch_exposure_hist_b(const int16_t *e, GraphRef gr, int64_t n_rows, int B, int Bp, int t0, int L,
                                    int32_t *H, cudaStream_t s);
 // counts [I][ldP][4] and newRM [I][ldP] of days t0..T-1 from H and the per-tile exposures
-// tile_new [T][ntiles][Bp]; newinf [I][ldP] is scratch, zeroed by the caller.
-cudaError_t launch_counts_b(const uint8_t *tile_new, int ntiles, const int32_t *d_tile0, const int32_t *d_ntiles,
-                            const int32_t *d_rows, int G, int B, int Bp, int max_tiles, int t0, int T, int ldP,
+// unit_new [T][nunits][Bp]; newinf [I][ldP] is scratch, zeroed by the caller.
+cudaError_t launch_counts_b(const uint8_t *unit_new, int nunits, const int32_t *d_unit0, const int32_t *d_nunits,
+                            const int32_t *d_rows, int G, int B, int Bp, int max_units, int t0, int T, int ldP,
                             int tau_EI, int L, const int32_t *H, int32_t *newinf, int32_t *counts, int32_t *newRM,
                             cudaStream_t s);
 // Q[g*B+s][t][a] = sum over graph g's tiles of P[t][tile][a][s], in a fixed order (two levels of
 // kReduceChunkTiles tiles); scratch holds T * G * max_chunks * 9 * Bp doubles.
-cudaError_t launch_bwd_reduce_b(const double *P, int ntiles, const int32_t *d_tile0, const int32_t *d_ntiles, int G,
+cudaError_t launch_bwd_reduce_b(const float *P, int nunits, const int32_t *d_tile0, const int32_t *d_ntiles, int G,
                                 int B, int Bp, int T, double *scratch, int max_chunks, const int32_t *sig,
                                 int ld_sig, double *Q, cudaStream_t s);
 constexpr int kReduceChunkTiles = 64;
@@ -515,7 +513,7 @@ cudaError_t launch_dc_seeds(Sell m_out, const int16_t *E, const float *r0, Graph
 cudaError_t launch_dc_reduce(const double *dc_tile, const int32_t *graph_tile0, const int32_t *graph_ntiles, int G,
                              int L, double *dc, cudaStream_t s);
 cudaError_t launch_dc_seeds_b(Csr m_out, const int16_t *E, const float *r0, GraphRef gr, const int32_t *sig,
-                              int ld_sig, int ntiles, int L, int B, int Bp, double *dc_tile, cudaStream_t s);
+                              int ld_sig, int nunits, int ru, int L, int B, int Bp, double *dc_tile, cudaStream_t s);
 cudaError_t launch_dc_reduce_b(const double *dc_tile, const int32_t *graph_tile0, const int32_t *graph_ntiles, int G,
                                int B, int Bp, int L, double *dc, cudaStream_t s);
 // Location hop of agent-location graphs (twohop.cu): pressures of day t and adjoints.  Small
@@ -535,9 +533,10 @@ int occupancy_loc();
 cudaError_t launch_lam_day(Sell m, const int16_t *E, const uint32_t *bits, GraphRef gr, int t, int L, int ntiles,
                            const float *c, const float *long_lam, float *lam_out, int grid, cudaStream_t s);
 // Q[g][t][a] = 2^sigma_g(t) x (sum over graph g's tiles of P[t][tile][a]), FP64.
-cudaError_t launch_bwd_reduce(const double *P, int ntiles, int ldP, const int32_t *graph_tile0,
-                              const int32_t *graph_ntiles, int T, int I, const int32_t *sig, int ld_sig,
-                              double *Q, cudaStream_t s);
+// parts: [T][I][kReduceParts][9] scratch.
+constexpr int kReduceParts = 8;
+cudaError_t launch_bwd_reduce(const float *P, int ntiles, const int32_t *graph_tile0, const int32_t *graph_ntiles,
+                              int T, int I, const int32_t *sig, int ld_sig, double *parts, double *Q, cudaStream_t s);
 // newRM_real (soft mode, [I][ldP]) replaces the integer newRM when non-null.
 cudaError_t launch_bwd_finalize(const double *Q, const float *R, const float *S, const double *gD,
                                 const int32_t *newRM, const double *newRM_real, int ldP, int T, int I, double *dR,

@@ -283,7 +283,7 @@ __global__ void __launch_bounds__(kBlock, 3) k_bwd_day_sirs(SirsBwdArgs a) {
 
         float mine = 0.f;   // lanes 2b, 2b + 1: bin b (the base kernel's tree)
         if (__any_sync(0xffffffffu, !(v == 0.f))) mine = warp_bin_sums(v, ai, lane, bin_s[wib]);
-        if (!(lane & 1) && (lane >> 1) < kAges) a.P_t[(size_t)tile * kAges + (lane >> 1)] = (double)mine;
+        if (!(lane & 1) && (lane >> 1) < kAges) a.P_t[(size_t)tile * kAges + (lane >> 1)] = mine;
     }
     if (cur_g >= 0) {
         const int sN = __reduce_add_sync(0xffffffffu, cN);

@@ -61,7 +61,7 @@ struct SirsBwdArgs {
     const float *R, *m_t, *S;
     const double *gD;
     int ldP;
-    double *P_t;                // [ntiles][9] per-tile sums of gl * Lam by age
+    float *P_t;                 // [ntiles][9] per-tile sums of gl * Lam by age
     int32_t *newRM;             // [I][ldP] recounted
     int32_t *sig, *emax;        // [G][ld_sig] per-day scale exponents
     int32_t *rnz;               // [G][ld_sig] 1: some r of that day is not 0
