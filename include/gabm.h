@@ -219,8 +219,8 @@ gabm_status gabm_mse_loss(gabm_ctx *ctx, const double *y, double *loss, double *
 
 /* Replace the infectiousness table c [L] (host floats; c[0] = 0, every entry finite
  * and >= 0, as at creation) for the forwards that follow, e.g. between the steps of a
- * calibration that learns the stage factors or the profile behind c.  Waits for the
- * ctx stream.  The last trajectory used the old table, so gabm_backward returns
+ * calibration that learns the stage factors or the profile behind c.  Takes effect on the
+ * ctx stream, behind the work already there.  The last trajectory used the old table, so gabm_backward returns
  * GABM_ESTATE until the next gabm_forward.  GABM_EINVAL for a NULL or invalid table. */
 gabm_status gabm_set_infectiousness(gabm_ctx *ctx, const float *c);
 
@@ -327,6 +327,13 @@ gabm_status gabm_get_profile(gabm_ctx *ctx, int kind, double *total_ms, int64_t 
  * ctr [count][4] uint32 and out [count][4] uint32, both device memory. */
 gabm_status gabm_philox(uint64_t seed, const uint32_t *ctr, uint32_t *out, int64_t count,
                         void *cuda_stream);
+
+/* MSE on cumulative deaths (Sec. 3.2, Stage 3) and its gradient, in FP64: with C = the running
+ * sums of D over the days, loss[0] = (1 / (instances T)) sum (C - y)^2 and gD = its gradient
+ * with respect to D.  D, y, gD [instances][T]; loss [1 + instances] (each instance's sum of
+ * squares follows the mean).  All device memory; enqueued on cuda_stream. */
+gabm_status gabm_cumulative_mse(const double *D, const double *y, int instances, int T, double *loss, double *gD,
+                                void *cuda_stream);
 
 /* Message for the last failing call on ctx (or for the last failing
  * gabm_create when ctx is NULL).  Valid until the next call on that ctx. */

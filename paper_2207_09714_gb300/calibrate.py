@@ -184,8 +184,43 @@ def synthetic_features(R_t: np.ndarray, t_N: int, F: int = 5, seed: int = 0) -> 
     return out
 
 
+class _CumulativeMse(torch.autograd.Function):
+    """The fused loss and its gradient (two launches for the five and their backward's nine of
+    the torch expression, 300 us of host time a step)."""
+
+    @staticmethod
+    def forward(fctx, D, y):
+        loss, gD = capi.gabm_cumulative_mse(D, y)
+        fctx.save_for_backward(D, y, gD)
+        return loss
+
+    @staticmethod
+    def backward(fctx, g):
+        D, y, gD = fctx.saved_tensors
+        if torch.is_grad_enabled():   # a graph of the gradient is wanted: keep it differentiable
+            r = torch.cumsum(D, dim=-1) - y
+            gD = torch.flip(torch.cumsum(torch.flip(r, (-1,)), dim=-1), (-1,)) * (2.0 / r.numel())
+        return g * gD, None
+
+
+def _plain_cuda(t: torch.Tensor) -> bool:
+    """An ordinary float64 matrix on the current device, outside any transform of torch."""
+    return (type(t) is torch.Tensor and t.is_cuda and t.dtype == torch.float64 and t.dim() == 2 and t.numel() > 0 and
+            t.is_contiguous() and t.device.index == torch.cuda.current_device() and
+            not torch._C._functorch.is_functorch_wrapped_tensor(t) and
+            torch.autograd.forward_ad.unpack_dual(t).tangent is None)
+
+
 def cumulative_mse(D: torch.Tensor, y_cum: torch.Tensor) -> torch.Tensor:
-    """Mean over instances and days of (sum_{s<=t} D_s - y_cum_t)^2 (Sec. 3.2, Stage 3)."""
+    """Mean over instances and days of (sum_{s<=t} D_s - y_cum_t)^2 (Sec. 3.2, Stage 3).
+
+    Float64 matrices on the GPU go through the library's fused kernel; everything else (other
+    types, the CPU, a target that broadcasts or wants a gradient, vmap, forward-mode
+    differentiation, tracing) through the torch expression."""
+    if (isinstance(y_cum, torch.Tensor) and not y_cum.requires_grad and D.shape == y_cum.shape and
+            D.device == y_cum.device and not torch.jit.is_tracing() and not torch.compiler.is_compiling() and
+            torch._C._len_torch_dispatch_stack() == 0 and _plain_cuda(D) and _plain_cuda(y_cum)):
+        return _CumulativeMse.apply(D, y_cum)
     return ((torch.cumsum(D, dim=-1) - y_cum) ** 2).mean()
 
 

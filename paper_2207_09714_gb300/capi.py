@@ -96,6 +96,8 @@ def load_library(path: str = LIB_PATH) -> ctypes.CDLL:
         L.gabm_set_profiling.argtypes = [P, i32]
         L.gabm_get_profile.argtypes = [P, i32, ctypes.POINTER(ctypes.c_double), ctypes.POINTER(i64)]
         L.gabm_philox.argtypes = [u64, P, P, i64, P]
+        L.gabm_cumulative_mse.argtypes = [P, P, i32, i32, P, P, P]
+        L.gabm_cumulative_mse.restype = ctypes.c_int
         L.gabm_last_error.argtypes = [P]
         L.gabm_last_error.restype = ctypes.c_char_p
         L.gabm_destroy.argtypes = [P]
@@ -543,6 +545,20 @@ def gabm_philox(seed: int, ctr, out=None, stream=None):
     st = load_library().gabm_philox(int(seed), _ptr(ctr, np.uint32), _ptr(out, np.uint32), int(ctr.shape[0]), s)
     _check(st, None)
     return out
+
+
+def gabm_cumulative_mse(D, y):
+    """MSE of the running sums of D [I, T] against y [I, T] (float64 CUDA tensors) and its
+    gradient with respect to D; returns (loss, a 0-d tensor, and gD [I, T])."""
+    import torch
+    I, T = D.shape
+    _shape(y, (I, T), "y")
+    loss = torch.empty(1 + I, dtype=torch.float64, device=D.device)
+    gD = torch.empty((I, T), dtype=torch.float64, device=D.device)
+    st = load_library().gabm_cumulative_mse(_ptr(D, np.float64), _ptr(y, np.float64), I, T, _ptr(loss), _ptr(gD),
+                                            ctypes.c_void_p(torch.cuda.current_stream(D.device).cuda_stream))
+    _check(st, None)
+    return loss[0], gD
 
 
 def gabm_destroy(ctx: GabmCtx):

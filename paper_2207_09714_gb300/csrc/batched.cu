@@ -278,18 +278,19 @@ __global__ void k_counts_b(const int32_t *H, const int32_t *newinf, const int32_
     auto cnt = [&](int d) -> int32_t { return d >= t0 ? ni[d] : h[2 + d - (t0 - L)]; };
     int32_t S = rows[inst / B];
     for (int b = 1; b < nb; ++b) S -= h[b];
+    // the stages on day t0, then each day's changes: who left E for I, I for RM, and S for E
+    int32_t E = 0, In = 0, RM = h[1];
+    for (int d = t0 - tau_EI + 1; d <= t0 - 1; ++d) E += cnt(d);
+    for (int d = t0 - L + 1; d <= t0 - tau_EI; ++d) In += cnt(d);
+    RM += cnt(t0 - L);
     for (int t = t0; t < T; ++t) {
-        int32_t E = 0, In = 0, RM = h[1];
-        for (int d = t - tau_EI + 1; d <= t - 1; ++d) E += cnt(d);
-        for (int d = t - L + 1; d <= t - tau_EI; ++d) In += cnt(d);
-        for (int d = t0 - L; d <= t - L; ++d) RM += cnt(d);
-        int32_t *cp = counts + ((size_t)inst * ldP + t) * 4;
-        cp[0] = S;
-        cp[1] = E;
-        cp[2] = In;
-        cp[3] = RM;
+        *reinterpret_cast<int4 *>(counts + ((size_t)inst * ldP + t) * 4) = make_int4(S, E, In, RM);
         newRM[(size_t)inst * ldP + t] = cnt(t - L);
-        S -= ni[t];
+        const int32_t born = ni[t], ripe = cnt(t + 1 - tau_EI), gone = cnt(t + 1 - L);
+        S -= born;
+        E += born - ripe;
+        In += ripe - gone;
+        RM += gone;
     }
 }
 

@@ -18,6 +18,8 @@
 #include "gabm_internal.cuh"
 #include "rowsum.cuh"
 
+#include <algorithm>
+
 // The share (percent) of a graph's agents in E or I on the previous day from which the
 // one-set forward gathers every entry's exposure day instead of testing the day's bitmap.
 #ifndef GABM_DENSE_MARKS_PCT
@@ -387,33 +389,52 @@ __global__ void k_infectious_bits(const int16_t *e, int t0, int ndays, int L, in
 // 32-bit word in three digits (11, 11, 10 bits), then ties on the final word
 // are broken by id.
 // ---------------------------------------------------------------------------
+template <int W>   // slots a thread writes together: 2 (as one word), or 1 for odd or unaligned arrays
 __global__ void k_init_state(int16_t *e, const int32_t *row0, const int32_t *rows, int G, int64_t n_rows,
-                             int B, int Bp) {
-    for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < n_rows;
-         r += (int64_t)gridDim.x * blockDim.x) {
-        // binary search the graph of row r
-        int lo = 0, hi = G - 1;
-        while (lo < hi) {
-            int mid = (lo + hi + 1) >> 1;
-            if (row0[mid] <= r) lo = mid; else hi = mid - 1;
+                             int B, int Bp, SeedState *st, const int32_t *n_seed, int I) {
+    const int64_t first = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (st)
+        for (int64_t i = first; i < I; i += (int64_t)gridDim.x * blockDim.x) {
+            SeedState v;
+            v.prefix = 0u;
+            v.k_rem = (uint32_t)n_seed[i];
+            v.eq_count = v.tie_n = v.done = 0u;
+            v.none = (n_seed[i] == 0);
+            v.overflow = 0;
+            st[i] = v;
         }
-        const bool agent = r - row0[lo] < rows[lo];
-        for (int b = 0; b < Bp; ++b)
-            e[(size_t)r * Bp + b] = (agent && b < B) ? (int16_t)kNever : (int16_t)kPad;
+    // slot by slot within a row, 64 sets of 200k agents took 120 us
+    const int shift = 31 - __clz(Bp);   // Bp is a power of two
+    for (int64_t w = first; w < n_rows * Bp / W; w += (int64_t)gridDim.x * blockDim.x) {
+        uint32_t out = 0u;
+#pragma unroll
+        for (int h = 0; h < W; ++h) {
+            const int64_t r = (W * w + h) >> shift;
+            const int b = (int)((W * w + h) & (Bp - 1));
+            int lo = 0, hi = G - 1;   // binary search the graph of row r
+            while (lo < hi) {
+                int mid = (lo + hi + 1) >> 1;
+                if (row0[mid] <= r) lo = mid; else hi = mid - 1;
+            }
+            const bool agent = b < B && r - row0[lo] < rows[lo];
+            out |= (uint32_t)(uint16_t)(int16_t)(agent ? kNever : kPad) << (16 * h);
+        }
+        if (W == 2) reinterpret_cast<uint32_t *>(e)[w] = out;
+        else e[w] = (int16_t)out;
     }
 }
 
-__global__ void k_seed_reset(SeedState *st, const int32_t *n_seed, int I) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= I) return;
-    SeedState s;
-    s.prefix = 0u;
-    s.k_rem = (uint32_t)n_seed[i];
-    s.eq_count = 0u;
-    s.tie_n = 0u;
-    s.none = (n_seed[i] == 0);
-    s.overflow = 0;
-    st[i] = s;
+// Whether this block is the last of its instance's to come here: what the others wrote
+// before is then visible to it.  Called by every thread of the block.
+__device__ __forceinline__ bool last_of_instance(SeedState *st) {
+    __shared__ uint32_t s_last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(&st->done, 1u) == gridDim.x - 1u;
+    __syncthreads();
+    const bool last = s_last != 0u;
+    if (last) __threadfence();
+    return last;
 }
 
 __device__ __forceinline__ void digit_of_pass(int pass, int &shift, int &nbins, uint32_t &himask) {
@@ -422,8 +443,12 @@ __device__ __forceinline__ void digit_of_pass(int pass, int &shift, int &nbins, 
     else { shift = 0; nbins = 1024; himask = 0xFFFFFC00u; }
 }
 
-__global__ void __launch_bounds__(256) k_seed_hist(const SeedArgs a) {
+// One digit of the selection: the histogram of the keys that match the prefix so far; the
+// instance's last block finds the bin holding the k_rem-th smallest key, and clears the
+// histogram for the next pass.
+__global__ void __launch_bounds__(256) k_seed_pass(const SeedArgs a) {
     __shared__ uint32_t h_s[kHistBins];
+    __shared__ uint32_t warp_s[8];
     const int inst = blockIdx.y;
     const SeedState st = a.st[inst];
     if (st.none) return;
@@ -442,53 +467,47 @@ __global__ void __launch_bounds__(256) k_seed_hist(const SeedArgs a) {
     uint32_t *gh = a.hist + (size_t)inst * kHistBins;
     for (int b = threadIdx.x; b < nbins; b += blockDim.x)
         if (h_s[b]) atomicAdd(gh + b, h_s[b]);
-}
+    if (!last_of_instance(a.st + inst)) return;
 
-// One warp per instance: find the digit bin holding the k_rem-th smallest key.
-__global__ void k_seed_scan(const SeedArgs a) {
-    const int inst = blockIdx.x;
-    const int lane = threadIdx.x;
-    SeedState st = a.st[inst];
-    int shift, nbins; uint32_t himask;
-    digit_of_pass(a.pass, shift, nbins, himask);
-    uint32_t *gh = a.hist + (size_t)inst * kHistBins;
-    if (!st.none) {
-        const int per = nbins / 32;
-        uint32_t mine = 0;
-        for (int b = 0; b < per; ++b) mine += gh[lane * per + b];
-        uint32_t incl = mine;
-        for (int o = 1; o < 32; o <<= 1) {
-            uint32_t v = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += v;
-        }
-        const uint32_t excl = incl - mine;
-        const bool here = (excl < st.k_rem) && (st.k_rem <= incl);
-        const unsigned who = __ballot_sync(0xffffffffu, here);
-        const int src = __ffs(who) - 1;
-        uint32_t digit = 0, below = 0, eq = 0;
-        if (lane == src) {
-            uint32_t cum = excl;
-            for (int b = 0; b < per; ++b) {
-                const uint32_t hb = gh[lane * per + b];
-                if (st.k_rem <= cum + hb) { digit = (uint32_t)(lane * per + b); below = cum; eq = hb; break; }
-                cum += hb;
+    constexpr int kMaxPer = kHistBins / 256;
+    const int per = nbins / 256, lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    uint32_t bin[kMaxPer], mine = 0u;
+#pragma unroll
+    for (int b = 0; b < kMaxPer; ++b) {
+        bin[b] = b < per ? __ldcg(gh + threadIdx.x * per + b) : 0u;
+        mine += bin[b];
+    }
+    uint32_t incl = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t v = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += v;
+    }
+    if (lane == 31) warp_s[wib] = incl;
+    __syncthreads();
+    for (int w = 0; w < wib; ++w) incl += warp_s[w];
+    uint32_t cum = incl - mine;
+    if (cum < st.k_rem && st.k_rem <= incl) {   // one thread
+#pragma unroll
+        for (int b = 0; b < kMaxPer; ++b) {
+            if (b < per && cum < st.k_rem && st.k_rem <= cum + bin[b]) {
+                SeedState out = st;
+                out.prefix |= (uint32_t)(threadIdx.x * per + b) << shift;
+                out.k_rem -= cum;
+                if (a.pass == 2) out.eq_count = bin[b];
+                out.done = 0u;
+                a.st[inst] = out;
+                break;
             }
-        }
-        digit = __shfl_sync(0xffffffffu, digit, src);
-        below = __shfl_sync(0xffffffffu, below, src);
-        eq = __shfl_sync(0xffffffffu, eq, src);
-        __syncwarp();
-        if (lane == 0) {
-            st.prefix |= digit << shift;
-            st.k_rem -= below;
-            if (a.pass == 2) st.eq_count = eq;
-            a.st[inst] = st;
+            cum += bin[b];
         }
     }
-    for (int b = lane; b < nbins; b += 32) gh[b] = 0u;
+    for (int b = threadIdx.x; b < nbins; b += blockDim.x) gh[b] = 0u;
 }
 
-__global__ void k_seed_mark(const SeedArgs a) {
+// Marks the chosen agents.  Ties on the threshold word: the instance's last block gives them
+// to the k_rem candidates with the smallest caller ids (the tie list holds local rows).
+__global__ void __launch_bounds__(256) k_seed_mark(const SeedArgs a) {
     const int inst = blockIdx.y;
     const SeedState st = a.st[inst];
     if (st.none) return;
@@ -510,29 +529,93 @@ __global__ void k_seed_mark(const SeedArgs a) {
         }
         if (mark) a.e[(size_t)(r0 + i) * a.Bp + set] = (int16_t)(-a.tau_EI);
     }
-}
-
-// Ties on the threshold word: the k_rem candidates with the smallest caller ids win.
-// The tie list holds local row indices.
-__global__ void k_seed_ties(const SeedArgs a) {
-    const int inst = blockIdx.x;
-    const SeedState st = a.st[inst];
-    if (st.none || st.eq_count == st.k_rem) return;
-    const uint32_t n = min(st.tie_n, (uint32_t)kTieCap);
+    if (st.eq_count == st.k_rem) return;
+    if (!last_of_instance(a.st + inst)) return;
+    const uint32_t n = min(*(volatile uint32_t *)&a.st[inst].tie_n, (uint32_t)kTieCap);
     const uint32_t *tl = a.ties + (size_t)inst * kTieCap;
-    const int g = inst / a.B;
-    const size_t set = (size_t)(inst - g * a.B);
-    const int32_t r0 = a.row0[g];
     for (uint32_t c = threadIdx.x; c < n; c += blockDim.x) {
-        const uint32_t i = tl[c];
+        const uint32_t i = __ldcg(tl + c);
         const uint32_t id = a.orig_id ? a.orig_id[r0 + i] : i;
         uint32_t rank = 0;
         for (uint32_t d = 0; d < n; ++d) {
-            const uint32_t idd = a.orig_id ? a.orig_id[r0 + tl[d]] : tl[d];
+            const uint32_t rd = __ldcg(tl + d);
+            const uint32_t idd = a.orig_id ? a.orig_id[r0 + rd] : rd;
             rank += (idd < id);
         }
         if (rank < st.k_rem) a.e[(size_t)(r0 + i) * a.Bp + set] = (int16_t)(-a.tau_EI);
     }
+}
+
+__global__ void k_stage(const float *R, const float *m, const float *S, float *R_ctx, float *m_ctx, float *S_ctx,
+                        int I, int T, int ldP) {
+    const int total = I * T;
+    for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < total; idx += gridDim.x * blockDim.x) {
+        const int inst = idx / T;
+        const size_t to = (size_t)inst * ldP + (idx - inst * T);
+        R_ctx[to] = R[idx];
+        m_ctx[to] = m[idx];
+    }
+    for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < I * kAges; idx += gridDim.x * blockDim.x)
+        S_ctx[idx] = S[idx];
+}
+
+// MSE on cumulative deaths (Sec. 3.2, Stage 3) over I instances and T days in FP64, one block
+// per instance: with C_t = sum of D up to t, out[1 + i] = sum_t (C_t - y_t)^2 and
+// gD_t = 2 / (I T) sum_{s >= t} (C_s - y_s).  The days go in pieces of one a thread, a scan
+// each way.  k_cumulative_mse_mean then writes out[0], the mean.
+constexpr int kCumBlock = 256;
+__device__ __forceinline__ double block_scan(double v, double *warp_s, double &total) {   // inclusive
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const double u = __shfl_up_sync(0xffffffffu, v, o);
+        if (lane >= o) v += u;
+    }
+    __syncthreads();   // warp_s free
+    if (lane == 31) warp_s[wib] = v;
+    __syncthreads();
+    double before = 0.0;
+    total = 0.0;
+    for (int w = 0; w < kCumBlock / 32; ++w) {
+        if (w < wib) before += warp_s[w];
+        total += warp_s[w];
+    }
+    return v + before;
+}
+
+__global__ void __launch_bounds__(kCumBlock) k_cumulative_mse(const double *D, const double *y, int I, int T,
+                                                              double *out, double *gD) {
+    __shared__ double warp_s[kCumBlock / 32];
+    const size_t base = (size_t)blockIdx.x * T;
+    const double scale = 2.0 / ((double)I * (double)T);
+    double run = 0.0, sq = 0.0, total;
+    for (int t0 = 0; t0 < T; t0 += kCumBlock) {   // C_t - y_t into gD
+        const int t = t0 + threadIdx.x;
+        const double C = run + block_scan(t < T ? D[base + t] : 0.0, warp_s, total);
+        run += total;
+        if (t < T) {
+            const double d = C - y[base + t];
+            gD[base + t] = d;
+            sq += d * d;
+        }
+    }
+    block_scan(sq, warp_s, total);
+    if (threadIdx.x == 0) out[1 + blockIdx.x] = total;
+    run = 0.0;
+    for (int t1 = T; t1 > 0; t1 -= kCumBlock) {   // suffix sums, from the end
+        const int t = t1 - 1 - (int)threadIdx.x;
+        const double v = run + block_scan(t >= 0 ? gD[base + t] : 0.0, warp_s, total);
+        run += total;
+        if (t >= 0) gD[base + t] = scale * v;
+    }
+}
+
+__global__ void k_cumulative_mse_mean(int I, int T, double *out) {
+    double v = 0.0;
+    for (int i = threadIdx.x; i < I; i += 32) v += out[1 + i];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (threadIdx.x == 0) out[0] = v / ((double)I * (double)T);
 }
 
 // Row order <-> caller order.
@@ -663,23 +746,17 @@ cudaError_t launch_infectious_bits_fate(const int16_t *e, GraphRef gr, FateRef f
 }
 
 cudaError_t launch_init_state(int16_t *e, const int32_t *row0, const int32_t *rows, int G,
-                              int64_t n_rows, int B, int Bp, int grid, cudaStream_t s) {
-    k_init_state<<<grid, 256, 0, s>>>(e, row0, rows, G, n_rows, B, Bp);
+                              int64_t n_rows, int B, int Bp, SeedState *st, const int32_t *n_seed, int I,
+                              cudaStream_t s) {
+    const bool pairs = (n_rows * Bp) % 2 == 0 && (uintptr_t)e % sizeof(uint32_t) == 0;
+    const int64_t grid = std::min<int64_t>((n_rows * Bp / (pairs ? 2 : 1) + 255) / 256, 65535);
+    (pairs ? k_init_state<2> : k_init_state<1>)<<<(int)std::max<int64_t>(grid, 1), 256, 0, s>>>(e, row0, rows, G, n_rows, B, Bp,
+                                                                                         st, n_seed, I);
     return cudaGetLastError();
 }
 
-cudaError_t launch_seed_reset(SeedState *st, const int32_t *n_seed, int I, cudaStream_t s) {
-    k_seed_reset<<<(I + 127) / 128, 128, 0, s>>>(st, n_seed, I);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_seed_hist(const SeedArgs &a, int I, int grid_x, cudaStream_t s) {
-    k_seed_hist<<<dim3(grid_x, I), 256, 0, s>>>(a);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_seed_scan(const SeedArgs &a, int I, cudaStream_t s) {
-    k_seed_scan<<<I, 32, 0, s>>>(a);
+cudaError_t launch_seed_pass(const SeedArgs &a, int I, int grid_x, cudaStream_t s) {
+    k_seed_pass<<<dim3(grid_x, I), 256, 0, s>>>(a);
     return cudaGetLastError();
 }
 
@@ -688,8 +765,17 @@ cudaError_t launch_seed_mark(const SeedArgs &a, int I, int grid_x, cudaStream_t 
     return cudaGetLastError();
 }
 
-cudaError_t launch_seed_ties(const SeedArgs &a, int I, cudaStream_t s) {
-    k_seed_ties<<<I, 256, 0, s>>>(a);
+cudaError_t launch_stage(const float *R, const float *m, const float *S, float *R_ctx, float *m_ctx, float *S_ctx,
+                         int I, int T, int ldP, cudaStream_t s) {
+    const int64_t n = std::max<int64_t>((int64_t)I * T, (int64_t)I * kAges);
+    k_stage<<<(int)std::min<int64_t>((n + 255) / 256, 1024), 256, 0, s>>>(R, m, S, R_ctx, m_ctx, S_ctx, I, T, ldP);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_cumulative_mse(const double *D, const double *y, int I, int T, double *out, double *gD,
+                                  cudaStream_t s) {
+    k_cumulative_mse<<<I, kCumBlock, 0, s>>>(D, y, I, T, out, gD);
+    k_cumulative_mse_mean<<<1, 32, 0, s>>>(I, T, out);
     return cudaGetLastError();
 }
 

@@ -214,7 +214,7 @@ struct FwdDayArgs {
     uint64_t seed;
     FateRef fate;               // sampled R/M split (fate.L_M > 0) or the single RM exit
     DurRef dur;                 // stochastic I-stage durations (dur.n > 0)
-    float c[kMaxL];
+    const float *c;             // [kMaxL] infectiousness table, 0 from L on (device: captured loops outlive a table)
 };
 
 // Fixed-noise soft relaxation (every draw uses y = sigmoid(logit p - logit u)):
@@ -236,7 +236,7 @@ struct SoftDayArgs {
     double *P_nrm_t;         // [ntiles] per-tile sums of n_i(t - L) (newRM of day t)
     int ntiles, t, L;
     uint64_t seed;
-    float c[kMaxL];
+    const float *c;
 };
 
 struct BwdDayArgs {
@@ -262,7 +262,7 @@ struct BwdDayArgs {
     int ntiles, t, T, tau_EI, L;
     int mode;                  // kBwdStore, kBwdFused or kBwdSplit
     uint64_t seed;
-    float c[kMaxL];
+    const float *c;
     int ring_slot[kMaxL];      // ring slot holding day t + k, k = 1..L-1
     int32_t *sig, *emax;       // [G][ld_sig] scale exponent and largest stored exponent per day
     int32_t *rnz;              // [G][ld_sig] 1: some r of that day is not 0 (see carries_adjoint)
@@ -286,6 +286,7 @@ struct SeedState {
     uint32_t k_rem;     // seeds still to choose among keys matching the prefix
     uint32_t eq_count;  // keys equal to the final threshold hash
     uint32_t tie_n;     // candidates appended to the tie list
+    uint32_t done;      // blocks of the running pass that are through (the last one goes on)
     int32_t none;       // 1 when no seed is to be chosen
     int32_t overflow;   // tie list overflowed
 };
@@ -331,7 +332,7 @@ struct FwdBatchArgs {
     uint32_t *bits_next;         // the same for day t + 1
     int nunits, ru, t, tau_EI, L, B;   // units of ru rows (see unit_rows)
     uint64_t seed;
-    float c[kMaxL];
+    const float *c;
 };
 
 struct BwdBatchArgs {
@@ -352,7 +353,7 @@ struct BwdBatchArgs {
     int *tile_ctr;
     int nunits, ru, t, T, tau_EI, L, B;
     uint64_t seed;
-    float c[kMaxL];
+    const float *c;
     int ring_slot[kMaxL];
     int32_t *sig, *emax;         // [G][ld_sig] per graph (shared by its sets)
     int32_t *rnz;                // [G][ld_sig] 1: some r of that day is not 0 in some set
@@ -475,13 +476,17 @@ cudaError_t launch_day(void (*kernel)(P...), int grid, int block, size_t smem, c
 }
 
 // Launchers (forward.cu / backward.cu)
+// st: also resets the seeding of I instances (nullptr: state only).
 cudaError_t launch_init_state(int16_t *e, const int32_t *row0, const int32_t *rows, int G,
-                              int64_t n_rows, int B, int Bp, int grid, cudaStream_t s);
-cudaError_t launch_seed_reset(SeedState *st, const int32_t *n_seed, int I, cudaStream_t s);
-cudaError_t launch_seed_hist(const SeedArgs &a, int I, int grid_x, cudaStream_t s);
-cudaError_t launch_seed_scan(const SeedArgs &a, int I, cudaStream_t s);
+                              int64_t n_rows, int B, int Bp, SeedState *st, const int32_t *n_seed, int I,
+                              cudaStream_t s);
+cudaError_t launch_seed_pass(const SeedArgs &a, int I, int grid_x, cudaStream_t s);
 cudaError_t launch_seed_mark(const SeedArgs &a, int I, int grid_x, cudaStream_t s);
-cudaError_t launch_seed_ties(const SeedArgs &a, int I, cudaStream_t s);
+// R, m [I][T] and S [I][9] into the ctx's arrays (stride ldP), device memory.
+cudaError_t launch_stage(const float *R, const float *m, const float *S, float *R_ctx, float *m_ctx, float *S_ctx,
+                         int I, int T, int ldP, cudaStream_t s);
+cudaError_t launch_cumulative_mse(const double *D, const double *y, int I, int T, double *out, double *gD,
+                                  cudaStream_t s);
 // overlap: the launch before it in the stream is a day kernel of the same loop (see pdl_wait).
 cudaError_t launch_fwd_day(const FwdDayArgs &a, int grid, bool smem_bits, bool overlap, cudaStream_t s);
 // Flags for day t of the rows with an in-neighbour infectious on day t (bits_t): every

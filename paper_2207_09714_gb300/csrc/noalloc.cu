@@ -123,8 +123,7 @@ gabm_status gabm_seed_state_noalloc(uint64_t seed, int64_t n, int num_instances,
     k_fill_offsets<<<1, kNoallocMaxInstances, 0, s>>>(sc, (int32_t)n, num_instances, counts);
     NA_CK(cudaGetLastError());
     const int64_t n_rows = n * num_instances;
-    const int grid = (int)std::min<int64_t>((n_rows + 255) / 256, 65535);
-    NA_CK(launch_init_state(e_out, sc->row0, sc->rows, num_instances, n_rows, 1, 1, grid, s));
+    NA_CK(launch_init_state(e_out, sc->row0, sc->rows, num_instances, n_rows, 1, 1, sc->st, sc->n_seed, num_instances, s));
     SeedArgs sa;
     sa.row0 = sc->row0;
     sa.rows = sc->rows;
@@ -139,14 +138,11 @@ gabm_status gabm_seed_state_noalloc(uint64_t seed, int64_t n, int num_instances,
     sa.tau_EI = tau_EI;
     sa.pass = 0;
     const int gx = (int)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, 1024));
-    NA_CK(launch_seed_reset(sc->st, sc->n_seed, num_instances, s));
     for (int pass = 0; pass < 3; ++pass) {
         sa.pass = pass;
-        NA_CK(launch_seed_hist(sa, num_instances, gx, s));
-        NA_CK(launch_seed_scan(sa, num_instances, s));
+        NA_CK(launch_seed_pass(sa, num_instances, gx, s));
     }
     NA_CK(launch_seed_mark(sa, num_instances, gx, s));
-    NA_CK(launch_seed_ties(sa, num_instances, s));
 #undef NA_CK
     return GABM_OK;
 }

@@ -40,7 +40,7 @@ struct SirsFwdArgs {
     const float *long_sum;      // the long in-rows' sums of today
     int ntiles, t, tau_EI, L, cycle;
     uint64_t seed;
-    float c[kMaxL];
+    const float *c;
 };
 
 struct SirsBwdArgs {
@@ -68,7 +68,7 @@ struct SirsBwdArgs {
     int ld_sig;
     int ntiles, t, T, tau_EI, L, cycle;
     uint64_t seed;
-    float c[kMaxL];
+    const float *c;
 };
 
 cudaError_t launch_sirs_hist_init(const int16_t *e, int64_t n_rows, int H, int16_t *hist, uint16_t *cnt,
