@@ -20,12 +20,6 @@
 
 #include <algorithm>
 
-// The share (percent) of a graph's agents in E or I on the previous day from which the
-// one-set forward gathers every entry's exposure day instead of testing the day's bitmap.
-#ifndef GABM_DENSE_MARKS_PCT
-#define GABM_DENSE_MARKS_PCT 25
-#endif
-
 namespace gabm {
 
 namespace {
@@ -68,6 +62,7 @@ __global__ void __launch_bounds__(NT, MINB) k_fwd_day(FwdDayArgs a) {
     __shared__ float c_s[kMaxL];
     __shared__ double F_s[kMaxL];
     __shared__ int32_t red_s[NW][6];
+    __shared__ float rs_s[NW][kAges];   // R_t S_a of the warp's graph
     if (threadIdx.x < kMaxL) c_s[threadIdx.x] = a.c[threadIdx.x];
     if (EXIT == kExitDur && threadIdx.x < kMaxL) F_s[threadIdx.x] = a.dur.F[threadIdx.x];
     if (SMEM_BITS) {
@@ -80,12 +75,11 @@ __global__ void __launch_bounds__(NT, MINB) k_fwd_day(FwdDayArgs a) {
     const int t = a.t, L = a.L, tau_EI = a.tau_EI, ntiles = a.ntiles;
     const int16_t *e = a.e;
     const uint32_t *bits = a.bits_cur;
-    // Only neighbours infectious today contribute.  While few rows are infectious the day's
-    // bitmap spares the gathers of the others' exposure days; once many are (use_bits
-    // false, base model only), every entry's exposure day is gathered and tested directly.
-    bool use_bits = true;
+    // Only neighbours infectious today contribute: those whose exposure day lies in the window,
+    // and, where the exit from I is a row's own draw, that the day's bitmap marks as well.
+    constexpr bool EXPOSED = EXIT == kExitBase && !SMEM_BITS && !PULL;
     auto contrib = [&](uint32_t j, float w, bool valid, float &out, bool &take) {
-        const bool pre = valid && (!use_bits || (SMEM_BITS ? ((bits_s[j >> 5] >> (j & 31u)) & 1u) : marked(bits, j)));
+        const bool pre = valid && (EXPOSED || (SMEM_BITS ? ((bits_s[j >> 5] >> (j & 31u)) & 1u) : marked(bits, j)));
         const int ej = ld_if(e + j, pre, kNever);
         const int k = t - ej;
         take = pre && (unsigned)(k - 1) < (unsigned)(L - 1);
@@ -93,6 +87,7 @@ __global__ void __launch_bounds__(NT, MINB) k_fwd_day(FwdDayArgs a) {
     };
 
     int cur_g = -1;
+    float inv_D = 0.f;
     int cS = 0, cE = 0, cI = 0, cR = 0, cN = 0;
 
     // Tiles come from the block's contiguous range; each tile's row data is loaded two
@@ -115,11 +110,12 @@ __global__ void __launch_bounds__(NT, MINB) k_fwd_day(FwdDayArgs a) {
             if (cur_g >= 0) flush_counts_warp(a.counts, a.newRM, a.ldP, cur_g, t, cS, cE, cI, cR, cN, lane);
             cur_g = g;
             cS = cE = cI = cR = cN = 0;
-            if (!PULL && EXIT == kExitBase && t > a.t_first) {   // the graph's E + I share yesterday
-                const int32_t *cp = a.counts + ((size_t)g * a.ldP + t - 1) * 4;
-                const int32_t ei_cnt = cp[1] + cp[2], all = cp[0] + cp[1] + cp[2] + cp[3];
-                use_bits = (int64_t)ei_cnt * 100 < (int64_t)GABM_DENSE_MARKS_PCT * all;
-            }
+            // a graph's scalars, all loads in flight together
+            const float RS_ld = lane < kAges ? a.R[(size_t)g * a.ldP + t] * a.S[g * kAges + lane] : 0.f;
+            inv_D = a.gr.inv_Dbar[g];
+            __syncwarp();
+            if (lane < kAges) rs_s[wib][lane] = RS_ld;
+            __syncwarp();
         }
         const int row = tile * kTile + lane;
         const bool isS = (ei == kNever);
@@ -155,18 +151,17 @@ __global__ void __launch_bounds__(NT, MINB) k_fwd_day(FwdDayArgs a) {
             sum = gather_sum(a.m, cur.p0, cur.len, act, lane, a.pull);
         } else if (flags && __popc(amask) <= GABM_COOP_ROWS) {   // few summing rows: warp-wide, together
             if (amask) sum = few_row_sums(a.m, cur.p0, cur.len, amask, lane, contrib);
-        } else if (use_bits) {
-            sum = marked_sum(a.m, cur.p0, cur.len, act, lane, SMEM_BITS ? bits_s : bits, e, c_s, t, L);
-        } else {
+        } else if constexpr (EXPOSED) {
             sum = exposed_sum(a.m, cur.p0, cur.len, act, lane, e, c_s, t, L);
+        } else {
+            sum = marked_sum(a.m, cur.p0, cur.len, act, lane, SMEM_BITS ? bits_s : bits, e, c_s, t, L);
         }
-
         if (cur.len & kLongBit) sum = a.long_sum[cur.len & ~kLongBit];
         int e_next = ei;
         if (act) {
-            const float Lam = sum * a.gr.inv_Dbar[g];
+            const float Lam = sum * inv_D;
             const int inst = g;
-            const float lam = (a.R[(size_t)inst * a.ldP + t] * a.S[inst * kAges + age_ld]) * Lam;
+            const float lam = rs_s[wib][age_ld] * Lam;
             const float p = -expm1f(-lam);
             const uint32_t id = id_ld;
             const float u = uniform_from_word(philox_word(a.seed, id, (uint32_t)t, (uint32_t)inst, 0u));
@@ -184,7 +179,7 @@ __global__ void __launch_bounds__(NT, MINB) k_fwd_day(FwdDayArgs a) {
         const unsigned inf_next = __ballot_sync(0xffffffffu, inf);
         if (lane == 0) a.bits_next[tile] = inf_next;
         if (!PULL && flags) {   // tomorrow's flags: the out-neighbours of tomorrow's infectious rows
-            push_flags(a.m_out, tile, lane, inf, a.flag_next);
+            push_flags(a.m, a.m_out, cur, lane, inf, a.flag_next);
             a.flag_clear[row] = 0;
         }
 
@@ -785,7 +780,11 @@ __global__ void k_flags_from_bits(const uint32_t *bits_t, Sell m_out, int ntiles
     const int lane = threadIdx.x & 31;
     const int warps = (gridDim.x * blockDim.x) >> 5;
     for (int tile = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; tile < ntiles; tile += warps)
-        push_flags(m_out, tile, lane, (bits_t[tile] >> lane) & 1u, flags);
+{
+        TileRows own;
+        load_tile_layout(m_out, nullptr, ntiles, tile, lane, own);
+        push_flags(m_out, m_out, own, lane, (bits_t[tile] >> lane) & 1u, flags);
+    }
 }
 
 cudaError_t launch_flags_from_bits(const uint32_t *bits_t, Sell m_out, int ntiles, uint8_t *flags, cudaStream_t s) {

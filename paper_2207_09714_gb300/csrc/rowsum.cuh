@@ -233,12 +233,15 @@ __device__ __forceinline__ const uint2 *entry_ptr(const Sell &m, uint32_t p0, ui
 // their order).  Up to two rows: one at a time, the lanes splitting the row's entries.
 // More: every lane walks its own row, kMP pairs in flight; taken one at a time, the rows
 // of a tile with a dozen infectious agents would cost a dozen load round trips in a row.
-// Called by all 32 lanes.
-__device__ __forceinline__ void push_flags(const Sell &m_out, int tile, int lane, bool push, uint8_t *flags) {
+// `own` is the tile's row data of the in-edges: the same as the out-edges' where the
+// weights are symmetric, which spares a round trip.  Called by all 32 lanes.
+__device__ __forceinline__ void push_flags(const Sell &m, const Sell &m_out, const TileRows &own, int lane, bool push,
+                                           uint8_t *flags) {
     unsigned rows = __ballot_sync(0xffffffffu, push);
     if (!rows) return;
-    const uint32_t base = m_out.slice_ptr[tile];
-    uint32_t my_len = push ? m_out.row_len[tile * kTile + lane] : 0u;
+    const bool same = m.cw == m_out.cw;
+    const uint32_t base = same ? own.p0 : m_out.slice_ptr[own.tile];
+    uint32_t my_len = !push ? 0u : (same ? own.len : m_out.row_len[own.tile * kTile + lane]);
     if (my_len & kLongBit) my_len = 0u;   // the next day's long-row launch pushes these
     if (__popc(rows) <= 2) {
         while (rows) {
@@ -466,8 +469,11 @@ __device__ __forceinline__ float marked_sum(const Sell &m, uint32_t p0, uint32_t
 }
 
 // marked_sum without the bitmap: every entry's exposure day is gathered and tested, which
-// takes the same entries (an exposure during day t itself gives t - e_j = 0).  One
-// scattered load per entry: the cheaper way once a good share of the rows is infectious.
+// takes the same entries (an exposure during day t itself gives t - e_j = 0): one round trip a
+// batch, where the bitmap costs one for the bits and two for the marks.  On every day of the
+// base model this is the faster way (250k agents x 120 days: 2.42 ms by the bitmap below a
+// quarter of the agents infected, 2.28 without it; 1M x 60: 37.3 and 35.6 us a day).  The
+// first pairs loaded ahead, during the tile before, cost more registers than they gave.
 __device__ __forceinline__ float exposed_sum(const Sell &m, uint32_t p0, uint32_t len, bool act, int lane,
                                              const int16_t *e, const float *c_s, int t, int L) {
     const TileSpan s = tile_span(m, p0, len, act, lane);

@@ -46,18 +46,20 @@ __global__ void k_sirs_hist_init(const int16_t *e, int64_t n_rows, int H, int16_
 // reads no entries: its lambda is 0 exactly.
 __global__ void __launch_bounds__(kBlock, 3) k_fwd_day_sirs(SirsFwdArgs a) {
     __shared__ float c_s[kMaxL];
+    __shared__ float rs_s[kBlock / 32][kAges];   // R_t S_a of the warp's graph
+    float inv_D = 0.f;
     pdl_trigger();
     if (threadIdx.x < kMaxL) c_s[threadIdx.x] = a.c[threadIdx.x];
     __syncthreads();
     const int lane = threadIdx.x & 31;
     const int t = a.t, L = a.L, ntiles = a.ntiles;
-    const uint32_t *bits = a.bits_cur;
     const int16_t *e = a.e;
-    // neighbours marked infectious today (never written by this launch) contribute
+    // neighbours infectious today contribute: those whose last exposure day lies in the window
+    // (one exposed again during the day gives t - e = 0, and was out of it before)
     auto contrib = [&](uint32_t j, float w, bool valid, float &out, bool &take) {
-        take = valid && marked(bits, j);
-        const int ej = ld_if(e + j, take, kNever);
-        out = take ? w * infectiousness(ej, c_s, t, L) : 0.f;
+        const int k = t - ld_if(e + j, valid, kNever);
+        take = valid && (unsigned)(k - 1) < (unsigned)(L - 1);
+        out = take ? w * c_s[k] : 0.f;
     };
     int cur_g = -1, cS = 0, cE = 0, cI = 0, cR = 0, cN = 0;
     BlockTiles disp;
@@ -76,6 +78,11 @@ __global__ void __launch_bounds__(kBlock, 3) k_fwd_day_sirs(SirsFwdArgs a) {
             if (cur_g >= 0) flush_counts(a.counts, a.newRM, a.ldP, cur_g, t, cS, cE, cI, cR, cN, lane);
             cur_g = g;
             cS = cE = cI = cR = cN = 0;
+            const float RS_ld = lane < kAges ? a.R[(size_t)g * a.ldP + t] * a.S[g * kAges + lane] : 0.f;
+            inv_D = a.gr.inv_Dbar[g];
+            __syncwarp();
+            if (lane < kAges) rs_s[threadIdx.x >> 5][lane] = RS_ld;
+            __syncwarp();
         }
         const int row = tile * kTile + lane;
         const int ei = cur.e;
@@ -88,20 +95,22 @@ __global__ void __launch_bounds__(kBlock, 3) k_fwd_day_sirs(SirsFwdArgs a) {
         }
         cS += isS;
         const bool act = isS && cur.flag;
+        const int age_ld = act ? (int)a.age[row] : 0;   // ahead of the sums
+        const uint32_t id_ld = act ? caller_id(a.gr, row, g) : 0u;
         float sum = 0.f;
         const unsigned amask = __ballot_sync(0xffffffffu, act);
         if (a.flag_cur && __popc(amask) <= GABM_COOP_ROWS) {   // few summing rows: warp-wide, together
             if (amask) sum = few_row_sums(a.m, cur.p0, cur.len, amask, lane, contrib);
         } else {
-            sum = marked_sum(a.m, cur.p0, cur.len, act, lane, bits, e, c_s, t, L);
+            sum = exposed_sum(a.m, cur.p0, cur.len, act, lane, e, c_s, t, L);
         }
         if (cur.len & kLongBit) sum = a.long_sum[cur.len & ~kLongBit];
         int e_next = ei;
         if (act) {
-            const float Lam = sum * a.gr.inv_Dbar[g];
-            const float lam = (a.R[(size_t)g * a.ldP + t] * a.S[g * kAges + a.age[row]]) * Lam;
+            const float Lam = sum * inv_D;
+            const float lam = rs_s[threadIdx.x >> 5][age_ld] * Lam;
             const float p = -expm1f(-lam);
-            const uint32_t id = caller_id(a.gr, row, g);
+            const uint32_t id = id_ld;
             const float u = uniform_from_word(philox_word(a.seed, id, (uint32_t)t, (uint32_t)g, 0u));
             if (u < p) {
                 a.e[row] = (int16_t)t;
@@ -123,7 +132,7 @@ __global__ void __launch_bounds__(kBlock, 3) k_fwd_day_sirs(SirsFwdArgs a) {
         const unsigned inf_next = __ballot_sync(0xffffffffu, inf);
         if (lane == 0) a.bits_next[tile] = inf_next;
         if (a.flag_cur) {   // tomorrow's flags: the out-neighbours of tomorrow's infectious rows
-            push_flags(a.m_out, tile, lane, inf, a.flag_next);
+            push_flags(a.m, a.m_out, cur, lane, inf, a.flag_next);
             a.flag_clear[row] = 0;
         }
         cur = nxt;
