@@ -75,14 +75,14 @@ struct RingTerm {
 // EXIT = kExitDur (stochastic I-stage durations, store policy): G of an exposure today
 // sums over the window L_i it would draw and takes the death term m gD of its own exit
 // day; the exits recounted for dm are at each row's drawn L_i.
-template <int MODE, bool DC, int EXIT = kExitBase>
-__global__ void __launch_bounds__(kBlock, (MODE == kBwdStore && !DC) ? GABM_BWD_MINBLOCKS : GABM_MINBLOCKS)
+template <int MODE, bool DC, int EXIT = kExitBase, int NT = kBlock, int MINB = GABM_BWD_MINBLOCKS, int GP = kGP>
+__global__ void __launch_bounds__(NT, MINB)
     k_bwd_day(BwdDayArgs a) {
     constexpr bool FATE = EXIT == kExitFate;
     constexpr bool DUR = EXIT == kExitDur;
     constexpr bool SOFT = MODE == kBwdSoft;
     constexpr int RB = GABM_RING_BATCH;   // ring slots loaded together in the epilogue
-    constexpr int NW = kBlock / 32;
+    constexpr int NW = NT / 32;
     __shared__ float c_s[kMaxL];
     __shared__ int32_t red_s[NW][4];
     __shared__ RingTerm term_s[NW][kMaxL];        // the warp's graph's ring terms, k ascending
@@ -132,9 +132,9 @@ __global__ void __launch_bounds__(kBlock, (MODE == kBwdStore && !DC) ? GABM_BWD_
     disp.init(ntiles, lane);
     TileRows cur, nxt;
     load_tile_rows(a.m, E, a.gr.tile_graph, ntiles, disp.get(), lane, cur);
-    uint4 ea[kGP];
+    uint4 ea[GP];
 #pragma unroll
-    for (int u = 0; u < kGP; ++u) ea[u] = make_uint4(0u, 0u, 0u, 0u);
+    for (int u = 0; u < GP; ++u) ea[u] = make_uint4(0u, 0u, 0u, 0u);
     // the first tile's first pairs before the wait, as if its rows gather (they do, but for
     // the last days of a horizon); the final exposure days are not written by the sweep
     live_k = 2u;
@@ -143,6 +143,18 @@ __global__ void __launch_bounds__(kBlock, (MODE == kBwdStore && !DC) ? GABM_BWD_
         load_pairs(sp.row, 0u, sp.lim, ea);
     }
     bool have = true;   // ea holds the current tile's first pairs
+    // the first graph's scalars that no launch of the sweep writes
+    float RS_ld = 0.f, gt_ld = 0.f;
+    int row0_ld = 0;
+    auto load_scalars = [&](int g) {
+        const size_t pg = (size_t)g * a.ldP;
+        RS_ld = lane < kAges ? a.R[pg + t] * a.S[g * kAges + lane] : 0.f;
+        const int td = t + (FATE ? a.fate.L_M : L);   // the day today's exposures die on
+        gt_ld = td < T ? (FATE ? 1.f : a.m_t[pg + td]) * (float)a.gD[pg + td] : 0.f;
+        inv_D = a.gr.inv_Dbar[g];
+        row0_ld = a.gr.row0[g];
+    };
+    if (cur.tile < ntiles) load_scalars(cur.g);
     pdl_wait();
     while (cur.tile < ntiles) {
         load_tile_rows(a.m, E, a.gr.tile_graph, ntiles, disp.get(), lane, nxt);   // a tile ahead of use
@@ -159,17 +171,13 @@ __global__ void __launch_bounds__(kBlock, (MODE == kBwdStore && !DC) ? GABM_BWD_
             }
             const bool first = cur_g < 0;
             // every load of this block goes out before any is used
-            const size_t pg = (size_t)g * a.ldP, ps = (size_t)g * a.ld_sig;
+            const size_t ps = (size_t)g * a.ld_sig;
             sg = a.sig + ps;
             const bool in = lane >= 1 && lane < L && t + lane < T;
             const int32_t nz_ld = in ? a.rnz[ps + t + lane] : 0;
             const int32_t sg_ld = (lane >= 1 && lane < L && t + lane <= T) ? sg[t + lane] : 0;
             const int32_t em_ld = a.emax[ps + t + 1];
-            const float RS_ld = lane < kAges ? a.R[pg + t] * a.S[g * kAges + lane] : 0.f;
-            const int td = t + (FATE ? a.fate.L_M : L);   // the day today's exposures die on
-            const float gt_ld = td < T ? (FATE ? 1.f : a.m_t[pg + td]) * (float)a.gD[pg + td] : 0.f;
-            inv_D = a.gr.inv_Dbar[g];
-            const int row0_ld = a.gr.row0[g];
+            if (!first) load_scalars(g);
             live_k = __ballot_sync(0xffffffffu, nz_ld != 0);   // days that carry adjoint (flush_rnz)
             // this day's scale for graph g (every warp computes the same value; the warp
             // holding the graph's first tile records it)
@@ -610,8 +618,11 @@ __global__ void __launch_bounds__(256) k_bwd_finalize(const double *Q, const flo
 
 }  // namespace
 
-cudaError_t launch_bwd_day(const BwdDayArgs &a, int grid, bool overlap, cudaStream_t s) {
+cudaError_t launch_bwd_day(const BwdDayArgs &a, int grid, bool small, bool overlap, cudaStream_t s) {
     const bool dc = a.dc_tile != nullptr;
+    if (small && !dc)
+        return launch_day(k_bwd_day<kBwdStore, false, kExitBase, kSmallBlock, 8, 6>,
+                          (a.ntiles * 32 + kSmallBlock - 1) / kSmallBlock, kSmallBlock, 0, s, overlap, a);
     auto go = [&](void (*k)(BwdDayArgs)) { return launch_day(k, grid, kBlock, 0, s, overlap, a); };
     if (a.fate.L_M > 0 || a.dur.n > 0) {   // store policy, plain instance only (checked at creation)
         if (a.mode != kBwdStore || dc) return cudaErrorInvalidValue;

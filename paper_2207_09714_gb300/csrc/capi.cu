@@ -130,6 +130,7 @@ struct gabm_ctx {
     int lam_from = -1;
     int bits_from = -1;             // first day whose infectious bitmap the last forward wrote
 
+    bool small = false;             // a tile a warp: the base model's small instances (launch_fwd_day)
     bool overlap = false;           // day launches overlap at their edges (see pdl_wait)
     int grid_fwd = 0, grid_bwd = 0, grid_bwd_dc = 0;   // grid_bwd_dc: the table-adjoint instance
     int grid_bwd_fate = 0;                              // the sampled R/M split's instance
@@ -1065,7 +1066,7 @@ gabm_status forward_days_plain(gabm_ctx *c, int t0, int T, cudaStream_t s) {
         }
         a.long_sum = long_lam_buf(c);
         TRY(long_lambda(c, a.bits_cur, a.flag_cur ? fbuf(t) : nullptr, t, c->overlap && t > t0, s));
-        LAUNCH(launch_fwd_day(a, c->grid_fwd, c->smem_bits, c->overlap && t > t0, s));
+        LAUNCH(launch_fwd_day(a, c->grid_fwd, c->smem_bits, c->small && !c->smem_bits, c->overlap && t > t0, s));
         prof_end(c, 0);
     }
     return GABM_OK;
@@ -1163,7 +1164,7 @@ gabm_status backward_days_plain(gabm_ctx *c, int T, cudaStream_t s) {
             }
             if (la.in.n + la.out.n > 0) LAUNCH(launch_long(la, overlap, s));
         }
-        LAUNCH(launch_bwd_day(a, grid, overlap, s));
+        LAUNCH(launch_bwd_day(a, grid, c->small && mode == kBwdStore, overlap, s));
         prof_end(c, 1);
     }
     if (c->fate || a.dc_tile) TRY(long_gather(c, c->r, nullptr, 0, false, s));   // the long rows' gx(0)
@@ -1381,6 +1382,8 @@ void apply_schedule(gabm_ctx *c) {
     if (c->grid_bwd_fate > max_grid) c->grid_bwd_fate = max_grid;
     c->grid_sirs_f = std::min(max_grid, c->num_sms * occupancy_sirs(false));
     c->grid_sirs_b = std::min(max_grid, c->num_sms * occupancy_sirs(true));
+    c->small = !c->batched && !c->soft && !c->two_hop && !c->fate && c->dur.n == 0 && !c->sirs &&
+               c->ntiles <= kSmallTiles * c->num_sms;
     c->overlap = !c->batched && !c->soft && !c->two_hop &&
                  c->ntiles <= kOverlapRounds * c->num_sms * GABM_RESIDENT_WARPS;
     for (auto &g : c->loop_graph) drop_graph(g);   // captured launches carry the old schedule

@@ -53,7 +53,7 @@ __device__ __forceinline__ void flush_counts_warp(int32_t *counts, int32_t *newR
 // one), and the deaths counted are the M entries.  EXIT = kExitDur (stochastic I-stage
 // durations): the exit is the row's drawn L_i (drawn again from its first possible day
 // on); deaths stay m_t newRM(t).
-template <bool SMEM_BITS, int NT, int MINB, bool PULL = false, int EXIT = kExitBase>
+template <bool SMEM_BITS, int NT, int MINB, bool PULL = false, int EXIT = kExitBase, int UP = kMP>
 __global__ void __launch_bounds__(NT, MINB) k_fwd_day(FwdDayArgs a) {
     constexpr int NW = NT / 32;
     extern __shared__ uint32_t bits_s[];
@@ -98,6 +98,13 @@ __global__ void __launch_bounds__(NT, MINB) k_fwd_day(FwdDayArgs a) {
     TileRows cur, nxt;
     load_tile_layout(a.m, a.gr.tile_graph, ntiles, disp.get(), lane, cur);
     load_tile_layout(a.m, a.gr.tile_graph, ntiles, disp.get(), lane, nxt);
+    // the first graph's scalars too are of what no launch of the loop writes
+    if (cur.tile < ntiles) {
+        cur_g = cur.g;
+        if (lane < kAges) rs_s[wib][lane] = a.R[(size_t)cur_g * a.ldP + t] * a.S[cur_g * kAges + lane];
+        inv_D = a.gr.inv_Dbar[cur_g];
+        __syncwarp();
+    }
     if (!SMEM_BITS) pdl_wait();
     load_tile_state(e, ntiles, lane, cur, flags);
     load_tile_state(e, ntiles, lane, nxt, flags);
@@ -152,7 +159,7 @@ __global__ void __launch_bounds__(NT, MINB) k_fwd_day(FwdDayArgs a) {
         } else if (flags && __popc(amask) <= GABM_COOP_ROWS) {   // few summing rows: warp-wide, together
             if (amask) sum = few_row_sums(a.m, cur.p0, cur.len, amask, lane, contrib);
         } else if constexpr (EXPOSED) {
-            sum = exposed_sum(a.m, cur.p0, cur.len, act, lane, e, c_s, t, L);
+            sum = exposed_sum<UP>(a.m, cur.p0, cur.len, act, lane, e, c_s, t, L);
         } else {
             sum = marked_sum(a.m, cur.p0, cur.len, act, lane, SMEM_BITS ? bits_s : bits, e, c_s, t, L);
         }
@@ -794,7 +801,10 @@ cudaError_t launch_flags_from_bits(const uint32_t *bits_t, Sell m_out, int ntile
     return cudaGetLastError();
 }
 
-cudaError_t launch_fwd_day(const FwdDayArgs &a, int grid, bool smem_bits, bool overlap, cudaStream_t s) {
+cudaError_t launch_fwd_day(const FwdDayArgs &a, int grid, bool smem_bits, bool small, bool overlap, cudaStream_t s) {
+    if (small)
+        return launch_day(k_fwd_day<false, kSmallBlock, 8, false, kExitBase, 8>, (a.ntiles * 32 + kSmallBlock - 1) / kSmallBlock,
+                          kSmallBlock, 0, s, overlap, a);
     if (a.fate.L_M > 0) {
         return launch_day(k_fwd_day<false, kBlock, GABM_MINBLOCKS, false, kExitFate>, grid, kBlock, 0, s, overlap, a);
     } else if (a.dur.n > 0) {

@@ -335,31 +335,32 @@ __device__ __forceinline__ void load_pairs(const uint4 *row, uint32_t q0, uint32
 // used.  Batches in which every lane's entries are valid run without predicates; in the
 // others an invalid entry adds y = 0, which leaves the sum as it is (entries are invalid
 // from some k on, so the compensation it spoils is not used again).
-__device__ __forceinline__ float gather_sum(const TileSpan &s, const float *x, uint4 (&ea)[kGP]) {
+template <int GP>
+__device__ __forceinline__ float gather_sum(const TileSpan &s, const float *x, uint4 (&ea)[GP]) {
     float sum = 0.f, comp = 0.f;
-    auto use = [&](uint32_t q0, const uint4 (&v)[kGP]) {
-        float g[2 * kGP];
-        if (2u * q0 + 2u * kGP <= s.kfull) {
+    auto use = [&](uint32_t q0, const uint4 (&v)[GP]) {
+        float g[2 * GP];
+        if (2u * q0 + 2u * GP <= s.kfull) {
 #pragma unroll
-            for (int u = 0; u < kGP; ++u) {
+            for (int u = 0; u < GP; ++u) {
                 g[2 * u] = x[v[u].x];
                 g[2 * u + 1] = x[v[u].z];
             }
 #pragma unroll
-            for (int u = 0; u < kGP; ++u) {
+            for (int u = 0; u < GP; ++u) {
                 kahan_add(sum, comp, __uint_as_float(v[u].y) * g[2 * u]);
                 kahan_add(sum, comp, __uint_as_float(v[u].w) * g[2 * u + 1]);
             }
             return;
         }
 #pragma unroll
-        for (int u = 0; u < kGP; ++u) {
+        for (int u = 0; u < GP; ++u) {
             const uint32_t k = 2u * (q0 + (uint32_t)u);
             g[2 * u] = k < s.len ? x[v[u].x] : 0.f;
             g[2 * u + 1] = k + 1u < s.len ? x[v[u].z] : 0.f;
         }
 #pragma unroll
-        for (int i = 0; i < 2 * kGP; ++i) {
+        for (int i = 0; i < 2 * GP; ++i) {
             const float w = __uint_as_float((i & 1) ? v[i >> 1].w : v[i >> 1].y);
             const float y = (2u * q0 + (uint32_t)i < s.len) ? __fsub_rn(w * g[i], comp) : 0.f;
             const float t = __fadd_rn(sum, y);
@@ -367,15 +368,15 @@ __device__ __forceinline__ float gather_sum(const TileSpan &s, const float *x, u
             sum = t;
         }
     };
-    uint4 eb[kGP];
+    uint4 eb[GP];
 #pragma unroll
-    for (int u = 0; u < kGP; ++u) eb[u] = make_uint4(0u, 0u, 0u, 0u);
-    for (uint32_t q = 0; q < s.np; q += 2 * kGP) {
-        if (q + kGP < s.np) load_pairs(s.row, q + kGP, s.lim, eb);
+    for (int u = 0; u < GP; ++u) eb[u] = make_uint4(0u, 0u, 0u, 0u);
+    for (uint32_t q = 0; q < s.np; q += 2 * GP) {
+        if (q + GP < s.np) load_pairs(s.row, q + GP, s.lim, eb);
         use(q, ea);
-        if (q + kGP >= s.np) break;
-        if (q + 2 * kGP < s.np) load_pairs(s.row, q + 2 * kGP, s.lim, ea);
-        use(q + kGP, eb);
+        if (q + GP >= s.np) break;
+        if (q + 2 * GP < s.np) load_pairs(s.row, q + 2 * GP, s.lim, ea);
+        use(q + GP, eb);
     }
     return sum;
 }
@@ -474,36 +475,37 @@ __device__ __forceinline__ float marked_sum(const Sell &m, uint32_t p0, uint32_t
 // base model this is the faster way (250k agents x 120 days: 2.42 ms by the bitmap below a
 // quarter of the agents infected, 2.28 without it; 1M x 60: 37.3 and 35.6 us a day).  The
 // first pairs loaded ahead, during the tile before, cost more registers than they gave.
+template <int UP = kMP>
 __device__ __forceinline__ float exposed_sum(const Sell &m, uint32_t p0, uint32_t len, bool act, int lane,
                                              const int16_t *e, const float *c_s, int t, int L) {
     const TileSpan s = tile_span(m, p0, len, act, lane);
     float sum = 0.f, comp = 0.f;
-    uint4 ea[kMP], eb[kMP];
+    uint4 ea[UP], eb[UP];
 #pragma unroll
-    for (int u = 0; u < kMP; ++u) ea[u] = eb[u] = make_uint4(0u, 0u, 0u, 0u);
+    for (int u = 0; u < UP; ++u) ea[u] = eb[u] = make_uint4(0u, 0u, 0u, 0u);
     load_pairs(s.row, 0u, s.lim, ea);
-    auto use = [&](uint32_t q0, const uint4 (&v)[kMP]) {
-        int ej[2 * kMP];
+    auto use = [&](uint32_t q0, const uint4 (&v)[UP]) {
+        int ej[2 * UP];
 #pragma unroll
-        for (int u = 0; u < kMP; ++u) {
+        for (int u = 0; u < UP; ++u) {
             const uint32_t k = 2u * (q0 + (uint32_t)u);
             ej[2 * u] = k < s.len ? (int)e[v[u].x] : kNever;
             ej[2 * u + 1] = k + 1u < s.len ? (int)e[v[u].z] : kNever;
         }
 #pragma unroll
-        for (int i = 0; i < 2 * kMP; ++i) {
+        for (int i = 0; i < 2 * UP; ++i) {
             const float w = __uint_as_float((i & 1) ? v[i >> 1].w : v[i >> 1].y);
             const int k = t - ej[i];
             const bool tk = (unsigned)(k - 1) < (unsigned)(L - 1);
             kahan_add_if(sum, comp, tk ? w * c_s[k] : 0.f, tk);
         }
     };
-    for (uint32_t q = 0; q < s.np; q += 2 * kMP) {
-        if (q + kMP < s.np) load_pairs(s.row, q + kMP, s.lim, eb);
+    for (uint32_t q = 0; q < s.np; q += 2 * UP) {
+        if (q + UP < s.np) load_pairs(s.row, q + UP, s.lim, eb);
         use(q, ea);
-        if (q + kMP >= s.np) break;
-        if (q + 2 * kMP < s.np) load_pairs(s.row, q + 2 * kMP, s.lim, ea);
-        use(q + kMP, eb);
+        if (q + UP >= s.np) break;
+        if (q + 2 * UP < s.np) load_pairs(s.row, q + 2 * UP, s.lim, ea);
+        use(q + UP, eb);
     }
     return sum;
 }
