@@ -63,10 +63,7 @@ struct RingTerm {
 
 // DC: accumulate the table adjoint (a.dc_tile); a separate instance, so the plain sweep
 // carries none of its code.
-// Resident blocks: see the launch bounds' measurements below.
-#ifndef GABM_BWD_MINBLOCKS
-#define GABM_BWD_MINBLOCKS 3
-#endif
+// MINB blocks an SM, GP pairs of entries a lane ahead of their use (see bwd_kernel).
 // EXIT = kExitFate (sampled R/M split, store policy): G of an exposure today takes the
 // fate it would draw (window L_R or L_M; the death term gD_{t+L_M} only if M-fated), and
 // the rows exposed today add H dphi/dm to day t + tau_EI's dL/dm, H = dL/dphi = sum over
@@ -75,7 +72,8 @@ struct RingTerm {
 // EXIT = kExitDur (stochastic I-stage durations, store policy): G of an exposure today
 // sums over the window L_i it would draw and takes the death term m gD of its own exit
 // day; the exits recounted for dm are at each row's drawn L_i.
-template <int MODE, bool DC, int EXIT = kExitBase, int NT = kBlock, int MINB = GABM_BWD_MINBLOCKS, int GP = kGP>
+template <int MODE, bool DC, int EXIT = kExitBase, int NT = kBlock, int MINB = 3,
+          int GP = kGP>
 __global__ void __launch_bounds__(NT, MINB)
     k_bwd_day(BwdDayArgs a) {
     constexpr bool FATE = EXIT == kExitFate;
@@ -618,22 +616,39 @@ __global__ void __launch_bounds__(256) k_bwd_finalize(const double *Q, const flo
 
 }  // namespace
 
-cudaError_t launch_bwd_day(const BwdDayArgs &a, int grid, bool small, bool overlap, cudaStream_t s) {
+// The instance of a day.  deep (deep_gather in capi.cu holds the rule): two blocks an SM with
+// most of an ordinary row in flight instead of three with two pairs a lane ahead.  A row sum
+// is a chain of round trips, so fewer and longer batches win wherever the fewer warps don't
+// cost more waves of tiles than that saves.  Us per day, three blocks against two: 1M town
+// 61.4 -> 58.5, twelve counties 29.2 -> 24.1, 300k power law 58.9 -> 50.2, deaths sampled at
+// 200k 24.1 -> 23.3 (at 1M, 4, 5 and 7 pairs: 62.4, 59.9, 61.5).  The instances with the
+// table's adjoint have other work between the loads: 15.5 -> 16.8 at 100k, so they stay.
+using BwdKernel = void (*)(BwdDayArgs);
+static BwdKernel bwd_kernel(int mode, bool dc, int exit_mode, bool deep) {
+    constexpr int D = kDeepPairs;
+    if (exit_mode == kExitFate)
+        return deep ? k_bwd_day<kBwdStore, false, kExitFate, kBlock, 2, D> : k_bwd_day<kBwdStore, false, kExitFate>;
+    if (exit_mode == kExitDur)
+        return deep ? k_bwd_day<kBwdStore, false, kExitDur, kBlock, 2, D> : k_bwd_day<kBwdStore, false, kExitDur>;
+    if (mode == kBwdSoft) return dc ? k_bwd_day<kBwdSoft, true> : k_bwd_day<kBwdSoft, false>;
+    if (mode == kBwdFused) {
+        if (dc) return k_bwd_day<kBwdFused, true>;
+        return deep ? k_bwd_day<kBwdFused, false, kExitBase, kBlock, 2, D> : k_bwd_day<kBwdFused, false>;
+    }
+    if (dc) return k_bwd_day<kBwdStore, true>;
+    return deep ? k_bwd_day<kBwdStore, false, kExitBase, kBlock, 2, D> : k_bwd_day<kBwdStore, false>;
+}
+
+cudaError_t launch_bwd_day(const BwdDayArgs &a, int grid, bool small, bool deep, bool overlap, cudaStream_t s) {
     const bool dc = a.dc_tile != nullptr;
+    const int exit_mode = a.fate.L_M > 0 ? kExitFate : a.dur.n > 0 ? kExitDur : kExitBase;
+    if (a.mode != kBwdStore && a.mode != kBwdFused && a.mode != kBwdSoft) return cudaErrorInvalidValue;
+    // store policy, plain instance only (checked at creation)
+    if (exit_mode != kExitBase && (a.mode != kBwdStore || dc)) return cudaErrorInvalidValue;
     if (small && !dc)
-        return launch_day(k_bwd_day<kBwdStore, false, kExitBase, kSmallBlock, 8, 6>,
+        return launch_day(k_bwd_day<kBwdStore, false, kExitBase, kSmallBlock, 8, kDeepPairs>,
                           (a.ntiles * 32 + kSmallBlock - 1) / kSmallBlock, kSmallBlock, 0, s, overlap, a);
-    auto go = [&](void (*k)(BwdDayArgs)) { return launch_day(k, grid, kBlock, 0, s, overlap, a); };
-    if (a.fate.L_M > 0 || a.dur.n > 0) {   // store policy, plain instance only (checked at creation)
-        if (a.mode != kBwdStore || dc) return cudaErrorInvalidValue;
-        return a.fate.L_M > 0 ? go(k_bwd_day<kBwdStore, false, kExitFate>) : go(k_bwd_day<kBwdStore, false, kExitDur>);
-    }
-    switch (a.mode) {
-        case kBwdStore: return dc ? go(k_bwd_day<kBwdStore, true>) : go(k_bwd_day<kBwdStore, false>);
-        case kBwdFused: return dc ? go(k_bwd_day<kBwdFused, true>) : go(k_bwd_day<kBwdFused, false>);
-        case kBwdSoft: return dc ? go(k_bwd_day<kBwdSoft, true>) : go(k_bwd_day<kBwdSoft, false>);
-        default: return cudaErrorInvalidValue;
-    }
+    return launch_day(bwd_kernel(a.mode, dc, exit_mode, deep), grid, kBlock, 0, s, overlap, a);
 }
 
 cudaError_t launch_dc_seeds(Sell m_out, const int16_t *E, const float *r0, GraphRef gr, const int32_t *sig,
@@ -669,29 +684,9 @@ cudaError_t launch_lam_day(Sell m, const int16_t *E, const uint32_t *bits, Graph
     return cudaGetLastError();
 }
 
-int occupancy_bwd(int mode, bool dc, int exit_mode) {
+int occupancy_bwd(int mode, bool dc, int exit_mode, bool deep) {
     int blocks = 0;
-    if (exit_mode != kExitBase) {
-        if (exit_mode == kExitFate)
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, k_bwd_day<kBwdStore, false, kExitFate>, kBlock, 0);
-        else
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, k_bwd_day<kBwdStore, false, kExitDur>, kBlock, 0);
-        return blocks > 0 ? blocks : 1;
-    }
-    switch (mode) {
-        case kBwdFused:
-            if (dc) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, k_bwd_day<kBwdFused, true>, kBlock, 0);
-            else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, k_bwd_day<kBwdFused, false>, kBlock, 0);
-            break;
-        case kBwdSoft:
-            if (dc) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, k_bwd_day<kBwdSoft, true>, kBlock, 0);
-            else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, k_bwd_day<kBwdSoft, false>, kBlock, 0);
-            break;
-        default:
-            if (dc) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, k_bwd_day<kBwdStore, true>, kBlock, 0);
-            else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, k_bwd_day<kBwdStore, false>, kBlock, 0);
-            break;
-    }
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, bwd_kernel(mode, dc, exit_mode, deep), kBlock, 0);
     return blocks > 0 ? blocks : 1;
 }
 

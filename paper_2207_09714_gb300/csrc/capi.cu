@@ -130,9 +130,12 @@ struct gabm_ctx {
     int lam_from = -1;
     int bits_from = -1;             // first day whose infectious bitmap the last forward wrote
 
+    double mean_len = 0, near_share = 0;   // entries per agent; those within kNearRows of their row
+    bool deep = false;              // the reverse sweep's deep instances (deep_gather)
     bool small = false;             // a tile a warp: the base model's small instances (launch_fwd_day)
     bool overlap = false;           // day launches overlap at their edges (see pdl_wait)
     int grid_fwd = 0, grid_bwd = 0, grid_bwd_dc = 0;   // grid_bwd_dc: the table-adjoint instance
+    int grid_lam = 0;                                   // k_lam_day
     int grid_bwd_fate = 0;                              // the sampled R/M split's instance
     bool smem_bits = false;         // forward keeps the infectious bitmap in shared memory
     // agent-location graphs: the location hop (SELL-32 of locations -> members) and its values
@@ -1130,7 +1133,7 @@ gabm_status backward_days_plain(gabm_ctx *c, int T, cudaStream_t s) {
         if (mode == kBwdSplit) {
             TRY(long_lambda(c, c->bits + (size_t)t * c->ntiles, nullptr, t, false, s));
             LAUNCH(launch_lam_day(sell_view(c, false), c->e, c->bits + (size_t)t * c->ntiles, graph_ref(c), t, c->L,
-                                  c->ntiles, c->c_dev, long_lam_buf(c), c->lam_tmp, c->grid_bwd, s));
+                                  c->ntiles, c->c_dev, long_lam_buf(c), c->lam_tmp, c->grid_lam, s));
         }
         a.r_next = c->r + (size_t)((t + 1) & 1) * c->n_rows;
         a.r_cur = c->r + (size_t)(t & 1) * c->n_rows;
@@ -1164,7 +1167,7 @@ gabm_status backward_days_plain(gabm_ctx *c, int T, cudaStream_t s) {
             }
             if (la.in.n + la.out.n > 0) LAUNCH(launch_long(la, overlap, s));
         }
-        LAUNCH(launch_bwd_day(a, grid, c->small && mode == kBwdStore, overlap, s));
+        LAUNCH(launch_bwd_day(a, grid, c->small && mode == kBwdStore, c->deep, overlap, s));
         prof_end(c, 1);
     }
     if (c->fate || a.dc_tile) TRY(long_gather(c, c->r, nullptr, 0, false, s));   // the long rows' gx(0)
@@ -1346,6 +1349,22 @@ gabm_status backward_core(gabm_ctx *c, int T) {
     return run_day_loop(c, kLoopBackward, 0, T, false);
 }
 
+// Whether the reverse sweep runs its deep instances (bwd_kernel): fewer warps, more of each
+// row in flight.  Rows of a few entries have nothing to put in flight (agents' locations at
+// 300k: 17.7 us a day, deep 19.4; 200k random pairs, 3 a row: 391 us a sweep, 451).  Fewer warps
+// must not double the waves of tiles (100k random, 8 a row: 349 us a sweep, 381; 200k: 544,
+// 533; 300k, 20 a row: 1204, 1121).  And where most entries lie beyond the reach of the SM's
+// L1, warps hide its misses better from some size on (400k random, 8 a row: 912, 948; 600k:
+// 1235, 1319); with most entries near, as in towns, the deep instances stay ahead up to 1M.
+bool deep_gather(const gabm_ctx *c, int mode) {
+    if (c->mean_len < 8.0) return false;
+    const auto waves = [&](bool deep) {
+        const int warps = c->num_sms * occupancy_bwd(mode, false, kExitBase, deep) * (kBlock / 32);
+        return (c->ntiles + warps - 1) / warps;
+    };
+    return waves(true) < 2 * waves(false) && (c->near_share >= 0.5 || c->ntiles <= kDeepTiles * c->num_sms);
+}
+
 // Grid sizes for the current schedule (resident blocks per SM x SMs, at most one warp per tile).
 void apply_schedule(gabm_ctx *c) {
     const int mode = c->soft ? kBwdSoft
@@ -1366,9 +1385,11 @@ void apply_schedule(gabm_ctx *c) {
         // finish early leave their SM to the next wave's blocks
         const int waves = std::max(1, GABM_DAY_WAVES);
         c->grid_fwd = c->num_sms * (c->smem_bits ? bps : occupancy_fwd(c->ntiles, false) * waves);
-        c->grid_bwd = c->num_sms * occupancy_bwd(mode) * waves;
+        c->deep = deep_gather(c, mode);
+        c->grid_lam = c->num_sms * occupancy_bwd(mode) * waves;
+        c->grid_bwd = c->num_sms * occupancy_bwd(mode, false, kExitBase, c->deep) * waves;
         c->grid_bwd_dc = c->num_sms * occupancy_bwd(mode, true);
-        c->grid_bwd_fate = c->num_sms * occupancy_bwd(mode, false, c->fate ? kExitFate : kExitDur);
+        c->grid_bwd_fate = c->num_sms * occupancy_bwd(mode, false, c->fate ? kExitFate : kExitDur, c->deep);
     }
     if (c->two_hop) {
         c->smem_bits = false;
@@ -1378,6 +1399,7 @@ void apply_schedule(gabm_ctx *c) {
     const int max_grid = ((c->batched ? c->nunits : c->ntiles) + kBlock / 32 - 1) / (kBlock / 32);
     if (!c->smem_bits && c->grid_fwd > max_grid) c->grid_fwd = max_grid;
     if (c->grid_bwd > max_grid) c->grid_bwd = max_grid;
+    if (c->grid_lam > max_grid) c->grid_lam = max_grid;
     if (c->grid_bwd_dc > max_grid) c->grid_bwd_dc = max_grid;
     if (c->grid_bwd_fate > max_grid) c->grid_bwd_fate = max_grid;
     c->grid_sirs_f = std::min(max_grid, c->num_sms * occupancy_sirs(false));
@@ -1435,6 +1457,7 @@ struct HostLayout {
     std::vector<double> Dbar;
     bool symmetric = true, batched = false, reorder = true;
     uint32_t max_degree = 0;
+    double mean_len = 0, near_share = 0;
     int64_t n_rows = 0, nnz = 0, nnz_pad = 0, n_total = 0;
     int ntiles = 0, sigma = 1024, num_graphs = 1;
 };
@@ -1467,6 +1490,8 @@ static gabm_status create_on_device(const HostLayout &H, const gabm_model_desc *
         c->Bp = 2;
         while (c->Bp < sets_per_graph) c->Bp *= 2;
     }
+    c->mean_len = H.mean_len;
+    c->near_share = H.near_share;
     c->kahan_b = max_degree > (uint32_t)kPlainSumMaxDegree;
     {
         int mx = 1;
@@ -1799,7 +1824,10 @@ gabm_status gabm_create(const gabm_graph_desc *graphs, int num_graphs, int sets_
                      (!symmetric && !build_sell(t_rowptr, t_col, t_w, n_rows, sell_out, true))))
         return fail(nullptr, GABM_EUNSUPPORTED, "SELL-32 layout needs >= 2^32 entries");
     uint32_t max_degree = 0;
+    int64_t near = 0;
     for (int64_t r = 0; r < n_rows; ++r) {
+        for (uint32_t p = t_rowptr[r]; p < t_rowptr[r + 1]; ++p)
+            near += std::abs((int64_t)t_col[p] - r) < kNearRows;
         max_degree = std::max(max_degree, h_rowptr[r + 1] - h_rowptr[r]);
         max_degree = std::max(max_degree, t_rowptr[r + 1] - t_rowptr[r]);
     }
@@ -1826,6 +1854,8 @@ gabm_status gabm_create(const gabm_graph_desc *graphs, int num_graphs, int sets_
     H.batched = batched;
     H.reorder = reorder;
     H.max_degree = max_degree;
+    H.mean_len = n_total > 0 ? (double)nnz / (double)n_total : 0.0;
+    H.near_share = nnz > 0 ? (double)near / (double)nnz : 0.0;
     H.n_rows = n_rows;
     H.nnz = nnz;
     H.nnz_pad = nnz_pad;

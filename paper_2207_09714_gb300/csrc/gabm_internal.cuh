@@ -511,9 +511,12 @@ cudaError_t launch_fwd_finalize(const int32_t *newRM, const int32_t *counts, con
                                 int32_t *counts_out, cudaStream_t s);
 cudaError_t launch_mse(const double *D, int ldP, const double *y, int T, int I, double *loss,
                        double *gD_ctx, double *gD_out, cudaStream_t s);
-cudaError_t launch_bwd_day(const BwdDayArgs &a, int grid, bool small, bool overlap, cudaStream_t s);
+cudaError_t launch_bwd_day(const BwdDayArgs &a, int grid, bool small, bool deep, bool overlap, cudaStream_t s);
 constexpr int kSmallBlock = 64;   // threads of those blocks; eight an SM at 128 registers
 constexpr int kSmallTiles = 16;
+constexpr int kDeepTiles = 64;    // tiles an SM (deep_gather)
+constexpr int kNearRows = 1024;
+constexpr int kDeepPairs = 6;     // pairs of entries a lane ahead of use, reverse sweep (bwd_kernel)
 // Adjoint of the infectiousness table (hard mode, one set per graph): the seeds'
 // share through their day-0 infectiousness, then the per-graph sums of dc_tile.
 cudaError_t launch_dc_seeds(Sell m_out, const int16_t *E, const float *r0, GraphRef gr, const int32_t *sig,
@@ -577,6 +580,6 @@ cudaError_t launch_rows_to_caller_f32(const float *src, float *dst, GraphRef gr,
 cudaError_t launch_caller_to_rows_i16(const int16_t *src, int16_t *dst, GraphRef gr, const int32_t *rows,
                                       const int64_t *goff, int64_t n_rows, SetLayout sl, cudaStream_t s);
 int occupancy_fwd(int ntiles, bool smem_bits);
-int occupancy_bwd(int mode, bool dc = false, int exit_mode = kExitBase);
+int occupancy_bwd(int mode, bool dc = false, int exit_mode = kExitBase, bool deep = false);
 
 }  // namespace gabm
