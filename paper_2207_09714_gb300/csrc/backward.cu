@@ -14,9 +14,9 @@
 // lambda_i(t) comes from the forward's store or is recomputed from the final
 // exposure days E (no reinfection, A3/A4 of App. A, so E determines every
 // day's state and no checkpoints are needed): in the same pass when in- and
-// out-edges coincide, else by k_lam_day over the in-edges first.  Each warp
-// prefetches the next tile's id, row data and (into L2) its edge range while
-// it works on the current tile.
+// out-edges coincide, else by k_lam_day over the in-edges first.  The next tile's
+// row data are loaded while the current tile is worked on.  Days no adjoint has
+// reached yet (rnz) gather nothing.
 #include "gabm_internal.cuh"
 #include "rowsum.cuh"
 

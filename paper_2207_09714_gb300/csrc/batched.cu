@@ -13,19 +13,20 @@
 // row, lane q of the group owning the SPL sets [q SPL, (q+1) SPL); 32/LPR rows
 // are in flight per warp and the unit takes as many passes as that needs.  For each chunk of LPR
 // entries of the row, the group loads the columns and weights coalesced, tests
-// each neighbour against the day's bitmap (rows infectious in some set, or
-// susceptible in some set in the backward), compacts the marked entries with a
-// ballot and broadcasts them one by one; every lane gathers its SPL sets'
-// values with one vector load and accumulates them in entry order.  Unmarked
-// entries contribute nothing in any set, so skipping them changes no sum.
+// each neighbour against the day's bitmap (rows infectious in some set),
+// compacts the marked entries with a ballot and broadcasts them one by one;
+// every lane gathers its SPL sets' values with one vector load and accumulates
+// them in entry order.  Unmarked entries contribute nothing in any set, so
+// skipping them changes no sum.  The reverse sweep gathers every entry: nearly
+// all neighbours are susceptible in some set, and r is 0 where they are not.
 //
 // Summation: compensated (as in the single-set kernels) when some row has more
 // than kPlainSumMaxDegree entries, else fused multiply-add in entry order,
 // whose relative error is below (entries + 3) * 2^-24 < 1e-5 for a sum of
 // non-negative terms.
 //
-// Counting (Aggregate, Sec. 3.1): the forward writes, per tile and set, how
-// many agents were exposed that day (tile_new, one byte each); the stage
+// Counting (Aggregate, Sec. 3.1): the forward writes, per unit and set, how
+// many agents were exposed that day (unit_new, one byte each); the stage
 // counts and newRM of every day follow from those and the exposure-day
 // histogram of the starting state (k_counts_b), with no atomics in the day
 // kernel.

@@ -3,12 +3,13 @@
 // One launch per day (Sec. 3.1, Eq. 1-3; A1: one-day steps).  Each block takes
 // a contiguous range of 32-row tiles, its warps one tile at a time (neighbours
 // stay in the SM's L1 this way); each lane sums its own susceptible
-// row over the in-edges (a pull gather, no atomics) read from the tile's
-// SELL-32 slice with coalesced loads: w_ji * c[t - e_j] for the neighbours
-// marked infectious in today's bitmap (an L1-resident bit array), whose
-// exposure days are gathered from the L2-resident state.  Each warp prefetches
-// the next tile's id, row data and (into L2) its slice while it works on the
-// current tile.  Each lane then runs the fused epilogue for its own
+// row over the in-edges (a pull gather, no atomics) read from the tile's SELL-32
+// slice with coalesced 16-byte loads: w_ji * c[t - e_j], the neighbours' exposure
+// days gathered from the L2-resident state (the progression variants, whose exit
+// from I is a row's own draw, go by the day's infectious bitmap first).  The next
+// tile's row data are loaded while the current tile is worked on, and a launch's
+// layout and scalars before the day ahead of it has ended (pdl_wait).  Each lane
+// then runs the fused epilogue for its own
 // row: lambda, p = 1 - exp(-lambda) (Eq. 3), the Philox uniform, the hard draw
 // and the in-place state update e_i = t.
 //
@@ -42,9 +43,8 @@ __device__ __forceinline__ void flush_counts_warp(int32_t *counts, int32_t *newR
     }
 }
 
-// SMEM_BITS: today's infectious bitmap is copied into shared memory (one large
-// block per SM), so the per-edge test is a shared-memory lookup instead of a
-// scattered L1 load; otherwise it is read through L1 from global memory.
+// SMEM_BITS: entries go by today's infectious bitmap, which is copied into shared memory (one large
+// block per SM), so the per-edge test is a shared-memory lookup.
 // PULL (agent-location graphs): the row's entries are the agent's locations, and each
 // contributes w_il * P_l from the day's location pressures (a.pull) instead of a marked
 // neighbour's infectiousness.
