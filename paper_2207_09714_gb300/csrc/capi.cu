@@ -1355,14 +1355,17 @@ gabm_status backward_core(gabm_ctx *c, int T) {
 // must not double the waves of tiles (100k random, 8 a row: 349 us a sweep, 381; 200k: 544,
 // 533; 300k, 20 a row: 1204, 1121).  And where most entries lie beyond the reach of the SM's
 // L1, warps hide its misses better from some size on (400k random, 8 a row: 912, 948; 600k:
-// 1235, 1319); with most entries near, as in towns, the deep instances stay ahead up to 1M.
+// 1235, 1319); with most entries near, as in towns, the deep instances stay ahead up to 1M
+// (us a sweep at 200k and 1M, three blocks against two: 1105 and 3522, 952 and 3426; drawn
+// durations 1307 and 4360, 1197 and 4333), but for the sampled deaths (1217 and 4190, 1143
+// and 4286), whose draw keeps more registers.
 bool deep_gather(const gabm_ctx *c, int mode) {
     if (c->mean_len < 8.0) return false;
     const auto waves = [&](bool deep) {
         const int warps = c->num_sms * occupancy_bwd(mode, false, kExitBase, deep) * (kBlock / 32);
         return (c->ntiles + warps - 1) / warps;
     };
-    return waves(true) < 2 * waves(false) && (c->near_share >= 0.5 || c->ntiles <= kDeepTiles * c->num_sms);
+    return waves(true) < 2 * waves(false) && ((c->near_share >= 0.5 && !c->fate) || c->ntiles <= kDeepTiles * c->num_sms);
 }
 
 // Grid sizes for the current schedule (resident blocks per SM x SMs, at most one warp per tile).
