@@ -318,16 +318,16 @@ __global__ void __launch_bounds__(kBlock, SPL <= 4 ? 3 : 2) k_bwd_day_b(const Bw
     }
 }
 
+// The 48 KB that need no opt-in hold the kernel's static arrays too (20 KB with 64 sets), so
+// L decides on which side of it a launch lies; the limit is raised to that of the longest table, the
+// same value from every ctx and thread.
 template <int LPR, int SPL, bool KAHAN>
 cudaError_t launch_bwd_dc(const BwdBatchArgs &a, int grid, cudaStream_t s) {
-    const size_t bytes = sizeof(float) * (size_t)(kBlock / 32) * a.L * (LPR * SPL);
-    if (bytes > 48 * 1024) {
-        const cudaError_t e =
-            cudaFuncSetAttribute(k_bwd_day_b<LPR, SPL, KAHAN, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)bytes);
-        if (e != cudaSuccess) return e;
-    }
-    k_bwd_day_b<LPR, SPL, KAHAN, true><<<grid, kBlock, bytes, s>>>(a);
+    constexpr size_t day = sizeof(float) * (size_t)(kBlock / 32) * (LPR * SPL);
+    const cudaError_t e = cudaFuncSetAttribute(k_bwd_day_b<LPR, SPL, KAHAN, true>,
+                                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(day * kMaxL));
+    if (e != cudaSuccess) return e;
+    k_bwd_day_b<LPR, SPL, KAHAN, true><<<grid, kBlock, day * a.L, s>>>(a);
     return cudaGetLastError();
 }
 
