@@ -185,30 +185,49 @@ def synthetic_features(R_t: np.ndarray, t_N: int, F: int = 5, seed: int = 0) -> 
 
 
 class _CumulativeMse(torch.autograd.Function):
-    """The fused loss and its gradient (two launches for the five and their backward's nine of
-    the torch expression, 300 us of host time a step)."""
+    """The fused loss and its gradient, gD = 2/n S (C - y) with C = the running sums of D and S = the
+    sums from each day to the last (three launches with the backward, for the fourteen of the
+    torch expression).  gD is an output too, so that it needs neither operand to be
+    differentiated again: its adjoint h gives 2/n S (the running sums of h)."""
 
     @staticmethod
     def forward(fctx, D, y):
         loss, gD = capi.gabm_cumulative_mse(D, y)
-        fctx.save_for_backward(D, y, gD)
-        return loss
+        fctx.set_materialize_grads(False)
+        fctx.save_for_backward(gD)
+        return loss, gD
 
     @staticmethod
-    def backward(fctx, g):
-        D, y, gD = fctx.saved_tensors
-        if torch.is_grad_enabled():   # a graph of the gradient is wanted: keep it differentiable
-            r = torch.cumsum(D, dim=-1) - y
-            gD = torch.flip(torch.cumsum(torch.flip(r, (-1,)), dim=-1), (-1,)) * (2.0 / r.numel())
-        return g * gD, None
+    def backward(fctx, g, h):
+        gD, = fctx.saved_tensors
+        out = None if g is None else g * gD
+        if h is not None:
+            back = torch.flip(torch.cumsum(torch.flip(torch.cumsum(h, -1), (-1,)), -1), (-1,)) * (2.0 / h.numel())
+            out = back if out is None else out + back
+        return out, None
 
 
-def _plain_cuda(t: torch.Tensor) -> bool:
-    """An ordinary float64 matrix on the current device, outside any transform of torch."""
+# What tells whether torch works under a transform (vmap, grad, jvp) or a mode that looks at or
+# replaces its operations (tracing, fake tensors); without one of these, always "yes".
+_MODES = [getattr(torch._C, name, None) for name in
+          ("_are_functorch_transforms_active", "_len_torch_dispatch_stack", "_len_torch_function_stack")]
+
+
+def _transformed() -> bool:
+    return (torch.jit.is_tracing() or torch.compiler.is_compiling() or
+            any(probe is None or probe() for probe in _MODES))
+
+
+def _plain_cuda(t) -> bool:
+    """An ordinary float64 matrix on the current device."""
     return (type(t) is torch.Tensor and t.is_cuda and t.dtype == torch.float64 and t.dim() == 2 and t.numel() > 0 and
-            t.is_contiguous() and t.device.index == torch.cuda.current_device() and
-            not torch._C._functorch.is_functorch_wrapped_tensor(t) and
+            t.is_contiguous() and not t.is_neg() and t.device.index == torch.cuda.current_device() and
             torch.autograd.forward_ad.unpack_dual(t).tangent is None)
+
+
+def _fusable(D, y_cum) -> bool:
+    return (not _transformed() and _plain_cuda(D) and _plain_cuda(y_cum) and not y_cum.requires_grad and
+            D.shape == y_cum.shape and D.device == y_cum.device)
 
 
 def cumulative_mse(D: torch.Tensor, y_cum: torch.Tensor) -> torch.Tensor:
@@ -216,11 +235,11 @@ def cumulative_mse(D: torch.Tensor, y_cum: torch.Tensor) -> torch.Tensor:
 
     Float64 matrices on the GPU go through the library's fused kernel; everything else (other
     types, the CPU, a target that broadcasts or wants a gradient, vmap, forward-mode
-    differentiation, tracing) through the torch expression."""
-    if (isinstance(y_cum, torch.Tensor) and not y_cum.requires_grad and D.shape == y_cum.shape and
-            D.device == y_cum.device and not torch.jit.is_tracing() and not torch.compiler.is_compiling() and
-            torch._C._len_torch_dispatch_stack() == 0 and _plain_cuda(D) and _plain_cuda(y_cum)):
-        return _CumulativeMse.apply(D, y_cum)
+    differentiation, tracing and scripting) through the torch expression.  Neither keeps an
+    operand for its backward: both may be written again before it runs."""
+    if not torch.jit.is_scripting():
+        if _fusable(D, y_cum):
+            return _CumulativeMse.apply(D, y_cum)[0]
     return ((torch.cumsum(D, dim=-1) - y_cum) ** 2).mean()
 
 

@@ -558,7 +558,7 @@ def gabm_cumulative_mse(D, y):
     st = load_library().gabm_cumulative_mse(_ptr(D, np.float64), _ptr(y, np.float64), I, T, _ptr(loss), _ptr(gD),
                                             ctypes.c_void_p(torch.cuda.current_stream(D.device).cuda_stream))
     _check(st, None)
-    return loss[0], gD
+    return loss.resize_(()), gD   # the mean, in a tensor of its own (a view could not be written in place by callers)
 
 
 def gabm_destroy(ctx: GabmCtx):
