@@ -551,6 +551,8 @@ def gabm_cumulative_mse(D, y):
     """MSE of the running sums of D [I, T] against y [I, T] (float64 CUDA tensors) and its
     gradient with respect to D; returns (loss, a 0-d tensor, and gD [I, T])."""
     import torch
+    if _space(D, y) != GABM_DEVICE or D.device != y.device:
+        raise ValueError("D and y must be CUDA tensors on one device")
     I, T = D.shape
     _shape(y, (I, T), "y")
     loss = torch.empty(1 + I, dtype=torch.float64, device=D.device)
