@@ -27,14 +27,7 @@ class GabmFunction(torch.autograd.Function):
 
     @staticmethod
     def backward(fctx, gD):
-        gD = gD.detach().to(torch.float64).contiguous()
-        (I, T), A = gD.shape, capi.GABM_NUM_AGES
-        # one buffer, so that one conversion serves the three gradients
-        flat = torch.empty(I * (2 * T + A), dtype=torch.float64, device=gD.device)
-        dR, dm, dS = flat.split((I * T, I * T, I * A))
-        capi.gabm_backward(fctx.handle, gD, dR.view(I, T), dm.view(I, T), dS.view(I, A))
-        if len(set(fctx.dtypes)) == 1:
-            dR, dm, dS = flat.to(fctx.dtypes[0]).split((I * T, I * T, I * A))
-        else:
-            dR, dm, dS = (x.to(t) for x, t in zip((dR, dm, dS), fctx.dtypes))
-        return None, dR.view(I, T), dm.view(I, T), dS.view(I, A), None
+        # tensors of their own, each: as views of one buffer, writing one in place would count as
+        # a change of the others, and keeping one would keep all three
+        dR, dm, dS = capi.gabm_backward(fctx.handle, gD.detach().to(torch.float64).contiguous())
+        return None, dR.to(fctx.dtypes[0]), dm.to(fctx.dtypes[1]), dS.to(fctx.dtypes[2]), None
