@@ -129,6 +129,7 @@ struct gabm_ctx {
     int T_last = -1;
     int lam_from = -1;
     int bits_from = -1;             // first day whose infectious bitmap the last forward wrote
+    bool seeds_captured = false;     // the caller captured a seeding: its replays change d_nseed unseen
 
     double mean_len = 0, near_share = 0;   // entries per agent; those within kNearRows of their row
     bool deep = false;              // the reverse sweep's deep instances (deep_gather)
@@ -1320,9 +1321,16 @@ gabm_status forward_prologue(gabm_ctx *c, bool seeding, cudaStream_t s) {
 // Forward over days t0..T-1 from the staged parameters, seeding the state (from last_seeds)
 // when `seeding`.
 gabm_status forward_core(gabm_ctx *c, int t0, int T, bool seeding) {
-    if (seeding && c->seeds_on_device != c->last_seeds) {
-        CK(cudaMemcpyAsync(c->d_nseed, c->last_seeds.data(), sizeof(int32_t) * c->I, cudaMemcpyHostToDevice, c->stream));
-        c->seeds_on_device = c->last_seeds;
+    if (seeding) {
+        cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+        CK(cudaStreamIsCapturing(c->stream, &capture));
+        c->seeds_captured |= capture != cudaStreamCaptureStatusNone;
+        if (c->seeds_captured || c->seeds_on_device != c->last_seeds) {
+            c->seeds_on_device.clear();   // unknown until every launch has gone out
+            for (int i0 = 0; i0 < c->I; i0 += kSeedArgs)
+                LAUNCH(launch_set_seeds(c->last_seeds.data() + i0, std::min(kSeedArgs, c->I - i0), c->d_nseed + i0, c->stream));
+            c->seeds_on_device = c->last_seeds;
+        }
     }
     return run_day_loop(c, kLoopForward, t0, T, seeding);
 }

@@ -20,6 +20,7 @@
 #include "rowsum.cuh"
 
 #include <algorithm>
+#include <cstring>
 
 namespace gabm {
 
@@ -561,6 +562,13 @@ __global__ void k_stage(const float *R, const float *m, const float *S, float *R
         S_ctx[idx] = S[idx];
 }
 
+struct SeedCounts {
+    int32_t n[kSeedArgs];
+};
+__global__ void k_set_seeds(const SeedCounts v, int n, int32_t *out) {
+    for (int i = threadIdx.x; i < n; i += blockDim.x) out[i] = v.n[i];
+}
+
 // MSE on cumulative deaths (Sec. 3.2, Stage 3) over I instances and T days in FP64, one block
 // per instance: with C_t = sum of D up to t, out[1 + i] = sum_t (C_t - y_t)^2 and
 // gD_t = 2 / (I T) sum_{s >= t} (C_s - y_s).  The days go in pieces of one a thread, a scan
@@ -771,6 +779,14 @@ cudaError_t launch_stage(const float *R, const float *m, const float *S, float *
                          int I, int T, int ldP, cudaStream_t s) {
     const int64_t n = std::max<int64_t>((int64_t)I * T, (int64_t)I * kAges);
     k_stage<<<(int)std::min<int64_t>((n + 255) / 256, 1024), 256, 0, s>>>(R, m, S, R_ctx, m_ctx, S_ctx, I, T, ldP);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_set_seeds(const int32_t *n_seed, int n, int32_t *n_seed_dev, cudaStream_t s) {
+    if (n < 1 || n > kSeedArgs) return cudaErrorInvalidValue;
+    SeedCounts v;
+    memcpy(v.n, n_seed, sizeof(int32_t) * (size_t)n);
+    k_set_seeds<<<1, 256, 0, s>>>(v, n, n_seed_dev);
     return cudaGetLastError();
 }
 

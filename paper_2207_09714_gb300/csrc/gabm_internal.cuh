@@ -484,6 +484,11 @@ cudaError_t launch_seed_mark(const SeedArgs &a, int I, int grid_x, cudaStream_t 
 // R, m [I][T] and S [I][9] into the ctx's arrays (stride ldP), device memory.
 cudaError_t launch_stage(const float *R, const float *m, const float *S, float *R_ctx, float *m_ctx, float *S_ctx,
                          int I, int T, int ldP, cudaStream_t s);
+// n <= kSeedArgs instances' seed counts (host) into the ctx's, as the stream reaches it.  By value in
+// the launch: an asynchronous copy may read the host's array after the next call has changed it, and
+// a captured one would bring whatever it holds when the graph is replayed.
+constexpr int kSeedArgs = 4000;
+cudaError_t launch_set_seeds(const int32_t *n_seed, int n, int32_t *n_seed_dev, cudaStream_t s);
 cudaError_t launch_cumulative_mse(const double *D, const double *y, int I, int T, double *out, double *gD,
                                   cudaStream_t s);
 // overlap: the launch before it in the stream is a day kernel of the same loop (see pdl_wait).
