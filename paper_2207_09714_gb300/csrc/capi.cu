@@ -2364,9 +2364,8 @@ gabm_status gabm_set_infectiousness(gabm_ctx *ctx, const float *c_in) {
     for (int k = 0; k < c->L; ++k) c->c[k] = c_in[k];
     // ordered behind the launches that read the old table; captured loops read the table from
     // here (carried by value, each change cost both loops' capture: a step of a calibration
-    // that learns the table took 2.4 ms on 100k agents, of which the GPU worked 1.3).  By value in
-    // the launch, since an asynchronous copy may read the host's array after the next change of it.
-    LAUNCH(launch_set_table(c->c, c->c_dev, c->stream));
+    // that learns the table took 2.4 ms on 100k agents, of which the GPU worked 1.3)
+    CK(cudaMemcpyAsync(c->c_dev, c->c, sizeof(float) * kMaxL, cudaMemcpyHostToDevice, c->stream));
     c->T_last = -1;                                // the last trajectory used the old table
     return GABM_OK;
 }
@@ -2402,10 +2401,6 @@ gabm_status gabm_autotune(gabm_ctx *ctx, int repetitions) {
     if (c->T_last < 1 || !c->last_from_seeding)
         return fail(c, GABM_ESTATE, "autotune needs a preceding forward that started from seeding");
     const int T = c->T_last, ld = c->Tcap;
-    // the ctx would hold this table at once, the device only when the captured graph is replayed
-    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-    CK(cudaStreamIsCapturing(c->stream, &capture));
-    if (capture != cudaStreamCaptureStatusNone) return fail(c, GABM_ECUDA, "the ctx stream is being captured");
     cudaStream_t s = c->stream;
     if (!c->gD_staged) CK(cudaMemsetAsync(c->gD, 0, sizeof(double) * (size_t)c->I * ld, s));
     gabm_schedule cur{};

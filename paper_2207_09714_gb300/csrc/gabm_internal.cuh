@@ -495,8 +495,6 @@ cudaError_t launch_cumulative_mse(const double *D, const double *y, int I, int T
 // small: the base model's instance for graphs of at most kSmallTiles tiles an SM (a tile a
 // warp): blocks of two warps spread over the chip, registers for most of a row in flight
 // (10k agents x 30 days forward: 173 us against 204).
-// The infectiousness table (host, [kMaxL]) into the ctx's, as the stream reaches it.
-cudaError_t launch_set_table(const float *c, float *c_dev, cudaStream_t s);
 cudaError_t launch_fwd_day(const FwdDayArgs &a, int grid, bool smem_bits, bool small, bool overlap, cudaStream_t s);
 // Flags for day t of the rows with an in-neighbour infectious on day t (bits_t): every
 // out-neighbour of a marked row gets flag 1.  flags must be zero on entry.
