@@ -2361,11 +2361,16 @@ gabm_status gabm_set_infectiousness(gabm_ctx *ctx, const float *c_in) {
     if (c_in[0] != 0.0f) return fail(c, GABM_EINVAL, "c[0] must be 0 (no onward infection on the day of exposure)");
     for (int k = 0; k < c->L; ++k)
         if (!std::isfinite(c_in[k]) || c_in[k] < 0.0f) return fail(c, GABM_EINVAL, "c[%d] must be finite and >= 0", k);
+    // the ctx would hold this table at once, the device only when the captured graph is replayed
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    CK(cudaStreamIsCapturing(c->stream, &capture));
+    if (capture != cudaStreamCaptureStatusNone) return fail(c, GABM_ECUDA, "the ctx stream is being captured");
     for (int k = 0; k < c->L; ++k) c->c[k] = c_in[k];
     // ordered behind the launches that read the old table; captured loops read the table from
     // here (carried by value, each change cost both loops' capture: a step of a calibration
-    // that learns the table took 2.4 ms on 100k agents, of which the GPU worked 1.3)
-    CK(cudaMemcpyAsync(c->c_dev, c->c, sizeof(float) * kMaxL, cudaMemcpyHostToDevice, c->stream));
+    // that learns the table took 2.4 ms on 100k agents, of which the GPU worked 1.3).  By value in
+    // the launch, since an asynchronous copy may read the host's array after the next change of it.
+    LAUNCH(launch_set_table(c->c, c->c_dev, c->stream));
     c->T_last = -1;                                // the last trajectory used the old table
     return GABM_OK;
 }

@@ -569,6 +569,11 @@ __global__ void k_set_seeds(const SeedCounts v, int n, int32_t *out) {
     for (int i = threadIdx.x; i < n; i += blockDim.x) out[i] = v.n[i];
 }
 
+struct TableArg {
+    float c[kMaxL];
+};
+__global__ void k_set_table(const TableArg t, float *c) { c[threadIdx.x] = t.c[threadIdx.x]; }
+
 // MSE on cumulative deaths (Sec. 3.2, Stage 3) over I instances and T days in FP64, one block
 // per instance: with C_t = sum of D up to t, out[1 + i] = sum_t (C_t - y_t)^2 and
 // gD_t = 2 / (I T) sum_{s >= t} (C_s - y_s).  The days go in pieces of one a thread, a scan
@@ -787,6 +792,13 @@ cudaError_t launch_set_seeds(const int32_t *n_seed, int n, int32_t *n_seed_dev, 
     SeedCounts v;
     memcpy(v.n, n_seed, sizeof(int32_t) * (size_t)n);
     k_set_seeds<<<1, 256, 0, s>>>(v, n, n_seed_dev);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_set_table(const float *c, float *c_dev, cudaStream_t s) {
+    TableArg t;
+    for (int k = 0; k < kMaxL; ++k) t.c[k] = c[k];
+    k_set_table<<<1, kMaxL, 0, s>>>(t, c_dev);
     return cudaGetLastError();
 }
 

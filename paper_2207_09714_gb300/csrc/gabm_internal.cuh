@@ -489,6 +489,8 @@ cudaError_t launch_stage(const float *R, const float *m, const float *S, float *
 // a captured one would bring whatever it holds when the graph is replayed.
 constexpr int kSeedArgs = 4000;
 cudaError_t launch_set_seeds(const int32_t *n_seed, int n, int32_t *n_seed_dev, cudaStream_t s);
+// The infectiousness table (host, [kMaxL]) into the ctx's, as the stream reaches it.
+cudaError_t launch_set_table(const float *c, float *c_dev, cudaStream_t s);
 cudaError_t launch_cumulative_mse(const double *D, const double *y, int I, int T, double *out, double *gD,
                                   cudaStream_t s);
 // overlap: the launch before it in the stream is a day kernel of the same loop (see pdl_wait).

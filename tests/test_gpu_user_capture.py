@@ -1,5 +1,6 @@
 """A caller that captures the ctx stream (day loops launched one by one, GABM_CUDA_GRAPHS=0): a
-captured forward leaves the eager ones right before and after it is replayed."""
+captured forward leaves the eager ones right before and after it is replayed, and a table
+is not exchanged inside a capture."""
 import numpy as np
 import pytest
 import torch
@@ -50,3 +51,43 @@ def test_eager_forward_after_a_captured_one(setting):
     torch.cuda.synchronize()
     assert np.array_equal(capi.gabm_get_state(ctx), want[25])
     assert np.array_equal(run(ctx, 10), want[10])   # nor do the seeds of the replay stay
+
+
+def test_no_table_is_set_inside_a_capture(setting):
+    make, run, dev, stream = setting
+    ctx = make()
+    want = run(ctx, 10)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=stream):
+        D = dev[0] + 1.0
+        with pytest.raises(capi.GabmError):
+            capi.gabm_set_infectiousness(ctx, synth.infectiousness_table(T_E=0.2, T_I=1.3))
+    assert np.array_equal(run(ctx, 10), want)
+    graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(D, dev[0] + 1.0)
+
+
+def test_seeds_and_tables_of_forwards_still_queued(setting):
+    """Calls that return before the stream has reached them keep the values they were given."""
+    make, run, dev, stream = setting
+    tables = [synth.infectiousness_table(T_E=e, T_I=1.3) for e in (0.2, 0.9)]
+    want = []
+    for k, c in enumerate(tables):
+        ctx = make()
+        capi.gabm_set_infectiousness(ctx, c)
+        want.append(run(ctx, 10 + k))
+    ctx = make()
+    with torch.cuda.stream(stream):
+        busy = torch.rand((4096, 4096), device="cuda")
+        got = []
+        for _ in range(8):
+            for k, c in enumerate(tables):
+                for _ in range(4):
+                    busy = busy @ busy / 2048.0
+                capi.gabm_set_infectiousness(ctx, c)
+                capi.gabm_forward(ctx, T, *dev, [10 + k])
+                got.append(capi.gabm_get_state(ctx, device=True))
+    stream.synchronize()
+    for i, e in enumerate(got):
+        assert np.array_equal(e.cpu().numpy(), want[i % 2])
