@@ -295,15 +295,16 @@ __global__ void k_counts_b(const int32_t *H, const int32_t *newinf, const int32_
     }
 }
 
-// Level 1 of the parameter-gradient reduction: Pc[t][g][c][a][s] = sum over the
-// tiles [c K, min((c+1) K, ntiles_g)) of graph g of P[t][tile][a][s], K = kReduceChunkTiles.
+// Level 1 of the parameter-gradient reduction of the days [t0, t0 + gridDim.y), whose sums
+// are P's days 0, 1, ...: Pc[t][g][c][a][s] = sum over the units [c K, min((c+1) K, nu_g))
+// of graph g of P[t - t0][unit][a][s], K = kReduceChunkTiles.
 __global__ void k_reduce_b1(const float *P, int nunits, const int32_t *unit0, const int32_t *nu, int G, int Bp,
-                            int max_chunks, double *Pc) {
-    const int c = blockIdx.x, t = blockIdx.y, g = blockIdx.z;
+                            int t0, int max_chunks, double *Pc) {
+    const int c = blockIdx.x, d = blockIdx.y, g = blockIdx.z;
     const int wdt = kAges * Bp;
     const int nt = nu[g];
     const int i0 = c * kReduceChunkTiles, i1 = min(nt, i0 + kReduceChunkTiles);
-    const float *base = P + ((size_t)t * nunits + unit0[g]) * wdt;
+    const float *base = P + ((size_t)d * nunits + unit0[g]) * wdt;
     for (int k = threadIdx.x; k < wdt; k += blockDim.x) {
         double acc = 0.0;
         int i = i0;
@@ -315,7 +316,7 @@ __global__ void k_reduce_b1(const float *P, int nunits, const int32_t *unit0, co
             for (int u = 0; u < 4; ++u) acc += (double)v[u];
         }
         for (; i < i1; ++i) acc += (double)base[(size_t)i * wdt + k];
-        Pc[(((size_t)t * G + g) * max_chunks + c) * wdt + k] = acc;
+        Pc[(((size_t)(t0 + d) * G + g) * max_chunks + c) * wdt + k] = acc;
     }
 }
 
@@ -442,15 +443,18 @@ cudaError_t launch_counts_b(const uint8_t *unit_new, int nunits, const int32_t *
     return cudaGetLastError();
 }
 
-cudaError_t launch_bwd_reduce_b(const float *P, int nunits, const int32_t *d_tile0, const int32_t *d_ntiles, int G,
-                                int B, int Bp, int T, double *scratch, int max_chunks, const int32_t *sig,
-                                int ld_sig, double *Q, cudaStream_t s) {
-    const int wdt = kAges * Bp;
-    const int threads = std::min(1024, (wdt + 31) / 32 * 32);
-    k_reduce_b1<<<dim3(max_chunks, T, G), threads, 0, s>>>(P, nunits, d_tile0, d_ntiles, G, Bp, max_chunks, scratch);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    k_reduce_b2<<<dim3(T, G), threads, 0, s>>>(scratch, G, B, Bp, T, max_chunks, sig, ld_sig, Q);
+static int reduce_threads(int Bp) { return std::min(1024, (kAges * Bp + 31) / 32 * 32); }
+
+cudaError_t launch_reduce_units_b(const float *P, int nunits, const int32_t *d_unit0, const int32_t *d_nunits, int G,
+                                  int Bp, int t0, int days, int max_chunks, double *Pc, cudaStream_t s) {
+    k_reduce_b1<<<dim3(max_chunks, days, G), reduce_threads(Bp), 0, s>>>(P, nunits, d_unit0, d_nunits, G, Bp, t0,
+                                                                        max_chunks, Pc);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_reduce_chunks_b(const double *Pc, int G, int B, int Bp, int T, int max_chunks, const int32_t *sig,
+                                   int ld_sig, double *Q, cudaStream_t s) {
+    k_reduce_b2<<<dim3(T, G), reduce_threads(Bp), 0, s>>>(Pc, G, B, Bp, T, max_chunks, sig, ld_sig, Q);
     return cudaGetLastError();
 }
 

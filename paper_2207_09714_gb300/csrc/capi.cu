@@ -104,7 +104,8 @@ struct gabm_ctx {
     float *lam = nullptr;
     int32_t *counts = nullptr, *newRM = nullptr, *newRM_b = nullptr;
     double *D = nullptr, *gD = nullptr, *y = nullptr, *Q = nullptr, *Qp = nullptr;   // Qp [Tcap][I][kReduceParts][9] (one set per graph)
-    float *P = nullptr;
+    float *P = nullptr;             // [Tcap][ntiles][9], batched [P_days][nunits][9][Bp]
+    int P_days = 0;                 // batched: days the sweep keeps before it adds them up (ensure_days)
     float *R = nullptr, *m = nullptr, *S = nullptr;
     double *dR_s = nullptr, *dm_s = nullptr, *dS_s = nullptr, *loss_s = nullptr;
     double *dc_tile = nullptr;      // [ntiles][kMaxL] table-adjoint accumulators (on request)
@@ -627,7 +628,12 @@ gabm_status ensure_days(gabm_ctx *c, int T) {
     TRY(dalloc(c, &c->D, IT));
     TRY(dalloc(c, &c->gD, IT));
     TRY(dalloc(c, &c->y, IT));
-    TRY(dalloc(c, &c->P, (size_t)cap * (c->batched ? c->nunits : c->ntiles) * kAges * c->Bp));
+    // Sums of parts of tiles are added up some days at a time (with quarters 3/8 of the days, with
+    // halves 3/4), so that they, the chunks' sums, unit_new and the table's accumulators take no
+    // more together than whole tiles' sums of all days in FP64 did; the quarters' of all
+    // days would take twice that.
+    c->P_days = c->batched ? std::min(cap, cap * 3 * c->ru / (2 * kTile)) : cap;
+    TRY(dalloc(c, &c->P, (size_t)c->P_days * (c->batched ? c->nunits : c->ntiles) * kAges * c->Bp));
     if (!c->batched) TRY(dalloc(c, &c->Qp, IT * kAges * kReduceParts));
     if (c->fate) TRY(dalloc(c, &c->Pm, (size_t)cap * c->ntiles));
     if (c->soft) {
@@ -881,7 +887,8 @@ gabm_status backward_days_batched(gabm_ctx *c, int T, cudaStream_t s) {
         a.r_next = c->r + (size_t)((t + 1) & 1) * nb;
         a.r_cur = c->r + (size_t)(t & 1) * nb;
 
-        a.P_t = c->P + (size_t)t * c->nunits * kAges * c->Bp;
+        const int t0 = std::max(0, T - ((T - 1 - t) / c->P_days + 1) * c->P_days);   // P holds the days from here
+        a.P_t = c->P + (size_t)(t - t0) * c->nunits * kAges * c->Bp;
         for (int k = 0; k < kMaxL; ++k) a.ring_slot[k] = (k >= 1 && k < c->L) ? (t + k) % Lm1 : 0;
         prof_begin(c, 1);
         for (int ch = 0; ch < nch; ++ch) {   // the row's sets in launches of bwd_chunk sets
@@ -890,12 +897,14 @@ gabm_status backward_days_batched(gabm_ctx *c, int T, cudaStream_t s) {
             LAUNCH(launch_bwd_day_b(a, c->bwd_chunk, c->spl_bwd, c->kahan_b, c->grid_bwd, s));
         }
         prof_end(c, 1);
+        if (t == t0)
+            LAUNCH(launch_reduce_units_b(c->P, c->nunits, c->d_unit0, c->d_nunits, c->G, c->Bp, t0,
+                                         (T - 1 - t) % c->P_days + 1, c->max_chunks, c->Pc, s));
     }
+    LAUNCH(launch_reduce_chunks_b(c->Pc, c->G, c->B, c->Bp, T, c->max_chunks, c->sig, ld + 1, c->Q, s));
     if (a.dc_tile)   // the seeds' share through day 0 (r of day 0 is in slot 0)
         LAUNCH(launch_dc_seeds_b(csr_view(c, true), c->e, c->r, graph_ref(c), c->sig, ld + 1, c->nunits,
                                  c->ru, c->L, c->B, c->Bp, c->dc_tile, s));
-    LAUNCH(launch_bwd_reduce_b(c->P, c->nunits, c->d_unit0, c->d_nunits, c->G, c->B, c->Bp, T, c->Pc, c->max_chunks,
-                               c->sig, ld + 1, c->Q, s));
     return GABM_OK;
 }
 

@@ -381,11 +381,13 @@ cudaError_t launch_counts_b(const uint8_t *unit_new, int nunits, const int32_t *
                             const int32_t *d_rows, int G, int B, int Bp, int max_units, int t0, int T, int ldP,
                             int tau_EI, int L, const int32_t *H, int32_t *newinf, int32_t *counts, int32_t *newRM,
                             cudaStream_t s);
-// Q[g*B+s][t][a] = sum over graph g's tiles of P[t][tile][a][s], in a fixed order (two levels of
-// kReduceChunkTiles tiles); scratch holds T * G * max_chunks * 9 * Bp doubles.
-cudaError_t launch_bwd_reduce_b(const float *P, int nunits, const int32_t *d_tile0, const int32_t *d_ntiles, int G,
-                                int B, int Bp, int T, double *scratch, int max_chunks, const int32_t *sig,
-                                int ld_sig, double *Q, cudaStream_t s);
+// Q[g*B+s][t][a] = the sum over graph g's units of their P[unit][a][s] of day t, in a fixed order of
+// two levels: kReduceChunkTiles units each into Pc [T][G][max_chunks][9][Bp], from P holding
+// the days [t0, t0 + days), then the chunks of all T days.
+cudaError_t launch_reduce_units_b(const float *P, int nunits, const int32_t *d_unit0, const int32_t *d_nunits, int G,
+                                  int Bp, int t0, int days, int max_chunks, double *Pc, cudaStream_t s);
+cudaError_t launch_reduce_chunks_b(const double *Pc, int G, int B, int Bp, int T, int max_chunks, const int32_t *sig,
+                                   int ld_sig, double *Q, cudaStream_t s);
 constexpr int kReduceChunkTiles = 64;
 
 // ---------------------------------------------------------------------------
