@@ -549,7 +549,7 @@ __global__ void __launch_bounds__(256) k_dc_reduce(const double *dc_tile, const 
     if (threadIdx.x == 0) dc[(size_t)g * L + k] = s[0];
 }
 
-// parts[t][inst][c][a] = sum over the c-th of kReduceParts shares of the graph's tiles of
+// parts[t][inst][c][a] = sum over the c-th of gridDim.z shares of the graph's tiles of
 // P[t][tile][a], fixed order, FP64.  The shares' elements are taken in a row by kReduceBlock
 // threads, a multiple of nine, so a thread keeps one age bin and the loads are coalesced; one
 // block of 256 threads a day with nine accumulators each took 130 us on the 1M-agent graph.
@@ -559,7 +559,7 @@ __global__ void __launch_bounds__(kReduceBlock) k_bwd_reduce(const float *P, int
     __shared__ double s[kReduceBlock];
     const int t = blockIdx.x, inst = blockIdx.y, c = blockIdx.z, tid = threadIdx.x;
     const int tile0 = graph_tile0[inst], nt = graph_ntiles[inst];
-    const int i0 = (int)((long long)nt * c / kReduceParts), i1 = (int)((long long)nt * (c + 1) / kReduceParts);
+    const int np = gridDim.z, i0 = (int)((long long)nt * c / np), i1 = (int)((long long)nt * (c + 1) / np);
     const float *p = P + ((size_t)t * ntiles + tile0 + i0) * kAges;
     const int n = (i1 - i0) * kAges;
     double acc = 0.0;
@@ -577,17 +577,17 @@ __global__ void __launch_bounds__(kReduceBlock) k_bwd_reduce(const float *P, int
     if (tid < kAges) {   // 56 values of bin tid, in order
         double v = 0.0;
         for (int k = 0; k < kReduceBlock / kAges; ++k) v += s[k * kAges + tid];
-        parts[(((size_t)t * gridDim.y + inst) * kReduceParts + c) * kAges + tid] = v;
+        parts[(((size_t)t * gridDim.y + inst) * np + c) * kAges + tid] = v;
     }
 }
 
-// Q[inst][t][a] = 2^sigma(t) x the sum of the shares, in order.
-__global__ void k_bwd_reduce_parts(const double *parts, int T, int I, const int32_t *sig, int ld_sig, double *Q) {
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= T * I * kAges) return;
-    const int a = idx % kAges, ti = idx / kAges, inst = ti % I, t = ti / I;
+// Q[inst][t][a] = 2^sigma(t) x the sum of the np shares, in order.
+__global__ void k_bwd_reduce_parts(const double *parts, int np, int T, const int32_t *sig, int ld_sig, double *Q) {
+    const int t = blockIdx.x, inst = blockIdx.y, a = threadIdx.x;
+    if (a >= kAges) return;
+    const double *p = parts + ((size_t)t * gridDim.y + inst) * np * kAges + a;
     double v = 0.0;
-    for (int c = 0; c < kReduceParts; ++c) v += parts[((size_t)ti * kReduceParts + c) * kAges + a];
+    for (int c = 0; c < np; ++c) v += p[c * kAges];
     Q[((size_t)inst * T + t) * kAges + a] = ldexp(v, sig[(size_t)inst * ld_sig + t]);
 }
 
@@ -691,9 +691,10 @@ int occupancy_bwd(int mode, bool dc, int exit_mode, bool deep) {
 }
 
 cudaError_t launch_bwd_reduce(const float *P, int ntiles, const int32_t *graph_tile0, const int32_t *graph_ntiles,
-                              int T, int I, const int32_t *sig, int ld_sig, double *parts, double *Q, cudaStream_t s) {
-    k_bwd_reduce<<<dim3(T, I, kReduceParts), kReduceBlock, 0, s>>>(P, ntiles, graph_tile0, graph_ntiles, parts);
-    k_bwd_reduce_parts<<<(T * I * kAges + 255) / 256, 256, 0, s>>>(parts, T, I, sig, ld_sig, Q);
+                              int T, int I, const int32_t *sig, int ld_sig, double *parts, int np, double *Q,
+                              cudaStream_t s) {
+    k_bwd_reduce<<<dim3(T, I, np), kReduceBlock, 0, s>>>(P, ntiles, graph_tile0, graph_ntiles, parts);
+    k_bwd_reduce_parts<<<dim3(T, I), 32, 0, s>>>(parts, np, T, sig, ld_sig, Q);
     return cudaGetLastError();
 }
 

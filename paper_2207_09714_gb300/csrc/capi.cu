@@ -103,7 +103,8 @@ struct gabm_ctx {
     int Tcap = 0;
     float *lam = nullptr;
     int32_t *counts = nullptr, *newRM = nullptr, *newRM_b = nullptr;
-    double *D = nullptr, *gD = nullptr, *y = nullptr, *Q = nullptr, *Qp = nullptr;   // Qp [Tcap][I][kReduceParts][9] (one set per graph)
+    double *D = nullptr, *gD = nullptr, *y = nullptr, *Q = nullptr, *Qp = nullptr;   // Qp [Tcap][I][reduce_parts][9] (one set per graph)
+    int reduce_parts = 1;
     float *P = nullptr;             // [Tcap][ntiles][9], batched [P_days][nunits][9][Bp]
     int P_days = 0;                 // batched: days the sweep keeps before it adds them up (ensure_days)
     float *R = nullptr, *m = nullptr, *S = nullptr;
@@ -634,7 +635,10 @@ gabm_status ensure_days(gabm_ctx *c, int T) {
     // days would take twice that.
     c->P_days = c->batched ? std::min(cap, cap * 3 * c->ru / (2 * kTile)) : cap;
     TRY(dalloc(c, &c->P, (size_t)c->P_days * (c->batched ? c->nunits : c->ntiles) * kAges * c->Bp));
-    if (!c->batched) TRY(dalloc(c, &c->Qp, IT * kAges * kReduceParts));
+    // at most a share per two tiles, on average: Qp then takes no more than P (or, with one share,
+    // 72 bytes an instance and day), however many graphs of a tile or two there are
+    c->reduce_parts = std::max(1, std::min(kReduceParts, c->ntiles / (2 * c->I)));
+    if (!c->batched) TRY(dalloc(c, &c->Qp, IT * kAges * c->reduce_parts));
     if (c->fate) TRY(dalloc(c, &c->Pm, (size_t)cap * c->ntiles));
     if (c->soft) {
         TRY(dalloc(c, &c->s_hist, (size_t)cap * c->n_rows));
@@ -1002,7 +1006,8 @@ gabm_status backward_days_sirs(gabm_ctx *c, int T, cudaStream_t s) {
         LAUNCH(launch_bwd_day_sirs(a, c->grid_sirs_b, c->overlap && t < T - 1, s));
         prof_end(c, 1);
     }
-    LAUNCH(launch_bwd_reduce(c->P, c->ntiles, c->d_tile0, c->d_ntiles, T, c->I, c->sig, ld + 1, c->Qp, c->Q, s));
+    LAUNCH(launch_bwd_reduce(c->P, c->ntiles, c->d_tile0, c->d_ntiles, T, c->I, c->sig, ld + 1, c->Qp,
+                             c->reduce_parts, c->Q, s));
     return GABM_OK;
 }
 
@@ -1194,7 +1199,8 @@ gabm_status backward_days_plain(gabm_ctx *c, int T, cudaStream_t s) {
         LAUNCH(launch_dc_seeds(sell_view(c, true), c->e, r0, graph_ref(c), c->sig, ld + 1, c->ntiles, c->L,
                                long_gx_buf(c), c->dc_tile, c->grid_bwd, s));
     }
-    LAUNCH(launch_bwd_reduce(c->P, c->ntiles, c->d_tile0, c->d_ntiles, T, c->I, c->sig, ld + 1, c->Qp, c->Q, s));
+    LAUNCH(launch_bwd_reduce(c->P, c->ntiles, c->d_tile0, c->d_ntiles, T, c->I, c->sig, ld + 1, c->Qp,
+                             c->reduce_parts, c->Q, s));
     return GABM_OK;
 }
 

@@ -554,10 +554,11 @@ int occupancy_loc();
 cudaError_t launch_lam_day(Sell m, const int16_t *E, const uint32_t *bits, GraphRef gr, int t, int L, int ntiles,
                            const float *c, const float *long_lam, float *lam_out, int grid, cudaStream_t s);
 // Q[g][t][a] = 2^sigma_g(t) x (sum over graph g's tiles of P[t][tile][a]), FP64.
-// parts: [T][I][kReduceParts][9] scratch.
+// parts: [T][I][np][9] scratch, np <= kReduceParts shares of a graph's tiles each.
 constexpr int kReduceParts = 8;
 cudaError_t launch_bwd_reduce(const float *P, int ntiles, const int32_t *graph_tile0, const int32_t *graph_ntiles,
-                              int T, int I, const int32_t *sig, int ld_sig, double *parts, double *Q, cudaStream_t s);
+                              int T, int I, const int32_t *sig, int ld_sig, double *parts, int np, double *Q,
+                              cudaStream_t s);
 // newRM_real (soft mode, [I][ldP]) replaces the integer newRM when non-null.
 cudaError_t launch_bwd_finalize(const double *Q, const float *R, const float *S, const double *gD,
                                 const int32_t *newRM, const double *newRM_real, int ldP, int T, int I, double *dR,
