@@ -3,6 +3,7 @@
 // transpose, the per-day launch sequences of the forward and the reverse
 // sweep, and the host/device staging of arguments.
 #include <algorithm>
+#include <climits>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -440,11 +441,11 @@ void sort_windows_by_degree(const HostGraph &h, std::vector<uint32_t> &order, in
     }
 }
 
-// Rows much longer than the rest (hubs of a power-law contact graph) cost a SELL tile
-// its longest row in every lane's loop.  Rows of more than kLongRow entries therefore
-// leave their degree window: they are sorted by length and put, 32 to a tile, at evenly
-// spaced window boundaries of the order, so that each such tile holds rows of similar
-// length and the heavy tiles spread over the launch's tile ranges.
+// Rows of more than kLongRow entries leave their degree window: they are sorted by length
+// and put, 32 to a tile, at evenly spaced window boundaries of the order.  On a graph of
+// shorter rows they are hubs, summed apart from the tiles (long_from): together they leave
+// no idle lanes among the other rows.  On a graph whose rows are that long anyway, a tile of
+// them holds rows of similar length, and the heavy tiles spread over the launch's tile ranges.
 constexpr uint64_t kLongRow = 128;
 
 void group_long_rows(const HostGraph &h, std::vector<uint32_t> &order, int sigma) {
@@ -487,8 +488,20 @@ struct HostSell {
     std::vector<uint2> lcw;
 };
 
+// A graph's rows of more entries than this are long ones (LongRows): more than kLongEntries, and
+// three times its mean row.  Hubs are few then (less than a third of the rows whatever the graph,
+// in practice a few in a thousand); by the first number alone a graph of 100 contacts an
+// agent had all its rows summed by a block each, day after day: 100k agents x 40 days took
+// 13.1 ms a step, 2.8 in slices.
+uint32_t long_from(int64_t n, int64_t nnz) {
+    const double mean = n > 0 ? (double)nnz / (double)n : 0.0;
+    return (uint32_t)std::max((double)kLongEntries, std::min(3.0 * mean, 2147483647.0));
+}
+
+// limit: long_from by graph, with each tile's graph; nullptr: no long rows.
 bool build_sell(const std::vector<uint32_t> &rowptr, const std::vector<uint32_t> &col, const std::vector<float> &w,
-                int64_t n_rows, HostSell &hs, bool long_rows) {
+                int64_t n_rows, HostSell &hs, const std::vector<uint32_t> *limit,
+                const std::vector<uint16_t> &tile_graph) {
     const int64_t ns = n_rows / kTile;
     hs.slice_ptr.assign((size_t)ns + 1, 0u);
     hs.row_len.assign((size_t)n_rows, 0u);
@@ -499,7 +512,7 @@ bool build_sell(const std::vector<uint32_t> &rowptr, const std::vector<uint32_t>
             const int64_t r = sl * kTile + l;
             const uint32_t len = rowptr[r + 1] - rowptr[r];
             hs.row_len[r] = len;
-            if (long_rows && len > kLongEntries) {
+            if (limit && len > (*limit)[tile_graph[sl]]) {
                 hs.row_len[r] = kLongBit | (uint32_t)hs.lrow.size();
                 hs.lrow.push_back((uint32_t)r);
                 continue;
@@ -780,17 +793,20 @@ LongArgs long_args(const gabm_ctx *c, int t) {
     a.ld_sig = c->Tcap + 1;
     a.t = t;
     a.L = c->L;
+    a.cycle = c->sirs ? c->cycle : 0;
+    a.gx_from = INT_MIN;
     a.c = c->c_dev;
     return a;
 }
 float *long_lam_buf(const gabm_ctx *c) { return c->long_sums; }
 float *long_gx_buf(const gabm_ctx *c) { return c->long_sums + c->long_cap; }
 
-// Sums of w x[j] over the long out-rows, into long_gx_buf.
-gabm_status long_gather(gabm_ctx *c, const float *x, const int32_t *rnz, int t, bool overlap, cudaStream_t s) {
+// Sums of w x[j] over the long out-rows exposed on day `from` or later, into long_gx_buf.
+gabm_status long_gather(gabm_ctx *c, const float *x, const int32_t *rnz, int t, int from, bool overlap, cudaStream_t s) {
     if (!c->long_cap) return GABM_OK;
     LongArgs a = long_args(c, t);
     a.in.n = 0;
+    a.gx_from = from;
     a.x = x;
     a.gx = long_gx_buf(c);
     a.rnz = rnz;
@@ -1002,7 +1018,7 @@ gabm_status backward_days_sirs(gabm_ctx *c, int T, cudaStream_t s) {
         for (int k = 0; k < kMaxL; ++k) a.ring_slot[k] = (k >= 1 && k < c->L) ? (t + k) % Lm1 : 0;
         a.long_gx = long_gx_buf(c);
         prof_begin(c, 1);
-        if (t < T - 1) TRY(long_gather(c, a.r_next, c->rnz, t, c->overlap, s));
+        if (t < T - 1) TRY(long_gather(c, a.r_next, c->rnz, t, INT_MIN, c->overlap, s));
         LAUNCH(launch_bwd_day_sirs(a, c->grid_sirs_b, c->overlap && t < T - 1, s));
         prof_end(c, 1);
     }
@@ -1168,6 +1184,7 @@ gabm_status backward_days_plain(gabm_ctx *c, int T, cudaStream_t s) {
         if (c->long_cap) {   // the long rows' gx(t+1), and their lambda sums when not stored
             LongArgs la = long_args(c, t);
             la.rnz = c->rnz;
+            if (!c->soft) la.gx_from = t + 2 - c->L;   // k_bwd_day's needs(), seeds included
             if (t < T - 1) {
                 la.x = a.r_next;
                 la.gx = long_gx_buf(c);
@@ -1185,7 +1202,7 @@ gabm_status backward_days_plain(gabm_ctx *c, int T, cudaStream_t s) {
         LAUNCH(launch_bwd_day(a, grid, c->small && mode == kBwdStore, c->deep, overlap, s));
         prof_end(c, 1);
     }
-    if (c->fate || a.dc_tile) TRY(long_gather(c, c->r, nullptr, 0, false, s));   // the long rows' gx(0)
+    if (c->fate || a.dc_tile) TRY(long_gather(c, c->r, nullptr, 0, 1 - c->L, false, s));   // the long rows' gx(0)
     if (c->fate)   // the fate draws of agents exposed before day 0 (r of day 0 is in slot 0)
         LAUNCH(launch_fate_seeds(sell_view(c, true), c->e, c->r, c->ring, Lm1, graph_ref(c), a.fate,
                                  c->gD, c->sig, ld + 1, c->rnz, c->ntiles, T, c->c_dev, long_gx_buf(c), c->Pm, c->grid_bwd, s));
@@ -1846,8 +1863,10 @@ gabm_status gabm_create(const gabm_graph_desc *graphs, int num_graphs, int sets_
     const bool batched = sets_per_graph > 1;
     if (batched && model->lambda_policy != GABM_STORE_LAMBDA && !symmetric)
         return fail(nullptr, GABM_EUNSUPPORTED, "sets_per_graph > 1 with GABM_RECOMPUTE needs symmetric weights in this build");
-    if (!batched && (!build_sell(h_rowptr, h_col, h_w, n_rows, sell_in, true) ||
-                     (!symmetric && !build_sell(t_rowptr, t_col, t_w, n_rows, sell_out, true))))
+    std::vector<uint32_t> limit;
+    for (const HostGraph &h : hg) limit.push_back(long_from(h.n, h.nnz));
+    if (!batched && (!build_sell(h_rowptr, h_col, h_w, n_rows, sell_in, &limit, tile_graph) ||
+                     (!symmetric && !build_sell(t_rowptr, t_col, t_w, n_rows, sell_out, &limit, tile_graph))))
         return fail(nullptr, GABM_EUNSUPPORTED, "SELL-32 layout needs >= 2^32 entries");
     uint32_t max_degree = 0;
     int64_t near = 0;
@@ -2058,8 +2077,8 @@ gabm_status gabm_create_bipartite(const gabm_bipartite_desc *graphs, int num_gra
             }
     }
     HostSell loc_sell;
-    if (!build_sell(H.h_rowptr, H.h_col, H.h_w, n_rows, H.sell_in, false) ||
-        !build_sell(lrow, lcol, lw, ns_rows, loc_sell, false))
+    if (!build_sell(H.h_rowptr, H.h_col, H.h_w, n_rows, H.sell_in, nullptr, H.tile_graph) ||
+        !build_sell(lrow, lcol, lw, ns_rows, loc_sell, nullptr, H.tile_graph))
         return fail(nullptr, GABM_EUNSUPPORTED, "SELL-32 layout needs >= 2^32 entries");
     H.t_rowptr = H.h_rowptr;
     H.t_col = H.h_col;

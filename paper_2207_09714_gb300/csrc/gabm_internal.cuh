@@ -153,12 +153,14 @@ struct Sell {
                                 // (neighbour row) and weight bits of each (0 in padding)
 };
 
-// Rows of more than kLongEntries entries (the hubs of a power-law contact graph) are kept out
-// of the SELL slices and summed by a block each, in a launch before the day kernel
-// (longrows.cu): in a slice, one lane walks its row and the whole tile waits for it -- on
-// the 300k-agent power-law graph (90 days, recompute policy) a step took 30.7 ms that way
-// and takes 8.0 (with rows of more than 32, 48 and 96 entries taken out: 13.1, 7.7 and 8.8; at
-// 48 the 1M-agent typed graph, whose longest rows hold about 50, loses 4%).  The sum of a long row is compensated per thread and over a fixed tree.
+// Rows of more than kLongEntries entries (the hubs of a power-law contact graph; on a graph of
+// long rows, those far above its mean, see long_from in capi.cu) are kept out of the SELL slices
+// and summed by a block each, in a launch before the day kernel (longrows.cu): in a slice, one
+// lane walks its row and the whole tile waits for it -- on the 300k-agent power-law graph (90
+// days, recompute policy) a step took 30.7 ms that way and 8.0 with them taken out (rows of
+// more than 32, 48 and 96 entries: 13.1, 7.7 and 8.8; at 48 the 1M-agent typed graph, whose
+// longest rows hold about 50, loses 4%).  The sum of a long row is compensated per thread and
+// over a fixed tree.
 constexpr uint32_t kLongEntries = 64;
 constexpr uint32_t kLongBit = 0x80000000u;
 struct LongRows {
@@ -169,9 +171,12 @@ struct LongRows {
 };
 
 // One launch over a ctx's long rows.  Each part runs when its output is given:
-// lam[i] = sum over in-row i of w c[t - e_j] over the neighbours marked in bits (marked_sum);
-// gx[i] = sum over out-row i of w x[j], 0 when rnz says that day t + 1 carries no adjoint;
+// lam[i] = sum over in-row i of w c[t - e_j] over the neighbours marked in bits (marked_sum), for
+// rows susceptible on day t: not exposed before it, or `cycle` days past it (0: none returns);
+// gx[i] = sum over out-row i of w x[j] for rows with e >= gx_from, 0 when rnz says that day t + 1
+// carries no adjoint;
 // flags: out-neighbours of the out-rows marked in bits get flag 1.
+// The other rows' sums are left as they are: the day kernels do not use them.
 struct LongArgs {
     LongRows in, out;
     const uint32_t *bits;
@@ -181,7 +186,7 @@ struct LongArgs {
     uint8_t *flags;
     const int32_t *rnz;       // [G][ld_sig] or nullptr: gather always
     const uint16_t *tile_graph;
-    int ld_sig, t, L;
+    int ld_sig, t, L, cycle, gx_from;
     const float *c;           // device table [kMaxL]
 };
 cudaError_t launch_long(const LongArgs &a, bool overlap, cudaStream_t s);

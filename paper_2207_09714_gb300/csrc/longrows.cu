@@ -38,6 +38,8 @@ __global__ void __launch_bounds__(kLongBlock) k_long(LongArgs a) {
     if (!in && a.flags && marked(a.bits, row))
         for (uint32_t p = p0 + threadIdx.x; p < p1; p += kLongBlock) a.flags[lr.cw[p].x] = 1;
     if (in ? !a.lam : !a.gx) return;
+    const int er = a.e[row];
+    if (in ? er < a.t && !(a.cycle > 0 && a.t - er >= a.cycle) : er < a.gx_from) return;
     const int g = a.tile_graph ? (int)a.tile_graph[row / kTile] : 0;
     const bool dead = !in && a.rnz && a.rnz[(size_t)g * a.ld_sig + a.t + 1] == 0;
     float s = 0.f, c = 0.f;
