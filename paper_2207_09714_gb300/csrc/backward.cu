@@ -233,15 +233,21 @@ __global__ void __launch_bounds__(NT, MINB)
         {
             const TileSpan sp = tile_span(a.m, cur.p0, cur.len, needA || dc_row, lane);
             if (!have) load_pairs(sp.row, 0u, sp.lim, ea);
-            gx_mine = gather_sum(sp, a.r_next, ea);
+            if constexpr (MODE == kBwdFused) {   // lambda from the final exposure days, the forward's sum
+                if (gather) {                    // rows susceptible today are among those that gather
+                    gx_mine = gather_and_exposed_sum(sp, a.r_next, isS, E, c_s, t, L, ea, Lam);
+                } else {
+                    gx_mine = 0.f;
+                    Lam = exposed_sum<2>(a.m, cur.p0, cur.len, isS, lane, E, c_s, t, L);
+                }
+                if (cur.len & kLongBit) Lam = a.long_lam[cur.len & ~kLongBit];
+                Lam *= inv_D;
+            } else {
+                gx_mine = gather_sum(sp, a.r_next, ea);
+            }
         }
         if ((cur.len & kLongBit) && gather) gx_mine = a.long_gx[cur.len & ~kLongBit];
         if (a.self_q && gather) gx_mine = __fmaf_rn(-a.self_q[row], a.self_r[row], gx_mine);
-        if constexpr (MODE == kBwdFused) {   // lambda from the final exposure days, the forward's sum
-            Lam = marked_sum<2>(a.m, cur.p0, cur.len, isS, lane, a.bits_t, E, c_s, t, L);
-            if (cur.len & kLongBit) Lam = a.long_lam[cur.len & ~kLongBit];
-            Lam *= inv_D;
-        }
         // the next tile's first pairs are in flight during this tile's epilogue
         have = nxt.tile < ntiles && nxt.g == cur_g;
         if (have) {
@@ -620,7 +626,7 @@ __global__ void __launch_bounds__(256) k_bwd_finalize(const double *Q, const flo
 // most of an ordinary row in flight instead of three with two pairs a lane ahead.  A row sum
 // is a chain of round trips, so fewer and longer batches win wherever the fewer warps don't
 // cost more waves of tiles than that saves.  Us per day, three blocks against two: 1M town
-// 61.4 -> 58.5, twelve counties 29.2 -> 24.1, 300k power law 58.9 -> 50.2, deaths sampled at
+// 61.0 -> 58.9, twelve counties 29.2 -> 24.1, 300k power law 52.2 -> 37.1, deaths sampled at
 // 200k 24.1 -> 23.3 (at 1M, 4, 5 and 7 pairs: 62.4, 59.9, 61.5).  The instances with the
 // table's adjoint have other work between the loads: 15.5 -> 16.8 at 100k, so they stay.
 using BwdKernel = void (*)(BwdDayArgs);

@@ -1133,7 +1133,7 @@ gabm_status backward_days_plain(gabm_ctx *c, int T, cudaStream_t s) {
     a.seed = c->seed;
     a.c = c->c_dev;
     const int Lm1 = c->L - 1;
-    if (mode == kBwdFused || mode == kBwdSplit)   // every day's infectious rows, from the final state
+    if (mode == kBwdSplit || (mode == kBwdFused && c->long_cap))   // every day's infectious rows, from the final state
         LAUNCH(launch_infectious_bits(c->e, 0, T, c->L, c->ntiles, c->bits, (size_t)c->ntiles, s));
     a.s_hist_t = a.y_hist_t = nullptr;
     a.s_hist = c->s_hist;
@@ -1152,7 +1152,6 @@ gabm_status backward_days_plain(gabm_ctx *c, int T, cudaStream_t s) {
     if (c->fate)   // draw days 0..tau_EI-1 hold only the seeds' shares (k_fate_seeds)
         CK(cudaMemsetAsync(c->Pm, 0, sizeof(double) * (size_t)std::min(c->tau_EI, T) * c->ntiles, s));
     for (int t = T - 1; t >= 0; --t) {
-        a.bits_t = (mode == kBwdFused || mode == kBwdSplit) ? c->bits + (size_t)t * c->ntiles : nullptr;
         a.t = t;
         a.lam_t = (mode == kBwdStore || mode == kBwdSoft) ? c->lam + (size_t)t * c->n_rows
                                                           : (mode == kBwdSplit ? c->lam_tmp : nullptr);
@@ -1192,7 +1191,7 @@ gabm_status backward_days_plain(gabm_ctx *c, int T, cudaStream_t s) {
                 la.out.n = 0;
             }
             if (mode == kBwdFused) {
-                la.bits = a.bits_t;
+                la.bits = c->bits + (size_t)t * c->ntiles;
                 la.lam = long_lam_buf(c);
             } else {
                 la.in.n = 0;

@@ -248,7 +248,6 @@ struct BwdDayArgs {
     const uint8_t *age;
     GraphRef gr;
     const int16_t *E;          // final exposure days
-    const uint32_t *bits_t;    // [ntiles] rows infectious on day t (recompute policy) or nullptr
     const float *lam_t;        // stored normalised sums for day t (store policy) or nullptr
     const float *r_next;       // coefficients of day t+1 [n_rows]
     const float *long_gx, *long_lam;   // the long rows' gx(t+1), and (recompute policy) lambda sums of day t

@@ -510,6 +510,54 @@ __device__ __forceinline__ float exposed_sum(const Sell &m, uint32_t p0, uint32_
     return sum;
 }
 
+// gather_sum, and for the rows with `lam` the sum of w c[t - e_j] over the neighbours infectious on
+// day t (exposed_sum), in one pass over the entries: each pair is read once and its neighbours'
+// coefficients and exposure days are gathered together.  (Two passes, gather_sum and then the
+// marked neighbours by the day's bitmap: 110 us a day on the 1M-agent town against 91, 50 on the
+// 300k-agent power-law graph against 37; one pass that tests the bitmap before it gathers an
+// exposure day: 111 and 52.)
+template <int GP>
+__device__ __forceinline__ float gather_and_exposed_sum(const TileSpan &s, const float *x, bool lam, const int16_t *e,
+                                                        const float *c_s, int t, int L, uint4 (&ea)[GP],
+                                                        float &lam_sum) {
+    float sum = 0.f, comp = 0.f, ls = 0.f, lc = 0.f;
+    auto use = [&](uint32_t q0, const uint4 (&v)[GP]) {
+        float g[2 * GP];
+        int ej[2 * GP];
+#pragma unroll
+        for (int u = 0; u < GP; ++u) {
+            const uint32_t k = 2u * (q0 + (uint32_t)u);
+            g[2 * u] = k < s.len ? x[v[u].x] : 0.f;
+            g[2 * u + 1] = k + 1u < s.len ? x[v[u].z] : 0.f;
+            ej[2 * u] = lam && k < s.len ? (int)e[v[u].x] : kNever;
+            ej[2 * u + 1] = lam && k + 1u < s.len ? (int)e[v[u].z] : kNever;
+        }
+#pragma unroll
+        for (int i = 0; i < 2 * GP; ++i) {
+            const float w = __uint_as_float((i & 1) ? v[i >> 1].w : v[i >> 1].y);
+            const float y = (2u * q0 + (uint32_t)i < s.len) ? __fsub_rn(w * g[i], comp) : 0.f;
+            const float tt = __fadd_rn(sum, y);
+            comp = __fsub_rn(__fsub_rn(tt, sum), y);
+            sum = tt;
+            const int k = t - ej[i];
+            const bool tk = (unsigned)(k - 1) < (unsigned)(L - 1);
+            kahan_add_if(ls, lc, tk ? w * c_s[k] : 0.f, tk);
+        }
+    };
+    uint4 eb[GP];
+#pragma unroll
+    for (int u = 0; u < GP; ++u) eb[u] = make_uint4(0u, 0u, 0u, 0u);
+    for (uint32_t q = 0; q < s.np; q += 2 * GP) {
+        if (q + GP < s.np) load_pairs(s.row, q + GP, s.lim, eb);
+        use(q, ea);
+        if (q + GP >= s.np) break;
+        if (q + 2 * GP < s.np) load_pairs(s.row, q + 2 * GP, s.lim, ea);
+        use(q + GP, eb);
+    }
+    lam_sum = ls;
+    return sum;
+}
+
 // Tiles with at most this many summing rows have them summed one row at a time by the
 // whole warp (warp_row_sum) instead of lane by lane over the tile's longest row.
 #ifndef GABM_COOP_ROWS
