@@ -1392,19 +1392,27 @@ gabm_status backward_core(gabm_ctx *c, int T) {
 // row in flight.  Rows of a few entries have nothing to put in flight (agents' locations at
 // 300k: 17.7 us a day, deep 19.4; 200k random pairs, 3 a row: 391 us a sweep, 451).  Fewer warps
 // must not double the waves of tiles (100k random, 8 a row: 349 us a sweep, 381; 200k: 544,
-// 533; 300k, 20 a row: 1204, 1121).  And where most entries lie beyond the reach of the SM's
-// L1, warps hide its misses better from some size on (400k random, 8 a row: 912, 948; 600k:
-// 1235, 1319); with most entries near, as in towns, the deep instances stay ahead up to 1M
-// (us a sweep at 200k and 1M, three blocks against two: 1105 and 3522, 952 and 3426; drawn
-// durations 1307 and 4360, 1197 and 4333), but for the sampled deaths (1217 and 4190, 1143
-// and 4286), whose draw keeps more registers.
+// 533; 300k, 20 a row: 1204, 1121).  From some size on more warps hide the misses of the SM's L1
+// better, the later the more entries lie within its reach and the more a row has to load.
+// Us a day with three blocks and with two:
+//   towns (most entries near)      1M 61.0, 58.9; 1.5M 92.4, 94.6; 2M 120, 124; 4M 224, 236; 32
+//                                  counties of 12M in all 533, 567
+//   towns, drawn durations         300k 33.5, 30.1; 1M 75.0, 74.7; 2M 142, 146
+//   towns, sampled deaths          300k 31.4, 28.6; 1M 71.7, 73.2 (the draw keeps more registers)
+//   towns, lambda recomputed       100k 21.1, 20.2; 1M 107, 91; 4M 388, 343; power law 8M 774, 672
+//   random                         400k, 8 a row: 912, 948 us a sweep; 600k: 1235, 1319
+//   random, lambda recomputed      400k, 8 a row: 34.1, 31.8; 1M, 12: 89.6, 85.1; 3M, 16: 309, 318
 bool deep_gather(const gabm_ctx *c, int mode) {
     if (c->mean_len < 8.0) return false;
     const auto waves = [&](bool deep) {
         const int warps = c->num_sms * occupancy_bwd(mode, false, kExitBase, deep) * (kBlock / 32);
         return (c->ntiles + warps - 1) / warps;
     };
-    return waves(true) < 2 * waves(false) && ((c->near_share >= 0.5 && !c->fate) || c->ntiles <= kDeepTiles * c->num_sms);
+    if (waves(true) >= 2 * waves(false)) return false;
+    const bool near = c->near_share >= 0.5;
+    if (mode == kBwdFused && near) return true;
+    const int tiles = (mode == kBwdFused || near) && !c->fate ? kDeepNearTiles : kDeepTiles;
+    return c->ntiles <= (int64_t)tiles * c->num_sms;
 }
 
 // Grid sizes for the current schedule (resident blocks per SM x SMs, at most one warp per tile).

@@ -527,7 +527,7 @@ cudaError_t launch_mse(const double *D, int ldP, const double *y, int T, int I, 
 cudaError_t launch_bwd_day(const BwdDayArgs &a, int grid, bool small, bool deep, bool overlap, cudaStream_t s);
 constexpr int kSmallBlock = 64;   // threads of those blocks; eight an SM at 128 registers
 constexpr int kSmallTiles = 16;
-constexpr int kDeepTiles = 64;    // tiles an SM (deep_gather)
+constexpr int kDeepTiles = 64, kDeepNearTiles = 256;   // tiles an SM (deep_gather)
 constexpr int kNearRows = 1024;
 constexpr int kDeepPairs = 6;     // pairs of entries a lane ahead of use, reverse sweep (bwd_kernel)
 // Adjoint of the infectiousness table (hard mode, one set per graph): the seeds'
