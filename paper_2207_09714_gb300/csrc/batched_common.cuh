@@ -317,10 +317,6 @@ template <int SPL>
 struct EWords {
     uint32_t w[SPL / 2];
 };
-template <int SPL>
-struct FVec {
-    float v[SPL];
-};
 
 template <class K>
 int blocks_of(K kernel) {

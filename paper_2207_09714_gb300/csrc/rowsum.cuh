@@ -288,12 +288,6 @@ __device__ __forceinline__ uint32_t ld_if(const uint32_t *p, bool pred) {
     asm("{ .reg .pred q; setp.ne.u32 q, %2, 0; @q ld.global.u32 %0, [%1]; }" : "+r"(v) : "l"(p), "r"((uint32_t)pred));
     return v;
 }
-__device__ __forceinline__ float2 ld_if(const float2 *p, bool pred) {
-    float2 v = make_float2(0.f, 0.f);
-    asm("{ .reg .pred q; setp.ne.u32 q, %3, 0; @q ld.global.v2.f32 {%0, %1}, [%2]; }"
-        : "+f"(v.x), "+f"(v.y) : "l"(p), "r"((uint32_t)pred));
-    return v;
-}
 __device__ __forceinline__ int ld_if(const int16_t *p, bool pred, int dflt) {
     int v = dflt;
     asm("{ .reg .pred q; setp.ne.u32 q, %2, 0; @q ld.global.s16 %0, [%1]; }" : "+r"(v) : "l"(p), "r"((uint32_t)pred));
@@ -559,7 +553,7 @@ __device__ __forceinline__ float gather_and_exposed_sum(const TileSpan &s, const
 }
 
 // Tiles with at most this many summing rows have them summed one row at a time by the
-// whole warp (warp_row_sum) instead of lane by lane over the tile's longest row.
+// whole warp (few_row_sums) instead of lane by lane over the tile's longest row.
 #ifndef GABM_COOP_ROWS
 #define GABM_COOP_ROWS 4
 #endif
