@@ -198,16 +198,22 @@ def frontier_counts(pop, E, T, L):
     return sf_rows, sf_nnz, push
 
 
-def trajectory_bytes(E, deg, T, L, n_rows, policy_store, frontier=None):
+def trajectory_bytes(E, deg, T, L, n_rows, policy_store, frontier=None, last=None):
     """Algorithmic (compulsory) HBM bytes of every forward and backward day launch, from
     the final exposure days E (which determine each day's state).  With ``frontier`` (from
     frontier_counts) the forward reads only the entries of susceptible rows with an
     infectious in-neighbour, plus every row's state, flag and length and the pushes of
-    tomorrow's flags; without it, every susceptible row's entries."""
+    tomorrow's flags; without it, every susceptible row's entries.  With ``last``, the last
+    day whose exposures still count in the loss (last_counting_day), the reverse days are
+    counted as the day kernels run them: the coefficients of the days after it are 0, so
+    nothing is gathered from those days and their ring slots are neither written nor read,
+    and a tile's partial sums are fp32 (36 bytes); without it every later day is charged,
+    and 72 bytes a tile."""
     E = E.astype(np.int64)
     NEVER = 32767
     seed = (E != NEVER) & (E < 0)
     live = ~seed
+    end = T if last is None else min(T, last + 1)      # days from here on carry no adjoint back
     never = E == NEVER
     Ec = np.where(never, T, E)          # never infected counts as susceptible every day
     Ec = np.where(seed, -1, Ec)
@@ -236,31 +242,40 @@ def trajectory_bytes(E, deg, T, L, n_rows, policy_store, frontier=None):
     bwd = np.zeros(T)
     for t in range(T):
         nS, eS = S_cnt[t], S_nnz[t]
-        # the last reverse day has no gx(t+1) to gather
-        nA, eA = ge(max(t + 2 - L, 0)) if t + 1 < T else (0, 0.0)
-        ring_reads = max(0, min(L - 1, T - 1 - t) - 1)      # slots k = 2..L-1 inside the horizon
+        # no gx(t+1) to gather where day t + 1 carries nothing back
+        nA, eA = ge(max(t + 2 - L, 0)) if t + 1 < end else (0, 0.0)
+        ring_reads = max(0, min(L - 1, end - 1 - t) - 1)    # slots k = 2..L-1 of the days before `end`
         # entries (col + w) of the gathering rows; state and row length of every row; age
         # of the susceptible rows
         b = 8.0 * eA + 6.0 * n_rows + 1.0 * nS
-        b += 4.0 * ring_reads * nS + (4.0 * nA if t + 1 < T else 0.0)   # ring reads and write
+        b += 4.0 * ring_reads * nS + 4.0 * nA                        # ring reads and write
         # A read by the susceptible rows exposed later (not today, not never), written by
         # today's exposures; r written by every susceptible row
         b += 4.0 * (nS - n_never - new[t]) + 4.0 * new[t] + 4.0 * nS
         if policy_store:
             b += 4.0 * nS
-        b += 72.0 * (n_rows // 32)                                   # per-tile partial sums
+        b += (72.0 if last is None else 36.0) * (n_rows // 32)       # per-tile partial sums
         bwd[t] = b
     return fwd, bwd, S_cnt, S_nnz
 
 
-def batched_trajectory_bytes(E, deg, T, L, n, B, l2_bytes):
+def last_counting_day(T, to_death):
+    """The last day of T whose exposures can still enter the loss: those die (or recover, in
+    expectation) `to_death` days later at the earliest, and what an exposure does to later ones
+    counts only through theirs."""
+    return T - 1 - to_death
+
+
+def batched_trajectory_bytes(E, deg, T, L, n, B, l2_bytes, last=None):
     """Algorithmic HBM bytes of the batched day launches (B sets sharing one graph) from the
     final exposure days E [B, n] of every set: rows are read once for all sets, per-set
     state once per set.  The backward's coefficient gather costs nothing per edge when
     the array fits in half of L2, else its B values per edge (every entry of a row that
     needs the transpose gather reads them).  The forward's exposure-day gathers are not
     charged: they are made for the marked neighbours only (infectious in some set), a
-    data-dependent share of the entries, and their DRAM cost is what ncu measures."""
+    data-dependent share of the entries, and their DRAM cost is what ncu measures.  ``last``
+    as in trajectory_bytes."""
+    end = T if last is None else min(T, last + 1)
     E = E.astype(np.int64)
     NEVER = 32767
     seed = (E != NEVER) & (E < 0)
@@ -282,10 +297,10 @@ def batched_trajectory_bytes(E, deg, T, L, n, B, l2_bytes):
     for t in range(T):
         fwd[t] = (8.0 * nnz_t[t] + 8.0 * rows_t[t] + 2.0 * n * B + n + 2.0 * new[t] + 4.0 * S_t[t]
                   + gath_f * nnz_t[t])
-        ring_reads = max(0, min(L - 1, T - 1 - t) - 1)
+        ring_reads = max(0, min(L - 1, end - 1 - t) - 1)
         thr = min(T, max(t + 2 - L, 0))
         b = 4.0 * S_t[t] + 2.0 * n * B + n + S_t[t] * (4.0 * ring_reads + 4.0 + 4.0)
-        if t + 1 < T:
+        if t + 1 < end:
             b += 8.0 * nnz_t[thr] + 8.0 * rows_t[thr] + 4.0 * n * B + gath_b * nnz_t[thr]
         bwd[t] = b
     return fwd, bwd
@@ -352,7 +367,8 @@ def bench_batched(args, stream, peak, peak_kind):
     capi.gabm_set_profiling(ctx, False)
     E = capi.gabm_get_state(ctx)
     l2 = torch.cuda.get_device_properties(0).L2_cache_size
-    fwd_b, bwd_b = batched_trajectory_bytes(E, pop.degrees().astype(np.float64), T, TAU_EI + TAU_IR, pop.n, B, l2)
+    fwd_b, bwd_b = batched_trajectory_bytes(E, pop.degrees().astype(np.float64), T, TAU_EI + TAU_IR, pop.n, B, l2,
+                                            last_counting_day(T, TAU_EI + TAU_IR))
     f_gbs = fwd_b.sum() / (f_ms / 1e3) / 1e9
     b_gbs = bwd_b.sum() / (b_ms / 1e3) / 1e9
     both_gbs = (fwd_b.sum() + bwd_b.sum()) / ((f_ms + b_ms) / 1e3) / 1e9
@@ -558,12 +574,12 @@ def bench_progression_variant(pop, stream, S, y_np, dist, peak, peak_kind, varia
     from paper_2207_09714_gb300 import capi, synth
 
     if variant == "rm_split":
-        L = TAU_EI + max(TAU_IR, TAU_IM)
+        L, to_death = TAU_EI + max(TAU_IR, TAU_IM), TAU_EI + TAU_IM
         md = capi.ModelDesc(TAU_EI, TAU_IR, synth.infectiousness_table(TAU_EI, max(TAU_IR, TAU_IM)), seed=0,
                             tau_IM=TAU_IM)
         what = f"sampled R/M split: tau_EI {TAU_EI}, tau_IR {TAU_IR}, tau_IM {TAU_IM}"
     elif variant == "durations":
-        L = TAU_EI + P_IR.size
+        L, to_death = TAU_EI + P_IR.size, TAU_EI + 1
         md = capi.ModelDesc(TAU_EI, P_IR.size, synth.infectiousness_table(TAU_EI, P_IR.size), seed=0, p_IR=P_IR)
         what = f"stochastic I-stage durations: tau_EI {TAU_EI}, I days ~ pmf {P_IR.round(2).tolist()} over 1..{P_IR.size}"
     else:
@@ -613,7 +629,8 @@ def bench_progression_variant(pop, stream, S, y_np, dist, peak, peak_kind, varia
         return out
     n_rows = ((pop.n + 31) // 32) * 32
     fwd_b, bwd_b, _, _ = trajectory_bytes(E, pop.degrees().astype(np.float64), DAYS, L, n_rows, True,
-                                          frontier=frontier_counts(pop, E, DAYS, L))
+                                          frontier=frontier_counts(pop, E, DAYS, L),
+                                          last=last_counting_day(DAYS, to_death))
     f_gbs = fwd_b.sum() * steps / (f_ms / 1e3) / 1e9
     b_gbs = bwd_b.sum() * steps / (b_ms / 1e3) / 1e9
     return {"workload": f"{what}, on the bench graph, m = {MORTALITY}, {DAYS} days, forward + MSE + backward",
@@ -739,11 +756,12 @@ def workload_bytes(pops, E, B, T, L, store, l2_bytes):
         off = np.concatenate([[0], np.cumsum([p.n for p in pops])])
         parts = [frontier_counts(p, E[0][off[g]:off[g + 1]], T, L) for g, p in enumerate(pops)]
         frontier = tuple(sum(pt[k] for pt in parts) for k in range(3))
-        fwd, bwd, _, _ = trajectory_bytes(E[0], deg, T, L, n_rows, store, frontier=frontier)
+        fwd, bwd, _, _ = trajectory_bytes(E[0], deg, T, L, n_rows, store, frontier=frontier,
+                                          last=last_counting_day(T, L))
         ffwd, fbwd, _, _ = trajectory_bytes(np.full(deg.size, NEVER, np.int16), deg, T, L, n_rows, store)
     else:
         n = pops[0].n
-        fwd, bwd = batched_trajectory_bytes(E, deg, T, L, n, B, l2_bytes)
+        fwd, bwd = batched_trajectory_bytes(E, deg, T, L, n, B, l2_bytes, last_counting_day(T, L))
         ffwd, fbwd = batched_trajectory_bytes(np.full((B, n), NEVER, np.int16), deg, T, L, n, B, l2_bytes)
     return fwd, bwd, ffwd, fbwd
 
@@ -1167,15 +1185,14 @@ def main():
     n_rows = ((pop.n + 31) // 32) * 32
     frontier = frontier_counts(pop, E, DAYS, TAU_EI + TAU_IR)
     fwd_b, bwd_b, S_cnt, S_nnz = trajectory_bytes(E, deg, DAYS, TAU_EI + TAU_IR, n_rows,
-                                                  policy == capi.GABM_STORE_LAMBDA, frontier=frontier)
+                                                  policy == capi.GABM_STORE_LAMBDA, frontier=frontier,
+                                                  last=last_counting_day(DAYS, TAU_EI + TAU_IR))
     fwd_gbs = fwd_b.sum() * args.steps / (fwd_ms_k / 1e3) / 1e9 if fwd_ms_k > 0 else None
     bwd_gbs = bwd_b.sum() * args.steps / (bwd_ms_k / 1e3) / 1e9 if bwd_ms_k > 0 else None
     peak, peak_kind = _peaks()
     dominant = "k_bwd_day" if bwd_ms_k >= fwd_ms_k else "k_fwd_day"
-    src = ["backward.cu", "rowsum.cuh", "gabm_internal.cuh"] if dominant == "k_bwd_day" else \
-          ["forward.cu", "rowsum.cuh", "gabm_internal.cuh"]
     workload_tag = f"typed1M_T{DAYS}_{args.policy}"
-    traffic = _ncu_traffic(dominant, _kernel_source_sha(src), workload_tag)
+    traffic = _ncu_traffic(dominant, _kernel_source_sha(_SRC[dominant]), workload_tag)
     fwd_dr = dram_rate("k_fwd_day", workload_tag, fwd_ms_k / fwd_n if fwd_n else 0.0, peak)
     bwd_dr = dram_rate("k_bwd_day", workload_tag, bwd_ms_k / bwd_n if bwd_n else 0.0, peak)
     dom_gbs = bwd_gbs if dominant == "k_bwd_day" else fwd_gbs
