@@ -221,7 +221,8 @@ gabm_status gabm_mse_loss(gabm_ctx *ctx, const double *y, double *loss, double *
  * and >= 0, as at creation) for the forwards that follow, e.g. between the steps of a
  * calibration that learns the stage factors or the profile behind c.  Takes effect on the
  * ctx stream, behind the work already there.  The last trajectory used the old table, so gabm_backward returns
- * GABM_ESTATE until the next gabm_forward.  GABM_EINVAL for a NULL or invalid table. */
+ * GABM_ESTATE until the next gabm_forward.  GABM_EINVAL for a NULL or invalid table,
+ * GABM_ECUDA while the ctx stream is being captured. */
 gabm_status gabm_set_infectiousness(gabm_ctx *ctx, const float *c);
 
 /* Straight-through adjoint of the last forward (App. B): given gD = dL/dD_t
