@@ -678,6 +678,7 @@ gabm_status ensure_days(gabm_ctx *c, int T) {
     c->Tcap = cap;
     c->T_last = -1;
     c->lam_from = -1;
+    c->gD_staged = false;
     c->buffer_generation++;
     return GABM_OK;
 }
@@ -2448,7 +2449,9 @@ gabm_status gabm_autotune(gabm_ctx *ctx, int repetitions) {
         return fail(c, GABM_ESTATE, "autotune needs a preceding forward that started from seeding");
     const int T = c->T_last, ld = c->Tcap;
     cudaStream_t s = c->stream;
-    if (!c->gD_staged) CK(cudaMemsetAsync(c->gD, 0, sizeof(double) * (size_t)c->I * ld, s));
+    // without a loss gradient yet, any that is not 0 (these bytes are 4.8e-4): days that carry no
+    // adjoint are skipped, and the backward schedules would be timed on nothing else
+    if (!c->gD_staged) CK(cudaMemsetAsync(c->gD, 0x3f, sizeof(double) * (size_t)c->I * ld, s));
     gabm_schedule cur{};
     TRY(gabm_get_schedule(c, &cur));
     // forward schedules (the backward schedule does not change the forward) ...
