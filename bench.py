@@ -379,10 +379,8 @@ def bench_batched(args, stream, peak, peak_kind):
     del ctx
     units = B * pop.n * T
     dom = "k_bwd_day_b" if b_ms >= f_ms else "k_fwd_day_b"
-    src = ["batched_bwd.cu" if dom == "k_bwd_day_b" else "batched.cu", "batched_common.cuh", "rowsum.cuh",
-           "gabm_internal.cuh"]
     wl = f"typed{pop.n // 1000}k_B{B}_T{T}_store"
-    traffic = _ncu_traffic(dom, _kernel_source_sha(src), wl)
+    traffic = _ncu_traffic(dom, _kernel_source_sha(_SRC[dom]), wl)
     f_dr = dram_rate("k_fwd_day_b", wl, f_ms / f_n, peak)
     b_dr = dram_rate("k_bwd_day_b", wl, b_ms / b_n, peak)
     result = {
