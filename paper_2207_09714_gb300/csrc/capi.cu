@@ -807,6 +807,7 @@ gabm_status long_gather(gabm_ctx *c, const float *x, const int32_t *rnz, int t, 
     if (!c->long_cap) return GABM_OK;
     LongArgs a = long_args(c, t);
     a.in.n = 0;
+    if (a.out.n == 0) return GABM_OK;
     a.gx_from = from;
     a.x = x;
     a.gx = long_gx_buf(c);
@@ -820,6 +821,7 @@ gabm_status long_lambda(gabm_ctx *c, const uint32_t *bits, uint8_t *flags, int t
     if (!c->long_cap) return GABM_OK;
     LongArgs a = long_args(c, t);
     if (!flags) a.out.n = 0;
+    if (a.in.n + a.out.n == 0) return GABM_OK;
     a.bits = bits;
     a.lam = long_lam_buf(c);
     a.flags = flags;
