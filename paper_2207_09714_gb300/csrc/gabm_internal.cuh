@@ -477,7 +477,9 @@ cudaError_t launch_day(void (*kernel)(P...), int grid, int block, size_t smem, c
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
     cfg.numAttrs = overlap ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+    if (e != cudaSuccess) (void)cudaGetLastError();   // reported here: not to the launch after it as well
+    return e;
 }
 
 // Launchers (forward.cu / backward.cu)
